@@ -227,6 +227,9 @@ int cc_graph_destroy(cc_graph* g) {
   dfree(g->nz_pos, s);
   dfree(g->dsort, s);
   dfree(g->dge, s);
+  dfree(g->up_row, s);
+  dfree(g->up_pos, s);
+  dfree(g->up_dlt, s);
   dfree(g->perm_ws, s);
   dfree(g->order, s);
   dfree(g->round_ws, s);
@@ -335,37 +338,54 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     if ((rc = from_cuda(dalloc(&g->nz_row, 4 * (size_t)(n > 0 ? n : 1), s))) != CC_OK) { dfree(vws, s); break; }
     if ((rc = from_cuda(dalloc(&g->nz_pos, 8 * (size_t)(n > 0 ? n : 1), s))) != CC_OK) { dfree(vws, s); break; }
     void* nws = nullptr;
+    int64_t* up_at = nullptr;
     if ((rc = from_cuda(dalloc(&nws, nonempty_workspace_bytes(n), s))) != CC_OK) { dfree(vws, s); break; }
+    if ((rc = from_cuda(dalloc(&up_at, 8 * (size_t)(n > 0 ? n : 1), s))) != CC_OK) {
+      dfree(vws, s); dfree(nws, s);
+      break;
+    }
     int64_t* nz_dev = reinterpret_cast<int64_t*>(static_cast<char*>(nws) + nonempty_workspace_bytes(n) - 256);
-    launch_nonempty_rows(n, g->off, g->nz_row, g->nz_pos, nws, nz_dev, g->num_sms, s);
+    launch_nonempty_rows(n, g->off, g->nz_row, g->nz_pos, up_at, nws, nz_dev, g->num_sms, s);
     cudaMemcpyAsync(&g->nz_n, nz_dev, 8, cudaMemcpyDeviceToHost, s);
-    if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) { dfree(vws, s); dfree(nws, s); break; }
-    // the non-isolated vertices by degree (for the round kernel's Delta)
+    if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }
+    // the non-isolated vertices by degree (for the round kernel's Delta) and
+    // the memory of the rows' upper parts (for the objective)
     {
+      const size_t nz = (size_t)(g->nz_n > 0 ? g->nz_n : 1);
       void* dws = nullptr;
-      if ((rc = from_cuda(dalloc(&g->dsort, 4 * (size_t)(g->nz_n > 0 ? g->nz_n : 1), s))) != CC_OK ||
+      if ((rc = from_cuda(dalloc(&g->dsort, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&g->dge, 8 * ((size_t)g->max_deg + 2), s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_row, 4 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_pos, 8 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_dlt, 8 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&dws, degree_order_workspace_bytes(g->max_deg), s))) != CC_OK) {
-        dfree(dws, s); dfree(vws, s); dfree(nws, s);
+        dfree(dws, s); dfree(vws, s); dfree(nws, s); dfree(up_at, s);
         break;
       }
       rc = from_cuda(launch_degree_order(g->nz_n, g->nz_row, g->off, g->max_deg, g->dsort, g->dge, dws, g->num_sms, s));
       dfree(dws, s);
-      if (rc != CC_OK) { dfree(vws, s); dfree(nws, s); break; }
+      if (rc != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }
     }
     for (int c = 0; c < chunks; ++c) {
       if (g->col_ready[c]) cudaStreamWaitEvent(s, g->col_ready[c], 0);
-      launch_validate_edges(n, cut[c], cut[c + 1], c == chunks - 1, g->nz_row, g->nz_pos, g->nz_n, g->col, vws,
+      launch_validate_edges(n, cut[c], cut[c + 1], c == chunks - 1, g->nz_row, g->nz_pos, g->nz_n, g->col, up_at, vws,
                             g->num_sms, s);
     }
+    unsigned long long* up_dev = reinterpret_cast<unsigned long long*>(nz_dev);
+    unsigned long long up_pack = 0;
+    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_row, g->up_pos, g->up_dlt, nws, up_dev,
+                      g->num_sms, s);
+    cudaMemcpyAsync(&up_pack, up_dev, 8, cudaMemcpyDeviceToHost, s);
     if (flags & CC_VALIDATE_EXACT)
       launch_validate_reverse(nnz, g->off, g->nz_row, g->nz_pos, g->nz_n, g->col, vws, g->num_sms, s);
     cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s);
     dfree(vws, s);
     dfree(nws, s);
+    dfree(up_at, s);
     if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) break;
     if ((rc = from_cuda(cudaGetLastError())) != CC_OK) break;
     if (vflags[0] != 0) { rc = CC_ERR_INVALID_GRAPH; break; }
+    g->up_n = (int64_t)(up_pack >> 33);
   } while (false);
   // the copy stream and its events are no longer needed (every chunk is
   // ordered before the work on s, or the graph is being thrown away)
@@ -443,8 +463,7 @@ static int cluster_async(cc_graph* g, uint64_t seed, int32_t* labels_out, int32_
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[1], s));
   CC_TRY(launch_async_c4(b, g->async_grid, lab, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[2], s));
-  CC_TRY(launch_disagreements(g->n, g->nnz, g->off, g->col, g->nz_row, g->nz_pos, g->nz_n, lab, g->obj_ws,
-                              g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->nnz, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   if (labels_out && !dev) CC_TRY(cudaMemcpyAsync(labels_out, lab, 4 * (size_t)g->n, cudaMemcpyDeviceToHost, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[3], s));
   CC_TRY(cudaMemcpyAsync(g->ctl_host, b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -475,7 +494,7 @@ static int cluster_async(cc_graph* g, uint64_t seed, int32_t* labels_out, int32_
   }
   if (stats_len) *stats_len = 1;
   if (rounds_out) *rounds_out = 0;
-  if (disagreements_out) *disagreements_out = g->nnz / 2 - (int64_t)g->obj_host[0] + (int64_t)g->obj_host[1];
+  if (disagreements_out) *disagreements_out = g->nnz / 2 - 2 * (int64_t)g->obj_host[0] + (int64_t)g->obj_host[1];
   return CC_OK;
 }
 
@@ -623,12 +642,11 @@ int cc_disagreements(cc_graph* g, const int32_t* labels, int64_t* out) {
     CC_TRY(cudaMemcpyAsync(g->labels_tmp, labels, 4 * (size_t)g->n, cudaMemcpyHostToDevice, s));
     lab = g->labels_tmp;
   }
-  CC_TRY(launch_disagreements(g->n, g->nnz, g->off, g->col, g->nz_row, g->nz_pos, g->nz_n, lab, g->obj_ws,
-                              g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->nnz, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   CC_TRY(cudaMemcpyAsync(g->obj_host, g->obj_out, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   CC_TRY(cudaStreamSynchronize(s));
   if (g->obj_host[2]) return CC_ERR_INVALID_ARG;
-  *out = g->nnz / 2 - (int64_t)g->obj_host[0] + (int64_t)g->obj_host[1];
+  *out = g->nnz / 2 - 2 * (int64_t)g->obj_host[0] + (int64_t)g->obj_host[1];
   return CC_OK;
 }
 

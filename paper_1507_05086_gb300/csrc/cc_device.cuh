@@ -176,6 +176,19 @@ __device__ __forceinline__ T block_max(T x, T* scratch) {
 }
 
 // ---------------------------------------------------------------------------
+// 4-bit signatures of cluster ids (objective): equal ids have equal ones.
+// pack_sig8: the eight signatures of lanes 8 i .. 8 i + 7 in one word (valid
+// in the first of the eight lanes).  All lanes must call it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_sig(uint32_t id) { return (id * 0x9E3779B1u) >> 28; }
+__device__ __forceinline__ uint32_t pack_sig8(uint32_t sig) {
+  uint32_t x = sig << ((threadIdx.x & 7) * 4);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x |= __shfl_xor_sync(FULL, x, o);
+  return x;
+}
+
+// ---------------------------------------------------------------------------
 // Edge-balanced walk over a list of adjacency rows.
 //
 // Item j of the list owns the virtual edges [epos[j], epos[j+1]) (epos[j] is

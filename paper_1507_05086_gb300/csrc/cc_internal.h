@@ -92,6 +92,16 @@ Tuning default_tuning();
 // classes and the round-kernel settings of their jobs.
 Tuning batch_settings(int64_t* small_n, int64_t* team_n, int* team_blocks);
 
+// The upper part of every row (columns above the row's vertex), which holds
+// each edge once: rows with a non-empty upper part, with their first virtual
+// edge and CSR delta (RowList in cc_device.cuh).  The objective walks it.
+struct UpperRows {
+  const int32_t* row;
+  const int64_t* pos;
+  const int64_t* dlt;
+  int64_t n;
+};
+
 struct RoundBuffers {
   int64_t n, nnz;
   int32_t max_deg;
@@ -184,12 +194,18 @@ cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, c
 
 // ---- objective and validation (cc_objective.cu) ------------------------------
 size_t objective_workspace_bytes(int64_t n);
-// out[0] = intra-cluster CSR entries, out[1] = sum_c C(s_c, 2), out[2] = 1 if a
+// out[0] = edges inside clusters, out[1] = sum_c C(s_c, 2), out[2] = 1 if a
 // label was outside [0, n).  out: 3 device words.
-cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int64_t* off, const int32_t* col,
-                                 const int32_t* nz_row, const int64_t* nz_pos, int64_t nz_n,
+cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int32_t* col, const UpperRows& up,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream);
+// *out += the number of edges (u, w) with id[u] == id[w]; `sig` (or null): a
+// 4-bit signature of id per vertex, eight to a word, that is equal when the
+// ids are.
+cudaError_t launch_intra(int64_t edges, const int32_t* col, const UpperRows& up, const uint32_t* id,
+                         const uint32_t* sig, unsigned long long* out, int num_sms, cudaStream_t stream);
+// Vertices above which the objective reads signatures before ids.
+bool intra_wants_signatures(int64_t n);
 size_t validate_workspace_bytes();
 // Validation in two steps sharing ws (validate_workspace_bytes()): offsets
 // first (zeroes ws), then the entries over the non-empty rows.  The int pair
@@ -198,9 +214,10 @@ cudaError_t launch_validate_offsets(int64_t n, int64_t nnz, const int64_t* off, 
                                     cudaStream_t stream);
 // Entries [e0, e1) of the CSR; `last` adds the symmetry verdict over every
 // range validated since launch_validate_offsets cleared the workspace.
+// Also writes up_at[j], the first entry of non-empty row j above its vertex.
 cudaError_t launch_validate_edges(int64_t n, int64_t e0, int64_t e1, bool last, const int32_t* nz_row,
-                                  const int64_t* nz_pos, int64_t nz_n, const int32_t* col, void* ws, int num_sms,
-                                  cudaStream_t stream);
+                                  const int64_t* nz_pos, int64_t nz_n, const int32_t* col, int64_t* up_at, void* ws,
+                                  int num_sms, cudaStream_t stream);
 // Exact symmetry check (CC_VALIDATE_EXACT): reverse-entry search for every
 // lower entry; shares ws (and its error word) with the validation above.
 cudaError_t launch_validate_reverse(int64_t nnz, const int64_t* off, const int32_t* nz_row, const int64_t* nz_pos,
@@ -213,7 +230,15 @@ size_t degree_order_workspace_bytes(int32_t max_deg);
 cudaError_t launch_degree_order(int64_t nz_n, const int32_t* nz_row, const int64_t* off, int32_t max_deg,
                                 int32_t* dsort, int64_t* dge, void* ws, int num_sms, cudaStream_t stream);
 size_t nonempty_workspace_bytes(int64_t n);
-cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, void* ws,
-                                 int64_t* count_dev, int num_sms, cudaStream_t stream);
+// up_at (int64[n]): per non-empty row its end, the start of its upper part
+// while no column above the row's vertex has been seen (launch_validate_edges
+// writes the starts).
+cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, int64_t* up_at,
+                                 void* ws, int64_t* count_dev, int num_sms, cudaStream_t stream);
+// The rows of UpperRows from up_at; *count_dev = their number << kPackShift |
+// their edges.  ws: nonempty_workspace_bytes(nz_n).
+cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
+                              const int64_t* up_at, int32_t* row, int64_t* pos, int64_t* dlt, void* ws,
+                              unsigned long long* count_dev, int num_sms, cudaStream_t stream);
 
 }  // namespace ccg

@@ -3,10 +3,10 @@
 //
 // Disagreements: with m positive edges, intra = positive edges inside a
 // cluster and s_c the cluster sizes,
-//     D = (m - intra) + (sum_c C(s_c, 2) - intra) = m - intra_dir + sum_c C(s_c, 2)
-// where intra_dir = 2 * intra counts CSR entries (u, w) with label[u] == label[w].
-// One pass counts cluster sizes, one edge-balanced pass over the non-empty
-// rows counts intra_dir, one pass sums C(s_c, 2).
+//     D = (m - intra) + (sum_c C(s_c, 2) - intra) = m - 2 intra + sum_c C(s_c, 2).
+// One pass over the vertices adds up the sizes and the pairs, one
+// edge-balanced pass over the upper parts of the rows (every edge once)
+// counts intra.
 #include <cstdint>
 
 #include "cc_device.cuh"
@@ -16,48 +16,83 @@ namespace ccg {
 namespace {
 
 constexpr int kObjThreads = 512;
+// Graphs above this many vertices read 4-bit signatures before ids: up to it
+// the ids (64 MB) fit the 129 MB L2 themselves.
+constexpr int64_t kSigMin = int64_t(1) << 24;
 
-__global__ void k_cluster_sizes(int64_t n, const int32_t* __restrict__ labels, int32_t* __restrict__ size,
-                                unsigned long long* out) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c = labels[v];
-    if (c < 0 || c >= n) { atomicExch(out + 2, 1ull); continue; }
-    atomicAdd(size + c, 1);
+// sum_c C(s_c, 2) = sum over the vertices of the number of members that their
+// cluster had before them, so the add that counts a member also gives its
+// pairs (no second pass over the sizes).  Lanes of a warp with the same label
+// share one add: the adds of a cluster queue on one word, which bound the
+// whole call on a planted partition (2M vertices, the largest cluster 0.77M
+// members: 915 us with one add per vertex and both ends of every edge read,
+// 310 us so).
+__global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int32_t* __restrict__ size,
+                              unsigned long long* out) {
+  __shared__ int64_t scr[33];
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t pairs = 0;
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; b < n; b += stride) {
+    const int64_t v = b + lane;
+    int32_t c = v < n ? __ldg(labels + v) : -1;
+    if (v < n && (c < 0 || c >= n)) { atomicExch(out + 2, 1ull); c = -1; }
+    const unsigned same = __match_any_sync(FULL, c);
+    if (c < 0 || lane != __ffs(same) - 1) continue;
+    const int64_t k = __popc(same);
+    const int64_t old = atomicAdd(size + c, (int32_t)k);
+    pairs += k * old + k * (k - 1) / 2;
   }
+  pairs = block_sum<int64_t>(pairs, scr);
+  if (threadIdx.x == 0 && pairs) atomicAdd(out + 1, (unsigned long long)pairs);
 }
 
-__global__ void __launch_bounds__(kObjThreads) k_intra(int64_t nz_n, const int32_t* __restrict__ nz_row,
-                                                      const int64_t* __restrict__ nz_pos, int64_t nnz,
-                                                      const int32_t* __restrict__ col,
-                                                      const int32_t* __restrict__ labels, unsigned long long* out) {
+// Edges (u, w) with id[u] == id[w], every edge read from its lower end only
+// (half of the CSR's entries).  Bound by the latency of the chain row data ->
+// column -> id.  With sig, a 4-bit signature per vertex decides first, so that
+// ids are read only where the signatures agree.  Objective of a ClusterWild!
+// labelling, both ends of every edge -> this: R-MAT 22 0.59 -> 0.40 ms, R-MAT
+// 24 2.43 -> 1.52 ms, R-MAT 26 12.5 -> 7.6 ms.
+template <bool kSig>
+__global__ void __launch_bounds__(kObjThreads) k_intra(int64_t edges, UpperRows up, const int32_t* __restrict__ col,
+                                                      const uint32_t* __restrict__ id,
+                                                      const uint32_t* __restrict__ sig, unsigned long long* out) {
   __shared__ LbsWarp lbs[kObjThreads / 32];
   __shared__ int64_t scr[33];
   int64_t cnt = 0;
-  // the non-empty rows are contiguous in the CSR, so virtual edge e is CSR entry e
-  lbs_for_each(nz_pos, nz_n, nnz, &lbs[threadIdx.x >> 5], [&](const Lbs& L) {
-    int32_t lu[kLbsK], w[kLbsK];
+  lbs_for_each_in((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, ((int64_t)gridDim.x * blockDim.x) >> 5,
+                  up.pos, up.n, edges, &lbs[threadIdx.x >> 5], [&](const Lbs& L) {
+    int32_t w[kLbsK];
 #pragma unroll
-    for (int t = 0; t < kLbsK; ++t) {
-      lu[t] = L.ok(t) ? __ldg(labels + __ldg(nz_row + L.item(t))) : 0;
-      w[t] = L.ok(t) ? __ldg(col + L.edge(t)) : 0;
+    for (int t = 0; t < kLbsK; ++t) w[t] = L.ok(t) ? __ldg(col + L.csr(t)) : 0;
+    uint32_t x[kLbsK];
+    if (kSig) {
+#pragma unroll
+      for (int t = 0; t < kLbsK; ++t) x[t] = __ldg(sig + (w[t] >> 3)) >> ((w[t] & 7) * 4);
+#pragma unroll
+      for (int t = 0; t < kLbsK; ++t)
+        if (L.ok(t) && ((x[t] ^ cluster_sig((uint32_t)L.vtx(t))) & 15u) == 0)
+          cnt += __ldg(id + w[t]) == (uint32_t)L.vtx(t) ? 1 : 0;
+    } else {
+#pragma unroll
+      for (int t = 0; t < kLbsK; ++t) x[t] = __ldg(id + w[t]);
+#pragma unroll
+      for (int t = 0; t < kLbsK; ++t) cnt += L.ok(t) && x[t] == (uint32_t)L.vtx(t) ? 1 : 0;
     }
-#pragma unroll
-    for (int t = 0; t < kLbsK; ++t)
-      if (L.ok(t)) cnt += (__ldg(labels + w[t]) == lu[t]) ? 1 : 0;
-  }, nullptr, nullptr, 0, col);
+  }, up.dlt, up.row, 0, id, 0, col);
   cnt = block_sum<int64_t>(cnt, scr);
-  if (threadIdx.x == 0 && cnt) atomicAdd(out + 0, (unsigned long long)cnt);
+  if (threadIdx.x == 0 && cnt) atomicAdd(out, (unsigned long long)cnt);
 }
 
-__global__ void k_pairs(int64_t n, const int32_t* __restrict__ size, unsigned long long* out) {
-  __shared__ int64_t scr[33];
-  int64_t acc = 0;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = size[c];
-    acc += s * (s - 1) / 2;
+// sig word i: the signatures of the ids of vertices 8 i .. 8 i + 7.
+__global__ void k_signatures(int64_t n, const uint32_t* __restrict__ id, uint32_t* __restrict__ sig) {
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; b < n; b += stride) {
+    const int64_t v = b + lane;
+    const uint32_t s = pack_sig8(v < n ? cluster_sig(__ldg(id + v)) : 0u);
+    if (v < n && (lane & 7) == 0) sig[v >> 3] = s;
   }
-  acc = block_sum<int64_t>(acc, scr);
-  if (threadIdx.x == 0 && acc) atomicAdd(out + 1, (unsigned long long)acc);
 }
 
 // ---- validation ---------------------------------------------------------------
@@ -91,7 +126,8 @@ constexpr int kValThreads = 512;
 __global__ void __launch_bounds__(kValThreads) k_validate_edges(int64_t n, int64_t e0, int64_t e1, int64_t nz_n,
                                                                const int32_t* __restrict__ nz_row,
                                                                const int64_t* __restrict__ nz_pos,
-                                                               const int32_t* __restrict__ col, int* flags,
+                                                               const int32_t* __restrict__ col,
+                                                               int64_t* __restrict__ up_at, int* flags,
                                                                unsigned long long* sums) {
   __shared__ LbsWarp lbs[kValThreads / 32];
   unsigned long long lo1 = 0, lo2 = 0, up1 = 0, up2 = 0;
@@ -106,7 +142,9 @@ __global__ void __launch_bounds__(kValThreads) k_validate_edges(int64_t n, int64
       const int32_t w = __ldg(col + e);
       if (w < 0 || w >= n) { bad = bad ? bad : kBadColumn; continue; }
       if (w == u) { bad = bad ? bad : kSelfLoop; continue; }
-      if (L.in_row(t) > 0 && __ldg(col + e - 1) >= w) bad = bad ? bad : kUnsorted;
+      const int32_t prev = L.in_row(t) > 0 ? __ldg(col + e - 1) : -1;
+      if (prev >= w) bad = bad ? bad : kUnsorted;
+      if (w > u && prev < u) up_at[L.item(t)] = e;      // the row's upper part starts here
       const uint64_t key = u < w ? (((uint64_t)u << 32) | (uint32_t)w) : (((uint64_t)w << 32) | (uint32_t)u);
       const uint64_t h1 = mix64(key ^ 0x9E3779B97F4A7C15ull), h2 = mix64(key + 0x632BE59BD9B4E019ull);
       if (u < w) { lo1 += h1; lo2 += h2; ++nlo; } else { up1 += h1; up2 += h2; ++nup; }
@@ -195,7 +233,7 @@ __global__ void k_nz_scan(int64_t ntiles, int64_t* __restrict__ tile_cnt, int64_
 }
 
 __global__ void k_nz_write(int64_t n, const int64_t* __restrict__ off, const int64_t* __restrict__ tile_off,
-                           int32_t* __restrict__ nz_row, int64_t* __restrict__ nz_pos) {
+                           int32_t* __restrict__ nz_row, int64_t* __restrict__ nz_pos, int64_t* __restrict__ up_at) {
   __shared__ int64_t scr[33];
   const int64_t ntiles = (n + kNzTile - 1) / kNzTile;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -206,6 +244,46 @@ __global__ void k_nz_write(int64_t n, const int64_t* __restrict__ off, const int
     if (c) {
       nz_row[tile_off[t] + ex] = (int32_t)v;
       nz_pos[tile_off[t] + ex] = off[v];
+      up_at[tile_off[t] + ex] = off[v + 1];
+    }
+  }
+}
+
+// Rows with a non-empty upper part, by the same three steps; counts are
+// packed (rows << kPackShift | edges).
+__device__ __forceinline__ int64_t upper_len(int64_t j, int64_t nz_n, int64_t nnz, const int64_t* nz_pos,
+                                             const int64_t* up_at) {
+  return j < nz_n ? (j + 1 < nz_n ? nz_pos[j + 1] : nnz) - up_at[j] : 0;
+}
+
+__global__ void k_up_count(int64_t nz_n, int64_t nnz, const int64_t* __restrict__ nz_pos,
+                           const int64_t* __restrict__ up_at, int64_t* __restrict__ tile_cnt) {
+  __shared__ int64_t scr[33];
+  const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int64_t len = upper_len(t * kNzTile + threadIdx.x, nz_n, nnz, nz_pos, up_at);
+    const int64_t c = block_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | len : 0, scr);
+    if (threadIdx.x == 0) tile_cnt[t] = c;
+  }
+}
+
+__global__ void k_up_write(int64_t nz_n, int64_t nnz, const int32_t* __restrict__ nz_row,
+                           const int64_t* __restrict__ nz_pos, const int64_t* __restrict__ up_at,
+                           const int64_t* __restrict__ tile_off, int32_t* __restrict__ row, int64_t* __restrict__ pos,
+                           int64_t* __restrict__ dlt) {
+  __shared__ int64_t scr[33];
+  const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int64_t j = t * kNzTile + threadIdx.x;
+    const int64_t len = upper_len(j, nz_n, nnz, nz_pos, up_at);
+    int64_t tot;
+    const int64_t ex = block_exclusive_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | len : 0, scr, &tot);
+    if (len > 0) {
+      const uint64_t at = (uint64_t)(tile_off[t] + ex);
+      const int64_t o = (int64_t)(at >> kPackShift), p = (int64_t)(at & kPackEdgeMask);
+      row[o] = nz_row[j];
+      pos[o] = p;
+      dlt[o] = up_at[j] - p;
     }
   }
 }
@@ -336,26 +414,42 @@ cudaError_t launch_degree_order(int64_t nz_n, const int32_t* nz_row, const int64
   return cudaGetLastError();
 }
 
+bool intra_wants_signatures(int64_t n) { return n > kSigMin; }
+
 size_t objective_workspace_bytes(int64_t n) {
-  return align_up(4 * (size_t)(n > 0 ? n : 1)) + align_up(8 * 4);
+  const size_t nn = (size_t)(n > 0 ? n : 1);
+  return align_up(4 * nn) + (intra_wants_signatures(n) ? align_up(4 * ((nn >> 3) + 1)) : 0);
 }
 
-cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int64_t* off, const int32_t* col,
-                                 const int32_t* nz_row, const int64_t* nz_pos, int64_t nz_n,
+cudaError_t launch_intra(int64_t edges, const int32_t* col, const UpperRows& up, const uint32_t* id,
+                         const uint32_t* sig, unsigned long long* out, int num_sms, cudaStream_t stream) {
+  if (edges <= 0) return cudaSuccess;
+  const int64_t want = (edges + kObjThreads * kLbsK - 1) / (kObjThreads * kLbsK);
+  const int g = (int)(want < (int64_t)num_sms * 4 ? want : (int64_t)num_sms * 4);
+  if (sig) k_intra<true><<<g, kObjThreads, 0, stream>>>(edges, up, col, id, sig, out);
+  else k_intra<false><<<g, kObjThreads, 0, stream>>>(edges, up, col, id, nullptr, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int32_t* col, const UpperRows& up,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream) {
-  (void)off;
   int32_t* size = static_cast<int32_t*>(ws);
   cudaError_t e = cudaMemsetAsync(size, 0, 4 * (size_t)(n > 0 ? n : 1), stream);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(out, 0, 3 * sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
-  const int g = num_sms * 4;
-  k_cluster_sizes<<<g, 256, 0, stream>>>(n, labels, size, out);
-  if (nnz > 0) k_intra<<<num_sms * 2, kObjThreads, 0, stream>>>(nz_n, nz_row, nz_pos, nnz, col, labels, out);
-  k_pairs<<<g, 256, 0, stream>>>(n, size, out);
-  return cudaGetLastError();
+  const int64_t want = (n + 255) / 256;
+  const int g = (int)(want < (int64_t)num_sms * 8 ? want : (int64_t)num_sms * 8);
+  k_sizes_pairs<<<g, 256, 0, stream>>>(n, labels, size, out);
+  const uint32_t* id = reinterpret_cast<const uint32_t*>(labels);
+  uint32_t* sig = nullptr;
+  if (intra_wants_signatures(n)) {
+    sig = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + align_up(4 * (size_t)n));
+    k_signatures<<<g, 256, 0, stream>>>(n, id, sig);
+  }
+  return launch_intra(nnz / 2, col, up, id, sig, out, num_sms, stream);
 }
 
 size_t validate_workspace_bytes() { return align_up(8 * sizeof(unsigned long long)) + align_up(2 * sizeof(int)); }
@@ -371,12 +465,13 @@ cudaError_t launch_validate_offsets(int64_t n, int64_t nnz, const int64_t* off, 
 }
 
 cudaError_t launch_validate_edges(int64_t n, int64_t e0, int64_t e1, bool last, const int32_t* nz_row,
-                                  const int64_t* nz_pos, int64_t nz_n, const int32_t* col, void* ws, int num_sms,
-                                  cudaStream_t stream) {
+                                  const int64_t* nz_pos, int64_t nz_n, const int32_t* col, int64_t* up_at, void* ws,
+                                  int num_sms, cudaStream_t stream) {
   unsigned long long* sums = static_cast<unsigned long long*>(ws);
   int* flags = reinterpret_cast<int*>(static_cast<char*>(ws) + align_up(8 * sizeof(unsigned long long)));
   if (e1 > e0)
-    k_validate_edges<<<num_sms * 2, kValThreads, 0, stream>>>(n, e0, e1, nz_n, nz_row, nz_pos, col, flags, sums);
+    k_validate_edges<<<num_sms * 2, kValThreads, 0, stream>>>(n, e0, e1, nz_n, nz_row, nz_pos, col, up_at, flags,
+                                                              sums);
   if (last) k_validate_symmetry<<<1, 1, 0, stream>>>(flags, sums);
   return cudaGetLastError();
 }
@@ -401,15 +496,28 @@ size_t nonempty_workspace_bytes(int64_t n) {
 
 // nz_row/nz_pos get the non-empty rows and their first CSR positions; the
 // count is written to *count_dev (device int64).
-cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, void* ws,
-                                 int64_t* count_dev, int num_sms, cudaStream_t stream) {
+cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, int64_t* up_at,
+                                 void* ws, int64_t* count_dev, int num_sms, cudaStream_t stream) {
   if (n <= 0) return cudaMemsetAsync(count_dev, 0, sizeof(int64_t), stream);
   const int64_t ntiles = (n + kNzTile - 1) / kNzTile;
   int64_t* tile = static_cast<int64_t*>(ws);
   const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
   k_nz_count<<<g, kNzTile, 0, stream>>>(n, off, tile);
   k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, count_dev);
-  k_nz_write<<<g, kNzTile, 0, stream>>>(n, off, tile, nz_row, nz_pos);
+  k_nz_write<<<g, kNzTile, 0, stream>>>(n, off, tile, nz_row, nz_pos, up_at);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
+                              const int64_t* up_at, int32_t* row, int64_t* pos, int64_t* dlt, void* ws,
+                              unsigned long long* count_dev, int num_sms, cudaStream_t stream) {
+  if (nz_n <= 0) return cudaMemsetAsync(count_dev, 0, sizeof(unsigned long long), stream);
+  const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
+  int64_t* tile = static_cast<int64_t*>(ws);
+  const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
+  k_up_count<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_pos, up_at, tile);
+  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, reinterpret_cast<int64_t*>(count_dev));
+  k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, row, pos, dlt);
   return cudaGetLastError();
 }
 
