@@ -227,9 +227,10 @@ int cc_graph_destroy(cc_graph* g) {
   dfree(g->nz_pos, s);
   dfree(g->dsort, s);
   dfree(g->dge, s);
+  dfree(g->up_v, s);
   dfree(g->up_row, s);
+  dfree(g->up_len, s);
   dfree(g->up_pos, s);
-  dfree(g->up_dlt, s);
   dfree(g->perm_ws, s);
   dfree(g->order, s);
   dfree(g->round_ws, s);
@@ -355,9 +356,10 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
       void* dws = nullptr;
       if ((rc = from_cuda(dalloc(&g->dsort, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&g->dge, 8 * ((size_t)g->max_deg + 2), s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_row, 4 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_pos, 8 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_dlt, 8 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_v, 4 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_row, 8 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_len, 4 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_pos, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&dws, degree_order_workspace_bytes(g->max_deg), s))) != CC_OK) {
         dfree(dws, s); dfree(vws, s); dfree(nws, s); dfree(up_at, s);
         break;
@@ -373,8 +375,8 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     }
     unsigned long long* up_dev = reinterpret_cast<unsigned long long*>(nz_dev);
     unsigned long long up_pack = 0;
-    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_row, g->up_pos, g->up_dlt, nws, up_dev,
-                      g->num_sms, s);
+    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_v, g->up_row, g->up_len, g->up_pos, nws,
+                      up_dev, g->num_sms, s);
     cudaMemcpyAsync(&up_pack, up_dev, 8, cudaMemcpyDeviceToHost, s);
     if (flags & CC_VALIDATE_EXACT)
       launch_validate_reverse(nnz, g->off, g->nz_row, g->nz_pos, g->nz_n, g->col, vws, g->num_sms, s);
@@ -386,6 +388,7 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     if ((rc = from_cuda(cudaGetLastError())) != CC_OK) break;
     if (vflags[0] != 0) { rc = CC_ERR_INVALID_GRAPH; break; }
     g->up_n = (int64_t)(up_pack >> 33);
+    g->up_units = (int64_t)(up_pack & ((1ull << 33) - 1));
   } while (false);
   // the copy stream and its events are no longer needed (every chunk is
   // ordered before the work on s, or the graph is being thrown away)
@@ -463,7 +466,7 @@ static int cluster_async(cc_graph* g, uint64_t seed, int32_t* labels_out, int32_
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[1], s));
   CC_TRY(launch_async_c4(b, g->async_grid, lab, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[2], s));
-  CC_TRY(launch_disagreements(g->n, g->nnz, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   if (labels_out && !dev) CC_TRY(cudaMemcpyAsync(labels_out, lab, 4 * (size_t)g->n, cudaMemcpyDeviceToHost, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[3], s));
   CC_TRY(cudaMemcpyAsync(g->ctl_host, b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -642,7 +645,7 @@ int cc_disagreements(cc_graph* g, const int32_t* labels, int64_t* out) {
     CC_TRY(cudaMemcpyAsync(g->labels_tmp, labels, 4 * (size_t)g->n, cudaMemcpyHostToDevice, s));
     lab = g->labels_tmp;
   }
-  CC_TRY(launch_disagreements(g->n, g->nnz, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   CC_TRY(cudaMemcpyAsync(g->obj_host, g->obj_out, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   CC_TRY(cudaStreamSynchronize(s));
   if (g->obj_host[2]) return CC_ERR_INVALID_ARG;

@@ -457,6 +457,108 @@ __device__ __forceinline__ void lbs_for_each(const int64_t* epos, int64_t nitems
                   epos, nitems, E, ws, f, delta, vtx, E0, nullptr, 0, colp);
 }
 
+// ---------------------------------------------------------------------------
+// Unit walk: the edge-balanced walk over rows cut into units of 32 entries.
+//
+// Item j of the list (a row of len >= 1 entries from CSR position row) owns
+// the units [pos, pos + units_of(len)); pos counts up over the list, U is the
+// total.  Warps take chunks of consecutive units and read kUnitB of them at a
+// time, so every lane has kUnitB independent column loads in flight, and the
+// item of a unit is known to the whole warp: the warp holds the data of 32
+// consecutive items, one per lane, and picks the unit's item by a ballot.
+// Against the 128-edge batches of lbs_for_each, which resolve the item of
+// every single edge through shared memory, a batch is twice as many entries
+// behind half as many dependent steps.  Short rows leave lanes idle (a row of
+// 8 entries fills a quarter of its unit), which costs little: the walk is
+// bound by latency, not by lanes.
+//
+// at(j) = pos of item j; load(j) = the item's data, read once per window of
+// items; f(X) gets the batch: the column of this lane's entry of each unit
+// (-1: none) and, the same in all lanes, the unit's item and payload.  All 32
+// lanes call f together.
+// ---------------------------------------------------------------------------
+constexpr int kUnitB = 8;
+__host__ __device__ __forceinline__ int64_t units_of(int64_t len) { return (len + 31) >> 5; }
+
+struct UnitItem {
+  uint32_t pos;          // below 2^33 / 32 + 2^31 units
+  int32_t len;
+  int64_t row;
+  int32_t aux;           // payload
+};
+
+struct UnitBatch {
+  int32_t w[kUnitB];     // column of this lane's entry, -1 when there is none
+  int32_t aux[kUnitB];   // payload of the unit's item
+  int32_t item[kUnitB];  // the unit's item relative to j0
+  int64_t j0;
+};
+
+// Number of items whose pos is <= x (pos ascending), by a 33-ary search of the warp.
+template <class At>
+__device__ __forceinline__ int64_t warp_count_upto(const At& at, int64_t n, uint32_t x) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = n;
+  while (hi - lo > 32) {
+    const int64_t p = lo + ((hi - lo) * (lane + 1)) / 33;
+    const int c = __popc(__ballot_sync(FULL, at(p) <= x));
+    const int64_t pp = __shfl_sync(FULL, p, c > 0 ? c - 1 : 0);
+    const int64_t pn = __shfl_sync(FULL, p, c < 32 ? c : 31);
+    lo = c > 0 ? pp + 1 : lo;
+    hi = c < 32 ? pn : hi;
+  }
+  const int64_t p = lo + lane;
+  const bool le = p < hi && at(p) <= x;
+  return lo + __popc(__ballot_sync(FULL, le));
+}
+
+template <class At, class Load, class F>
+__device__ __forceinline__ void unit_walk(int64_t gwarp, int64_t nwarps, int64_t nitems, int64_t U,
+                                          const int32_t* __restrict__ col, WalkShape shape, const At& at,
+                                          const Load& load, F&& f) {
+  const int lane = threadIdx.x & 31;
+  // up to 4 * shape.batches batches per chunk, fewer when the list is short
+  int64_t nb = U / (nwarps * (int64_t)kUnitB * 2);
+  nb = nb < 1 ? 1 : (nb > 4 * shape.batches ? 4 * shape.batches : nb);
+  const int64_t chunk = nb * kUnitB;
+  for (int64_t c0 = gwarp * chunk; c0 < U; c0 += nwarps * chunk) {
+    const int64_t cend = c0 + chunk < U ? c0 + chunk : U;
+    UnitBatch X;
+    X.j0 = warp_count_upto(at, nitems, (uint32_t)c0) - 1;
+    UnitItem it;
+    uint32_t wend = 0;                  // first unit after the window's items
+    for (int64_t t = c0; t < cend; t += kUnitB) {
+      const int64_t tend = t + kUnitB < cend ? t + kUnitB : cend;
+      if (t == c0 || tend > (int64_t)wend) {
+        if (t != c0) X.j0 += __popc(__ballot_sync(FULL, it.pos <= (uint32_t)t)) - 1;
+        const int64_t j = X.j0 + lane;
+        it = UnitItem{0xFFFFFFFFu, 0, 0, 0};
+        if (j < nitems) it = load(j);
+        const uint32_t e = it.pos + (uint32_t)units_of(it.len);
+        wend = __shfl_sync(FULL, e, 31);
+      }
+      int64_t pf = -1;
+#pragma unroll
+      for (int q = 0; q < kUnitB; ++q) {
+        const int64_t x = t + q;
+        const int i = __popc(__ballot_sync(FULL, it.pos <= (uint32_t)x)) - 1;
+        const uint32_t p = __shfl_sync(FULL, it.pos, i);
+        const int32_t len = __shfl_sync(FULL, it.len, i);
+        const int64_t row = __shfl_sync(FULL, it.row, i);
+        X.aux[q] = __shfl_sync(FULL, it.aux, i);
+        X.item[q] = i;
+        const int32_t k = (int32_t)((uint32_t)x - p) * 32 + lane;
+        X.w[q] = x < cend && k < len ? __ldg(col + row + k) : -1;
+        // lane q looks shape.pf_ahead batches ahead in the same row
+        const int32_t kp = k - lane + shape.pf_ahead * kUnitB * 32;
+        if (lane == q && shape.pf_ahead > 0 && kp < len) pf = row + kp;
+      }
+      if (pf >= 0) prefetch_l2(col + pf);
+      f(X);
+    }
+  }
+}
+
 // Lists of adjacency rows.  A list counter packs (items << 33 | edges): one
 // atomicAdd hands out an item index and the item's first virtual edge, so
 // epos stays non-decreasing in the item index.  For every item the list keeps

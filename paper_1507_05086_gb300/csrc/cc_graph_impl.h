@@ -25,11 +25,12 @@ struct cc_graph {
   int32_t* dsort = nullptr;
   int64_t* dge = nullptr;
   // the upper part of every row, each edge once (arrays of nz_n entries)
-  int32_t* up_row = nullptr;
-  int64_t* up_pos = nullptr;
-  int64_t* up_dlt = nullptr;
-  int64_t up_n = 0;
-  ccg::UpperRows upper() const { return ccg::UpperRows{up_row, up_pos, up_dlt, up_n}; }
+  int32_t* up_v = nullptr;
+  int64_t* up_row = nullptr;
+  int32_t* up_len = nullptr;
+  uint32_t* up_pos = nullptr;
+  int64_t up_n = 0, up_units = 0;
+  ccg::UpperRows upper() const { return ccg::UpperRows{up_v, up_row, up_len, up_pos, up_n, up_units}; }
   // cached workspaces (grown on demand)
   void* perm_ws = nullptr;
   size_t perm_ws_bytes = 0;

@@ -93,13 +93,15 @@ Tuning default_tuning();
 Tuning batch_settings(int64_t* small_n, int64_t* team_n, int* team_blocks);
 
 // The upper part of every row (columns above the row's vertex), which holds
-// each edge once: rows with a non-empty upper part, with their first virtual
-// edge and CSR delta (RowList in cc_device.cuh).  The objective walks it.
+// each edge once: per row with a non-empty upper part its vertex, the CSR
+// position and length of the part and its first unit (unit_walk in
+// cc_device.cuh).  The objective walks it.
 struct UpperRows {
-  const int32_t* row;
-  const int64_t* pos;
-  const int64_t* dlt;
-  int64_t n;
+  const int32_t* v;
+  const int64_t* row;
+  const int32_t* len;
+  const uint32_t* pos;
+  int64_t n, units;
 };
 
 struct RoundBuffers {
@@ -196,13 +198,13 @@ cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, c
 size_t objective_workspace_bytes(int64_t n);
 // out[0] = edges inside clusters, out[1] = sum_c C(s_c, 2), out[2] = 1 if a
 // label was outside [0, n).  out: 3 device words.
-cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int32_t* col, const UpperRows& up,
+cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows& up,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream);
 // *out += the number of edges (u, w) with id[u] == id[w]; `sig` (or null): a
 // 4-bit signature of id per vertex, eight to a word, that is equal when the
 // ids are.
-cudaError_t launch_intra(int64_t edges, const int32_t* col, const UpperRows& up, const uint32_t* id,
+cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id,
                          const uint32_t* sig, unsigned long long* out, int num_sms, cudaStream_t stream);
 // Vertices above which the objective reads signatures before ids.
 bool intra_wants_signatures(int64_t n);
@@ -235,10 +237,10 @@ size_t nonempty_workspace_bytes(int64_t n);
 // writes the starts).
 cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, int64_t* up_at,
                                  void* ws, int64_t* count_dev, int num_sms, cudaStream_t stream);
-// The rows of UpperRows from up_at; *count_dev = their number << kPackShift |
-// their edges.  ws: nonempty_workspace_bytes(nz_n).
+// The arrays of UpperRows from up_at; *count_dev = rows << kPackShift | units.
+// ws: nonempty_workspace_bytes(nz_n).
 cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
-                              const int64_t* up_at, int32_t* row, int64_t* pos, int64_t* dlt, void* ws,
+                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos, void* ws,
                               unsigned long long* count_dev, int num_sms, cudaStream_t stream);
 
 }  // namespace ccg

@@ -16,6 +16,7 @@ namespace ccg {
 namespace {
 
 constexpr int kObjThreads = 512;
+constexpr int kObjBlocks = 2;          // blocks of k_intra per SM
 // Graphs above this many vertices read 4-bit signatures before ids: up to it
 // the ids (64 MB) fit the 129 MB L2 themselves.
 constexpr int64_t kSigMin = int64_t(1) << 24;
@@ -48,38 +49,43 @@ __global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int
 }
 
 // Edges (u, w) with id[u] == id[w], every edge read from its lower end only
-// (half of the CSR's entries).  Bound by the latency of the chain row data ->
-// column -> id.  With sig, a 4-bit signature per vertex decides first, so that
-// ids are read only where the signatures agree.  Objective of a ClusterWild!
-// labelling, both ends of every edge -> this: R-MAT 22 0.59 -> 0.40 ms, R-MAT
-// 24 2.43 -> 1.52 ms, R-MAT 26 12.5 -> 7.6 ms.
+// (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 23
+// (130M edges, 0.49 ms, 265e9 edges/s) L2 runs at 65 % and L1 at 70 % of their
+// throughput, above the 236e9 reads/s of a library gather from a 32 MiB table.
+// With sig, a 4-bit signature per vertex decides first, so that ids are read
+// only where the signatures agree.  Whole objective of a ClusterWild! labelling
+// of R-MAT 22 / 24 / 26: both ends of every edge 0.59 / 2.43 / 12.5 ms, upper
+// ends over 128-edge batches (lbs_for_each) 0.40 / 1.52 / 7.6 ms, this 0.32 /
+// 1.22 / 5.8 ms.  Three blocks per SM at 40 registers spill: 0.49 / 1.90 / 7.4;
+// four units per batch at three blocks: 0.37 / 1.41 / 5.7.
 template <bool kSig>
-__global__ void __launch_bounds__(kObjThreads) k_intra(int64_t edges, UpperRows up, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(kObjThreads, kObjBlocks) k_intra(UpperRows up, const int32_t* __restrict__ col,
                                                       const uint32_t* __restrict__ id,
                                                       const uint32_t* __restrict__ sig, unsigned long long* out) {
-  __shared__ LbsWarp lbs[kObjThreads / 32];
   __shared__ int64_t scr[33];
   int64_t cnt = 0;
-  lbs_for_each_in((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, ((int64_t)gridDim.x * blockDim.x) >> 5,
-                  up.pos, up.n, edges, &lbs[threadIdx.x >> 5], [&](const Lbs& L) {
-    int32_t w[kLbsK];
-#pragma unroll
-    for (int t = 0; t < kLbsK; ++t) w[t] = L.ok(t) ? __ldg(col + L.csr(t)) : 0;
-    uint32_t x[kLbsK];
+  unit_walk((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, ((int64_t)gridDim.x * blockDim.x) >> 5, up.n,
+            up.units, col, WalkShape{}, [&](int64_t j) { return __ldg(up.pos + j); },
+            [&](int64_t j) {
+              return UnitItem{__ldg(up.pos + j), __ldg(up.len + j), __ldg(up.row + j),
+                              (int32_t)__ldg(id + __ldg(up.v + j))};
+            },
+            [&](const UnitBatch& X) {
+    uint32_t x[kUnitB];
     if (kSig) {
 #pragma unroll
-      for (int t = 0; t < kLbsK; ++t) x[t] = __ldg(sig + (w[t] >> 3)) >> ((w[t] & 7) * 4);
+      for (int q = 0; q < kUnitB; ++q) x[q] = X.w[q] >= 0 ? __ldg(sig + (X.w[q] >> 3)) >> ((X.w[q] & 7) * 4) : 0;
 #pragma unroll
-      for (int t = 0; t < kLbsK; ++t)
-        if (L.ok(t) && ((x[t] ^ cluster_sig((uint32_t)L.vtx(t))) & 15u) == 0)
-          cnt += __ldg(id + w[t]) == (uint32_t)L.vtx(t) ? 1 : 0;
+      for (int q = 0; q < kUnitB; ++q)
+        if (X.w[q] >= 0 && ((x[q] ^ cluster_sig((uint32_t)X.aux[q])) & 15u) == 0)
+          cnt += __ldg(id + X.w[q]) == (uint32_t)X.aux[q] ? 1 : 0;
     } else {
 #pragma unroll
-      for (int t = 0; t < kLbsK; ++t) x[t] = __ldg(id + w[t]);
+      for (int q = 0; q < kUnitB; ++q) x[q] = X.w[q] >= 0 ? __ldg(id + X.w[q]) : 0;
 #pragma unroll
-      for (int t = 0; t < kLbsK; ++t) cnt += L.ok(t) && x[t] == (uint32_t)L.vtx(t) ? 1 : 0;
+      for (int q = 0; q < kUnitB; ++q) cnt += X.w[q] >= 0 && x[q] == (uint32_t)X.aux[q] ? 1 : 0;
     }
-  }, up.dlt, up.row, 0, id, 0, col);
+  });
   cnt = block_sum<int64_t>(cnt, scr);
   if (threadIdx.x == 0 && cnt) atomicAdd(out, (unsigned long long)cnt);
 }
@@ -250,7 +256,7 @@ __global__ void k_nz_write(int64_t n, const int64_t* __restrict__ off, const int
 }
 
 // Rows with a non-empty upper part, by the same three steps; counts are
-// packed (rows << kPackShift | edges).
+// packed (rows << kPackShift | units).
 __device__ __forceinline__ int64_t upper_len(int64_t j, int64_t nz_n, int64_t nnz, const int64_t* nz_pos,
                                              const int64_t* up_at) {
   return j < nz_n ? (j + 1 < nz_n ? nz_pos[j + 1] : nnz) - up_at[j] : 0;
@@ -262,28 +268,29 @@ __global__ void k_up_count(int64_t nz_n, int64_t nnz, const int64_t* __restrict_
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int64_t len = upper_len(t * kNzTile + threadIdx.x, nz_n, nnz, nz_pos, up_at);
-    const int64_t c = block_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | len : 0, scr);
+    const int64_t c = block_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | units_of(len) : 0, scr);
     if (threadIdx.x == 0) tile_cnt[t] = c;
   }
 }
 
 __global__ void k_up_write(int64_t nz_n, int64_t nnz, const int32_t* __restrict__ nz_row,
                            const int64_t* __restrict__ nz_pos, const int64_t* __restrict__ up_at,
-                           const int64_t* __restrict__ tile_off, int32_t* __restrict__ row, int64_t* __restrict__ pos,
-                           int64_t* __restrict__ dlt) {
+                           const int64_t* __restrict__ tile_off, int32_t* __restrict__ v, int64_t* __restrict__ row,
+                           int32_t* __restrict__ len, uint32_t* __restrict__ pos) {
   __shared__ int64_t scr[33];
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int64_t j = t * kNzTile + threadIdx.x;
-    const int64_t len = upper_len(j, nz_n, nnz, nz_pos, up_at);
+    const int64_t l = upper_len(j, nz_n, nnz, nz_pos, up_at);
     int64_t tot;
-    const int64_t ex = block_exclusive_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | len : 0, scr, &tot);
-    if (len > 0) {
+    const int64_t ex = block_exclusive_sum<int64_t>(l > 0 ? (int64_t(1) << kPackShift) | units_of(l) : 0, scr, &tot);
+    if (l > 0) {
       const uint64_t at = (uint64_t)(tile_off[t] + ex);
-      const int64_t o = (int64_t)(at >> kPackShift), p = (int64_t)(at & kPackEdgeMask);
-      row[o] = nz_row[j];
-      pos[o] = p;
-      dlt[o] = up_at[j] - p;
+      const int64_t o = (int64_t)(at >> kPackShift);
+      v[o] = nz_row[j];
+      row[o] = up_at[j];
+      len[o] = (int32_t)l;
+      pos[o] = (uint32_t)(at & kPackEdgeMask);
     }
   }
 }
@@ -421,17 +428,18 @@ size_t objective_workspace_bytes(int64_t n) {
   return align_up(4 * nn) + (intra_wants_signatures(n) ? align_up(4 * ((nn >> 3) + 1)) : 0);
 }
 
-cudaError_t launch_intra(int64_t edges, const int32_t* col, const UpperRows& up, const uint32_t* id,
-                         const uint32_t* sig, unsigned long long* out, int num_sms, cudaStream_t stream) {
-  if (edges <= 0) return cudaSuccess;
-  const int64_t want = (edges + kObjThreads * kLbsK - 1) / (kObjThreads * kLbsK);
-  const int g = (int)(want < (int64_t)num_sms * 4 ? want : (int64_t)num_sms * 4);
-  if (sig) k_intra<true><<<g, kObjThreads, 0, stream>>>(edges, up, col, id, sig, out);
-  else k_intra<false><<<g, kObjThreads, 0, stream>>>(edges, up, col, id, nullptr, out);
+cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id, const uint32_t* sig,
+                         unsigned long long* out, int num_sms, cudaStream_t stream) {
+  if (up.units <= 0) return cudaSuccess;
+  const int64_t per = kObjThreads / 32 * kUnitB;
+  const int64_t want = (up.units + per - 1) / per;
+  const int g = (int)(want < (int64_t)num_sms * kObjBlocks ? want : (int64_t)num_sms * kObjBlocks);
+  if (sig) k_intra<true><<<g, kObjThreads, 0, stream>>>(up, col, id, sig, out);
+  else k_intra<false><<<g, kObjThreads, 0, stream>>>(up, col, id, nullptr, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int32_t* col, const UpperRows& up,
+cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows& up,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream) {
   int32_t* size = static_cast<int32_t*>(ws);
@@ -449,7 +457,7 @@ cudaError_t launch_disagreements(int64_t n, int64_t nnz, const int32_t* col, con
     sig = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + align_up(4 * (size_t)n));
     k_signatures<<<g, 256, 0, stream>>>(n, id, sig);
   }
-  return launch_intra(nnz / 2, col, up, id, sig, out, num_sms, stream);
+  return launch_intra(col, up, id, sig, out, num_sms, stream);
 }
 
 size_t validate_workspace_bytes() { return align_up(8 * sizeof(unsigned long long)) + align_up(2 * sizeof(int)); }
@@ -509,7 +517,7 @@ cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row,
 }
 
 cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
-                              const int64_t* up_at, int32_t* row, int64_t* pos, int64_t* dlt, void* ws,
+                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos, void* ws,
                               unsigned long long* count_dev, int num_sms, cudaStream_t stream) {
   if (nz_n <= 0) return cudaMemsetAsync(count_dev, 0, sizeof(unsigned long long), stream);
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
@@ -517,7 +525,7 @@ cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, 
   const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
   k_up_count<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_pos, up_at, tile);
   k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, reinterpret_cast<int64_t*>(count_dev));
-  k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, row, pos, dlt);
+  k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, v, row, len, pos);
   return cudaGetLastError();
 }
 
