@@ -161,7 +161,7 @@ int ensure_cluster_ws(cc_graph* g) {
     CC_TRY(dalloc(&g->perm_ws, pb, g->stream));
     g->perm_ws_bytes = pb;
   }
-  if (!g->grid) g->grid = rounds_grid_size(g->device);
+  if (!g->grid) g->grid = rounds_grid_size(g->device, g->nnz);
   const size_t rb = rounds_workspace_bytes(g->n, g->max_deg, g->grid);
   if (g->round_ws_bytes < rb) {
     dfree(g->round_ws, g->stream);
@@ -231,6 +231,7 @@ int cc_graph_destroy(cc_graph* g) {
   dfree(g->up_row, s);
   dfree(g->up_len, s);
   dfree(g->up_pos, s);
+  dfree(g->up_epos, s);
   dfree(g->perm_ws, s);
   dfree(g->order, s);
   dfree(g->round_ws, s);
@@ -360,6 +361,7 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
           (rc = from_cuda(dalloc(&g->up_row, 8 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&g->up_len, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&g->up_pos, 4 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_epos, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&dws, degree_order_workspace_bytes(g->max_deg), s))) != CC_OK) {
         dfree(dws, s); dfree(vws, s); dfree(nws, s); dfree(up_at, s);
         break;
@@ -374,10 +376,10 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
                             g->num_sms, s);
     }
     unsigned long long* up_dev = reinterpret_cast<unsigned long long*>(nz_dev);
-    unsigned long long up_pack = 0;
-    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_v, g->up_row, g->up_len, g->up_pos, nws,
-                      up_dev, g->num_sms, s);
-    cudaMemcpyAsync(&up_pack, up_dev, 8, cudaMemcpyDeviceToHost, s);
+    unsigned long long up_pack[2] = {0, 0};
+    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_v, g->up_row, g->up_len, g->up_pos,
+                      g->up_epos, nws, up_dev, g->num_sms, s);
+    cudaMemcpyAsync(up_pack, up_dev, sizeof(up_pack), cudaMemcpyDeviceToHost, s);
     if (flags & CC_VALIDATE_EXACT)
       launch_validate_reverse(nnz, g->off, g->nz_row, g->nz_pos, g->nz_n, g->col, vws, g->num_sms, s);
     cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s);
@@ -387,8 +389,9 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) break;
     if ((rc = from_cuda(cudaGetLastError())) != CC_OK) break;
     if (vflags[0] != 0) { rc = CC_ERR_INVALID_GRAPH; break; }
-    g->up_n = (int64_t)(up_pack >> 33);
-    g->up_units = (int64_t)(up_pack & ((1ull << 33) - 1));
+    g->up_n = (int64_t)(up_pack[0] >> 33);
+    g->up_units = (int64_t)(up_pack[0] & ((1ull << 33) - 1));
+    g->up_edges = (int64_t)up_pack[1];
   } while (false);
   // the copy stream and its events are no longer needed (every chunk is
   // ordered before the work on s, or the graph is being thrown away)
@@ -454,6 +457,7 @@ static int cluster_async(cc_graph* g, uint64_t seed, int32_t* labels_out, int32_
   b.nz_n = g->nz_n;
   b.dsort = g->dsort;
   b.dge = g->dge;
+  b.up = g->upper();
   const bool dev = is_device_ptr(labels_out);
   int32_t* lab = labels_out;
   if (!dev) {
@@ -543,6 +547,7 @@ int cc_cluster_ex(cc_graph* g, int algo, double eps, uint64_t seed, int32_t* lab
   b.nz_n = g->nz_n;
   b.dsort = g->dsort;
   b.dge = g->dge;
+  b.up = g->upper();
   b.stats = g->stats_dev;
   b.stats_cap = stats_cap;
   CC_TRY(cudaMemsetAsync(g->perm_err, 0, sizeof(int), s));
@@ -561,10 +566,10 @@ int cc_cluster_ex(cc_graph* g, int algo, double eps, uint64_t seed, int32_t* lab
   const bool dev = is_device_ptr(labels_out);
   if (labels_out && !dev) {
     if ((rc = ensure_labels_tmp(g)) != CC_OK) return rc;
-    CC_TRY(launch_finalize_labels(b, g->labels_tmp, s));
+    CC_TRY(launch_finalize_labels(b, g->labels_tmp, disagreements_out != nullptr, g->num_sms, s));
     CC_TRY(cudaMemcpyAsync(labels_out, g->labels_tmp, 4 * (size_t)g->n, cudaMemcpyDeviceToHost, s));
   } else {
-    CC_TRY(launch_finalize_labels(b, labels_out, s));   // also the objective's pair term
+    CC_TRY(launch_finalize_labels(b, labels_out, disagreements_out != nullptr, g->num_sms, s));
   }
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[3], s));
   CC_TRY(cudaMemcpyAsync(g->ctl_host, b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -591,7 +596,7 @@ int cc_cluster_ex(cc_graph* g, int algo, double eps, uint64_t seed, int32_t* lab
   if (rounds_out) *rounds_out = (int32_t)rounds;
   if (disagreements_out) {
     const int64_t m = g->nnz / 2;
-    *disagreements_out = m - 2 * (int64_t)c.mc - (int64_t)c.mm + (int64_t)c.pairs;
+    *disagreements_out = m - 2 * (int64_t)c.intra + (int64_t)c.pairs;
   }
   return CC_OK;
 }
@@ -683,7 +688,7 @@ int run_batch_jobs(cc_graph* const* gs, int32_t count, int algo, double eps, con
       const cc_graph* g = gs[i];
       jb = BatchJob{};
       jb.off = g->off; jb.col = g->col; jb.nz = g->nz_row; jb.nz_n = g->nz_n;
-      jb.dsort = g->dsort; jb.dge = g->dge;
+      jb.dsort = g->dsort; jb.dge = g->dge; jb.up = g->upper();
       jb.n = g->n; jb.nnz = g->nnz; jb.max_deg = g->max_deg;
       jb.seed = seeds[i] + (uint64_t)j;
       jb.err = 1;

@@ -38,6 +38,15 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -100,6 +109,18 @@ __device__ __forceinline__ T warp_inclusive_sum(T x) {
   return x;
 }
 
+// The same as a loop: a quarter of the code, for sums whose code runs once per
+// pass and so is fetched rather than found in the instruction cache.
+__device__ __forceinline__ int64_t warp_inclusive_sum_rolled(int64_t x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T x) {
 #pragma unroll
@@ -132,21 +153,15 @@ template <class T>
 __device__ __forceinline__ T block_exclusive_sum(T x, T* scratch, T* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = (blockDim.x + 31) >> 5;
-  T inc = warp_inclusive_sum(x);
-  __syncthreads();
+  const T inc = warp_inclusive_sum(x);
+  __syncthreads();                       // earlier readers of scratch
   if (lane == 31) scratch[warp] = inc;
   __syncthreads();
-  if (warp == 0) {
-    T w = lane < nwarps ? scratch[lane] : T(0);
-    T wi = warp_inclusive_sum(w);
-    scratch[lane] = wi - w;
-    if (lane == 31) scratch[32] = wi;   // lane 31 holds the grand total
-  }
-  __syncthreads();
-  T res = scratch[warp] + inc - x;
-  *total = scratch[32];
-  __syncthreads();
-  return res;
+  // every warp scans the warps' totals itself: no third barrier
+  const T w = lane < nwarps ? scratch[lane] : T(0);
+  const T wi = warp_inclusive_sum(w);
+  *total = __shfl_sync(FULL, wi, 31);
+  return __shfl_sync(FULL, wi - w, warp) + inc - x;
 }
 
 template <class T>
@@ -154,6 +169,24 @@ __device__ __forceinline__ T block_sum(T x, T* scratch) {
   T tot;
   block_exclusive_sum(x, scratch, &tot);
   return tot;
+}
+
+__device__ __forceinline__ int32_t block_max_i32(int32_t x, int32_t* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  x = __reduce_max_sync(FULL, x);
+  __syncthreads();
+  if (lane == 0) scratch[warp] = x;
+  __syncthreads();
+  return __reduce_max_sync(FULL, lane < (int)((blockDim.x + 31) >> 5) ? scratch[lane] : INT32_MIN);
+}
+
+__device__ __forceinline__ int32_t block_sum_i32(int32_t x, int32_t* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  x = __reduce_add_sync(FULL, x);
+  __syncthreads();
+  if (lane == 0) scratch[warp] = x;
+  __syncthreads();
+  return __reduce_add_sync(FULL, lane < (int)((blockDim.x + 31) >> 5) ? scratch[lane] : 0);
 }
 
 template <class T>
@@ -559,6 +592,125 @@ __device__ __forceinline__ void unit_walk(int64_t gwarp, int64_t nwarps, int64_t
   }
 }
 
+// ---------------------------------------------------------------------------
+// Row walk: the edge-balanced walk of the round kernel.
+//
+// Item j of the list is a row of len >= 1 entries from CSR position row; pos(j)
+// counts the entries of the items before it, E is the total.  Warps take
+// chunks of consecutive entries.  A warp holds a window of 32 items, one per
+// lane, in registers, and reads up to kB times 32 entries of the window at a
+// time, so every lane has kB independent column loads in flight.  A lane finds
+// the item of its entry by a five-step search over the lanes' starts (none
+// when the batch lies inside one row), so rows of any length fill the warp.
+// lbs_for_each does the same through marks in shared memory and a scan, behind
+// twice as many dependent steps.
+//
+// at(j) = pos of item j; load(j) = the item's data, read once per window;
+// f(X) gets a batch, g(j) follows the last batch of a window, with this lane's
+// item (j >= nitems: none).  All 32 lanes call f and g together.
+// ---------------------------------------------------------------------------
+struct RowItem {
+  int64_t pos;
+  int64_t row;
+  int32_t len;
+  int32_t aux;           // payload
+};
+
+template <int kB>
+struct RowBatch {
+  int32_t w[kB];         // column of this lane's entry, -1 when there is none
+  int32_t aux[kB];       // payload of its item
+  int32_t item[kB];      // its item
+  int32_t from, to;      // where this lane's window item lies, relative to the batch (from > 32 kB: after it)
+};
+
+// The last item whose pos is <= x (pos ascending from 0, x >= 0), by a 32-ary
+// search of the warp.
+template <class At>
+__device__ __forceinline__ int32_t warp_item_at(const At& at, int32_t n, int64_t x) {
+  const int lane = threadIdx.x & 31;
+  int32_t lo = 0, span = n;
+#pragma unroll 1
+  while (span > 1) {
+    const int32_t step = (int32_t)(((uint32_t)span + 31u) >> 5), p = lane * step;     // p < 2^31 + 31
+    const int c = __popc(__ballot_sync(FULL, (uint32_t)p < (uint32_t)span && at(lo + p) <= x));    // >= 1
+    lo += (c - 1) * step;
+    span = span - (c - 1) * step < step ? span - (c - 1) * step : step;
+  }
+  return lo;
+}
+
+template <int kB, class At, class Load, class F, class G>
+__device__ __forceinline__ void row_walk(int gwarp, int nwarps, int32_t nitems, int64_t E,
+                                         const int32_t* __restrict__ col, WalkShape shape, const At& at,
+                                         const Load& load, F&& f, G&& g) {
+  constexpr int32_t kFar = 1 << 30;     // relative positions from here on lie behind the chunk
+  constexpr int kW = 32 * kB;
+  const int lane = threadIdx.x & 31;
+  // up to 2 * shape.batches batches per chunk, fewer when the list is short
+  const int64_t most = (int64_t)nwarps * kW * 4 * shape.batches;
+  int nb = E >= most ? 2 * shape.batches : (int)((uint32_t)E / (uint32_t)(nwarps * kW * 2));
+  nb = nb < 1 ? 1 : nb;
+  const int32_t chunk = nb * kW;
+  for (int64_t cs = (int64_t)gwarp * chunk; cs < E; cs += (int64_t)nwarps * chunk) {
+    const int32_t cend = E - cs < chunk ? (int32_t)(E - cs) : chunk;
+    int32_t j0 = nitems > 32 ? warp_item_at(at, nitems, cs) : 0;       // a short list is one window
+    for (int32_t e = 0; e < cend; j0 += 32) {
+      // the window: starts and ends relative to the chunk
+      int32_t p = kFar, end = kFar, aux = 0;
+      int64_t rel = 0;                  // CSR position of the chunk's first entry, were it in this row
+      if (j0 + lane < nitems) {
+        const RowItem it = load(j0 + lane);
+        const int64_t d = it.pos - cs;
+        rel = it.row - d;
+        aux = it.aux;
+        p = d < kFar ? (int32_t)d : kFar;
+        end = d + it.len < kFar ? (int32_t)(d + it.len) : kFar;
+      }
+      int32_t wend = __shfl_sync(FULL, end, 31);
+      wend = wend < cend ? wend : cend;
+      for (; e < wend; e += kW) {
+        const int32_t stop = e + kW < wend ? e + kW : wend;
+        RowBatch<kB> X;
+        X.from = p - e;
+        X.to = (end < stop ? end : stop) - e;
+        const int i0 = __popc(__ballot_sync(FULL, p <= e)) - 1;
+        const int32_t end0 = __shfl_sync(FULL, end, i0);
+#pragma unroll
+        for (int q = 0; q < kB; ++q) {
+          const int32_t x = e + lane + 32 * q;
+          int i = i0;
+          if (end0 < stop) {            // warp-uniform: several rows in the batch
+            i = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+              if (__shfl_sync(FULL, p, i + o) <= x) i += o;
+          }
+          const int64_t at0 = __shfl_sync(FULL, rel, i);
+          X.aux[q] = __shfl_sync(FULL, aux, i);
+          X.item[q] = j0 + i;
+          X.w[q] = x < stop ? __ldg(col + at0 + x) : -1;
+        }
+        if (kB > 1 && shape.pf_ahead > 0 && end0 >= stop) {       // stream a long row ahead
+          const int32_t x = e + shape.pf_ahead * kW + 32 * lane;
+          const int64_t at0 = __shfl_sync(FULL, rel, i0);
+          if (lane < kB && x < end0) prefetch_l2(col + at0 + x);
+        }
+        f(X);
+      }
+      e = wend;
+      g(j0 + lane);
+    }
+  }
+}
+
+template <int kB, class At, class Load, class F>
+__device__ __forceinline__ void row_walk(int gwarp, int nwarps, int32_t nitems, int64_t E,
+                                         const int32_t* __restrict__ col, WalkShape shape, const At& at,
+                                         const Load& load, F&& f) {
+  row_walk<kB>(gwarp, nwarps, nitems, E, col, shape, at, load, f, [](int32_t) {});
+}
+
 // Lists of adjacency rows.  A list counter packs (items << 33 | edges): one
 // atomicAdd hands out an item index and the item's first virtual edge, so
 // epos stays non-decreasing in the item index.  For every item the list keeps
@@ -603,69 +755,6 @@ __device__ __forceinline__ void warp_append_rows(bool want, int32_t v, int64_t r
     L.delta[j] = row - ep;
     if (L.aux) L.aux[j] = aux;
   }
-}
-
-// Per-warp staging of list appends, so that many items share one atomic on
-// the list counter.
-constexpr int kAppCap = 128;
-
-struct AppendBuf {
-  int32_t v[kAppCap];
-  int32_t len[kAppCap];
-  int64_t row[kAppCap];
-  int n;
-};
-
-__device__ __forceinline__ void append_flush(AppendBuf* b, const RowList& L) {
-  const int lane = threadIdx.x & 31;
-  __syncwarp();
-  const int n = b->n;
-  if (n == 0) return;
-  constexpr int kPer = kAppCap / 32;
-  int64_t loc = 0;
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int i = lane * kPer + q;
-    if (i < n) loc += b->len[i];
-  }
-  const int64_t ex = warp_inclusive_sum<int64_t>(loc) - loc;
-  const int64_t tot = __shfl_sync(FULL, ex + loc, 31);
-  unsigned long long old = 0;
-  if (lane == 0) old = atomicAdd(L.counter, ((unsigned long long)n << kPackShift) | (unsigned long long)tot);
-  old = __shfl_sync(FULL, old, 0);
-  const int64_t j0 = (int64_t)(old >> kPackShift);
-  int64_t ep = (int64_t)(old & kPackEdgeMask) + ex;
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int i = lane * kPer + q;
-    if (i < n && CC_IN_BOUNDS(j0 + i, L.cap, L.err)) {
-      L.v[j0 + i] = b->v[i];
-      L.epos[j0 + i] = ep;
-      L.delta[j0 + i] = b->row[i] - ep;
-      ep += b->len[i];
-    }
-  }
-  __syncwarp();
-  if (lane == 0) b->n = 0;
-  __syncwarp();
-}
-
-__device__ __forceinline__ void append_stage(AppendBuf* b, bool want, int32_t v, int64_t row, int32_t len,
-                                             const RowList& L) {
-  const int lane = threadIdx.x & 31;
-  const unsigned mask = __ballot_sync(FULL, want);
-  if (mask == 0) return;
-  __syncwarp();
-  if (b->n + __popc(mask) > kAppCap) append_flush(b, L);
-  const int pos = b->n + __popc(mask & ((1u << lane) - 1u));
-  if (want) {
-    b->v[pos] = v;
-    b->len[pos] = len;
-    b->row[pos] = row;
-  }
-  __syncwarp();
-  if (lane == 0) b->n += __popc(mask);
-  __syncwarp();
 }
 
 }  // namespace ccg

@@ -29,8 +29,9 @@ struct cc_graph {
   int64_t* up_row = nullptr;
   int32_t* up_len = nullptr;
   uint32_t* up_pos = nullptr;
-  int64_t up_n = 0, up_units = 0;
-  ccg::UpperRows upper() const { return ccg::UpperRows{up_v, up_row, up_len, up_pos, up_n, up_units}; }
+  uint32_t* up_epos = nullptr;
+  int64_t up_n = 0, up_units = 0, up_edges = 0;
+  ccg::UpperRows upper() const { return ccg::UpperRows{up_v, up_row, up_len, up_pos, up_epos, up_n, up_units, up_edges}; }
   // cached workspaces (grown on demand)
   void* perm_ws = nullptr;
   size_t perm_ws_bytes = 0;

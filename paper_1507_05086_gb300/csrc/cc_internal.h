@@ -33,21 +33,22 @@ struct RoundStat {
 };
 
 // Plan of the next phase, published by the coordinator block at every grid
-// barrier (128 bytes, copied by every block with one vector load).
+// barrier.
 struct Plan {
   int64_t k, need, win_lo, win_len;
-  int64_t take, act_n, act_E, new_n;
-  int64_t new_E, b_n, b_E, undecided;
-  int32_t th, r0, pad3, pad4;
-  int32_t state, pad0, tag, pad2;      // tag: removal tag of the current round
+  int64_t take, act_n, act_E, long_n;
+  int64_t long_E, b_n, b_E, undecided;
+  int32_t th, r0, d_lb, by_warp;
+  int16_t pad0, hv_sel;                // hv_sel: buffer of the heavy list
+  int32_t state, tag, drop;            // tag: removal tag of the current round
 };
 static_assert(sizeof(Plan) == 128, "plan layout");
-static_assert(offsetof(Plan, state) == 112, "the state word opens the last 16 bytes of the plan");
+constexpr int kPlanCopies = 8;
 
 // Device control block of one clustering job.  Zeroed by the host before
 // each launch; written by the kernels only.
 struct Ctl {
-  unsigned arrive, gen;           // grid barrier (monotonic counters)
+  unsigned long long arrive;      // grid barrier (monotonic counter; the top bit: an error)
   int err;
   int algo;                       // 1 / 2: C4 / ClusterWild!; 3 / 4: the same with the Sec. 5 schedule
   int64_t eps_ppm;
@@ -55,18 +56,22 @@ struct Ctl {
   // test hook: 1 + the round after which the coordinator withholds its
   // release, so that every other block's bounded wait runs out (0: off)
   int32_t withhold;
-  alignas(16) Plan plan;
+  // the published plan: word i in the low half, the barrier's number above it
+  alignas(256) unsigned long long plan_ll[kPlanCopies * sizeof(Plan) / 4];
   // per-round counters, written by every block (lists pack items << 33 | edges)
-  unsigned long long act_pack, new_pack, blk_pack;
-  long long r_centers, r_attached, r_noncenter, r_blocked;
+  unsigned long long act_pack, long_pack, blk_pack;
+  long long r_centers, r_attached, r_noncenter, r_blocked, r_edges;
   long long undecided;
   unsigned long long h_pack;      // heavy-list appends
+  unsigned long long nz_pack;     // alive non-isolated vertices counted
   unsigned long long blk_maxlen;  // C4: longest row of a blocked active this round
   int32_t r0;
   int64_t cursor_next;
-  // objective tallies: member-center edges, member-member edges (counted from
-  // both ends), sum over clusters of C(size, 2)
-  unsigned long long mc, mm, pairs;
+  // exact Delta: the largest degree recounted, the largest bound of an alive
+  // heavy-list vertex that was / was not listed for the recount
+  int32_t best, listed_max, other_max;
+  // objective tallies: edges inside clusters, sum over clusters of C(size, 2)
+  unsigned long long intra, pairs;
   // results, written by the coordinator at the end
   int64_t round, n_alive;
   int done;
@@ -94,14 +99,16 @@ Tuning batch_settings(int64_t* small_n, int64_t* team_n, int* team_blocks);
 
 // The upper part of every row (columns above the row's vertex), which holds
 // each edge once: per row with a non-empty upper part its vertex, the CSR
-// position and length of the part and its first unit (unit_walk in
-// cc_device.cuh).  The objective walks it.
+// position and length of the part, its first unit (unit_walk in
+// cc_device.cuh) and the entries before it (row_walk; batched jobs, whose rows
+// are short).  The objective walks it.
 struct UpperRows {
   const int32_t* v;
   const int64_t* row;
   const int32_t* len;
   const uint32_t* pos;
-  int64_t n, units;
+  const uint32_t* epos;
+  int64_t n, units, edges;
 };
 
 struct RoundBuffers {
@@ -113,20 +120,21 @@ struct RoundBuffers {
   uint32_t* st;                // per-vertex state word
   uint32_t* rtag;              // per-vertex removal tag, 4 bits (8 vertices per word)
   int32_t* arank;              // rank of a vertex while it is active
-  // row lists (see RowList in cc_device.cuh): vertex, first virtual edge,
-  // CSR delta; actives also keep their rank, the blocked list stores the
-  // active-list index in place of a vertex
+  // the actives: vertex, rank, entries before the row (row_walk in
+  // cc_device.cuh), CSR row start, row length.  (C4 without rounds: act_e / act_d as in RowList.)
+  // The blocked list holds active-list indices, entries before the row and
+  // (CSR row start) - that.  Between rounds act_n counts the alive entries of the
+  // long heavy rows, which the blocked list's arrays then hold (length in pull).
   int32_t* act_v;
   int32_t* act_r;
   int64_t* act_e;
   int64_t* act_d;
-  int32_t* new_v;
-  int64_t* new_e;
-  int64_t* new_d;
+  int32_t* act_n;
+  unsigned* h_acc;             // recount of a short heavy list: alive entries per list slot
   int32_t* size;
-  int32_t* hv;                 // heavy list (Delta candidates)
-  int32_t* nz0;                // alive non-isolated vertices (double buffer)
-  int32_t* nz1;
+  int32_t* hv;                 // heavy list (Delta candidates), two buffers
+  int32_t* hv2;
+  int32_t* nz0;                // alive non-isolated vertices, a segment per block
   const int32_t* nz_static;    // the graph's non-isolated vertices
   int64_t nz_n;
   // the graph's non-isolated vertices by degree, largest first, and the
@@ -134,6 +142,7 @@ struct RoundBuffers {
   // rebuild reads the prefix that can still hold the maximum)
   const int32_t* dsort;
   const int64_t* dge;
+  UpperRows up;                // the graph's edges, each once (objective)
   uint8_t* blk_flag;
   uint8_t* hit_c;
   uint8_t* hit_p;
@@ -162,6 +171,7 @@ struct BatchJob {
   int64_t nz_n;
   const int32_t* dsort;
   const int64_t* dge;
+  UpperRows up;
   int64_t n, nnz;
   int32_t max_deg;
   int32_t err;          // result: device status (0 = ok, 1 = not run)
@@ -187,12 +197,14 @@ size_t rounds_workspace_bytes(int64_t n, int32_t max_deg, int grid);
 // Carve a workspace of rounds_workspace_bytes() into RoundBuffers (pointers only).
 void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* b);
 // Largest co-resident grid for the persistent round kernel on this device.
-int rounds_grid_size(int device);
+int rounds_grid_size(int device, int64_t nnz);
 cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint64_t seed, int grid,
                           cudaStream_t stream, int32_t withhold = 0);
 // labels_out[v] = center vertex id (order[center rank]) when labels_out is
-// not null; always adds the pair term sum_c C(s_c, 2) to ctl->pairs.
-cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, cudaStream_t stream);
+// not null; with `objective` also the two terms of D: ctl->pairs = sum_c
+// C(s_c, 2) and ctl->intra = the number of edges inside clusters.
+cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, bool objective, int num_sms,
+                                   cudaStream_t stream);
 
 // ---- objective and validation (cc_objective.cu) ------------------------------
 size_t objective_workspace_bytes(int64_t n);
@@ -201,11 +213,11 @@ size_t objective_workspace_bytes(int64_t n);
 cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows& up,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream);
-// *out += the number of edges (u, w) with id[u] == id[w]; `sig` (or null): a
+// *out += the number of edges (u, w) with id[u] == id[w] in [lo, hi); `sig` (or null): a
 // 4-bit signature of id per vertex, eight to a word, that is equal when the
 // ids are.
-cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id,
-                         const uint32_t* sig, unsigned long long* out, int num_sms, cudaStream_t stream);
+cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id, const uint32_t* sig, uint32_t lo,
+                         uint32_t hi, unsigned long long* out, int num_sms, cudaStream_t stream);
 // Vertices above which the objective reads signatures before ids.
 bool intra_wants_signatures(int64_t n);
 size_t validate_workspace_bytes();
@@ -237,10 +249,12 @@ size_t nonempty_workspace_bytes(int64_t n);
 // writes the starts).
 cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row, int64_t* nz_pos, int64_t* up_at,
                                  void* ws, int64_t* count_dev, int num_sms, cudaStream_t stream);
-// The arrays of UpperRows from up_at; *count_dev = rows << kPackShift | units.
+// The arrays of UpperRows from up_at; count_dev[0] = rows << kPackShift | units,
+// count_dev[1] = their entries.
 // ws: nonempty_workspace_bytes(nz_n).
 cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
-                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos, void* ws,
+                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos,
+                              uint32_t* epos, void* ws,
                               unsigned long long* count_dev, int num_sms, cudaStream_t stream);
 
 }  // namespace ccg

@@ -48,7 +48,7 @@ __global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int
   if (threadIdx.x == 0 && pairs) atomicAdd(out + 1, (unsigned long long)pairs);
 }
 
-// Edges (u, w) with id[u] == id[w], every edge read from its lower end only
+// Edges (u, w) with id[u] == id[w] in [lo, hi), every edge read from its lower end only
 // (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 23
 // (130M edges, 0.49 ms, 265e9 edges/s) L2 runs at 65 % and L1 at 70 % of their
 // throughput, above the 236e9 reads/s of a library gather from a 32 MiB table.
@@ -60,6 +60,7 @@ __global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int
 // four units per batch at three blocks: 0.37 / 1.41 / 5.7.
 template <bool kSig>
 __global__ void __launch_bounds__(kObjThreads, kObjBlocks) k_intra(UpperRows up, const int32_t* __restrict__ col,
+                                                      uint32_t lo, uint32_t hi,
                                                       const uint32_t* __restrict__ id,
                                                       const uint32_t* __restrict__ sig, unsigned long long* out) {
   __shared__ int64_t scr[33];
@@ -67,8 +68,9 @@ __global__ void __launch_bounds__(kObjThreads, kObjBlocks) k_intra(UpperRows up,
   unit_walk((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, ((int64_t)gridDim.x * blockDim.x) >> 5, up.n,
             up.units, col, WalkShape{}, [&](int64_t j) { return __ldg(up.pos + j); },
             [&](int64_t j) {
+              const uint32_t x = __ldg(id + __ldg(up.v + j));
               return UnitItem{__ldg(up.pos + j), __ldg(up.len + j), __ldg(up.row + j),
-                              (int32_t)__ldg(id + __ldg(up.v + j))};
+                              (int32_t)(x >= lo && x < hi ? x : 0xFFFFFFFFu)};
             },
             [&](const UnitBatch& X) {
     uint32_t x[kUnitB];
@@ -256,27 +258,30 @@ __global__ void k_nz_write(int64_t n, const int64_t* __restrict__ off, const int
 }
 
 // Rows with a non-empty upper part, by the same three steps; counts are
-// packed (rows << kPackShift | units).
+// packed (rows << kPackShift | units); the entries are counted beside them.
 __device__ __forceinline__ int64_t upper_len(int64_t j, int64_t nz_n, int64_t nnz, const int64_t* nz_pos,
                                              const int64_t* up_at) {
   return j < nz_n ? (j + 1 < nz_n ? nz_pos[j + 1] : nnz) - up_at[j] : 0;
 }
 
 __global__ void k_up_count(int64_t nz_n, int64_t nnz, const int64_t* __restrict__ nz_pos,
-                           const int64_t* __restrict__ up_at, int64_t* __restrict__ tile_cnt) {
+                           const int64_t* __restrict__ up_at, int64_t* __restrict__ tile_cnt,
+                           int64_t* __restrict__ tile_len) {
   __shared__ int64_t scr[33];
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int64_t len = upper_len(t * kNzTile + threadIdx.x, nz_n, nnz, nz_pos, up_at);
     const int64_t c = block_sum<int64_t>(len > 0 ? (int64_t(1) << kPackShift) | units_of(len) : 0, scr);
-    if (threadIdx.x == 0) tile_cnt[t] = c;
+    const int64_t e = block_sum<int64_t>(len, scr);
+    if (threadIdx.x == 0) { tile_cnt[t] = c; tile_len[t] = e; }
   }
 }
 
 __global__ void k_up_write(int64_t nz_n, int64_t nnz, const int32_t* __restrict__ nz_row,
                            const int64_t* __restrict__ nz_pos, const int64_t* __restrict__ up_at,
-                           const int64_t* __restrict__ tile_off, int32_t* __restrict__ v, int64_t* __restrict__ row,
-                           int32_t* __restrict__ len, uint32_t* __restrict__ pos) {
+                           const int64_t* __restrict__ tile_off, const int64_t* __restrict__ tile_len_off,
+                           int32_t* __restrict__ v, int64_t* __restrict__ row, int32_t* __restrict__ len,
+                           uint32_t* __restrict__ pos, uint32_t* __restrict__ epos) {
   __shared__ int64_t scr[33];
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -284,6 +289,7 @@ __global__ void k_up_write(int64_t nz_n, int64_t nnz, const int32_t* __restrict_
     const int64_t l = upper_len(j, nz_n, nnz, nz_pos, up_at);
     int64_t tot;
     const int64_t ex = block_exclusive_sum<int64_t>(l > 0 ? (int64_t(1) << kPackShift) | units_of(l) : 0, scr, &tot);
+    const int64_t ee = block_exclusive_sum<int64_t>(l, scr, &tot);
     if (l > 0) {
       const uint64_t at = (uint64_t)(tile_off[t] + ex);
       const int64_t o = (int64_t)(at >> kPackShift);
@@ -291,6 +297,7 @@ __global__ void k_up_write(int64_t nz_n, int64_t nnz, const int32_t* __restrict_
       row[o] = up_at[j];
       len[o] = (int32_t)l;
       pos[o] = (uint32_t)(at & kPackEdgeMask);
+      epos[o] = (uint32_t)(tile_len_off[t] + ee);
     }
   }
 }
@@ -429,13 +436,13 @@ size_t objective_workspace_bytes(int64_t n) {
 }
 
 cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id, const uint32_t* sig,
-                         unsigned long long* out, int num_sms, cudaStream_t stream) {
+                         uint32_t lo, uint32_t hi, unsigned long long* out, int num_sms, cudaStream_t stream) {
   if (up.units <= 0) return cudaSuccess;
   const int64_t per = kObjThreads / 32 * kUnitB;
   const int64_t want = (up.units + per - 1) / per;
   const int g = (int)(want < (int64_t)num_sms * kObjBlocks ? want : (int64_t)num_sms * kObjBlocks);
-  if (sig) k_intra<true><<<g, kObjThreads, 0, stream>>>(up, col, id, sig, out);
-  else k_intra<false><<<g, kObjThreads, 0, stream>>>(up, col, id, nullptr, out);
+  if (sig) k_intra<true><<<g, kObjThreads, 0, stream>>>(up, col, lo, hi, id, sig, out);
+  else k_intra<false><<<g, kObjThreads, 0, stream>>>(up, col, lo, hi, id, nullptr, out);
   return cudaGetLastError();
 }
 
@@ -457,7 +464,7 @@ cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows&
     sig = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + align_up(4 * (size_t)n));
     k_signatures<<<g, 256, 0, stream>>>(n, id, sig);
   }
-  return launch_intra(col, up, id, sig, out, num_sms, stream);
+  return launch_intra(col, up, id, sig, 0u, 0xFFFFFFFFu, out, num_sms, stream);
 }
 
 size_t validate_workspace_bytes() { return align_up(8 * sizeof(unsigned long long)) + align_up(2 * sizeof(int)); }
@@ -499,7 +506,7 @@ cudaError_t launch_offsets_i32_to_i64(int64_t n, const int32_t* in, int64_t* out
 
 size_t nonempty_workspace_bytes(int64_t n) {
   const int64_t ntiles = (n + kNzTile - 1) / kNzTile;
-  return align_up(8 * (size_t)(ntiles + 1)) + align_up(8);
+  return 2 * align_up(8 * (size_t)(ntiles + 1)) + align_up(8);
 }
 
 // nz_row/nz_pos get the non-empty rows and their first CSR positions; the
@@ -517,15 +524,18 @@ cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row,
 }
 
 cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, const int64_t* nz_pos,
-                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos, void* ws,
-                              unsigned long long* count_dev, int num_sms, cudaStream_t stream) {
-  if (nz_n <= 0) return cudaMemsetAsync(count_dev, 0, sizeof(unsigned long long), stream);
+                              const int64_t* up_at, int32_t* v, int64_t* row, int32_t* len, uint32_t* pos,
+                              uint32_t* epos, void* ws, unsigned long long* count_dev, int num_sms,
+                              cudaStream_t stream) {
+  if (nz_n <= 0) return cudaMemsetAsync(count_dev, 0, 2 * sizeof(unsigned long long), stream);
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   int64_t* tile = static_cast<int64_t*>(ws);
+  int64_t* tile_len = tile + align_up(8 * (size_t)(ntiles + 1)) / 8;
   const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
-  k_up_count<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_pos, up_at, tile);
+  k_up_count<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_pos, up_at, tile, tile_len);
   k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, reinterpret_cast<int64_t*>(count_dev));
-  k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, v, row, len, pos);
+  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile_len, reinterpret_cast<int64_t*>(count_dev + 1));
+  k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, tile_len, v, row, len, pos, epos);
   return cudaGetLastError();
 }
 

@@ -5,12 +5,12 @@
 // barriers; block 0 is the coordinator: at every barrier it waits for all
 // blocks, does the serial bookkeeping of the round (Delta walk, batch size,
 // selection windows, statistics) on state it keeps in its own shared memory,
-// publishes a 128-byte plan and releases the others, which copy the plan with
-// one vector load.  Every wait is bounded.  The host is not involved between
+// publishes a 128-byte plan, whose words carry the barrier's number and so
+// release the others.  Every wait is bounded.  The host is not involved between
 // rounds.
 //
 // Per-vertex state: one 32-bit word st[v]
-//   alive ............ kAlive | residual degree
+//   alive ............ kAlive | bound of the residual degree
 //   clustered ........ kLab + center rank
 //   active ............ kActive / kActCenter / kActNon (undecided or
 //                       ClusterWild! center / C4 center / C4 non-center)
@@ -23,27 +23,28 @@
 // active markers below, so one compare-then-atomicMin does rule 2 and skips
 // clustered and active vertices.
 //
-// Residual degrees live in the alive word itself, so the decrement that
-// follows the removal of a vertex is a fire-and-forget atomic on that word.
-// The alive tests of the hot passes read a separate removal tag instead:
-// 4 bits per vertex, 0 while alive, else 1 + (removal round mod 15), an
-// eighth of the state words' footprint, so the random reads of the edge
-// passes and of the selection scans mostly hit L2.  A tag equal to the
-// current round's only says "maybe removed this round" (a vertex removed
-// 15, 30, ... rounds earlier carries it too); the state word decides.
+// The alive word holds an upper bound of the residual degree: the full degree
+// at first, later the exact residual degree as of the vertex's last recount
+// (degrees only fall, so a value once exact stays a bound).  Nothing is
+// decremented when a vertex leaves; only the few vertices that can hold the
+// maximum are recounted, once per round (see co_delta).
+// The alive tests of the adjacency passes and of the selection scans read a
+// removal tag instead of the state word: 4 bits per vertex, 0 while alive,
+// else 1 + (removal round mod 15), an eighth of the state words' footprint, so
+// that the random reads mostly hit L2.  A tag equal to the current round's
+// only says "maybe removed this round" (a vertex removed 15, 30, ... rounds
+// earlier carries it too); the state word decides.
 //
-// Delta_i (max residual degree, exact every round) comes from a heavy list H:
-// every alive vertex whose degree was >= tau when H was built.  Degrees only
-// fall, so if the largest current degree in H is still >= tau it is the
-// maximum over the whole graph; otherwise a rebuild scans the compact list of
-// alive non-isolated vertices, takes the exact maximum D, sets tau = D/2 and
-// refills H.  No work per decrement.  Selection scans pi itself from a cursor
-// (entry i is the vertex of rank i) and skips removed vertices by their tag;
-// a selected vertex of residual degree 0 is a singleton center for which
+// Delta_i (max residual degree, exact every round) comes from a heavy list H
+// that holds every alive vertex whose bound was >= tau when H was built: the
+// rows of H's vertices with the largest bounds are recounted until the largest
+// exact degree found is at least every other bound.  Selection scans pi itself
+// from a cursor (entry i is the vertex of rank i) and skips removed vertices
+// by their tag; a selected vertex of bound 0 is a singleton center for which
 // nothing is written (the label pass reads its alive word of degree 0).
 //
-// Every adjacency pass is edge-balanced (lbs_for_each), so hub rows of
-// power-law graphs are split across many warps.
+// Every adjacency pass is edge-balanced (row_walk), so hub rows of power-law
+// graphs are split across many warps.
 #include <cstdint>
 
 #include "cc_device.cuh"
@@ -53,13 +54,28 @@ namespace ccg {
 namespace {
 
 constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
+constexpr int kRowB = 4;                     // entries in flight per lane (8 spill at 64 registers)
 constexpr int kScanU = 4;                    // list entries per thread per scan step
 constexpr int kSelU = 2;                     // window entries per thread per selection step
+// Up to this many vertices (64 MB of state words, which L2 holds) selection
+// also reads the bounds and spares the rows of vertices known to have no alive
+// neighbour; above, those rows cost less than a random DRAM read per active.
+constexpr int64_t kStateInL2 = int64_t(1) << 24;
 constexpr int64_t kDescStride = 16;          // look-back descriptors: one per 128-byte line
 constexpr int kAlgoC4 = 1, kAlgoCW = 2;
-constexpr int kRun = 0, kDone = 1, kAbort = 3, kRebuildDelta = 4, kScanH = 5, kDrawBatch = 6;
-constexpr int kRebuildDeg = 7, kRebuildHeavy = 8;   // Delta search over the degree order, heavy refill
+constexpr int kRun = 0, kDone = 1, kSelect = 2, kAbort = 3, kDrawBatch = 6;   // kRun: the active set is there
+constexpr int kRebuildOrder = 7, kRebuildAlive = 8; // heavy list from the degree order, from the alive vertices
+constexpr int kRecount = 9, kRecountLong = 10;      // degree recounts
+// where co_delta takes up again, or what it does next
+constexpr int kDScan = 0, kDCounted = 1, kDRebuild = 2, kDPlanned = 3, kDDone = 4;
+constexpr int kHList = kThreads;             // heavy lists up to this long: every block lists all of them
+constexpr int kHere = 16 * kThreads;         // heavy lists up to this long are looked at inside the barrier
+constexpr int kHRows = 1024;                 // rows that one block recounts at once
+constexpr int kHPick = 4096;                 // vertices that one block picks at once
+constexpr int kInlineWindow = 1024;          // selection windows up to this long are scanned inside the barrier
+constexpr int kInlineEdges = 8192;           // recounts up to this many entries run inside the barrier
+constexpr int32_t kLongRow = 1024;           // rows above this are not recounted by one block alone
+constexpr int32_t kTightest = 8;             // heavy lists reach down to 1 - 2^-8 of the largest bound at most
 // Defaults of the run-time schedule settings (Tuning; cc_tuning in the C ABI)
 constexpr int32_t kInlineH = 8192;           // heavy lists up to this size are scanned by the coordinator
 constexpr int32_t kInlineDecide = 4096;      // C4 blocked lists up to this size are decided by the coordinator
@@ -70,7 +86,7 @@ constexpr int32_t kHeavyShift = 1;           // heavy-list threshold tau = max(1
 constexpr int32_t kWarpResolveRow = 1024;
 
 // State word of a vertex (uint32):
-//   alive ........... kAlive | residual degree
+//   alive ........... kAlive | bound of the residual degree
 //   clustered ....... kLab + center rank
 //   active this round kActive (undecided, or a ClusterWild! center),
 //                     kActCenter / kActNon (C4 center / non-center)
@@ -80,6 +96,11 @@ constexpr int kTagCycle = 15;                // removal tags 1..15
 __device__ __forceinline__ bool is_alive(uint32_t x) { return x >= kAlive; }
 __device__ __forceinline__ uint32_t deg_of(uint32_t x) { return x & kDegMask; }
 __device__ __forceinline__ bool is_active(uint32_t x) { return x < kLab; }
+
+// The cluster of a member as the objective compares it: its state word; a
+// center or singleton matches nothing (member-center edges are counted by
+// finish_vertices).
+__device__ __forceinline__ uint32_t member_id(uint32_t x) { return x >= kLab && x < kAlive ? x : 0xFFFFFFFFu; }
 
 __device__ __forceinline__ int64_t rtag_words(int64_t n) { return (n >> 3) + 1; }
 __device__ __forceinline__ uint32_t rtag_of(const uint32_t* rtag, int32_t v) {
@@ -117,7 +138,7 @@ __device__ __forceinline__ uint64_t sec5_threshold(int64_t eps_ppm, int64_t dhat
   *all = (uint64_t)eps_ppm >= den;
   if (*all) return ~0ull;
   uint64_t r = (uint64_t)eps_ppm, t = 0;
-#pragma unroll
+#pragma unroll 1
   for (int s = 0; s < 5; ++s) {
     r <<= 12;
     t = (t << 12) | (r / den);
@@ -135,9 +156,17 @@ __device__ __forceinline__ uint64_t sec5_draw(uint64_t s, uint64_t j) {
 template <class T>
 __device__ __forceinline__ T vload(const T* p) { return *reinterpret_cast<const volatile T*>(p); }
 
-__device__ __forceinline__ void atom_add_release(unsigned* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void atom_add_release(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+constexpr unsigned long long kArriveError = 1ull << 63;
+
+constexpr int kPlanWords = sizeof(Plan) / 4;
+// Teams above kPlanAlone blocks wait on kPlanCopies copies of the plan: the 300
+// blocks of a grid polling one copy keep its L2 slice busy for longer than a
+// copy costs.
+constexpr unsigned kPlanAlone = 32;
+static_assert(kPlanWords == 32, "one warp reads the plan");
 
 // Coordinator state, in block 0's shared memory for the whole kernel.
 struct Coord {
@@ -145,16 +174,21 @@ struct Coord {
   int64_t need, win_lo, win_len, r_edges, fix_iter;
   int64_t clusters;              // centers opened so far
   int64_t h_len;                 // heavy list length
-  int64_t nz_len, nz_total;      // compact list of alive non-isolated vertices
-  int64_t rb_lo, rb_hi;          // degree-order search: next segment of the prefix
-  int32_t rb_t, rb_D;            // every vertex of full degree >= rb_t read; largest current degree seen
-  int32_t tau, delta, max_deg, d_new;
+  int64_t nz_len;                // alive non-isolated vertices, as of the last look at all of them
+  int32_t tau, delta, max_deg;
+  int32_t d_lb;                  // largest exact degree recounted this round (-1: none)
+  int32_t d_th;                  // heavy-list vertices of this bound or more are recounted
+  int32_t d_other;               // largest bound among the others
+  int32_t tight;                 // the heavy list reaches down to ub - (ub >> tight)
+  int32_t tau_next;              // the raised tau of a planned look
+  int32_t hv_sel;                // which of the two heavy-list buffers is current
+  int32_t d_top, d_drop;         // largest bound at the first look; how far Delta fell below it lately
   int algo, rebuilds_in_row;
-  int nz_sel, nz_static;
   int delta_zero;                // a rebuild found no alive vertex with an alive neighbour
   int est;                       // the Sec. 5 schedule: Delta-hat and binomial batches
   int64_t period, rank_cursor;   // rounds per halving of Delta-hat; ranks of pi passed
   int32_t withhold;              // test hook (Ctl::withhold)
+  int32_t round_ended;           // this barrier ended a round
   int64_t batch_end;             // rank (index in pi) that ends the round's batch
   unsigned long long t0, round_t0;
   unsigned long long ph_ns[8];
@@ -176,64 +210,105 @@ struct PermSmem {
   int32_t hist[kPermMaxBuckets];
 };
 
+// Round tallies of a block (Shared::tal), added up over the team at the end of
+// a round.
+enum { kTCenters = 0, kTAttached, kTNonCenter, kTBlocked, kTEdges, kTallies };
+
+// Rows to be recounted (slot order = heavy-list order).
+struct HeavyList {
+  int64_t pos[kHRows];
+  int64_t row[kHRows];
+  int32_t len[kHRows];
+  int32_t v[kHRows];             // -1: recounted elsewhere
+  unsigned cnt[kHRows];          // alive entries found (recount by one block)
+  int32_t pick[kHPick];          // vertices whose rows are recounted next
+};
+
 struct Shared {
   Plan plan;
   Coord co;
   int ok;
+  int failed;                    // this block has recorded an error
   int dec;
   int64_t scr[33];
   int64_t bcast[8];
-  unsigned long long tal[5];     // round tallies of the block (flushed at round end)
+  unsigned long long tal[kTallies];     // round tallies of the block (flushed at round end)
+  int32_t scr32[32];
+  // the selection's outcome: alive entries of the window, the round's first
+  // active rank, the next cursor, the active list (items << 33 | entries)
+  int64_t sel_total, sel_cursor;
+  int32_t sel_r0;
+  unsigned long long sel_pack;
+  int32_t h_picked, h_kept;      // vertices picked for the recount; entries of a compacted list
+  int32_t h_best;                // largest exact degree that this block knows of
+  int64_t nz_cnt;                // alive non-isolated vertices of this block's segment (-1: not looked at yet)
   union {
-    struct {
-      LbsWarp lbs[kWarps];
-      AppendBuf app[kWarps];
-    } w;
+    HeavyList hl;
     PermSmem perm;
   } u;
 };
 
-// Per-thread tallies of one round (flushed at every round end).
-// The member-center edges of the objective need no tally: every member of a
-// cluster is adjacent to its center (it was attached through that edge) and
-// to no other center of its cluster, so they number n - (number of clusters).
-struct Tally {
-  int32_t centers, attached, noncenter, blocked;
-  uint32_t mm;                  // member-member entries inside a cluster
-};
-
 // The blocks that run one clustering job: the whole grid, or a team of
 // G blocks inside a batched launch (bid = this block's rank in the team).
+// It lives in shared memory: the passes are functions of their own (each with
+// its own register allocation), and from there they read a field in one step.
+template <int kPerSM>
 struct K {
-  const RoundBuffers& B;
+  RoundBuffers B;
   Ctl* C;
   Shared* S;
   unsigned G;
   unsigned bid;
   unsigned epoch;
-  Tally t;
+  int algo;                      // C4 or ClusterWild!
 
-  template <class F>
-  __device__ __forceinline__ void lbs(const int64_t* epos, int64_t nitems, int64_t E, F&& f,
-                                      const int64_t* delta = nullptr, const int32_t* vtx = nullptr,
-                                      const uint32_t* vmap = nullptr, uint32_t vsub = 0) {
-    // every walk with a delta array walks CSR rows: stream them ahead.
-    // Warps are numbered across the blocks first (warp w of block b is
-    // w * G + b), so a short walk spreads over every SM instead of the
-    // first few blocks.
-    lbs_for_each_in((int64_t)(threadIdx.x >> 5) * G + bid, ((int64_t)G * blockDim.x) >> 5, epos, nitems,
-                    E, lbs_ws(), f, delta, vtx, 0, vmap, vsub, delta ? B.col : nullptr,
-                    WalkShape{B.tune.walk_batches, B.tune.prefetch_ahead});
+  // One round tally of this block; all lanes of the warp call it.
+  __device__ __forceinline__ void tally(int which, int32_t x) {
+    const int32_t sum = __reduce_add_sync(FULL, x);
+    if (sum && (threadIdx.x & 31) == 0) atomicAdd(&S->tal[which], (unsigned long long)sum);
+  }
+  // Block-wide sums as one copy of the code (see sync).
+  struct Scan {
+    int64_t ex, tot;
+  };
+  __device__ __noinline__ Scan scan(int64_t x) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t inc = warp_inclusive_sum_rolled(x);
+    __syncthreads();                       // earlier readers of scr
+    if (lane == 31) S->scr[warp] = inc;
+    __syncthreads();
+    const int64_t w = lane < kThreads / 32 ? S->scr[lane] : 0, wi = warp_inclusive_sum_rolled(w);
+    return Scan{__shfl_sync(FULL, wi - w, warp) + inc - x, __shfl_sync(FULL, wi, 31)};
+  }
+  __device__ __noinline__ int32_t sum_i32(int32_t x) { return block_sum_i32(x, S->scr32); }
+  __device__ __noinline__ int32_t max_i32(int32_t x) { return block_max_i32(x, S->scr32); }
+
+  // This warp among the team's warps.
+  __device__ __forceinline__ int team_warp() const { return (int)((threadIdx.x >> 5) * G + bid); }
+  __device__ __forceinline__ int team_warps() const { return (int)((G * blockDim.x) >> 5); }
+
+  // A walk of the team over the E entries of n rows.  Warps are numbered across
+  // the blocks first (warp w of block b is w * G + b), so a short walk spreads
+  // over every SM instead of the first few blocks.
+  // A walk of at most two batches of 32 entries per warp takes one entry per
+  // lane at a time: a third of the code, which such a walk spends its time
+  // fetching (f takes either batch).
+  template <class At, class Load, class F>
+  __device__ __forceinline__ void walk(int64_t n, int64_t E, const At& at, const Load& load, F&& f) {
+    const WalkShape shape{B.tune.walk_batches, B.tune.prefetch_ahead};
+    if (E <= 64 * (int64_t)team_warps()) row_walk<1>(team_warp(), team_warps(), (int32_t)n, E, B.col, shape, at, load, f);
+    else row_walk<kRowB>(team_warp(), team_warps(), (int32_t)n, E, B.col, shape, at, load, f);
   }
 
   __device__ __forceinline__ const Plan& P() const { return S->plan; }
-  // heavy-list threshold for a maximum degree D
-  __device__ __forceinline__ int32_t tau_of(int32_t D) const {
-    const int32_t t = D >> B.tune.heavy_shift;
-    return t >= 1 ? t : 1;
-  }
+  // The current heavy list (its buffer changes when the grid cuts it down).
+  __device__ __forceinline__ int32_t* hv() const { return S->plan.hv_sel ? B.hv2 : B.hv; }
   __device__ __forceinline__ Coord& co() const { return S->co; }
-  __device__ void fail(int code) { atomicCAS(&C->err, kOk, code); }
+  // Records an error; the coordinator sees it in the arrivals.
+  __device__ __noinline__ void fail(int code) {
+    if (atomicCAS(&C->err, kOk, code) == kOk) atomicOr(&C->arrive, kArriveError);
+    S->failed = 1;
+  }
 
   // ---------------- grid barrier with the coordinator -------------------------
   // All blocks call sync(); block 0 waits for every arrival, books the time
@@ -241,110 +316,118 @@ struct K {
   // block (writing S->plan), publishes the plan and releases.  The others
   // wait for the release and copy the plan.  Returns false once the run
   // must stop (error, or the plan says so).
+  // The waits are functions of their own: a phase is mostly straight-line code
+  // that runs once, so what the phases share should be fetched once.
   template <class A>
-  __device__ bool sync(int cat, A&& act) {
+  __device__ __forceinline__ bool sync(int cat, A&& act) {
+    if (bid != 0) return wait_release();
+    if (co_arrived(cat)) act();
+    return co_release();
+  }
+
+  // Coordinator: waits for every arrival; false after an error.
+  __device__ __noinline__ bool co_arrived(int cat) {
     __syncthreads();
-    ++epoch;
-    if (G == 1) {                       // a one-block team is its own coordinator
-      if (threadIdx.x == 0) {
-        const unsigned long long now = globaltimer_ns();
-        S->co.ph_ns[cat] += now - S->co.t0;
-        S->co.t0 = now;
-      }
-      __syncthreads();
-      if (ld_volatile_int(&C->err) == kOk) act();
-      __syncthreads();
-      if (threadIdx.x == 0 && ld_volatile_int(&C->err) != kOk) S->plan.state = kAbort;
-      __syncthreads();
-      return S->plan.state != kAbort;
-    }
-    if (threadIdx.x == 0) atom_add_release(&C->arrive, 1u);
-    if (bid == 0) {
-      if (threadIdx.x == 0) {
-        const unsigned target = G * epoch;
+    if (threadIdx.x == 0) {
+      ++epoch;
+      int ok = 1;
+      if (G > 1) {
+        atom_add_release(&C->arrive, 1ull);
+        const unsigned long long target = (unsigned long long)G * epoch;
         const uint64_t t0 = globaltimer_ns();
         unsigned spins = 0;
-        int ok = 1;
-        while (ld_acquire(&C->arrive) < target) {
-          if ((++spins & 63) == 0) {
-            if (ld_volatile_int(&C->err) != kOk) { ok = 0; break; }
-            if (globaltimer_ns() - t0 > kBarrierLimitNs) { atomicCAS(&C->err, kOk, kErrTimeout); ok = 0; break; }
-          }
+        unsigned long long x;
+        while ((x = ld_relaxed_u64(&C->arrive)) < target) {
+          if ((++spins & 63) == 0 && globaltimer_ns() - t0 > kBarrierLimitNs) { fail(kErrTimeout); ok = 0; break; }
         }
-        if (ld_volatile_int(&C->err) != kOk) ok = 0;
-        const unsigned long long now = globaltimer_ns();
-        S->co.ph_ns[cat] += now - S->co.t0;
-        S->co.t0 = now;
-        S->ok = ok;
+        if (x & kArriveError) ok = 0;
+        fence_gpu();
       }
-      __syncthreads();
-      if (S->ok) act();
-      __syncthreads();
+      if (S->failed || (kDebugChecks && ld_volatile_int(&C->err) != kOk)) ok = 0;
+      const unsigned long long now = globaltimer_ns();
+      S->co.ph_ns[cat] += now - S->co.t0;
+      S->co.t0 = now;
+      S->co.round_ended = 0;
+      S->ok = ok;
+    }
+    __syncthreads();
+    return S->ok != 0;
+  }
+
+  // Coordinator: publishes the plan.  Every word goes out in one 8-byte store
+  // with the barrier's number above it, so whoever sees the number has the
+  // word; the fence orders what this block and, through the arrivals, every
+  // block wrote before it.
+  __device__ __noinline__ bool co_release() {
+    __syncthreads();
+    if (threadIdx.x == 0) {
       // an error (here or in any block) travels in the plan as the abort state
-      if (threadIdx.x == 0 && (!S->ok || ld_volatile_int(&C->err) != kOk)) S->plan.state = kAbort;
+      if (!S->ok || S->failed || (kDebugChecks && ld_volatile_int(&C->err) != kOk)) S->plan.state = kAbort;
       // test hook: after the chosen round the release is withheld; the other
       // blocks' bounded waits run out (kErrTimeout) and every block unwinds
-      if (threadIdx.x == 0 && cat == 6 && S->co.withhold != 0 && S->co.round == S->co.withhold) {
+      if (G > 1 && S->co.round_ended && S->co.withhold != 0 && S->co.round == S->co.withhold) {
         S->plan.state = kAbort;
         S->ok = 2;
       }
-      __syncthreads();
-      if (S->ok != 2) {
-        // publish: 128 bytes as eight 16-byte stores, then release
-        if (threadIdx.x < sizeof(Plan) / 16)
-          reinterpret_cast<int4*>(&C->plan)[threadIdx.x] = reinterpret_cast<const int4*>(&S->plan)[threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x == 0) st_release(&C->gen, epoch);
-      }
-    } else {
-      if (threadIdx.x == 0) {
-        const uint64_t t0 = globaltimer_ns();
-        unsigned spins = 0;
-        int released = 1;
-        while (ld_acquire(&C->gen) < epoch) {
-          if ((++spins & 63) == 0) {
-            if (ld_volatile_int(&C->err) != kOk) { released = 0; break; }
-            if (globaltimer_ns() - t0 > kBarrierLimitNs) {
-              atomicCAS(&C->err, kOk, kErrTimeout);
-              released = 0;
-              break;
-            }
-          }
-        }
-        S->ok = released;
-      }
-      __syncthreads();
-      // the plan (its last 16 bytes hold the state word; without a release
-      // the copy is stale and the state becomes the abort state)
-      if (threadIdx.x < sizeof(Plan) / 16) {
-        int4 q = __ldcg(reinterpret_cast<const int4*>(&C->plan) + threadIdx.x);
-        if (threadIdx.x == sizeof(Plan) / 16 - 1 && !S->ok) q.x = kAbort;
-        reinterpret_cast<int4*>(&S->plan)[threadIdx.x] = q;
-      }
-      __syncthreads();
+    }
+    __syncthreads();
+    const unsigned copies = G > kPlanAlone ? kPlanCopies : G > 1 ? 1 : 0;
+    if (S->ok != 2 && threadIdx.x < kPlanWords * copies) {
+      const uint32_t w = reinterpret_cast<const uint32_t*>(&S->plan)[threadIdx.x % kPlanWords];
+      fence_gpu();
+      st_relaxed_u64(C->plan_ll + threadIdx.x, ((unsigned long long)epoch << 32) | w);
     }
     return S->plan.state != kAbort;
   }
+
+  // The other blocks: arrive, wait for the release and take the plan over.
+  __device__ __noinline__ bool wait_release() {
+    __syncthreads();
+    if (threadIdx.x < kPlanWords) {          // the first warp
+      if (threadIdx.x == 0) {
+        ++epoch;
+        atom_add_release(&C->arrive, 1ull);
+      }
+      __syncwarp();
+      const unsigned long long* const src =
+          C->plan_ll + (G > kPlanAlone ? bid % kPlanCopies : 0) * kPlanWords + threadIdx.x;
+      const unsigned e = epoch;
+      const uint64_t t0 = globaltimer_ns();
+      unsigned spins = 0;
+      bool released = true;
+      unsigned long long x = ld_relaxed_u64(src);
+      while (!__all_sync(FULL, (unsigned)(x >> 32) == e)) {
+        if ((++spins & 63) == 0) {
+          if (ld_volatile_int(&C->err) != kOk) released = false;
+          else if (globaltimer_ns() - t0 > kBarrierLimitNs) {
+            fail(kErrTimeout);
+            released = false;
+          }
+          if (__any_sync(FULL, !released)) break;
+        }
+        x = ld_relaxed_u64(src);
+      }
+      fence_gpu();
+      reinterpret_cast<uint32_t*>(&S->plan)[threadIdx.x] = (uint32_t)x;
+      __syncwarp();
+      // without a release the copy is stale and the state becomes the abort state
+      if (__any_sync(FULL, !released) && threadIdx.x == 0) S->plan.state = kAbort;
+    }
+    __syncthreads();
+    return S->plan.state != kAbort;
+  }
+
   __device__ bool sync(int cat) {
     return sync(cat, [] {});
   }
 
-  __device__ RowList new_list() const { return RowList{B.new_v, B.new_e, B.new_d, nullptr, &C->new_pack CC_ROWLIST_CHECK(B.n, &C->err)}; }
   // blocked actives; the payload initialises each one's pull slot (no center yet)
   __device__ RowList blk_list() const { return RowList{B.b_j, B.b_e, B.b_d, B.pull, &C->blk_pack CC_ROWLIST_CHECK(B.n, &C->err)}; }
-  __device__ LbsWarp* lbs_ws() const { return &S->u.w.lbs[threadIdx.x >> 5]; }
-  __device__ AppendBuf* app_buf() const { return &S->u.w.app[threadIdx.x >> 5]; }
-
-  // Entry i of the rank-ordered candidate list: (rank, vertex) = (i, pi(i)).
-  // Selection scans it from the cursor and skips removed vertices by their
-  // removal tag; the list is never compacted (every entry is scanned about
-  // once anyway, so a compaction pass would cost more than it saves).
-  __device__ int2 al_at(int64_t i) const { return make_int2((int32_t)i, __ldg(B.order + i)); }
 
   // contiguous slice of [lo, lo+len) for this block
-  __device__ void slice(int64_t lo, int64_t len, int64_t* s, int64_t* e) const {
-    const int64_t chunk = (len + G - 1) / G;
-    *s = lo + chunk * bid;
+  __device__ __forceinline__ void slice(int64_t lo, int64_t len, int64_t* s, int64_t* e) const {
+    const uint32_t chunk = ((uint32_t)len + G - 1) / G;           // len < 2^31
+    *s = lo + (int64_t)chunk * bid;
     *e = *s + chunk < lo + len ? *s + chunk : lo + len;
     if (*s > *e) *s = *e;
   }
@@ -376,9 +459,11 @@ struct K {
       c.tau = 0x7FFFFFFF;         // empty heavy list: the first round rebuilds it
       c.h_len = 0;
       c.nz_len = B.nz_n;          // non-isolated vertices, from the graph
-      c.nz_static = 1;
-      c.nz_sel = 0;
       c.delta_zero = 0;
+      c.d_drop = 0;
+      c.tight = 1;
+      c.hv_sel = 0;
+      c.r_edges = 0;
       c.round = 0;
       c.clusters = 0;
       c.rebuilds_in_row = 0;
@@ -394,12 +479,15 @@ struct K {
       p = Plan{};
       p.r0 = -1;
     }
+    if (threadIdx.x < kHList) B.h_acc[threadIdx.x] = 0;
     __syncthreads();
-    co_decide_delta();
+    if (threadIdx.x == 0) S->dec = co_next();
+    __syncthreads();
+    co_go_on();
   }
 
   // Coordinator: with Delta known, set k and the first selection window.
-  __device__ void plan_selection(int32_t delta) {
+  __device__ __noinline__ void plan_selection(int32_t delta) {
     if (threadIdx.x == 0) {
       Coord& c = co();
       Plan& p = S->plan;
@@ -417,7 +505,7 @@ struct K {
       c.need = k;
       c.win_lo = c.cursor;
       const int64_t avail = c.al_len - c.cursor;
-      const int64_t est = (int64_t)((double)k * (double)avail / (double)c.n_alive * 1.05) + 256;
+      const int64_t est = (int64_t)((float)k * ((float)avail / (float)c.n_alive) * 1.05f) + 256;   // a guess
       c.win_len = est < avail ? est : avail;
       if (c.est) {
         // Sec. 5: the whole window of the round's batch, every alive entry of it
@@ -425,11 +513,13 @@ struct K {
         c.need = INT64_MAX / 4;
         c.win_len = c.batch_end - c.cursor;
       }
-      c.r_edges = 0;
-      C->act_pack = 0; C->new_pack = 0; C->blk_pack = 0; C->blk_maxlen = 0;
-      C->r_centers = 0; C->r_attached = 0; C->r_noncenter = 0; C->r_blocked = 0;
+      C->act_pack = 0; C->blk_pack = 0; C->blk_maxlen = 0;
+      C->r_centers = 0; C->r_attached = 0; C->r_noncenter = 0; C->r_blocked = 0; C->r_edges = 0;
       C->r0 = -1;
-      p.state = kRun;
+      S->sel_r0 = -1;
+      S->sel_cursor = 0;
+      S->sel_pack = 0;
+      p.state = kSelect;
       p.k = c.k;
       p.need = c.need;
       p.win_lo = c.win_lo;
@@ -439,235 +529,633 @@ struct K {
       p.tag = (int32_t)(c.round % kTagCycle) + 1;
     }
     __syncthreads();
+    select_here();
   }
 
-  // Coordinator, at a round boundary: finish, draw the Sec. 5 batch, or get
-  // Delta from the heavy list (inline when short, else by a grid scan), or
-  // rebuild the heavy list.
-  __device__ __noinline__ void co_decide_delta() {
+  // Coordinator, at a round boundary (thread 0): finish or draw the Sec. 5 batch
+  // (1), a round with Delta known (2), or find Delta (0).
+  __device__ __forceinline__ int co_next() {
     Coord& c = co();
     Plan& p = S->plan;
-    if (threadIdx.x == 0) {
-      int dec = 1;
-      if (c.n_alive <= 0) p.state = kDone;
-      else if (c.est) {
-        p.state = kDrawBatch;             // Sec. 5: draw the batch, no Delta
-        const int64_t dh = sec5_delta_hat(c.max_deg, c.period, c.round);
-        bool all;
-        const uint64_t thr = sec5_threshold(c.eps_ppm, dh, &all);
-        c.delta = (int32_t)dh;
-        p.win_len = c.n - c.rank_cursor;                            // trials
-        p.need = (int64_t)thr;                                      // threshold bits
-        p.take = all ? 1 : 0;
-        p.k = (int64_t)perm_key(vload(&C->seed) ^ 0x5851F42D4C957F2Dull, (uint64_t)c.round);   // stream seed
-      } else if (c.delta_zero) {
-        dec = 2;                          // every alive vertex is isolated: Delta = 0
-      } else if (c.h_len == 0) {
-        dec = 3;                          // no heavy list yet: build it
-      } else if (c.h_len > B.tune.inline_heavy) {
-        p.state = kScanH; p.win_lo = 0; p.win_len = c.h_len;
-      } else {
-        dec = 0;                          // scan the short heavy list here
-      }
-      S->dec = dec;
+    if (c.n_alive <= 0) { p.state = kDone; return 1; }
+    if (c.est) { plan_draw(); return 1; }
+    if (c.round == 0) {                   // every degree is still the full one
+      c.delta = c.max_deg;
+      if (c.max_deg <= 0) c.delta_zero = 1;
+      return 2;
     }
-    __syncthreads();
-    if (S->dec == 2) { plan_selection(0); return; }
-    if (S->dec == 3) {
-      // before the first round every vertex is alive with its full degree:
-      // the search starts at the largest degree, which it finds at once
-      start_rebuild(co().round == 0 ? co().max_deg : 1);
-      return;
+    if (c.delta_zero) {                   // every alive vertex is isolated: Delta = 0
+      c.delta = 0;
+      return 2;
     }
-    if (S->dec) return;
-    // the whole block reads the heavy list, eight entries per thread at a time
-    // so that the dependent loads overlap
-    int64_t mx = -1;
-    for (int64_t base = 0; base < c.h_len; base += 8 * (int64_t)blockDim.x) {
-      int32_t h[8];
-      uint32_t x[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int64_t i = base + threadIdx.x + (int64_t)q * blockDim.x;
-        h[q] = i < c.h_len ? ldcg(B.hv + i) : -1;
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = h[q] >= 0 ? ldcg(B.st + h[q]) : 0u;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (is_alive(x[q])) mx = (int64_t)deg_of(x[q]) > mx ? (int64_t)deg_of(x[q]) : mx;
-    }
-    mx = block_max<int64_t>(mx, S->scr);
-    co_after_heavy((int32_t)mx);
+    // every bound is at most the last Delta: start a little below it
+    c.d_lb = -1;
+    c.d_top = -1;
+    c.d_th = below(c.delta, c.d_drop);
+    return 0;
+  }
+  // Sec. 5: the batch is drawn by the grid; no Delta.
+  __device__ __noinline__ void plan_draw() {
+    Coord& c = co();
+    Plan& p = S->plan;
+    p.state = kDrawBatch;
+    const int64_t dh = sec5_delta_hat(c.max_deg, c.period, c.round);
+    bool all;
+    const uint64_t thr = sec5_threshold(c.eps_ppm, dh, &all);
+    c.delta = (int32_t)dh;
+    p.win_len = c.n - c.rank_cursor;                            // trials
+    p.need = (int64_t)thr;                                      // threshold bits
+    p.take = all ? 1 : 0;
+    p.k = (int64_t)perm_key(vload(&C->seed) ^ 0x5851F42D4C957F2Dull, (uint64_t)c.round);   // stream seed
+  }
+  __device__ __forceinline__ void co_go_on() {
+    const int dec = S->dec;
+    if (dec == 2) plan_selection(co().delta);
+    else if (dec == 0) co_delta(kDScan);
   }
 
-  // Coordinator: the largest current degree in the heavy list is mx (-1 if
-  // none is alive).  It is the global maximum when it is still >= tau.
-  __device__ void co_after_heavy(int32_t mx) {
-    if (threadIdx.x == 0) S->dec = mx >= co().tau ? 1 : 0;
-    __syncthreads();
-    if (S->dec) { plan_selection(mx); return; }
-    // The new maximum D lies in [max(mx, 0), tau): every vertex outside the
-    // heavy list had a degree below tau when the list was built.
-    start_rebuild(co().tau >= 2 ? co().tau >> 1 : 1);
+  // The recount threshold when the largest bound is x: as far below it as
+  // Delta fell lately, but by no more than a quarter.
+  __device__ static int32_t below(int32_t x, int32_t drop) {
+    const int32_t lo = x - (x >> 2);
+    const int32_t t = x - drop > lo ? x - drop : lo;
+    return t > 1 ? t : 1;
   }
 
-  // ---------------- Delta rebuild: where to look -------------------------------
-  // A rebuild needs the exact maximum D over the alive vertices and a new heavy
-  // list holding every alive vertex of degree >= max(1, D/2).  Degrees only
-  // fall, so a vertex of current degree >= x has full degree >= x.  The search
-  // reads the degree order (dsort, largest full degree first) in segments:
-  // after every vertex of full degree >= t has been read, the largest current
-  // degree seen is D exactly if it is >= t (no unread vertex can reach t);
-  // otherwise t halves and the next segment is read.  The heavy list then
-  // comes from the prefix of full degree >= D/2.  Segments up to
-  // inline_rebuild vertices (a tuning setting) are read by the coordinator block inside the
-  // barrier; longer ones by the grid.  Once the prefix to read exceeds a
-  // quarter of the compact list of alive non-isolated vertices (vertex order,
-  // dead vertices dropped at each of its rebuilds), that list is cheaper and
-  // the rebuild switches to it.
-  __device__ __noinline__ void start_rebuild(int32_t t0) {
-    if (threadIdx.x == 0) {
-      Coord& c = co();
-      const int32_t hi = c.max_deg + 1;
-      c.rb_t = t0 < 1 ? 1 : (t0 > hi ? hi : t0);
-      c.rb_lo = 0;
-      c.rb_hi = __ldg(B.dge + c.rb_t);
-      c.rb_D = 0;
-      c.rebuilds_in_row += 1;
-      if (c.rebuilds_in_row > 2) fail(kErrInternal);
-    }
-    __syncthreads();
-    rebuild_advance();
-  }
-
-  // Coordinator block: read segments inline until D is known (then refill the
-  // heavy list, inline or by planning a grid pass), or plan a grid step.
-  __device__ __noinline__ void rebuild_advance() {
+  // Exact Delta without decrements.  Every alive vertex outside H has a bound
+  // < tau.  Alive vertices of H with a bound >= some threshold are picked and
+  // their degrees recounted; d_lb is the largest exact degree found, d_other
+  // the largest bound that was not picked.  Then, until Delta is known:
+  //   a bound above d_lb is left: recount those as well;
+  //   d_lb >= tau - 1: no vertex can have more, Delta = d_lb;
+  //   else H no longer holds the maximum: rebuild it with a lower tau.
+  // A pass with threshold d_lb + 1 leaves no larger bound, so each H is
+  // recounted at most twice.  The first threshold decides between rows
+  // recounted in vain and second passes: taking the recent fall of Delta, the
+  // recounted rows hold 0.15-0.6 of the graph's entries over a whole clustering
+  // (R-MAT 26 0.15, planted 10^6 0.55, eps 0.5 and 0.1) and 10-15 % of the rounds
+  // need a second pass; recounting all of H every round reads 1.6-3.3.
+  // Decrementing the neighbours of every removed vertex instead read 0.85-0.9
+  // of the entries, with an atomic for half of them.
+  // A list of up to kHere vertices is looked at here (inline_heavy), and
+  // recounted here while its rows are short: a grid phase would cost a barrier
+  // and the same dependent loads.
+  __device__ __noinline__ void co_delta(int step) {
+    Coord& c = co();
     for (;;) {
-      if (threadIdx.x == 0) {
-        Coord& c = co();
-        Plan& p = S->plan;
-        const int64_t limit = c.nz_len / 4;
-        const int64_t seg = c.rb_hi - c.rb_lo;
-        int dec;
-        if (seg > 0) {
-          dec = seg <= B.tune.inline_rebuild ? 0 : (c.rb_hi > limit ? 4 : 1);
-        } else if (c.rb_D >= c.rb_t || c.rb_t <= 1) {
-          if (c.rb_D <= 0) {
-            dec = 5;                                  // nothing alive has an alive neighbour
-          } else {
-            c.tau = tau_of(c.rb_D);
-            c.rb_hi = __ldg(B.dge + c.tau);           // heavy candidates: full degree >= tau
-            dec = c.rb_hi <= B.tune.inline_rebuild ? 2 : (c.rb_hi > limit ? 4 : 3);
-          }
-        } else {
-          c.rb_t = c.rb_t >= 2 ? c.rb_t >> 1 : 1;
-          c.rb_hi = __ldg(B.dge + c.rb_t);
-          dec = -1;
-        }
-        if (dec == 1) { p.state = kRebuildDeg; p.win_lo = c.rb_lo; p.win_len = seg; }
-        if (dec == 3) { p.state = kRebuildHeavy; p.win_lo = 0; p.win_len = c.rb_hi; p.th = c.tau; C->h_pack = 0; }
-        if (dec == 4) { p.state = kRebuildDelta; set_nz_plan(); }
-        S->dec = dec;
-      }
-      __syncthreads();
-      const int dec = S->dec;
-      __syncthreads();
-      if (dec == -1) continue;
-      if (dec == 0) {                                 // read a short segment here
-        const int64_t m = deg_max_over(co().rb_lo, co().rb_hi);
-        if (threadIdx.x == 0) {
-          Coord& c = co();
-          c.rb_D = m > c.rb_D ? (int32_t)m : c.rb_D;
-          c.rb_lo = c.rb_hi;
-        }
-        __syncthreads();
-        continue;
-      }
-      if (dec == 2) {                                 // refill a short heavy list here
-        const int32_t tau = co().tau;
-        const int64_t len = co().rb_hi;
-        if (threadIdx.x == 0) S->bcast[0] = 0;
-        __syncthreads();
-        for (int64_t base = threadIdx.x; base < len; base += (int64_t)kScanU * blockDim.x) {
-          int32_t v[kScanU];
-          uint32_t x[kScanU];
-#pragma unroll
-          for (int q = 0; q < kScanU; ++q) {
-            const int64_t i = base + (int64_t)q * blockDim.x;
-            v[q] = i < len ? __ldg(B.dsort + i) : -1;
-          }
-#pragma unroll
-          for (int q = 0; q < kScanU; ++q) x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
-#pragma unroll
-          for (int q = 0; q < kScanU; ++q)
-            if (is_alive(x[q]) && deg_of(x[q]) > 0 && (int64_t)deg_of(x[q]) >= tau)
-            {
-              const int64_t h = (int64_t)atomicAdd(reinterpret_cast<unsigned long long*>(&S->bcast[0]), 1ull);
-              if (CC_IN_BOUNDS(h, B.n, &C->err)) B.hv[h] = v[q];
+      if (step == kDScan) {
+        const int64_t hl = c.h_len;
+        step = kDPlanned;
+        if (hl <= kHere && (hl <= B.tune.inline_heavy || hl == 0)) {
+          look_here();
+          const int picked = S->h_picked;
+          int64_t E = 0;
+          if (picked > 0 && picked <= kHRows) E = prepare_rows(0, picked, false);
+          if (picked <= kHRows && (E <= kInlineEdges || G == 1)) {
+            if (picked > 0) {
+              const int32_t best = block_recount(picked, E);
+              if (threadIdx.x == 0) {
+                c.r_edges += E;
+                if (best > c.d_lb) c.d_lb = best;
+              }
             }
+            step = kDCounted;
+          }
+        }
+        if (step == kDPlanned && threadIdx.x == 0) {
+          Plan& p = S->plan;
+          p.state = kRecount;
+          p.win_len = c.h_len;
+          p.pad0 = G > 1 && c.h_len <= kHList ? 1 : 0;       // every block lists all of H
+          p.th = c.d_lb < 0 && c.h_len <= kHere && c.d_top > 0 ? below(c.d_top, c.d_drop) : c.d_th;
+          p.d_lb = c.d_lb;
+          p.drop = c.d_drop;
+          p.long_n = 0;
+          if (c.h_len > kHere && G > 1) {
+            // the list is too long: keep what the next rounds will ask for
+            if (c.tight < kTightest) c.tight += 1;
+            const int32_t d2 = c.delta - 2 * c.d_drop - 1, t = c.delta - (c.delta >> c.tight);
+            const int32_t up = d2 < t ? d2 : t;
+            c.tau_next = up > c.tau && c.d_lb < 0 && c.rebuilds_in_row == 0 ? up : c.tau;     // not after a rebuild
+            p.long_n = c.tau_next;
+            C->h_pack = 0;
+          }
+          reset_looked();
         }
         __syncthreads();
-        finish_rebuild(co().rb_D, S->bcast[0]);
-        return;
       }
-      if (dec == 5) { finish_rebuild(0, 0); return; }
-      return;                                         // a grid step is planned
+      if (step == kDPlanned) return;
+      if (threadIdx.x == 0) {
+        int next = kDScan;
+        if (c.d_other > c.d_lb && c.d_other > 0) {
+          c.d_th = c.d_lb < 0 ? below(c.d_other, c.d_drop) : c.d_lb + 1;
+        } else {
+          const int32_t D = c.d_lb > 0 ? c.d_lb : 0;
+          if (D + 1 >= c.tau) {
+            const int32_t fall = c.d_top > D ? c.d_top - D : 0;
+            c.d_drop = fall > c.d_drop ? fall : c.d_drop - ((c.d_drop - fall) >> 2);
+            if (D <= 0) c.delta_zero = 1;
+            c.delta = D;
+            next = kDDone;
+          } else {
+            next = kDRebuild;
+          }
+        }
+        S->dec = next;
+      }
+      __syncthreads();
+      step = S->dec;
+      __syncthreads();
+      if (step == kDDone) { plan_selection(c.delta); return; }
+      if (step == kDRebuild) {
+        if (!rebuild()) return;
+        step = kDScan;
+      }
     }
   }
 
-  // Coordinator block: the largest current degree of an alive vertex among
-  // dsort[lo, hi) (0 if none).
-  __device__ int64_t deg_max_over(int64_t lo, int64_t hi) {
-    int64_t mx = 0;
-    for (int64_t base = lo + threadIdx.x; base < hi; base += (int64_t)kScanU * blockDim.x) {
+  // The largest bounds of a look over H (thread 0 of the coordinator).
+  __device__ void note_looked(int32_t other, int32_t top) {
+    co().d_other = other;
+    if (co().d_top <= 0) co().d_top = top;
+  }
+
+  // Appends v to S->u.hl.pick where take is set (all lanes call it).
+  __device__ __forceinline__ void pick(bool take, int32_t v) {
+    const unsigned m = __ballot_sync(FULL, take);
+    if (m == 0) return;
+    int at = 0;
+    if ((threadIdx.x & 31) == 0) at = atomicAdd(&S->h_picked, __popc(m));
+    at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+    if (take) S->u.hl.pick[at] = v;
+  }
+
+  // Coordinator block, a heavy list of up to kHere vertices: picks the alive ones
+  // with a bound >= th, th = d_lb + 1 or a little below the largest bound while
+  // d_lb < 0, and compacts the list to its alive vertices.
+  __device__ __noinline__ void look_here() {
+    Coord& c = co();
+    const int len = (int)c.h_len;
+    constexpr int step = kScanU * kThreads;
+    int32_t v[kScanU], ub[kScanU], top = 0, alive = 0;
+    const auto read = [&](int base) {
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        const int i = base + q * kThreads + (int)threadIdx.x;
+        v[q] = i < len ? ldcg(hv() + i) : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        const uint32_t x = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+        ub[q] = is_alive(x) ? (int32_t)deg_of(x) : 0;
+      }
+    };
+#pragma unroll 1
+    for (int base = 0; base < len; base += step) {
+      read(base);
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        top = ub[q] > top ? ub[q] : top;
+        alive += ub[q] > 0 ? 1 : 0;
+      }
+    }
+    if (threadIdx.x == 0) S->h_picked = S->h_kept = 0;
+    top = max_i32(top);
+    // a second look costs no barrier here: a fraction of the recent fall
+    const int32_t th = c.d_lb < 0 ? below(top, c.d_drop >> 2) : c.d_lb + 1;
+    const bool pack = sum_i32(alive) < len - (len >> 2);    // a quarter has left
+    int32_t other = 0;
+#pragma unroll 1
+    for (int base = 0; base < len; base += step) {
+      if (len > step) read(base);                        // a longer list is read again (L2)
+      if (pack) __syncthreads();                         // the step is read before it is written over
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        const bool take = v[q] >= 0 && ub[q] >= th;      // th >= 1
+        other = !take && ub[q] > other ? ub[q] : other;
+        const unsigned m = __ballot_sync(FULL, take);
+        if (m) {
+          int at = 0;
+          if ((threadIdx.x & 31) == 0) at = atomicAdd(&S->h_picked, __popc(m));
+          at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+          if (take && at < kHPick) S->u.hl.pick[at] = v[q];
+        }
+        if (!pack) continue;
+        const unsigned k = __ballot_sync(FULL, ub[q] > 0);
+        int at = 0;
+        if (k && (threadIdx.x & 31) == 0) at = atomicAdd(&S->h_kept, __popc(k));
+        at = __shfl_sync(FULL, at, 0) + __popc(k & ((1u << (threadIdx.x & 31)) - 1u));
+        if (ub[q] > 0) hv()[at] = v[q];
+      }
+    }
+    other = max_i32(other);
+    if (threadIdx.x == 0) {
+      if (pack) c.h_len = S->h_kept;
+      c.d_th = th;
+      note_looked(other, top);
+    }
+    __syncthreads();
+  }
+
+  // Block-wide, for a heavy list of len <= kHList vertices: the alive ones with a
+  // bound >= th become the rows S->u.hl (in list order: every block makes the
+  // same list), th as in look_here.  Returns their number and entries.
+  __device__ __noinline__ void list_heavy(int64_t len, int32_t lb, int32_t drop, int64_t* items, int64_t* E) {
+    HeavyList& hl = S->u.hl;
+    const int32_t v = threadIdx.x < len ? ldcg(hv() + threadIdx.x) : -1;
+    const uint32_t x = v >= 0 ? ldcg(B.st + v) : 0u;
+    const int32_t ub = is_alive(x) ? (int32_t)deg_of(x) : 0;
+    int64_t row = 0, end = 0;
+    if (ub > 0) {                          // the row is asked for before the threshold is known
+      row = __ldg(B.off + v);
+      end = __ldg(B.off + v + 1);
+    }
+    const int32_t top = max_i32(ub);
+    const int32_t th = lb < 0 ? below(top, drop) : lb + 1;
+    const bool take = ub >= th;
+    const int32_t other = max_i32(take ? 0 : ub);
+    const int32_t n = take ? (int32_t)(end - row) : 0;
+    const Scan sc = scan(take ? (int64_t(1) << kPackShift) | n : 0);
+    if (take) {
+      const int j = (int)(sc.ex >> kPackShift);
+      hl.pos[j] = sc.ex & (int64_t)kPackEdgeMask;
+      hl.len[j] = n;
+      hl.row[j] = row;
+      hl.v[j] = v;
+    }
+    if (bid == 0 && threadIdx.x == 0) {    // the coordinator's copy counts
+      S->tal[kTEdges] += (unsigned long long)(sc.tot & (int64_t)kPackEdgeMask);
+      note_looked(other, top);
+    }
+    *items = sc.tot >> kPackShift;
+    *E = sc.tot & (int64_t)kPackEdgeMask;
+    __syncthreads();
+  }
+
+  // Block-wide: the rows of pick[base, base + items), items <= kHRows, into
+  // S->u.hl; returns their entries.  split: rows above kLongRow go to the
+  // grid-wide list instead.
+  __device__ __noinline__ int64_t prepare_rows(int base, int items, bool split) {
+    constexpr int kPer = kHRows / kThreads;
+    HeavyList& hl = S->u.hl;
+    int32_t v[kPer], len[kPer];
+    int64_t row[kPer];
+    int64_t mine = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = threadIdx.x * kPer + q;
+      v[q] = i < items ? hl.pick[base + i] : -1;
+      row[q] = v[q] >= 0 ? __ldg(B.off + v[q]) : 0;
+      len[q] = v[q] >= 0 ? (int32_t)(__ldg(B.off + v[q] + 1) - row[q]) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      if (split && len[q] > kLongRow) {
+        const unsigned long long old = atomicAdd(&C->long_pack, (1ull << kPackShift) | (unsigned long long)len[q]);
+        const int64_t j = (int64_t)(old >> kPackShift);
+        if (CC_IN_BOUNDS(j, B.n, &C->err)) {
+          B.b_j[j] = v[q];
+          B.b_e[j] = (int64_t)(old & kPackEdgeMask);
+          B.b_d[j] = row[q];
+          B.pull[j] = len[q];
+          B.act_n[j] = 0;
+        }
+        v[q] = -1;
+        len[q] = 0;
+      }
+      mine += len[q];
+    }
+    const Scan sc = scan(mine);
+    int64_t ex = sc.ex;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = threadIdx.x * kPer + q;
+      hl.pos[i] = ex;
+      hl.row[i] = row[q];
+      hl.len[i] = len[q];
+      hl.v[i] = v[q];
+      hl.cnt[i] = 0;
+      ex += len[q];
+    }
+    __syncthreads();
+    return sc.tot;
+  }
+
+  // Block-wide: recount of every picked vertex; the largest degree known to the
+  // block, and to the team so far, goes to S->h_best.
+  __device__ __noinline__ void recount_picked() {
+    const int n = S->h_picked;
+    int32_t best = -1;
+    int64_t edges = 0;
+    for (int base = 0; base < n; base += kHRows) {
+      const int items = n - base < kHRows ? n - base : kHRows;
+      const int64_t E = prepare_rows(base, items, G > 1);
+      const int32_t b = block_recount(items, E);
+      best = b > best ? b : best;
+      edges += E;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      S->h_picked = 0;
+      if (best > S->h_best) {
+        const int32_t old = atomicMax(&C->best, best);
+        S->h_best = old > best ? old : best;
+      }
+      S->tal[kTEdges] += (unsigned long long)edges;
+    }
+    __syncthreads();
+  }
+
+  // Counts the alive entries of `items` rows (lists in shared or global memory)
+  // into acc: warp gw of nw takes its share of the E entries.  The alive entries
+  // of a batch come as ballots, of which every lane counts the part of its own
+  // window item, so an item costs one add per window.
+  __device__ __noinline__ void count_alive(int gw, int nw, int32_t items, int64_t E, const int64_t* pos,
+                                           const int64_t* row, const int32_t* len, unsigned* acc) {
+    const uint32_t* const rtag = B.rtag;
+    unsigned cnt = 0;
+    const auto at = [&](int32_t j) { return vload(pos + j); };
+    const auto load = [&](int32_t j) { return RowItem{vload(pos + j), vload(row + j), vload(len + j), 0}; };
+    const auto count = [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+      uint32_t tg[kB];
+#pragma unroll
+      for (int q = 0; q < kB; ++q) {
+        const bool in = X.w[q] >= 0 && CC_IN_BOUNDS(X.w[q], B.n, &C->err);
+        tg[q] = in ? ldcg(rtag + (X.w[q] >> 3)) >> ((X.w[q] & 7) * 4) : 1u;
+      }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) {
+        const unsigned m = __ballot_sync(FULL, (tg[q] & 15u) == 0);
+        const int lo = X.from - 32 * q > 0 ? X.from - 32 * q : 0, hi = X.to - 32 * q < 32 ? X.to - 32 * q : 32;
+        if (hi > lo) cnt += __popc(m & (0xFFFFFFFFu >> (32 - (hi - lo)) << lo));
+      }
+    };
+    const auto flush = [&](int32_t j) {
+      if (cnt) atomicAdd(acc + j, cnt);
+      cnt = 0;
+    };
+    const WalkShape shape{B.tune.walk_batches, B.tune.prefetch_ahead};
+    if (E <= 64 * (int64_t)nw) row_walk<1>(gw, nw, items, E, B.col, shape, at, load, count, flush);
+    else row_walk<kRowB>(gw, nw, items, E, B.col, shape, at, load, count, flush);
+  }
+
+  // Recount of the block's list by the block itself; returns the largest
+  // degree found to every thread.
+  __device__ __noinline__ int32_t block_recount(int32_t items, int64_t E) {
+    HeavyList& hl = S->u.hl;
+    count_alive((int)(threadIdx.x >> 5), (int)(blockDim.x >> 5), items, E, hl.pos, hl.row, hl.len, hl.cnt);
+    __syncthreads();
+    int32_t best = -1;
+    for (int i = threadIdx.x; i < items; i += blockDim.x) {
+      const int32_t v = hl.v[i], d = (int32_t)hl.cnt[i];
+      if (v < 0 || !CC_IN_BOUNDS(v, B.n, &C->err)) continue;
+      B.st[v] = kAlive | (uint32_t)d;
+      best = d > best ? d : best;
+    }
+    return max_i32(best);
+  }
+
+  // Grid phase over a heavy list of up to kHList vertices: every block makes
+  // the same list (no state word changes in this phase), the grid's warps share
+  // its entries, and the coordinator writes the degrees inside the barrier.
+  // Longer lists: every block picks the vertices to recount out of its share
+  // (dealt out by 32 entries: neighbours in the list have similar rows) and
+  // recounts them, rows above kLongRow are left to a second phase of the whole
+  // grid.  A block that has recounted some raises its threshold to the largest
+  // degree known.
+  __device__ __noinline__ bool recount_phase() {
+    const int64_t len = P().win_len;
+    if (P().pad0) {
+      int64_t items, E;
+      list_heavy(len, P().d_lb, P().drop, &items, &E);
+      HeavyList& hl = S->u.hl;
+      count_alive(team_warp(), team_warps(), (int32_t)items, E, hl.pos, hl.row, hl.len, B.h_acc);
+      return sync(6, [&] {
+        int32_t best = -1;
+        if (threadIdx.x < items) {
+          const int32_t v = hl.v[threadIdx.x];
+          best = (int32_t)ldcg(B.h_acc + threadIdx.x);
+          B.h_acc[threadIdx.x] = 0;
+          if (CC_IN_BOUNDS(v, B.n, &C->err)) B.st[v] = kAlive | (uint32_t)best;
+        }
+        best = max_i32(best);
+        if (threadIdx.x == 0 && best > co().d_lb) co().d_lb = best;
+        __syncthreads();
+        co_delta(kDCounted);
+      });
+    }
+    Look k = look_begin(P().th);
+    const int64_t all = (int64_t)G * blockDim.x;
+    const int32_t keep = (int32_t)P().long_n;       // > 0: the list is rewritten with the bounds >= keep
+    int32_t* const to = S->plan.hv_sel ? B.hv : B.hv2;
+    for (int64_t base = 0; base < len; base += all * kScanU) {
+      int32_t v[kScanU];
       uint32_t x[kScanU];
 #pragma unroll
       for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)q * blockDim.x;
-        x[q] = i < hi ? ldcg(B.st + __ldg(B.dsort + i)) : 0u;
+        const int64_t i = base + q * all + (int64_t)(threadIdx.x >> 5) * G * 32 + bid * 32 + (threadIdx.x & 31);
+        v[q] = i < len ? ldcg(hv() + i) : -1;
       }
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q)
-        if (is_alive(x[q])) mx = (int64_t)deg_of(x[q]) > mx ? (int64_t)deg_of(x[q]) : mx;
+      for (int q = 0; q < kScanU; ++q) x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+      if (keep > 0) append_heavy<kScanU>(v, x, keep, to);
+      look_step(k, v, x, keep > 0 ? keep : 1, base + all * kScanU >= len);
     }
-    return block_max<int64_t>(mx, S->scr);
+    look_end(k);
+    return sync(6, [&] {
+      if (threadIdx.x == 0 && S->plan.long_n > 0) {
+        co().h_len = (int64_t)vload(&C->h_pack);
+        co().tau = co().tau_next;
+        S->plan.hv_sel ^= 1;
+      }
+      __syncthreads();
+      looked();
+    });
   }
 
-  __device__ void set_nz_plan() {
-    Coord& c = co();
-    S->plan.win_lo = 0;
-    S->plan.win_len = c.nz_len;
-    S->plan.pad0 = (c.nz_static ? 2 : 0) | c.nz_sel;
-  }
-
-  // Coordinator: the new maximum D and heavy list of hcount entries are in
-  // place; plan the round's selection.
-  __device__ void finish_rebuild(int32_t D, int64_t hcount) {
+  // A block's look at its share of the heavy vertices: the vertices of a bound
+  // >= th are picked and recounted, at first a small number of them, after
+  // which th is the largest degree known + 1.
+  struct Look {
+    int32_t th, other, top;
+    int limit;
+  };
+  __device__ __forceinline__ Look look_begin(int32_t th) {
     if (threadIdx.x == 0) {
-      Coord& c = co();
-      c.tau = tau_of(D);
-      c.h_len = D > 0 ? hcount : 0;
-      if (D <= 0) c.delta_zero = 1;
+      S->h_picked = 0;
+      S->h_best = -1;
     }
     __syncthreads();
-    plan_selection(D > 0 ? D : 0);
+    return Look{th, 0, 0, 256};
+  }
+  // Vertices v with state words x; bounds below tau are not heavy.
+  __device__ __forceinline__ void look_step(Look& k, const int32_t* v, const uint32_t* x, int32_t tau, bool last) {
+#pragma unroll
+    for (int q = 0; q < kScanU; ++q) {
+      const int32_t d = is_alive(x[q]) ? (int32_t)deg_of(x[q]) : 0;
+      const int32_t ub = d >= tau ? d : 0;
+      const bool take = ub >= k.th;         // th >= 1
+      k.top = ub > k.top ? ub : k.top;
+      k.other = !take && ub > k.other ? ub : k.other;
+      pick(take, v[q]);                     // room for a whole step is left (below)
+    }
+    __syncthreads();
+    if (S->h_picked > k.limit || (last && S->h_picked > 0)) {    // uniform
+      recount_picked();
+      if (S->h_best >= k.th) k.th = S->h_best + 1;
+      k.limit = k.limit * 4 < kHPick / 2 ? k.limit * 4 : kHPick / 2;
+    }
+  }
+  __device__ __forceinline__ void look_end(const Look& k) {
+    const int32_t other = __reduce_max_sync(FULL, k.other), top = __reduce_max_sync(FULL, k.top);
+    if ((threadIdx.x & 31) == 0) {
+      if (other > ld_volatile_int(&C->other_max)) atomicMax(&C->other_max, other);
+      if (top > ld_volatile_int(&C->listed_max)) atomicMax(&C->listed_max, top);
+    }
+  }
+  // Coordinator, after the blocks' looks.
+  __device__ __forceinline__ void looked() {
+    if (threadIdx.x < 4) {
+      const int i = threadIdx.x;
+      S->bcast[i] = i == 0 ? (int64_t)vload(&C->best) : i == 1 ? (int64_t)vload(&C->other_max)
+                    : i == 2 ? (int64_t)vload(&C->listed_max) : (int64_t)vload(&C->long_pack);
+    }
+    __syncthreads();
+    const unsigned long long lp = (unsigned long long)S->bcast[3];
+    if (threadIdx.x == 0) {
+      note_looked((int32_t)S->bcast[1], (int32_t)S->bcast[2]);
+      if ((int32_t)S->bcast[0] > co().d_lb) co().d_lb = (int32_t)S->bcast[0];
+      if (lp) {
+        S->plan.state = kRecountLong;
+        S->plan.long_n = (int64_t)(lp >> kPackShift);
+        S->plan.long_E = (int64_t)(lp & kPackEdgeMask);
+        co().r_edges += S->plan.long_E;
+      }
+    }
+    __syncthreads();
+    if (!lp) co_delta(kDCounted);
+  }
+  // What a planned look starts from (thread 0 of the coordinator).
+  __device__ __forceinline__ void reset_looked() {
+    C->best = -1; C->listed_max = 0; C->other_max = 0; C->long_pack = 0;
+  }
+
+  // The long rows of a long heavy list, shared by the grid.
+  __device__ __noinline__ bool recount_long() {
+    unsigned* const acc = reinterpret_cast<unsigned*>(B.act_n);
+    count_alive(team_warp(), team_warps(), (int32_t)P().long_n, P().long_E, B.b_e, B.b_d, B.pull, acc);
+    return sync(6, [&] {
+      int32_t best = -1;
+      for (int64_t j = threadIdx.x; j < S->plan.long_n; j += blockDim.x) {
+        const int32_t v = ldcg(B.b_j + j), d = (int32_t)ldcg(acc + j);
+        if (CC_IN_BOUNDS(v, B.n, &C->err)) B.st[v] = kAlive | (uint32_t)d;
+        best = d > best ? d : best;
+      }
+      best = max_i32(best);
+      if (threadIdx.x == 0 && best > co().d_lb) co().d_lb = best;
+      __syncthreads();
+      co_delta(kDCounted);
+    });
+  }
+
+  // ---------------- rebuild of the heavy list ----------------------------------
+  // A new H of every alive vertex with a bound >= tau, for a lower tau.  All
+  // bounds are at most ub = min(the last Delta, the old tau - 1).  tau = ub -
+  // (ub >> tight): a long list is costly every round, a short one is soon used
+  // up, so tight follows the length (from 1; up while the list is too long for
+  // the coordinator, down again when it is very short), and a list that is too
+  // long is cut down to a higher tau when the grid looks at it.  (R-MAT 26: with
+  // half of ub throughout, rounds below Delta = 100 scanned up to 10M entries
+  // each.)  A second rebuild in one round goes down to d_lb, at most to half of
+  // ub: only larger bounds matter.
+  // A vertex of bound >= tau has full degree >= tau, so the list comes from a
+  // prefix of the degree order (dsort): up to inline_rebuild vertices (a tuning
+  // setting) are read by the coordinator block inside the barrier, longer
+  // prefixes by the grid, and once the prefix exceeds a quarter of the alive
+  // non-isolated vertices, the grid reads those instead (vertex order).  True:
+  // the list is in place; false: a grid step is planned.
+  __device__ __noinline__ bool rebuild() {
+    Coord& c = co();
+    if (threadIdx.x == 0) {
+      Plan& p = S->plan;
+      c.rebuilds_in_row += 1;
+      if (c.rebuilds_in_row > 64) fail(kErrInternal);     // tau falls every time
+      const int32_t ub = c.delta < c.tau ? c.delta : c.tau - 1;     // >= 1: with tau = 1 Delta is known
+      const int32_t loose = ub >> B.tune.heavy_shift > 1 ? ub >> B.tune.heavy_shift : 1;
+      int32_t t = ub - (ub >> c.tight);
+      if (t > ub - 2 * c.d_drop) t = ub - 2 * c.d_drop;      // meant to last for more than a round
+      if (t < loose) t = loose;
+      if (c.rebuilds_in_row > 1) {
+        const int32_t lb = c.d_lb < t ? c.d_lb : t;
+        t = lb > loose ? lb : loose;
+      }
+      c.tau = t;
+      c.d_th = c.d_lb < 0 ? below(ub, c.d_drop) : c.d_lb + 1;
+      const int64_t prefix = __ldg(B.dge + t);
+      int dec = 0;
+      if (prefix > B.tune.inline_rebuild) {
+        dec = 1;
+        p.th = t;
+        p.take = c.d_th;                    // the grid looks at the new list while it makes it
+        p.win_len = prefix;
+        reset_looked();
+        p.state = prefix > c.nz_len / 4 ? kRebuildAlive : kRebuildOrder;
+        C->h_pack = 0;
+        C->nz_pack = 0;
+      }
+      S->dec = dec;
+      S->bcast[0] = prefix;
+      S->h_kept = 0;
+    }
+    __syncthreads();
+    if (S->dec) return false;
+    const int32_t tau = c.tau;
+    const int64_t len = S->bcast[0];
+    for (int64_t base = 0; base < len; base += (int64_t)kScanU * blockDim.x) {
+      int32_t v[kScanU];
+      uint32_t x[kScanU];
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        const int64_t i = base + threadIdx.x + (int64_t)q * blockDim.x;
+        v[q] = i < len ? __ldg(B.dsort + i) : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        if (!is_alive(x[q]) || (int32_t)deg_of(x[q]) < tau) continue;
+        const int h = atomicAdd(&S->h_kept, 1);
+        if (CC_IN_BOUNDS(h, B.n, &C->err)) hv()[h] = v[q];
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      c.h_len = S->h_kept;
+      follow_length();
+    }
+    __syncthreads();
+    return true;
+  }
+
+  // Thread 0 of the coordinator, with a new heavy list in place.
+  __device__ __forceinline__ void follow_length() {
+    Coord& c = co();
+    if (c.h_len > kHere && c.tight < kTightest) c.tight += 1;
+    else if (c.h_len < kHere / 16 && c.tight > 1) c.tight -= 1;
   }
 
   // Statistics and n_i update after the removal phase, then the next plan.
-  __device__ void co_end_round() {
+  __device__ __noinline__ void co_end_round() {
     Coord& c = co();
-    if (threadIdx.x < 6) {
-      const long long* src[6] = {&C->r_centers, &C->r_attached, &C->r_noncenter, &C->r_blocked,
-                                 reinterpret_cast<const long long*>(&C->new_pack), nullptr};
-      if (threadIdx.x < 5) S->bcast[threadIdx.x] = vload(src[threadIdx.x]);
+    if (threadIdx.x < 5) {
+      const long long* src[5] = {&C->r_centers, &C->r_attached, &C->r_noncenter, &C->r_blocked, &C->r_edges};
+      S->bcast[threadIdx.x] = vload(src[threadIdx.x]);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       const int64_t centers_seen = S->bcast[0], attached = S->bcast[1], noncenter = S->bcast[2];
       const int64_t blocked = S->bcast[3];
-      const unsigned long long np = (unsigned long long)S->bcast[4];
       const int64_t k = c.k;
       const int64_t removed = k + attached;
       const int64_t centers = k - noncenter;
@@ -675,11 +1163,13 @@ struct K {
       if (r < c.stats_cap) {
         RoundStat s;
         s.n_alive = c.n_alive; s.delta = c.delta; s.k = k; s.centers = centers;
-        s.removed = removed; s.blocked = blocked; s.edges = c.r_edges + (int64_t)(np & kPackEdgeMask);
+        s.removed = removed; s.blocked = blocked; s.edges = c.r_edges + S->bcast[4];
         s.ns = (int64_t)(globaltimer_ns() - c.round_t0);
         B.stats[r] = s;
       }
       c.round_t0 = globaltimer_ns();
+      c.round_ended = 1;
+      c.r_edges = 0;
       if (centers_seen != centers) fail(kErrInternal);
       c.n_alive -= removed;
       c.clusters += centers;
@@ -687,9 +1177,10 @@ struct K {
       c.round = r + 1;
       c.rebuilds_in_row = 0;
       if (!c.est && c.round > c.n + 1) fail(kErrInternal);   // Sec. 5 rounds may hold no active vertex
+      S->dec = co_next();
     }
     __syncthreads();
-    co_decide_delta();
+    co_go_on();
   }
 
   // ---------------- Sec. 5: the round's binomial batch ------------------------
@@ -698,7 +1189,7 @@ struct K {
   // succeeds, k = stream seed); the coordinator adds them up, moves the rank
   // cursor past the batch and plans the round's single selection window, the
   // batch's ranks of pi.
-  __device__ bool draw_batch() {
+  __device__ __noinline__ bool draw_batch() {
     const int64_t trials = P().win_len;
     const uint64_t thr = (uint64_t)P().need, s = (uint64_t)P().k;
     int64_t cnt = 0;
@@ -726,265 +1217,210 @@ struct K {
     });
   }
 
-  // ---------------- heavy list: per-round maximum ----------------------------
-  __device__ bool heavy_scan() {
-    int64_t s, e;
-    slice(0, P().win_len, &s, &e);
-    int64_t mx = -1;
-    for (int64_t base = s; base < e; base += (int64_t)blockDim.x * kScanU) {
-      int32_t v[kScanU];
+  // ---------------- rebuild of the heavy list: grid passes ---------------------
+  // Appends v (with its state word x) to the list `to` where its bound is >= tau.
+  template <int kN>
+  __device__ __forceinline__ void append_heavy(const int32_t* v, const uint32_t* x, int32_t tau, int32_t* to) {
+    int64_t heavy = 0;
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
-        v[q] = i < e ? ldcg(B.hv + i) : -1;
-      }
+    for (int q = 0; q < kN; ++q) heavy += is_alive(x[q]) && (int32_t)deg_of(x[q]) >= tau ? 1 : 0;
+    const Scan sc = scan(heavy);
+    if (sc.tot == 0) return;                // uniform
+    if (threadIdx.x == 0) S->bcast[0] = (int64_t)atomicAdd(&C->h_pack, (unsigned long long)sc.tot);
+    __syncthreads();
+    int64_t ho = S->bcast[0] + sc.ex;
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        if (v[q] < 0) continue;
-        const uint32_t x = ldcg(B.st + v[q]);
-        if (is_alive(x)) mx = (int64_t)deg_of(x) > mx ? (int64_t)deg_of(x) : mx;
-      }
-    }
-    mx = block_max<int64_t>(mx, S->scr);
-    if (threadIdx.x == 0) B.blk_b[bid] = mx;
-    return sync(0, [&] {
-      const int64_t m = max_blocks_signed();
-      co_after_heavy((int32_t)m);
-    });
+    for (int q = 0; q < kN; ++q)
+      if (is_alive(x[q]) && (int32_t)deg_of(x[q]) >= tau && CC_IN_BOUNDS(ho, B.n, &C->err)) to[ho++] = v[q];
   }
 
-  // ---------------- Delta rebuild: grid passes ---------------------------------
-  // Over the compact list (vertex order): A, count the vertices that are still
-  // alive with a degree > 0 and find the largest degree D; B, compact the list
-  // and put every survivor of degree >= tau = max(1, D/2) on the heavy list.
-  __device__ int32_t nz_at(int flags, int64_t i) const {
-    if (flags & 2) return __ldg(B.nz_static + i);
-    return ldcg(((flags & 1) ? B.nz1 : B.nz0) + i);
-  }
-
-  __device__ bool delta_rebuild() {
-    const int flags = P().pad0;
+  // H from the first win_len vertices of the degree order (dealt out by 32, as
+  // in recount_phase); the vertices of the largest bounds are recounted at once.
+  __device__ __noinline__ bool rebuild_from_order() {
     const int64_t len = P().win_len;
-    int64_t s, e;
-    slice(0, len, &s, &e);
-    int64_t cnt = 0, mx = 0;
-    for (int64_t base = s; base < e; base += (int64_t)blockDim.x * kScanU) {
-      int32_t v[kScanU];
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
-        v[q] = i < e ? nz_at(flags, i) : -1;
-      }
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        if (v[q] < 0) continue;
-        const uint32_t x = ldcg(B.st + v[q]);
-        if (is_alive(x) && deg_of(x) > 0) {
-          ++cnt;
-          mx = (int64_t)deg_of(x) > mx ? (int64_t)deg_of(x) : mx;
-        }
-      }
-    }
-    cnt = block_sum<int64_t>(cnt, S->scr);
-    mx = block_max<int64_t>(mx, S->scr);
-    if (threadIdx.x == 0) { B.blk_a[bid] = cnt; B.blk_b[bid] = mx; }
-    if (!sync(0, [&] {
-          const int64_t tot = prefix_blocks();
-          const int64_t D = max_blocks_signed();
-          if (threadIdx.x == 0) {
-            Coord& c = co();
-            c.nz_total = tot;
-            c.d_new = (int32_t)(D > 0 ? D : 0);
-            S->plan.th = tau_of((int32_t)D);
-            C->h_pack = 0;
-          }
-        }))
-      return false;
     const int32_t tau = P().th;
-    int32_t* dst = (flags & 2) ? B.nz0 : ((flags & 1) ? B.nz0 : B.nz1);
-    int64_t run = ldcg(B.blk_a + bid);
-    for (int64_t base = s; base < e; base += (int64_t)blockDim.x * kScanU) {
+    Look k = look_begin((int32_t)P().take);
+    const int64_t all = (int64_t)G * blockDim.x;
+    for (int64_t base = 0; base < len; base += all * kScanU) {
       int32_t v[kScanU];
-      uint32_t d[kScanU];
-      int64_t mine = 0, heavy = 0;
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
-        v[q] = i < e ? nz_at(flags, i) : -1;
-      }
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        d[q] = 0;
-        if (v[q] < 0) continue;
-        const uint32_t x = ldcg(B.st + v[q]);
-        if (is_alive(x)) d[q] = deg_of(x);
-        mine += d[q] > 0 ? 1 : 0;
-        heavy += (d[q] > 0 && (int64_t)d[q] >= tau) ? 1 : 0;
-      }
-      int64_t tot, htot;
-      int64_t o = run + block_exclusive_sum<int64_t>(mine, S->scr, &tot);
-      int64_t ho = block_exclusive_sum<int64_t>(heavy, S->scr, &htot);
-      if (htot > 0) {
-        if (threadIdx.x == 0) S->bcast[0] = (int64_t)atomicAdd(&C->h_pack, (unsigned long long)htot);
-        __syncthreads();
-        ho += S->bcast[0];
-        __syncthreads();
-      }
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        if (d[q] == 0) continue;
-        if (CC_IN_BOUNDS(o, B.n, &C->err)) dst[o++] = v[q];
-        if ((int64_t)d[q] >= tau && CC_IN_BOUNDS(ho, B.n, &C->err)) B.hv[ho++] = v[q];
-      }
-      run += tot;
-    }
-    return sync(1, [&] {
-      if (threadIdx.x == 0) {
-        Coord& c = co();
-        c.nz_sel = (flags & 2) ? 0 : ((flags & 1) ? 0 : 1);
-        c.nz_static = 0;
-        c.nz_len = c.nz_total;
-      }
-      __syncthreads();
-      finish_rebuild(co().d_new, (int64_t)vload(&C->h_pack));
-    });
-  }
-
-  // One segment dsort[win_lo, win_lo + win_len) of the degree-order search:
-  // the largest current degree of an alive vertex in it.
-  __device__ bool rebuild_segment() {
-    int64_t s, e;
-    slice(P().win_lo, P().win_len, &s, &e);
-    int64_t mx = 0;
-    for (int64_t base = s; base < e; base += (int64_t)blockDim.x * kScanU) {
       uint32_t x[kScanU];
 #pragma unroll
       for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
-        x[q] = i < e ? ldcg(B.st + __ldg(B.dsort + i)) : 0u;
+        const int64_t i = base + q * all + (int64_t)(threadIdx.x >> 5) * G * 32 + bid * 32 + (threadIdx.x & 31);
+        v[q] = i < len ? __ldg(B.dsort + i) : -1;
       }
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q)
-        if (is_alive(x[q])) mx = (int64_t)deg_of(x[q]) > mx ? (int64_t)deg_of(x[q]) : mx;
+      for (int q = 0; q < kScanU; ++q) x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+      append_heavy<kScanU>(v, x, tau, hv());
+      look_step(k, v, x, tau, base + all * kScanU >= len);
     }
-    mx = block_max<int64_t>(mx, S->scr);
-    if (threadIdx.x == 0) B.blk_b[bid] = mx;
+    look_end(k);
+    return sync(1, [&] { rebuilt(); });
+  }
+
+  // The same from the alive non-isolated vertices.  Every block keeps its own
+  // segment of them (vertex order; of the graph's list at first) and drops from
+  // it, in place, those that have left or have no alive neighbour.
+  __device__ __noinline__ bool rebuild_from_alive() {
+    int64_t s, e;
+    slice(0, B.nz_n, &s, &e);
+    const bool first = S->nz_cnt < 0;
+    const int32_t* const src = first ? B.nz_static : B.nz0;
+    if (!first) e = s + S->nz_cnt;
+    const int32_t tau = P().th;
+    int64_t out = s;
+    Look k = look_begin((int32_t)P().take);
+    const int64_t step = (int64_t)blockDim.x * kScanU;
+    for (int64_t base = s; base < e; base += step) {
+      int32_t v[kScanU];
+      uint32_t x[kScanU];
+      int64_t mine = 0;
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) {
+        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
+        v[q] = i < e ? ldcg(src + i) : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q) mine += is_alive(x[q]) && deg_of(x[q]) > 0 ? 1 : 0;
+      const Scan sc = scan(mine);           // every entry of the step is read by now
+      int64_t o = out + sc.ex;
+#pragma unroll
+      for (int q = 0; q < kScanU; ++q)
+        if (is_alive(x[q]) && deg_of(x[q]) > 0 && CC_IN_BOUNDS(o, B.n, &C->err)) B.nz0[o++] = v[q];
+      out += sc.tot;
+      append_heavy<kScanU>(v, x, tau, hv());
+      look_step(k, v, x, tau, base + step >= e);
+    }
+    look_end(k);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      S->nz_cnt = out - s;
+      atomicAdd(&C->nz_pack, (unsigned long long)(out - s));
+    }
     return sync(0, [&] {
-      const int64_t m = max_blocks_signed();
-      if (threadIdx.x == 0) {
-        Coord& c = co();
-        c.rb_D = m > c.rb_D ? (int32_t)m : c.rb_D;
-        c.rb_lo = c.rb_hi;
-      }
-      __syncthreads();
-      rebuild_advance();
+      if (threadIdx.x == 0) co().nz_len = (int64_t)vload(&C->nz_pack);
+      rebuilt();
     });
   }
 
-  // The heavy list from dsort[0, win_len): every alive vertex of current
-  // degree >= th (> 0).
-  __device__ bool heavy_fill() {
-    int64_t s, e;
-    slice(0, P().win_len, &s, &e);
-    const int64_t tau = P().th;
-    for (int64_t base = s; base < e; base += (int64_t)blockDim.x * kScanU) {
-      int32_t v[kScanU];
-      uint32_t x[kScanU];
-      int64_t heavy = 0;
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const int64_t i = base + (int64_t)threadIdx.x * kScanU + q;
-        v[q] = i < e ? __ldg(B.dsort + i) : -1;
-      }
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        x[q] = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
-        if (!(is_alive(x[q]) && deg_of(x[q]) > 0 && (int64_t)deg_of(x[q]) >= tau)) v[q] = -1;
-        heavy += v[q] >= 0 ? 1 : 0;
-      }
-      int64_t htot;
-      int64_t ho = block_exclusive_sum<int64_t>(heavy, S->scr, &htot);
-      if (htot > 0) {
-        if (threadIdx.x == 0) S->bcast[0] = (int64_t)atomicAdd(&C->h_pack, (unsigned long long)htot);
-        __syncthreads();
-        ho += S->bcast[0];
-        __syncthreads();
-      }
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q)
-        if (v[q] >= 0 && CC_IN_BOUNDS(ho, B.n, &C->err)) B.hv[ho++] = v[q];
+  // Coordinator: the grid has filled H and looked at it.
+  __device__ void rebuilt() {
+    if (threadIdx.x == 0) {
+      co().h_len = (int64_t)vload(&C->h_pack);
+      follow_length();
     }
-    return sync(1, [&] { finish_rebuild(co().rb_D, (int64_t)vload(&C->h_pack)); });
-  }
-
-  __device__ int64_t max_blocks_signed() {
-    int64_t m = -1;
-    for (unsigned b = threadIdx.x; b < G; b += blockDim.x) {
-      const int64_t x = ldcg(B.blk_b + b);
-      m = x > m ? x : m;
-    }
-    return block_max<int64_t>(m, S->scr);
+    __syncthreads();
+    looked();
   }
 
   // ---------------- active-set selection (Alg. 2: A = next k alive of pi) ----
-  // Called by every thread of the block for one tile of the window; entry q
-  // of a thread is an active vertex (rank a[q].x, vertex a[q].y) when want[q].
-  __device__ void emit_actives(const int2* a, const bool* want, int algo) {
-    int64_t deg0[kSelU], row[kSelU];
-    bool listed[kSelU];
-    int64_t nl = 0, el = 0;
+  // One tile of the window as one thread sees it: kSelU consecutive entries of
+  // pi from rank `first`, their vertices (-1: none or removed) and rows.
+  struct SelTile {
+    int64_t first;
+    int32_t v[kSelU];
+    int32_t len[kSelU];
+    int64_t row[kSelU];
+  };
+  __device__ __forceinline__ void sel_vertices(SelTile& T, int64_t base, int64_t e) const {
+    T.first = base + (int64_t)threadIdx.x * kSelU;
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q) T.v[q] = T.first + q < e ? __ldg(B.order + T.first + q) : -1;
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q)
+      if (T.v[q] >= 0 && rtag_of(B.rtag, T.v[q]) != 0) T.v[q] = -1;
+  }
+  __device__ __forceinline__ void sel_rows(SelTile& T) const {
 #pragma unroll
     for (int q = 0; q < kSelU; ++q) {
-      listed[q] = false;
-      deg0[q] = 0;
-      row[q] = 0;
-      if (!want[q]) continue;
-      const int32_t r = a[q].x, v = a[q].y;
-      const uint32_t d = deg_of(ldcg(B.st + v));
-      if (d == 0) {
-        // no alive neighbour: a singleton center.  No pass can reach it
-        // again (its neighbours are all clustered, and later windows start
-        // past it), so it keeps its alive word and zero tag; the label pass
-        // reads an alive word of degree 0 as its own cluster.
-        t.centers += 1;
-      } else {
-        set_rtag(B.rtag, v, (uint32_t)P().tag);
-        row[q] = __ldg(B.off + v);
-        deg0[q] = __ldg(B.off + v + 1) - row[q];
-        B.arank[v] = r;
-        B.st[v] = kActive;
-        listed[q] = true;
-        nl += 1;
-        el += deg0[q];
-        if (algo == kAlgoCW) t.centers += 1;
-      }
+      T.row[q] = T.v[q] >= 0 ? __ldg(B.off + T.v[q]) : 0;
+      T.len[q] = T.v[q] >= 0 ? (int32_t)(__ldg(B.off + T.v[q] + 1) - T.row[q]) : 0;
     }
-    // one atomic per block and tile on the packed list counter
-    int64_t tot;
-    const int64_t pkx = block_exclusive_sum<int64_t>((nl << 40) | el, S->scr, &tot);
-    const int64_t jx = pkx >> 40, ex = pkx & ((1ll << 40) - 1);
-    const int64_t cnt_tot = tot >> 40, e_tot = tot & ((1ll << 40) - 1);
-    if (cnt_tot == 0) return;
+    if (B.n > kStateInL2) return;
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q)
+      if (T.v[q] >= 0 && deg_of(ldcg(B.st + T.v[q])) == 0) T.len[q] = 0;
+  }
+
+  // Emits the entries of a tile that are numbered below `need`, the tile's first
+  // alive entry being number `run` of the window; returns the tile's alive
+  // count.  A vertex without neighbours, or without alive ones by its bound,
+  // is a singleton center for which nothing is written (no pass can reach it,
+  // and later windows start past it); the label pass reads an alive word of
+  // degree 0 as its own cluster.  One scan and one
+  // atomic on the packed list counter per tile (solo: none); the tile that
+  // reaches need is scanned again without its rest.
+  __device__ __forceinline__ int64_t sel_emit(const SelTile& T, int64_t run, int64_t need, bool solo) {
+    const uint32_t tag = (uint32_t)P().tag;
+    // alive << 48 | listed << 36 | entries of the listed rows
+    constexpr int kA = 48, kL = 36;
+    constexpr int64_t kEM = (int64_t(1) << kL) - 1;
+    int64_t pk = 0;
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q)
+      if (T.v[q] >= 0) pk += (int64_t(1) << kA) + (T.len[q] > 0 ? (int64_t(1) << kL) + T.len[q] : 0);
+    Scan sc = scan(pk);
+    const int64_t alive = sc.tot >> kA;
+    int64_t g = run + (sc.ex >> kA);
+    bool want[kSelU];
+    pk = 0;
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q) {
+      want[q] = T.v[q] >= 0 && g < need;
+      if (want[q]) {
+        if (g == 0) *(solo ? &S->sel_r0 : &C->r0) = (int32_t)(T.first + q);
+        if (g == need - 1) *(solo ? &S->sel_cursor : &C->cursor_next) = T.first + q + 1;
+        pk += T.len[q] > 0 ? (int64_t(1) << kL) + T.len[q] : 0;
+      }
+      g += T.v[q] >= 0 ? 1 : 0;
+    }
+    if (run + alive > need) sc = scan(pk);          // uniform
+    const int64_t cnt_tot = (sc.tot >> kL) & 0xFFF, e_tot = sc.tot & kEM;
     if (threadIdx.x == 0) {
-      const unsigned long long old =
-          atomicAdd(&C->act_pack, ((unsigned long long)cnt_tot << kPackShift) | (unsigned long long)e_tot);
+      // ClusterWild!: every one is a center; C4: so far those without neighbours
+      const int64_t wanted = run + alive < need ? alive : need - run;
+      S->tal[kTCenters] += (unsigned long long)(algo == kAlgoCW ? wanted : wanted - cnt_tot);
+      S->tal[kTEdges] += (unsigned long long)(algo == kAlgoCW ? e_tot : 2 * e_tot);      // C4 reads them twice
+    }
+    if (cnt_tot == 0) return alive;
+    if (threadIdx.x == 0) {
+      const unsigned long long add = ((unsigned long long)cnt_tot << kPackShift) | (unsigned long long)e_tot;
+      unsigned long long old;
+      if (solo) {
+        old = S->sel_pack;
+        S->sel_pack = old + add;
+      } else {
+        old = atomicAdd(&C->act_pack, add);
+      }
       S->bcast[0] = (int64_t)(old >> kPackShift);
       S->bcast[1] = (int64_t)(old & kPackEdgeMask);
     }
-    __syncthreads();
-    int64_t j = S->bcast[0] + jx, ep = S->bcast[1] + ex;
-    __syncthreads();
 #pragma unroll
     for (int q = 0; q < kSelU; ++q) {
-      if (!listed[q] || !CC_IN_BOUNDS(j, B.n, &C->err)) continue;
-      B.act_v[j] = a[q].y;
-      B.act_r[j] = a[q].x;
-      B.act_e[j] = ep;
-      B.act_d[j] = row[q] - ep;
-      B.blk_flag[j] = 0;
-      ++j;
-      ep += deg0[q];
+      if (!want[q] || T.len[q] == 0) continue;
+      set_rtag(B.rtag, T.v[q], tag);
+      B.st[T.v[q]] = kActive;
+      if (algo == kAlgoC4) B.arank[T.v[q]] = (int32_t)(T.first + q);
     }
+    __syncthreads();
+    int64_t j = S->bcast[0] + ((sc.ex >> kL) & 0xFFF), ep = S->bcast[1] + (sc.ex & kEM);
+#pragma unroll
+    for (int q = 0; q < kSelU; ++q) {
+      if (!want[q] || T.len[q] == 0 || !CC_IN_BOUNDS(j, B.n, &C->err)) continue;
+      B.act_r[j] = (int32_t)(T.first + q);
+      B.act_e[j] = ep;
+      B.act_d[j] = T.row[q];
+      B.act_n[j] = T.len[q];
+      if (algo == kAlgoC4) {
+        B.act_v[j] = T.v[q];
+        B.blk_flag[j] = 0;
+      }
+      ++j;
+      ep += T.len[q];
+    }
+    return alive;
   }
 
   // Look-back over the team (one pass instead of count, barrier, emit):
@@ -1007,244 +1443,215 @@ struct K {
     volatile unsigned long long* d = B.desc;
     if (threadIdx.x == 0) d[(int64_t)bid * kDescStride] = pack_desc(1, mine);
     const unsigned tag = epoch & 0xFFFFFFu;
-    long long v = 0;
+    int32_t v = 0;
     const uint64_t t0 = globaltimer_ns();
-    for (int64_t q = threadIdx.x; q < (int64_t)bid; q += blockDim.x) {
-      unsigned long long x = d[q * kDescStride];
+    for (unsigned q = threadIdx.x; q < bid; q += blockDim.x) {
+      unsigned long long x = d[(int64_t)q * kDescStride];
       unsigned spins = 0;
       while ((unsigned)(x >> 40) != tag || ((x >> 38) & 3u) == 0) {
         if ((++spins & 63) == 0 && (ld_volatile_int(&C->err) != kOk || globaltimer_ns() - t0 > kBarrierLimitNs)) {
-          atomicCAS(&C->err, kOk, kErrTimeout);
+          fail(kErrTimeout);
           x = 0;
           break;
         }
-        x = d[q * kDescStride];
+        x = d[(int64_t)q * kDescStride];
       }
-      v += (long long)(x & kDescVal);
+      v += (int32_t)(x & kDescVal);          // counts of one window: below 2^31 together
     }
-    const long long excl = block_sum<int64_t>(v, S->scr);
+    const long long excl = sum_i32(v);
     if (threadIdx.x == 0 && bid == G - 1) d[(int64_t)G * kDescStride] = pack_desc(2, excl + mine);
     return excl;
   }
 
-  __device__ bool select(int algo) {
-    for (;;) {
-      const int64_t wlo = P().win_lo, wlen = P().win_len;
-      int64_t s, e;
-      slice(wlo, wlen, &s, &e);
-      // Centers keep their active marker for good (a center's label is its
-      // arank): an active of this round is told from an earlier round's
-      // center by its rank, which is >= r0, the round's first active rank.
-      // count this block's alive entries (the first tile stays in registers)
-      const int64_t tile = (int64_t)blockDim.x * kSelU;
-      int2 a0[kSelU];
-      bool alive0[kSelU];
-      int64_t mine0 = 0;
-#pragma unroll
-      for (int q = 0; q < kSelU; ++q) {
-        const int64_t i = s + (int64_t)threadIdx.x * kSelU + q;
-        a0[q] = i < e ? al_at(i) : make_int2(0, -1);
-      }
-#pragma unroll
-      for (int q = 0; q < kSelU; ++q) {
-        alive0[q] = a0[q].y >= 0 && rtag_of(B.rtag, a0[q].y) == 0;
-        mine0 += alive0[q] ? 1 : 0;
-      }
-      int64_t cnt = mine0;
-      for (int64_t base = s + tile; base < e; base += 2 * tile) {
-        int2 a[2 * kSelU];
-#pragma unroll
-        for (int q = 0; q < 2 * kSelU; ++q) {
-          const int64_t i = base + (int64_t)q * blockDim.x + threadIdx.x;
-          a[q] = i < e ? al_at(i) : make_int2(0, -1);
-        }
-#pragma unroll
-        for (int q = 0; q < 2 * kSelU; ++q)
-          cnt += (a[q].y >= 0 && rtag_of(B.rtag, a[q].y) == 0) ? 1 : 0;
-      }
-      cnt = block_sum<int64_t>(cnt, S->scr);
-      // this block's first alive entry is number `run` of the window
-      int64_t run = lookback(cnt);
-      // emit the alive entries of the window numbered below `need`
-      const int64_t need = P().need;
-      const bool first_window = P().r0 < 0;
-      if (run < need) {
-        for (int64_t base = s; base < e; base += tile) {
-          int2 a[kSelU];
-          bool alive[kSelU];
-          int64_t mine = 0;
-          if (base == s) {
-#pragma unroll
-            for (int q = 0; q < kSelU; ++q) {
-              a[q] = a0[q];
-              alive[q] = alive0[q];
-            }
-            mine = mine0;
-          } else {
-#pragma unroll
-            for (int q = 0; q < kSelU; ++q) {
-              const int64_t i = base + (int64_t)threadIdx.x * kSelU + q;
-              a[q] = i < e ? al_at(i) : make_int2(0, -1);
-            }
-#pragma unroll
-            for (int q = 0; q < kSelU; ++q) {
-              alive[q] = a[q].y >= 0 && rtag_of(B.rtag, a[q].y) == 0;
-              mine += alive[q] ? 1 : 0;
-            }
-          }
-          int64_t tot;
-          int64_t g = run + block_exclusive_sum<int64_t>(mine, S->scr, &tot);
-          bool want[kSelU];
-#pragma unroll
-          for (int q = 0; q < kSelU; ++q) {
-            want[q] = alive[q] && g < need;
-            if (want[q] && g == 0 && first_window) C->r0 = a[q].x;
-            if (want[q] && g == need - 1) C->cursor_next = base + (int64_t)threadIdx.x * kSelU + q + 1;
-            g += alive[q] ? 1 : 0;
-          }
-          emit_actives(a, want, algo);
-          run += tot;
-          if (run >= need) break;           // uniform across the block
-        }
-      }
-      if (!sync(3, [&] {
-            // the four words this decision reads, loaded side by side
-            if (threadIdx.x < 4) {
-              const int i = threadIdx.x;
-              S->bcast[i] = i == 0 ? (int64_t)(ldcg(B.desc + (int64_t)G * kDescStride) & kDescVal)
-                                   : i == 1 ? (int64_t)vload(&C->r0)
-                                   : i == 2 ? vload(&C->cursor_next) : (int64_t)vload(&C->act_pack);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-              Coord& c = co();
-              Plan& p = S->plan;
-              // the last block's inclusive prefix: the window's alive count
-              const int64_t total = S->bcast[0];
-              p.take = total < c.need ? total : c.need;
-              if (c.est) { c.k = total; p.k = total; }   // Sec. 5: all of the window
-              if (p.r0 < 0) p.r0 = (int32_t)S->bcast[1];
-              const int64_t left = c.est ? 0 : c.need - p.take;
-              c.need = left;
-              p.need = left;
-              if (left == 0) {
-                c.cursor = c.est ? c.batch_end : S->bcast[2];
-                const unsigned long long pk = (unsigned long long)S->bcast[3];
-                p.act_n = (int64_t)(pk >> kPackShift);
-                p.act_E = (int64_t)(pk & kPackEdgeMask);
-                // adjacency passes over the active rows: attach (and C4 detection)
-                c.r_edges = p.act_E * (c.algo == kAlgoC4 ? 2 : 1);
-              } else {
-                const int64_t lo2 = c.win_lo + c.win_len;
-                const int64_t avail = c.al_len - lo2;
-                const int64_t alive_left = c.n_alive - (c.k - left);
-                if (avail <= 0 || alive_left <= 0) {
-                  fail(kErrInternal);
-                } else {
-                  const int64_t est = (int64_t)((double)left * (double)avail / (double)alive_left * 1.1) + 1024;
-                  c.win_lo = lo2;
-                  c.win_len = est < avail ? est : avail;
-                  p.win_lo = c.win_lo;
-                  p.win_len = c.win_len;
-                }
-              }
-            }
-          }))
-        return false;
-      if (P().need == 0) return true;
+  // This block's share of the window; solo: the coordinator block takes all of
+  // it, inside a barrier.
+  __device__ __noinline__ void select_window(bool solo) {
+    int64_t s, e;
+    if (solo) {
+      s = P().win_lo;
+      e = s + P().win_len;
+    } else {
+      slice(P().win_lo, P().win_len, &s, &e);
     }
+    // Centers keep their active marker for good: an active of this round is
+    // told from an earlier round's center by its rank (C4), which is >= r0,
+    // the round's first active rank.
+    // Count this block's alive entries; the first tile stays in registers and
+    // its rows are asked for while the block waits for the others' counts.
+    const int64_t tile = (int64_t)blockDim.x * kSelU, need = P().need;
+    int64_t base = s, run = 0;
+    do {
+      SelTile T;
+      sel_vertices(T, base, e);
+      sel_rows(T);
+      if (base == s && !solo) {
+        int32_t cnt = 0;
+#pragma unroll
+        for (int q = 0; q < kSelU; ++q) cnt += T.v[q] >= 0 ? 1 : 0;
+        for (int64_t b = s + tile; b < e; b += 2 * tile) {
+          int32_t v[2 * kSelU];
+#pragma unroll
+          for (int q = 0; q < 2 * kSelU; ++q) {
+            const int64_t i = b + (int64_t)q * blockDim.x + threadIdx.x;
+            v[q] = i < e ? __ldg(B.order + i) : -1;
+          }
+#pragma unroll
+          for (int q = 0; q < 2 * kSelU; ++q) cnt += (v[q] >= 0 && rtag_of(B.rtag, v[q]) == 0) ? 1 : 0;
+        }
+        run = lookback(sum_i32(cnt));       // this block's first alive entry is number `run` of the window
+      }
+      // emit the alive entries of the window numbered below `need`
+      if (run < need) run += sel_emit(T, run, need, solo);
+      base += tile;
+    } while (base < e && run < need);       // uniform across the block
+    if (solo && threadIdx.x == 0) S->sel_total = run;
   }
 
-  // Coordinator: list sizes after the attachment passes.
-  __device__ void co_lists_ready() {
+  // Coordinator: the round's active set is complete, or the next window follows.
+  __device__ __noinline__ void select_decide(bool solo) {
+    if (!solo && threadIdx.x < 4) {
+      const int i = threadIdx.x;            // side by side
+      const int64_t x = i == 0 ? (int64_t)(ldcg(B.desc + (int64_t)G * kDescStride) & kDescVal)
+                               : i == 1 ? (int64_t)vload(&C->r0)
+                               : i == 2 ? vload(&C->cursor_next) : (int64_t)vload(&C->act_pack);
+      if (i == 0) S->sel_total = x;
+      else if (i == 1) S->sel_r0 = (int32_t)x;
+      else if (i == 2) S->sel_cursor = x;
+      else S->sel_pack = (unsigned long long)x;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-      const unsigned long long pk = vload(&C->new_pack);
-      S->plan.new_n = (int64_t)(pk >> kPackShift);
-      S->plan.new_E = (int64_t)(pk & kPackEdgeMask);
+      Coord& c = co();
+      Plan& p = S->plan;
+      const int64_t total = S->sel_total;
+      p.take = total < c.need ? total : c.need;
+      if (c.est) { c.k = total; p.k = total; }   // Sec. 5: all of the window
+      if (p.r0 < 0) p.r0 = S->sel_r0;
+      const int64_t left = c.est ? 0 : c.need - p.take;
+      c.need = left;
+      p.need = left;
+      if (left == 0) {
+        c.cursor = c.est ? c.batch_end : S->sel_cursor;
+        p.act_n = (int64_t)(S->sel_pack >> kPackShift);
+        p.act_E = (int64_t)(S->sel_pack & kPackEdgeMask);
+        p.state = kRun;
+      } else {
+        const int64_t lo2 = c.win_lo + c.win_len;
+        const int64_t avail = c.al_len - lo2;
+        const int64_t alive_left = c.n_alive - (c.k - left);
+        if (avail <= 0 || alive_left <= 0) {
+          fail(kErrInternal);
+          p.state = kAbort;
+        } else {
+          const int64_t est = (int64_t)((float)left * ((float)avail / (float)alive_left) * 1.1f) + 1024;
+          c.win_lo = lo2;
+          c.win_len = est < avail ? est : avail;
+          p.win_lo = c.win_lo;
+          p.win_len = c.win_len;
+          if (solo) C->act_pack = S->sel_pack;   // a longer window goes on from here
+          p.state = kSelect;
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  // Coordinator: short windows at once (a grid phase would cost a barrier and
+  // the same dependent loads); a team of one block has nobody to share with.
+  __device__ __noinline__ void select_here() {
+    while (S->plan.state == kSelect && (G == 1 || P().win_len <= kInlineWindow)) {
+      select_window(true);
+      __syncthreads();
+      select_decide(true);
     }
   }
 
   // ---------------- createCluster: push a center's rank to its neighbours ----
-  // Lanes with push == true try to attach u (state word x, read earlier) to
-  // the center of rank r.  All 32 lanes must call it.
-  __device__ void attach_one(bool push, int32_t u, int32_t r, uint32_t x) {
-    bool fresh = false;
-    uint32_t d_old = 0;
+  // The arrays that the adjacency passes read and write, in registers: a pass
+  // is a function of its own (its own register allocation), and a field of B
+  // read inside its loops would be loaded again after every atomic.
+  struct Words {
+    uint32_t* st;
+    uint32_t* rtag;
+    uint32_t tag;
+  };
+  __device__ __forceinline__ Words words() const { return Words{B.st, B.rtag, (uint32_t)P().tag}; }
+
+  // Tries to attach u (state word x, read earlier; 0: cannot be) to the center
+  // of rank r; true when u was alive.
+  static __device__ __forceinline__ bool attach_one(const Words& W, int32_t u, int32_t r, uint32_t x) {
     const uint32_t nv = kLab + (uint32_t)r;
-    if (push && x > nv) {
-      const uint32_t old = atomicMin(B.st + u, nv);
-      if (is_alive(old)) {
-        fresh = true;
-        d_old = deg_of(old);
-        set_rtag(B.rtag, u, (uint32_t)P().tag);
-      }
+    if (x > nv && is_alive(atomicMin(W.st + u, nv))) {
+      set_rtag(W.rtag, u, W.tag);
+      return true;
     }
-    if (fresh) t.attached += 1;
-    // The center is the only alive neighbour of a fresh vertex of residual
-    // degree 1: nothing to decrement, and no other center can reach it, so
-    // its label is already final.
-    const bool single = fresh && d_old == 1;
-    if (single && CC_IN_BOUNDS(r, B.n, &C->err)) atomicAdd(B.size + r, 1);   // one more member (result unused)
-    const bool want = fresh && d_old != 1;
-    int64_t row = 0;
-    int32_t len = 0;
-    if (want) {
-      row = __ldg(B.off + u);
-      len = (int32_t)(__ldg(B.off + u + 1) - row);
-    }
-    append_stage(app_buf(), want, u, row, len, new_list());
+    return false;
   }
 
-  __device__ void attach_from_actives(bool skip_blocked) {
-    const int64_t an = P().act_n, aE = P().act_E;
-    lbs(B.act_e, an, aE, [&](const Lbs& L) {
-      bool push[kLbsK];
-      int32_t u[kLbsK];
-      uint32_t x[kLbsK];
-#pragma unroll
-      for (int q = 0; q < kLbsK; ++q) {
-        push[q] = L.ok(q) && (!skip_blocked || ldcg(B.blk_flag + L.item(q)) == 0);
-        u[q] = push[q] ? __ldg(B.col + L.csr(q)) : 0;
-        if (push[q] && !CC_IN_BOUNDS(u[q], B.n, &C->err)) push[q] = false;
-      }
+  // The entries of the active rows; aux(j) = payload of active j.
+  template <class Aux, class F>
+  __device__ __forceinline__ void walk_actives(const Aux& aux, F&& f) {
+    const int64_t* const pos = B.act_e;
+    const int64_t* const row = B.act_d;
+    const int32_t* const len = B.act_n;
+    walk(P().act_n, P().act_E, [&](int32_t j) { return ldcg(pos + j); },
+         [&](int32_t j) { return RowItem{ldcg(pos + j), ldcg(row + j), ldcg(len + j), aux(j)}; }, f);
+  }
+
+  __device__ __noinline__ void attach_from_actives(bool skip_blocked) {
+    const Words W = words();
+    const int32_t* const rank = B.act_r;
+    const uint8_t* const blocked = B.blk_flag;
+    int32_t attached = 0;
+    // payload: the center's rank, -1 for a blocked active
+    walk_actives([&](int32_t j) { return skip_blocked && ldcg(blocked + j) ? -1 : ldcg(rank + j); },
+                 [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+      uint32_t x[kB];
       // alive (tag 0): try the atomicMin directly; tagged this round (or 15k
       // rounds ago): the state word decides; removed earlier: nothing to do
-      uint32_t tg[kLbsK];
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) tg[q] = push[q] ? rtag_of(B.rtag, u[q]) : 16u;
+      for (int q = 0; q < kB; ++q) {
+        const bool push = X.w[q] >= 0 && X.aux[q] >= 0 && CC_IN_BOUNDS(X.w[q], B.n, &C->err);
+        x[q] = push ? rtag_of(W.rtag, X.w[q]) : 16u;
+      }
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q)
-        x[q] = tg[q] == 0 ? 0xFFFFFFFFu : (tg[q] == (uint32_t)P().tag ? ldcg(B.st + u[q]) : 0u);
+      for (int q = 0; q < kB; ++q) x[q] = x[q] == 0 ? 0xFFFFFFFFu : (x[q] == W.tag ? ldcg(W.st + X.w[q]) : 0u);
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) attach_one(push[q], u[q], L.vtx(q), x[q]);
-    }, B.act_d, B.act_r);
-    append_flush(app_buf(), new_list());
+      for (int q = 0; q < kB; ++q) attached += attach_one(W, X.w[q], X.aux[q], x[q]) ? 1 : 0;
+    });
+    tally(kTAttached, attached);
   }
 
   // ---------------- C4: blocked detection ------------------------------------
-  __device__ void c4_detect() {
-    const int64_t an = P().act_n, aE = P().act_E;
-    lbs(B.act_e, an, aE, [&](const Lbs& L) {
-      int32_t u[kLbsK];
+  __device__ __noinline__ void c4_detect() {
+    const Words W = words();
+    const int32_t* const rank = B.act_r;
+    const int32_t* const arank = B.arank;
+    uint8_t* const blocked = B.blk_flag;
+    const int32_t r0 = P().r0;
+    walk_actives([&](int32_t j) { return ldcg(rank + j); }, [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+      uint32_t tg[kB];
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) u[q] = L.ok(q) ? __ldg(B.col + L.csr(q)) : 0;
+      for (int q = 0; q < kB; ++q) tg[q] = X.w[q] >= 0 ? rtag_of(W.rtag, X.w[q]) : 16u;
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) {
-        if (!L.ok(q)) continue;
+      for (int q = 0; q < kB; ++q) {
         // an earlier active neighbour: v must wait (isCenter); actives carry
         // this round's tag
-        if (rtag_of(B.rtag, u[q]) != (uint32_t)P().tag) continue;
-        if (is_active(ldcg(B.st + u[q]))) {
-          const int32_t ru = ldcg(B.arank + u[q]);
-          if (ru >= P().r0 && ru < L.vtx(q)) B.blk_flag[L.item(q)] = 1;
+        if (tg[q] != W.tag) continue;
+        if (is_active(ldcg(W.st + X.w[q]))) {
+          const int32_t ru = ldcg(arank + X.w[q]);
+          if (ru >= r0 && ru < X.aux[q]) blocked[X.item[q]] = 1;
         }
       }
-    }, B.act_d, B.act_r);
+    });
   }
 
   // C4: unblocked actives become centers; blocked ones go to the blocked list.
-  __device__ void c4_classify() {
+  __device__ __noinline__ void c4_classify() {
     const int64_t an = P().act_n;
+    int32_t centers = 0, nblocked = 0;
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)G * blockDim.x) >> 5;
@@ -1253,22 +1660,24 @@ struct K {
       bool blocked = false;
       int64_t len = 0, row = 0;
       if (j < an) {
-        const int32_t v = ldcg(B.act_v + j), r = ldcg(B.act_r + j);
+        const int32_t v = ldcg(B.act_v + j);
         if (ldcg(B.blk_flag + j)) {
           blocked = true;
-          row = ldcg(B.act_e + j) + ldcg(B.act_d + j);
-          len = __ldg(B.off + v + 1) - __ldg(B.off + v);
-          t.blocked += 1;
+          row = ldcg(B.act_d + j);
+          len = ldcg(B.act_n + j);
+          nblocked += 1;
         } else {
           B.st[v] = kActCenter;
-          (void)r;
-          t.centers += 1;
+          centers += 1;
         }
       }
+      if (!__any_sync(FULL, blocked)) continue;
       warp_append_rows(blocked, (int32_t)j, row, len, 0x7FFFFFFF, blk_list());
       const int64_t ml = warp_max<int64_t>(len);
-      if (lane == 0 && ml > 0) atomicMax(&C->blk_maxlen, (unsigned long long)ml);
+      if (lane == 0) atomicMax(&C->blk_maxlen, (unsigned long long)ml);
     }
+    tally(kTCenters, centers);
+    tally(kTBlocked, nblocked);
   }
 
   // C4, a round's blocked actives one warp each (every one has a warp of its
@@ -1281,11 +1690,11 @@ struct K {
   // has a resident warp, so the earliest undecided vertex always progresses:
   // the same decisions as the fixpoint, in one grid phase.  Every wait is
   // bounded.
-  __device__ void c4_resolve_by_warp() {
+  __device__ __noinline__ void c4_resolve_by_warp() {
+    const Words W = words();
     const int64_t bn = P().b_n;
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)(threadIdx.x >> 5) * G + bid;     // warps numbered across the blocks first
-    const uint32_t tag = (uint32_t)P().tag;
     const int32_t r0 = P().r0;
     int32_t v = 0, rv = 0;
     int64_t row = 0, len = 0;
@@ -1294,7 +1703,7 @@ struct K {
       v = ldcg(B.act_v + j);
       rv = ldcg(B.act_r + j);
       row = ldcg(B.b_e + gw) + ldcg(B.b_d + gw);
-      len = __ldg(B.off + v + 1) - __ldg(B.off + v);
+      len = ldcg(B.act_n + j);
     }
     int32_t minc = 0x7FFFFFFF;
     bool late = false;
@@ -1303,7 +1712,7 @@ struct K {
       const int64_t e = base + lane;
       if (e >= len || late) continue;
       const int32_t u = __ldg(B.col + row + e);
-      if (rtag_of(B.rtag, u) != tag) continue;                     // not an active of this round
+      if (rtag_of(B.rtag, u) != W.tag) continue;                     // not an active of this round
       uint32_t x = ldcg(B.st + u);
       if (!is_active(x)) continue;                                 // a decided non-center, or attached
       const int32_t ru = ldcg(B.arank + u);
@@ -1324,47 +1733,51 @@ struct K {
     }
     minc = warp_min_i32(minc);
     const bool center = gw < bn && minc == 0x7FFFFFFF;
-    if (gw < bn && lane == 0) {
-      if (center) {
-        atomicExch(B.st + v, kActCenter);
-        t.centers += 1;
-      } else {
-        atomicExch(B.st + v, kLab + (uint32_t)minc);
-        t.noncenter += 1;
-      }
-    }
-    // a non-center leaves with its row (the removal phase walks it)
-    warp_append_rows(gw < bn && !center && lane == 0, v, row, len, 0, new_list());
+    if (gw < bn && lane == 0) atomicExch(B.st + v, center ? kActCenter : kLab + (uint32_t)minc);
+    tally(kTCenters, center && lane == 0 ? 1 : 0);
+    tally(kTNonCenter, gw < bn && !center && lane == 0 ? 1 : 0);
     if (!center) return;
+    int32_t attached = 0;
     for (int64_t base = 0; base < len; base += 32) {
       const int64_t e = base + lane;
       const bool in = e < len;
       const int32_t u = in ? __ldg(B.col + row + e) : 0;
       const uint32_t tg = in ? rtag_of(B.rtag, u) : 16u;
-      const uint32_t x = tg == 0 ? 0xFFFFFFFFu : (tg == tag ? ldcg(B.st + u) : 0u);
-      attach_one(in, u, rv, x);
+      const uint32_t x = tg == 0 ? 0xFFFFFFFFu : (tg == W.tag ? ldcg(B.st + u) : 0u);
+      attached += attach_one(W, u, rv, x) ? 1 : 0;
     }
-    append_flush(app_buf(), new_list());
+    tally(kTAttached, attached);
+  }
+
+  // The entries of the blocked rows; aux = payload(j, v) of active j, vertex v.
+  template <class Aux, class F>
+  __device__ __forceinline__ void walk_blocked(const Aux& aux, F&& f) {
+    walk(P().b_n, P().b_E, [&](int32_t q) { return ldcg(B.b_e + q); },
+         [&](int32_t q) {
+           const int32_t j = ldcg(B.b_j + q);
+           const int64_t e = ldcg(B.b_e + q);
+           return RowItem{e, e + ldcg(B.b_d + q), ldcg(B.act_n + j), aux(j, ldcg(B.act_v + j))};
+         }, f);
   }
 
   // C4 fixpoint, step 1: look at the earlier active neighbours of every
-  // undecided blocked vertex.
-  __device__ void c4_fix_scan() {
-    const int64_t bn = P().b_n, bE = P().b_E;
-    lbs(B.b_e, bn, bE, [&](const Lbs& L) {
+  // undecided blocked vertex (payload: its rank, -1 when decided).
+  __device__ __noinline__ void c4_fix_scan() {
+    const uint32_t tag = (uint32_t)P().tag;
+    const int32_t r0 = P().r0;
+    walk_blocked([&](int32_t j, int32_t v) { return ldcg(B.st + v) == kActive ? ldcg(B.act_r + j) : -1; },
+                 [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
 #pragma unroll
-      for (int i = 0; i < kLbsK; ++i) {
-        if (!L.ok(i)) continue;
-        const int32_t j = ldcg(B.b_j + L.item(i));
-        const int32_t v = ldcg(B.act_v + j), rv = ldcg(B.act_r + j);
-        if (ldcg(B.st + v) != kActive) continue;
-        const int32_t u = __ldg(B.col + L.edge(i) + ldcg(B.b_d + L.item(i)));
-        if (rtag_of(B.rtag, u) != (uint32_t)P().tag) continue;     // not an active of this round
+      for (int i = 0; i < kB; ++i) {
+        const int32_t u = X.w[i];
+        if (u < 0 || X.aux[i] < 0) continue;
+        if (rtag_of(B.rtag, u) != tag) continue;     // not an active of this round
         const uint32_t x = ldcg(B.st + u);
         const int32_t ru = is_active(x) ? ldcg(B.arank + u) : -1;
-        if (ru >= P().r0 && ru < rv) {
-          if (x == kActCenter) B.hit_c[L.item(i)] = 1;
-          else if (x == kActive) B.hit_p[L.item(i)] = 1;
+        if (ru >= r0 && ru < X.aux[i]) {
+          if (x == kActCenter) B.hit_c[X.item[i]] = 1;
+          else if (x == kActive) B.hit_p[X.item[i]] = 1;
         }
       }
     });
@@ -1376,139 +1789,103 @@ struct K {
   __device__ long long c4_fix_decide(int64_t first, int64_t stride) {
     const int64_t bn = P().b_n;
     long long left = 0;
+    int32_t centers = 0;
     for (int64_t q = first; q < bn; q += stride) {
       const int32_t j = ldcg(B.b_j + q);
       const int32_t v = ldcg(B.act_v + j), r = ldcg(B.act_r + j);
       (void)r;
       if (ldcg(B.st + v) != kActive) continue;
       if (ldcg(B.hit_c + q)) B.st[v] = kActNon;
-      else if (!ldcg(B.hit_p + q)) { B.st[v] = kActCenter; t.centers += 1; }
+      else if (!ldcg(B.hit_p + q)) { B.st[v] = kActCenter; centers += 1; }
       else left += 1;
       B.hit_c[q] = 0;
       B.hit_p[q] = 0;
     }
+    tally(kTCenters, centers);
     return left;
   }
 
   // C4 after the fixpoint: blocked centers push, blocked non-centers pull the
-  // lowest center rank among their neighbours.
-  __device__ void c4_blocked_attach() {
-    const int64_t bn = P().b_n, bE = P().b_E;
-    lbs(B.b_e, bn, bE, [&](const Lbs& L) {
+  // lowest center rank among their neighbours (payload: a center's rank, -1
+  // for a non-center).
+  __device__ __noinline__ void c4_blocked_attach() {
+    const Words W = words();
+    const int32_t r0 = P().r0;
+    int32_t attached = 0;
+    walk_blocked([&](int32_t j, int32_t v) { return ldcg(B.st + v) == kActCenter ? ldcg(B.act_r + j) : -1; },
+                 [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
 #pragma unroll
-      for (int i = 0; i < kLbsK; ++i) {
-        bool push = false;
-        int32_t u = 0, r = 0;
-        uint32_t x = 0;
-        if (L.ok(i)) {
-          const int32_t j = ldcg(B.b_j + L.item(i));
-          const int32_t v = ldcg(B.act_v + j);
-          r = ldcg(B.act_r + j);
-          u = __ldg(B.col + L.edge(i) + ldcg(B.b_d + L.item(i)));
-          x = ldcg(B.st + u);
-          if (ldcg(B.st + v) == kActCenter) {
-            push = true;
-          } else if (x == kActCenter) {
-            const int32_t ru = ldcg(B.arank + u);
-            if (ru >= P().r0) atomicMin(B.pull + L.item(i), ru);   // a center of this round
-          }
+      for (int i = 0; i < kB; ++i) {
+        const int32_t u = X.w[i];
+        if (u < 0) continue;
+        const uint32_t x = ldcg(B.st + u);
+        if (X.aux[i] >= 0) {
+          attached += attach_one(W, u, X.aux[i], x) ? 1 : 0;
+        } else if (x == kActCenter) {
+          const int32_t ru = ldcg(B.arank + u);
+          if (ru >= r0) atomicMin(B.pull + X.item[i], ru);   // a center of this round
         }
-        attach_one(push, u, r, x);
       }
     });
-    append_flush(app_buf(), new_list());
+    tally(kTAttached, attached);
   }
 
-  // C4: a non-center active takes its pulled label and joins the removal list.
-  __device__ void c4_pull_finalize() {
+  // C4: a non-center active takes its pulled label.
+  __device__ __noinline__ void c4_pull_finalize() {
     const int64_t bn = P().b_n;
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)G * blockDim.x) >> 5;
-    for (int64_t base = gw * 32; base < bn; base += nw * 32) {
-      const int64_t q = base + lane;
-      bool want = false;
-      int32_t v = 0;
-      int64_t len = 0, row = 0;
-      if (q < bn) {
-        const int32_t j = ldcg(B.b_j + q);
-        v = ldcg(B.act_v + j);
-        if (ldcg(B.st + v) == kActNon) {
-          const int32_t lab = ldcg(B.pull + q);
-          if (lab == 0x7FFFFFFF) fail(kErrInternal);   // a non-center always has a center neighbour
-          B.st[v] = kLab + (uint32_t)lab;
-          t.noncenter += 1;
-          row = ldcg(B.b_e + q) + ldcg(B.b_d + q);
-          len = __ldg(B.off + v + 1) - __ldg(B.off + v);
-          want = true;
-        }
-      }
-      warp_append_rows(want, v, row, len, 0, new_list());
+    int32_t noncenter = 0;
+    for (int64_t q = (int64_t)bid * blockDim.x + threadIdx.x; q < bn; q += (int64_t)G * blockDim.x) {
+      const int32_t v = ldcg(B.act_v + ldcg(B.b_j + q));
+      if (ldcg(B.st + v) != kActNon) continue;
+      const int32_t lab = ldcg(B.pull + q);
+      if (lab == 0x7FFFFFFF) fail(kErrInternal);   // a non-center always has a center neighbour
+      B.st[v] = kLab + (uint32_t)lab;
+      noncenter += 1;
     }
+    tally(kTNonCenter, noncenter);
   }
 
-  // ---------------- removal: residual degrees and the objective --------------
-  // ---------------- removal: residual degrees and the objective --------------
-  __device__ void decrement() {
-    const int64_t nn = P().new_n, nE = P().new_E;
-    lbs(B.new_e, nn, nE, [&](const Lbs& L) {
-      int32_t w[kLbsK];
-      uint32_t lu[kLbsK], x[kLbsK];
+  // ---------------- objective: edges inside clusters --------------------------
+  // This thread's share of the member-member edges inside clusters (batched
+  // jobs; k_intra is the same as a kernel).
+  __device__ __noinline__ int64_t intra_edges() {
+    int64_t cnt = 0;
+    walk(B.up.n, B.up.edges, [&](int32_t j) { return (int64_t)__ldg(B.up.epos + j); },
+         [&](int32_t j) {
+           return RowItem{(int64_t)__ldg(B.up.epos + j), __ldg(B.up.row + j), __ldg(B.up.len + j),
+                          (int32_t)member_id(ldcg(B.st + __ldg(B.up.v + j)))};
+         },
+         [&](const auto& X) {
+      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+      uint32_t x[kB];
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) {
-        w[q] = L.ok(q) ? __ldg(B.col + L.csr(q)) : 0;
-        lu[q] = (uint32_t)L.vtx(q);                             // the member's (final) label
-      }
-      uint32_t tg[kLbsK];
+      for (int q = 0; q < kB; ++q) x[q] = X.w[q] >= 0 ? ldcg(B.st + X.w[q]) : 0;
 #pragma unroll
-      for (int q = 0; q < kLbsK; ++q) tg[q] = L.ok(q) && CC_IN_BOUNDS(w[q], B.n, &C->err) ? rtag_of(B.rtag, w[q]) : 16u;
-      // alive: decrement; maybe removed this round: the state word decides
-      // whether w shares the member's cluster; removed earlier: nothing
-      const uint32_t tag = (uint32_t)P().tag;
-#pragma unroll
-      for (int q = 0; q < kLbsK; ++q) x[q] = tg[q] == tag ? ldcg(B.st + w[q]) : 0;
-#pragma unroll
-      for (int q = 0; q < kLbsK; ++q) {
-        if (!L.ok(q) || !CC_IN_BOUNDS(w[q], B.n, &C->err)) continue;
-        if (L.in_row(q) == 0 && CC_IN_BOUNDS(lu[q], B.n, &C->err)) atomicAdd(B.size + lu[q], 1);   // once per removed member
-        if (tg[q] == 0) {
-          atomicSub(B.st + w[q], 1u);                          // result unused
-        } else if (tg[q] != tag) {
-          continue;
-        } else if (is_active(x[q])) {                          // a center of this round: counted per member
-        } else if (x[q] - kLab == lu[q]) {
-          t.mm += 1;
-        }
-      }
-    }, B.new_d, B.new_v, B.st, kLab);       // payload: the member's label, st[v] - kLab
+      for (int q = 0; q < kB; ++q) cnt += X.w[q] >= 0 && x[q] == (uint32_t)X.aux[q] ? 1 : 0;
+    });
+    return cnt;
   }
 
   // Reduce the round tallies of this block into the control block.
   __device__ void flush_round_tallies() {
-    long long v[5] = {t.centers, t.attached, t.noncenter, t.blocked, (long long)t.mm};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) v[i] = warp_sum(v[i]);
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-      for (int i = 0; i < 5; ++i)
-        if (v[i]) atomicAdd(&S->tal[i], (unsigned long long)v[i]);
-    }
     __syncthreads();
-    if (threadIdx.x < 5) {
-      unsigned long long* dst[5] = {reinterpret_cast<unsigned long long*>(&C->r_centers),
-                                    reinterpret_cast<unsigned long long*>(&C->r_attached),
-                                    reinterpret_cast<unsigned long long*>(&C->r_noncenter),
-                                    reinterpret_cast<unsigned long long*>(&C->r_blocked), &C->mm};
+    if (threadIdx.x < kTallies) {
+      unsigned long long* dst[kTallies] = {reinterpret_cast<unsigned long long*>(&C->r_centers),
+                                           reinterpret_cast<unsigned long long*>(&C->r_attached),
+                                           reinterpret_cast<unsigned long long*>(&C->r_noncenter),
+                                           reinterpret_cast<unsigned long long*>(&C->r_blocked),
+                                           reinterpret_cast<unsigned long long*>(&C->r_edges)};
       const unsigned long long x = S->tal[threadIdx.x];
       if (x) { atomicAdd(dst[threadIdx.x], x); S->tal[threadIdx.x] = 0; }
     }
-    t = Tally{0, 0, 0, 0, 0};
   }
 };
 
 // All rounds of one clustering job, run by the team of blocks in k.  The
 // state words, the control block and the lists in k.B belong to this job.
-__device__ void run_job(K& k, int algo) {
+template <int kPerSM>
+__device__ void run_job(K<kPerSM>& k, int algo) {
   Shared& S = *k.S;
   Ctl* C = k.C;
   if (algo >= 3) algo -= 2;             // the Sec. 5 schedule: same rounds, C4 or ClusterWild!
@@ -1517,41 +1894,55 @@ __device__ void run_job(K& k, int algo) {
     S.co.t0 = globaltimer_ns();
     S.co.round_t0 = S.co.t0;
   }
+  if (threadIdx.x == 0) {
+    S.nz_cnt = -1;
+    k.algo = algo;
+  }
   __syncthreads();
   if (!k.sync(7, [&] { k.co_init(); })) goto out;
 
   for (;;) {
     if (S.plan.state == kDone) break;
-    if (S.plan.state == kRebuildDelta) {
-      if (!k.delta_rebuild()) goto out;
+    if (S.plan.state == kRebuildOrder) {
+      if (!k.rebuild_from_order()) goto out;
       continue;
     }
-    if (S.plan.state == kRebuildDeg) {
-      if (!k.rebuild_segment()) goto out;
+    if (S.plan.state == kRebuildAlive) {
+      if (!k.rebuild_from_alive()) goto out;
       continue;
     }
-    if (S.plan.state == kRebuildHeavy) {
-      if (!k.heavy_fill()) goto out;
+    if (S.plan.state == kRecount) {
+      if (!k.recount_phase()) goto out;
       continue;
     }
-    if (S.plan.state == kScanH) {
-      if (!k.heavy_scan()) goto out;
+    if (S.plan.state == kRecountLong) {
+      if (!k.recount_long()) goto out;
       continue;
     }
     if (S.plan.state == kDrawBatch) {
       if (!k.draw_batch()) goto out;
       continue;
     }
-    if (!k.select(algo)) goto out;
+    if (S.plan.state == kSelect) {
+      k.select_window(false);
+      if (!k.sync(3, [&] {
+            k.select_decide(false);
+            k.select_here();
+          }))
+        goto out;
+      continue;
+    }
     {
       if (algo == kAlgoCW) {
         k.attach_from_actives(false);
-        if (!k.sync(4, [&] { k.co_lists_ready(); })) goto out;
+        k.flush_round_tallies();
+        if (!k.sync(4, [&] { k.co_end_round(); })) goto out;
       } else {
         k.c4_detect();
         if (!k.sync(4)) goto out;
         k.c4_classify();
         k.attach_from_actives(true);
+        k.flush_round_tallies();
         if (!k.sync(4, [&] {
               if (threadIdx.x < 2) S.bcast[threadIdx.x] = (int64_t)vload(threadIdx.x == 0 ? &C->blk_pack : &C->blk_maxlen);
               __syncthreads();
@@ -1563,15 +1954,17 @@ __device__ void run_job(K& k, int algo) {
                 S.co.fix_iter = 0;
                 S.co.r_edges += 2 * S.plan.b_E;       // first fixpoint scan, blocked attach / pull
                 const int64_t warps = (int64_t)k.G * (blockDim.x >> 5);
-                S.plan.pad4 = (S.plan.b_n > 0 && S.plan.b_n <= warps &&
+                S.plan.by_warp = (S.plan.b_n > 0 && S.plan.b_n <= warps &&
                                S.bcast[1] <= (int64_t)k.B.tune.warp_resolve_row) ? 1 : 0;
               }
-              k.co_lists_ready();
+              __syncthreads();
+              if (S.plan.b_n == 0) k.co_end_round();       // nothing blocked: the round is over
             }))
           goto out;
-        if (S.plan.b_n > 0 && S.plan.pad4 == 1) {
+        if (S.plan.b_n > 0 && S.plan.by_warp == 1) {
           k.c4_resolve_by_warp();
-          if (!k.sync(5, [&] { k.co_lists_ready(); })) goto out;
+          k.flush_round_tallies();
+          if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
         } else if (S.plan.b_n > 0) {
           // the pull slots were set when the list was built; the hit flags are zero
           auto after_decide = [&](long long left) {
@@ -1603,12 +1996,10 @@ __device__ void run_job(K& k, int algo) {
           k.c4_blocked_attach();
           if (!k.sync(5)) goto out;
           k.c4_pull_finalize();
-          if (!k.sync(5, [&] { k.co_lists_ready(); })) goto out;
+          k.flush_round_tallies();
+          if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
         }
       }
-      k.decrement();
-      k.flush_round_tallies();
-      if (!k.sync(6, [&] { k.co_end_round(); })) goto out;
     }
   }
 out:
@@ -1616,18 +2007,26 @@ out:
   if (k.bid == 0 && threadIdx.x == 0) {
     C->round = S.co.round;
     C->n_alive = S.co.n_alive;
-    C->mc = (unsigned long long)(S.co.n - S.co.clusters);   // member-center edges
     C->done = S.plan.state == kDone ? 1 : 0;
     for (int i = 0; i < 8; ++i) C->ph_ns[i] = S.co.ph_ns[i];
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_rounds(const __grid_constant__ RoundBuffers B) {
+template <int kPerSM>
+__global__ void __launch_bounds__(kThreads, kPerSM) k_rounds(const __grid_constant__ RoundBuffers B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Shared& S = *reinterpret_cast<Shared*>(smem_raw);
-  K k{B, B.ctl, &S, gridDim.x, blockIdx.x, 0u, Tally{0, 0, 0, 0, 0}};
-  if ((threadIdx.x & 31) == 0) S.u.w.app[threadIdx.x >> 5].n = 0;
-  if (threadIdx.x < 5) S.tal[threadIdx.x] = 0;
+  __shared__ K<kPerSM> k;
+  if (threadIdx.x == 0) {
+    k.B = B;
+    k.C = B.ctl;
+    k.S = &S;
+    k.G = gridDim.x;
+    k.bid = blockIdx.x;
+    k.epoch = 0;
+    S.failed = 0;
+  }
+  if (threadIdx.x < kTallies) S.tal[threadIdx.x] = 0;
   // look-back descriptors of an earlier launch could carry the same epochs:
   // clear this block's before the first barrier
   if (threadIdx.x == 0) B.desc[(int64_t)blockIdx.x * kDescStride] = 0;
@@ -1635,6 +2034,56 @@ __global__ void __launch_bounds__(kThreads, 2) k_rounds(const __grid_constant__ 
   run_job(k, vload(&B.ctl->algo));
 }
 
+
+// Labels (center vertex id = order[center rank]) of the vertices first +
+// threadIdx.x + i * stride, by a block; with kObjective also this thread's share
+// of sum_c C(s_c, 2): the pairs that each member makes with its center and the
+// members counted before it (one add per cluster and warp, see k_sizes_pairs).
+// A center still carries its active word (an isolated vertex its alive word):
+// it is its own cluster.  *members: the members counted, which are also the
+// member-center edges (every member is adjacent to its center).  sig: the
+// signatures of the state words go there (eight per word).
+template <bool kObjective>
+__device__ __forceinline__ int64_t finish_vertices(const RoundBuffers& B, int32_t* labels, uint32_t* sig,
+                                                   int64_t first, int64_t stride, int64_t* members) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = B.n;
+  int64_t pairs = 0, mem = 0;
+  for (int64_t b = first + threadIdx.x - lane; b < n; b += stride) {
+    const int64_t v = b + lane;
+    const uint32_t x = v < n ? ldcg(B.st + v) : kAlive;
+    int32_t c = -1;                        // rank of the cluster that v joined as a member
+    if (v < n) {
+      int32_t lab = (int32_t)v;
+      if (!is_active(x) && x != kAlive) {
+        c = (int32_t)(x - kLab);
+        if (is_alive(x) || c < 0 || c >= n) {
+          atomicCAS(&B.ctl->err, kOk, kErrInternal);
+          c = lab = -1;
+        } else {
+          lab = ldcg(B.order + c);
+        }
+      }
+      if (labels) labels[v] = lab;
+    }
+    if (!kObjective) continue;
+    const unsigned same = __match_any_sync(FULL, c >= 0 ? c : ~lane);
+    if (c >= 0) {
+      mem += 1;
+      if (lane == __ffs(same) - 1) {
+        const int64_t k = __popc(same);
+        const int64_t old = atomicAdd(B.size + c, (int32_t)k);
+        pairs += k * old + k * (k + 1) / 2;
+      }
+    }
+    if (sig) {
+      const uint32_t w = pack_sig8(cluster_sig(x));
+      if (v < n && (lane & 7) == 0) sig[v >> 3] = w;
+    }
+  }
+  *members = mem;
+  return pairs;
+}
 
 // ---------------------------------------------------------------------------
 // Batched engine: many (graph, permutation) jobs in one persistent launch.
@@ -1648,7 +2097,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_rounds(const __grid_constant__ 
 // (histogram, exclusive scan, scatter), then a counting sort on the next
 // kPermSubBits bits plus an insertion sort inside each bucket.  Also writes
 // the initial state words.
-__device__ bool team_permutation(K& k, uint64_t seed) {
+template <int kPerSM>
+__device__ bool team_permutation(K<kPerSM>& k, uint64_t seed) {
   const RoundBuffers& B = k.B;
   Shared& S = *k.S;
   const int64_t n = B.n;
@@ -1767,18 +2217,27 @@ __device__ bool team_permutation(K& k, uint64_t seed) {
   return k.sync(7);
 }
 
-__global__ void __launch_bounds__(kThreads, 2)
+template <int kPerSM>
+__global__ void __launch_bounds__(kThreads, kPerSM)
 k_batch(BatchJob* __restrict__ jobs, int njobs, const RoundBuffers* __restrict__ slots, int team_size, int algo,
         int64_t eps_ppm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Shared& S = *reinterpret_cast<Shared*>(smem_raw);
-  __shared__ RoundBuffers rb;
+  __shared__ K<kPerSM> k;
+  RoundBuffers& rb = k.B;
   const unsigned G = (unsigned)team_size;
   const unsigned team = blockIdx.x / G, nteams = gridDim.x / G;
   if (team >= nteams) return;
   Ctl* C = slots[team].ctl;
-  K k{rb, C, &S, G, blockIdx.x % G, 0u, Tally{0, 0, 0, 0, 0}};
-  if (threadIdx.x == 0) S.plan.state = kDone;
+  if (threadIdx.x == 0) {
+    k.C = C;
+    k.S = &S;
+    k.G = G;
+    k.bid = blockIdx.x % G;
+    k.epoch = 0;
+    S.failed = 0;
+    S.plan.state = kDone;
+  }
   __syncthreads();
   for (int j = (int)team; j < njobs; j += (int)nteams) {
     if (threadIdx.x == 0) {
@@ -1791,6 +2250,7 @@ k_batch(BatchJob* __restrict__ jobs, int njobs, const RoundBuffers* __restrict__
       rb.col = jb.col;
       rb.dsort = jb.dsort;
       rb.dge = jb.dge;
+      rb.up = jb.up;
       rb.nz_static = jb.nz;
       rb.nz_n = jb.nz_n;
       rb.order = rb.order_w;
@@ -1806,51 +2266,41 @@ k_batch(BatchJob* __restrict__ jobs, int njobs, const RoundBuffers* __restrict__
     if (!k.sync(7, [&] {
           if (threadIdx.x == 0) {
             C->err = 0;
+            S.failed = 0;
             C->algo = algo;
             C->eps_ppm = eps_ppm;
             C->seed = jobs[j].seed;
-            C->mc = 0; C->mm = 0; C->pairs = 0;
+            C->intra = 0; C->pairs = 0;
             C->undecided = 0; C->h_pack = 0;
             S.plan.state = kRun;
           }
         }))
       break;
     if (!team_permutation(k, jobs[j].seed)) break;
-    if ((threadIdx.x & 31) == 0) S.u.w.app[threadIdx.x >> 5].n = 0;
-    if (threadIdx.x < 5) S.tal[threadIdx.x] = 0;
+      if (threadIdx.x < kTallies) S.tal[threadIdx.x] = 0;
     __syncthreads();
     run_job(k, algo);
     if (S.plan.state == kAbort) {
       if (k.bid == 0 && threadIdx.x == 0) jobs[j].err = ld_volatile_int(&C->err) ? ld_volatile_int(&C->err) : kErrInternal;
       break;
     }
-    // labels and the pair term of the objective (see k_finalize_labels)
-    unsigned long long pairs = 0;
-    int32_t* const lab = jobs[j].labels;
-    for (int64_t v = (int64_t)k.bid * blockDim.x + threadIdx.x; v < rb.n; v += (int64_t)G * blockDim.x) {
-      const uint32_t x = ldcg(rb.st + v);
-      if (x == kAlive) {                   // selected with residual degree 0: its own cluster
-        if (lab) lab[v] = (int32_t)v;
-        continue;
-      }
-      const int64_t c = is_active(x) ? (int64_t)ldcg(rb.arank + v) : (int64_t)x - kLab;
-      if (is_alive(x) || c < 0 || c >= rb.n) { k.fail(kErrInternal); continue; }
-      const int32_t cv = ldcg(rb.order + c);
-      if (lab) lab[v] = cv;
-      if (cv == v) {
-        const unsigned long long sz = 1ull + (unsigned long long)ldcg(rb.size + c);
-        pairs += sz * (sz - 1) / 2;
-      }
+    // labels and the objective (see k_finalize_labels; k_intra)
+    int64_t members;
+    const int64_t pairs = block_sum<int64_t>(
+        finish_vertices<true>(rb, jobs[j].labels, nullptr, (int64_t)k.bid * blockDim.x, (int64_t)G * blockDim.x,
+                              &members), S.scr);
+    const int64_t inside = block_sum<int64_t>(members + k.intra_edges(), S.scr);
+    if (threadIdx.x == 0) {
+      if (pairs) atomicAdd(&C->pairs, (unsigned long long)pairs);
+      if (inside) atomicAdd(&C->intra, (unsigned long long)inside);
     }
-    pairs = (unsigned long long)block_sum<int64_t>((int64_t)pairs, S.scr);
-    if (threadIdx.x == 0 && pairs) atomicAdd(&C->pairs, pairs);
     if (!k.sync(6, [&] {
           if (threadIdx.x == 0) {
             BatchJob& jb = jobs[j];
             const int done = S.plan.state == kDone && S.co.n_alive == 0;
             jb.rounds = S.co.round;
-            jb.D = jb.nnz / 2 - 2 * (int64_t)vload(&C->mc) - (int64_t)vload(&C->mm) + (int64_t)vload(&C->pairs);
-            jb.err = done ? 0 : kErrInternal;
+            jb.D = jb.nnz / 2 - 2 * (int64_t)vload(&C->intra) + (int64_t)vload(&C->pairs);
+            jb.err = done && vload(&C->err) == kOk ? 0 : kErrInternal;
             jb.t1 = (int64_t)globaltimer_ns();
             S.plan.state = kDone;
           }
@@ -1881,34 +2331,22 @@ __global__ void k_init_state(RoundBuffers B, int algo, int64_t eps_ppm, uint64_t
   }
 }
 
-// Labels (center vertex id = order[center rank]) and the pair term of the
-// objective: vertex v is the center of cluster c exactly when order[c] == v,
-// and its cluster has 1 + size[c] vertices.
-__global__ void k_finalize_labels(RoundBuffers B, int32_t* __restrict__ labels) {
+__global__ void k_finalize_labels(RoundBuffers B, int32_t* __restrict__ labels, bool objective, bool sig) {
   __shared__ int64_t scr[33];
-  const int64_t n = B.n;
-  unsigned long long pairs = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t x = B.st[v];
-    if (x == kAlive) {                     // selected with residual degree 0: its own cluster
-      if (labels) labels[v] = (int32_t)v;
-      continue;
-    }
-    const int64_t c = is_active(x) ? (int64_t)B.arank[v] : (int64_t)x - kLab;   // last round's centers
-    if (is_alive(x) || c < 0 || c >= n) {
-      atomicCAS(&B.ctl->err, kOk, kErrInternal);
-      if (labels) labels[v] = -1;
-      continue;
-    }
-    const int32_t cv = __ldg(B.order + c);
-    if (labels) labels[v] = cv;
-    if (cv == v) {
-      const unsigned long long sz = 1ull + (unsigned long long)B.size[c];
-      pairs += sz * (sz - 1) / 2;
-    }
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x, stride = (int64_t)gridDim.x * blockDim.x;
+  if (!objective) {
+    int64_t members;
+    finish_vertices<false>(B, labels, nullptr, first, stride, &members);
+    return;
   }
-  pairs = (unsigned long long)block_sum<int64_t>((int64_t)pairs, scr);
-  if (threadIdx.x == 0 && pairs) atomicAdd(&B.ctl->pairs, pairs);
+  int64_t members;
+  const int64_t pairs =
+      block_sum<int64_t>(finish_vertices<true>(B, labels, sig ? B.rtag : nullptr, first, stride, &members), scr);
+  members = block_sum<int64_t>(members, scr);
+  if (threadIdx.x == 0) {
+    if (pairs) atomicAdd(&B.ctl->pairs, (unsigned long long)pairs);
+    if (members) atomicAdd(&B.ctl->intra, (unsigned long long)members);
+  }
 }
 
 }  // namespace
@@ -1925,9 +2363,9 @@ size_t rounds_workspace_bytes(int64_t n, int32_t max_deg, int grid) {
   b += align_up(4 * ((nn >> 3) + 1));    // rtag
   b += align_up(4 * nn);                 // arank
   b += 2 * align_up(4 * nn) + 2 * align_up(8 * nn);   // act_v, act_r, act_e, act_d
-  b += align_up(4 * nn) + 2 * align_up(8 * nn);       // new_v, new_e, new_d
+  b += align_up(4 * nn) + align_up(4 * kHList);       // act_n, h_acc
   b += align_up(4 * nn);                 // size
-  b += 3 * align_up(4 * nn);             // hv, nz0, nz1
+  b += 3 * align_up(4 * nn);             // hv, hv2, nz0
   b += 3 * align_up(nn);                 // blk_flag, hit_c, hit_p
   b += align_up(4 * nn);                 // pull
   b += align_up(4 * nn) + 2 * align_up(8 * nn);       // b_j, b_e, b_d
@@ -1949,13 +2387,12 @@ void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* 
   B->act_r = reinterpret_cast<int32_t*>(take(4 * nn));
   B->act_e = reinterpret_cast<int64_t*>(take(8 * nn));
   B->act_d = reinterpret_cast<int64_t*>(take(8 * nn));
-  B->new_v = reinterpret_cast<int32_t*>(take(4 * nn));
-  B->new_e = reinterpret_cast<int64_t*>(take(8 * nn));
-  B->new_d = reinterpret_cast<int64_t*>(take(8 * nn));
+  B->act_n = reinterpret_cast<int32_t*>(take(4 * nn));
+  B->h_acc = reinterpret_cast<unsigned*>(take(4 * kHList));
   B->size = reinterpret_cast<int32_t*>(take(4 * nn));
   B->hv = reinterpret_cast<int32_t*>(take(4 * nn));
+  B->hv2 = reinterpret_cast<int32_t*>(take(4 * nn));
   B->nz0 = reinterpret_cast<int32_t*>(take(4 * nn));
-  B->nz1 = reinterpret_cast<int32_t*>(take(4 * nn));
   B->blk_flag = reinterpret_cast<uint8_t*>(take(nn));
   B->hit_c = reinterpret_cast<uint8_t*>(take(nn));
   B->hit_p = reinterpret_cast<uint8_t*>(take(nn));
@@ -1968,11 +2405,22 @@ void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* 
   B->desc = reinterpret_cast<unsigned long long*>(take(8 * kDescStride * ((size_t)grid + 1)));
 }
 
-int rounds_grid_size(int device) {
+// Blocks of k_rounds per SM.  Rounds of small graphs are a chain of barriers and
+// dependent reads: one block per SM, whose barrier has half the arrivals and
+// whose 128 registers spill nothing, is faster (R-MAT 20, 31M entries: 3.39 ms
+// against 3.98; R-MAT 22, 128M: 5.04 / 5.82; planted 0.7M, 24M: 2.20 / 2.48).
+// From here on the walks of a round are long enough for the entries in flight of
+// twice as many warps to count (planted 4M, 137M entries: 4.02 / 3.86 ms; R-MAT
+// 26, 2.1G: 20.1 / 17.8).
+constexpr int64_t kTwoPerSM = int64_t(1) << 27;
+inline int blocks_per_sm(int64_t nnz) { return nnz < kTwoPerSM ? 1 : 2; }
+
+int rounds_grid_size(int device, int64_t nnz) {
   int sms = 0, per = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  cudaFuncSetAttribute(k_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rounds, kThreads, sizeof(Shared));
+  if (blocks_per_sm(nnz) == 1) return sms;
+  cudaFuncSetAttribute(k_rounds<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rounds<2>, kThreads, sizeof(Shared));
   if (per < 1) per = 1;
   if (per > 2) per = 2;
   return sms * per;
@@ -1988,26 +2436,30 @@ cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint
   if (b.n <= 0) return cudaSuccess;
   RoundBuffers arg = b;
   void* args[] = {&arg};
-  e = cudaFuncSetAttribute(k_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+  const void* const f = blocks_per_sm(b.nnz) == 1 ? (const void*)k_rounds<1> : (const void*)k_rounds<2>;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel((const void*)k_rounds, dim3(grid), dim3(kThreads), args, sizeof(Shared),
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(kThreads), args, sizeof(Shared),
                                      stream);
 }
 
-cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, cudaStream_t stream) {
+cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, bool objective, int num_sms,
+                                   cudaStream_t stream) {
   if (b.n <= 0) return cudaSuccess;
   const int64_t want = (b.n + 255) / 256;
   const int grid = (int)(want < 2048 ? want : 2048);
-  k_finalize_labels<<<grid, 256, 0, stream>>>(b, labels_out);
-  return cudaGetLastError();
+  const bool sig = intra_wants_signatures(b.n);
+  k_finalize_labels<<<grid, 256, 0, stream>>>(b, labels_out, objective, sig);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || !objective) return e;
+  return launch_intra(b.col, b.up, b.st, sig ? b.rtag : nullptr, kLab, kAlive, &b.ctl->intra, num_sms, stream);
 }
-
 
 int batch_grid_size(int device) {
   int sms = 0, per = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch, kThreads, sizeof(Shared));
+  cudaFuncSetAttribute(k_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch<2>, kThreads, sizeof(Shared));
   if (per < 1) per = 1;
   if (per > 2) per = 2;
   return sms * per;
@@ -2033,20 +2485,20 @@ void batch_slot_carve(void* ws, int64_t n_max, int team_size, RoundBuffers* B) {
 // ordinary launch suffices and several batches can share the GPU.
 cudaError_t launch_batch_blocks(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int blocks,
                                 int algo, int64_t eps_ppm, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+  cudaError_t e = cudaFuncSetAttribute(k_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   if (e != cudaSuccess) return e;
-  k_batch<<<blocks, kThreads, sizeof(Shared), stream>>>(const_cast<BatchJob*>(jobs_dev), njobs, slots_dev, 1, algo,
+  k_batch<2><<<blocks, kThreads, sizeof(Shared), stream>>>(const_cast<BatchJob*>(jobs_dev), njobs, slots_dev, 1, algo,
                                                        eps_ppm);
   return cudaGetLastError();
 }
 
 cudaError_t launch_batch(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int team_size,
                          int grid, int algo, int64_t eps_ppm, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+  cudaError_t e = cudaFuncSetAttribute(k_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   if (e != cudaSuccess) return e;
   BatchJob* jobs = const_cast<BatchJob*>(jobs_dev);
   void* args[] = {&jobs, &njobs, &slots_dev, &team_size, &algo, &eps_ppm};
-  return cudaLaunchCooperativeKernel((const void*)k_batch, dim3(grid), dim3(kThreads), args, sizeof(Shared), stream);
+  return cudaLaunchCooperativeKernel((const void*)k_batch<2>, dim3(grid), dim3(kThreads), args, sizeof(Shared), stream);
 }
 
 }  // namespace ccg

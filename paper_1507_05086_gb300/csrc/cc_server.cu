@@ -213,7 +213,7 @@ int start_batch(cc_server* sv, Flight& f, int cls, std::vector<Request>& reqs) {
     BatchJob& jb = f.jobs_host[q];
     jb = BatchJob{};
     jb.off = g->off; jb.col = g->col; jb.nz = g->nz_row; jb.nz_n = g->nz_n;
-    jb.dsort = g->dsort; jb.dge = g->dge;
+    jb.dsort = g->dsort; jb.dge = g->dge; jb.up = g->upper();
     jb.n = g->n; jb.nnz = g->nnz; jb.max_deg = g->max_deg;
     jb.seed = reqs[q].seed;
     jb.labels = reqs[q].labels;
