@@ -13,7 +13,9 @@
 //     two thirds of the batched kernel's co-resident blocks, so that small
 //     jobs always find room);
 //   * larger graphs: the whole GPU per job (cc_cluster) on a worker thread of
-//     their own, one at a time, so that they never hold up the dispatcher.
+//     their own, one at a time, so that they never hold up the dispatcher.  Such
+//     a job starts once the requests submitted before it have been launched:
+//     while its grid waits for the GPU, later launches wait behind it.
 //
 // Every batch runs on its own stream (kStreams of them).  Whenever a stream
 // is free and the device-memory budget has room for a batch's scratch, the
@@ -112,6 +114,7 @@ struct cc_server {
   int64_t next_ticket = 1;
   bool stop = false;
   bool whole_busy = false;
+  bool starting = false;         // the dispatcher is launching requests that have left `pending`
   Flight fl[kStreams];
   cudaStream_t whole_stream = nullptr;
   std::thread worker;            // dispatcher
@@ -266,16 +269,20 @@ void finish_batch(cc_server* sv, Flight& f, cudaError_t ev) {
   f.busy = false;
 }
 
+// Whether the whole-GPU request at the front of its queue may start: nothing
+// submitted before it waits for its launch.  Called with the lock held.
+bool whole_ready(const cc_server* sv) {
+  return !sv->whole.empty() && !sv->starting &&
+         (sv->pending.empty() || sv->pending.front().ticket > sv->whole.front().ticket);
+}
+
 // Whole-GPU requests, one at a time, on their own thread.
 void whole_worker(cc_server* sv) {
   cudaSetDevice(sv->device);
   std::unique_lock<std::mutex> lk(sv->mu);
   for (;;) {
-    sv->cv_whole.wait(lk, [&] { return sv->stop || !sv->whole.empty(); });
-    if (sv->whole.empty()) {
-      if (sv->stop) break;
-      continue;
-    }
+    sv->cv_whole.wait(lk, [&] { return whole_ready(sv) || (sv->stop && sv->whole.empty()); });
+    if (sv->whole.empty()) break;
     Request q = sv->whole.front();
     sv->whole.pop_front();
     sv->whole_busy = true;
@@ -321,6 +328,7 @@ bool gather(cc_server* sv, int cls, bool any_busy, std::vector<Request>& batch, 
         sv->results[it->ticket].status = CC_ERR_OOM;
         it = sv->pending.erase(it);
         sv->cv_done.notify_all();
+        sv->cv_whole.notify_one();
         continue;
       }
       break;                                  // admit it when memory frees up
@@ -368,9 +376,12 @@ void dispatcher(cc_server* sv) {
       sv->in_use += need;
       free_f->share = need;
       free_f->busy = true;                    // reserved while the lock is released
+      sv->starting = true;
       lk.unlock();
       const int st = start_batch(sv, *free_f, cls, batch);
       lk.lock();
+      sv->starting = false;
+      sv->cv_whole.notify_one();
       if (st != CC_OK) {
         // this batch's requests fail; the server carries on
         free_f->busy = false;
