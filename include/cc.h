@@ -330,11 +330,12 @@ int cc_server_destroy(cc_server* s);
  *                    read inside the barrier, 0..65536 (8192)
  *   heavy_shift      heavy-list threshold tau = max(1, Delta >> heavy_shift),
  *                    1..4 (1)
- *   batch_small_n    batched jobs and served requests: one thread block per
- *                    job up to this many vertices, 1..2^20 (65536)
+ *   batch_small_n    served requests: one thread block per job up to this many
+ *                    vertices, 1..2^20 (65536)
  *   batch_team_n     one team of blocks per job up to this many vertices,
  *                    >= batch_small_n, <= 2^24 (2^21)
- *   batch_team_blocks  blocks per team, 2..16 (8)
+ *   batch_team_blocks  blocks per team, 2..16 (8); cc_batch_* calls: at most
+ *                    (the sizes and the number of the jobs decide)
  *   warp_resolve_row C4: a round's blocked actives are decided one warp per
  *                    vertex in one grid phase when each has a warp and no
  *                    blocked row is longer than this (else by the fixpoint of

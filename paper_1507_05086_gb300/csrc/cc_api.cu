@@ -67,9 +67,9 @@ extern "C" int cc_release_memory(void) {
 }
 
 namespace {
-// batched size classes (defaults): up to batch_small_n vertices one block
-// runs a job, up to batch_team_n a team of batch_team_blocks blocks, beyond
-// that the whole grid
+// size classes (defaults): served requests run on one block up to batch_small_n
+// vertices, jobs and requests up to batch_team_n on a team of (at most)
+// batch_team_blocks blocks, larger ones on the whole grid
 constexpr int64_t kBatchSmallN = 1 << 16;
 constexpr int64_t kBatchTeamN = 1 << 21;
 constexpr int kBatchTeamBlocks = 8;
@@ -662,6 +662,81 @@ int cc_disagreements(cc_graph* g, const int32_t* labels, int64_t* out) {
 
 namespace {
 
+// Time of a job on one block, in CSR entries (308 a microsecond): a job of 9K
+// entries takes as long as 0.3M, one of 6.9M no longer than its entries.
+int64_t job_work(const BatchJob& jb) { return jb.nnz + 350000; }
+
+// Cuts the jobs (largest work first) into classes, one per halving of the work,
+// and the blocks into teams.  One block per job gets the most out of the chip
+// (308 entries per microsecond and block; teams of two 279, four 238, eight 176
+// to 220 per block), but then the largest job decides: a job gets the fewest
+// blocks that bring it down to a block's share of all the work.  Jobs that can
+// all run at once that way, or with up to 2.25 times that share for the largest,
+// do: waiting for a second wave costs more (200 jobs of 20K vertices: 3.7 ms
+// against 6.3 queued; 150 of 1K to 500K: 13.9 against 10.8, where the largest
+// job would take 2.6 shares).  Larger classes get 1.3 times their share of the
+// blocks, so that they end first and their teams help the smaller ones (2048
+// jobs up to 1M vertices: 121 ms; 1.0 times 125, 2.0 times 122).  Against one
+// block up to 64K vertices and teams of eight above, one launch after the other
+// and jobs dealt out beforehand: those 2048 jobs 176 -> 121 ms, 144 jobs of 1K
+// to 60K vertices 7.6 -> 4.6.
+void plan_batch(const std::vector<BatchJob>& jobs, int blocks, int team_max, BatchPlan* plan,
+                std::vector<int64_t>* slot_n) {
+  const int nj = (int)jobs.size();
+  BatchPlan p{};
+  std::vector<double> work;              // per class
+  double total = 0;
+  for (int q = 0; q < nj; ++q) {
+    const int64_t w = job_work(jobs[(size_t)q]);
+    if (q == 0 || (p.n < kBatchClasses && 2 * w <= job_work(jobs[(size_t)p.job0[p.n - 1]]))) {
+      p.job0[p.n++] = q;
+      work.push_back(0);
+    }
+    work.back() += (double)w;
+    total += (double)w;
+  }
+  p.job0[p.n] = nj;
+  const int team_cap = std::min(team_max, blocks);
+  const double share = total / blocks;
+  // team sizes that bring every job down to `limit`; returns the blocks they take if all run at once
+  auto teams_for = [&](double limit) {
+    int64_t all = 0;
+    for (int c = 0; c < p.n; ++c) {
+      int g = 1;
+      while (g < team_cap && (double)job_work(jobs[(size_t)p.job0[c]]) > limit * g) g = std::min(2 * g, team_cap);
+      p.team[c] = g;
+      all += (int64_t)g * (p.job0[c + 1] - p.job0[c]);
+    }
+    return all;
+  };
+  double limit = share;
+  if (nj <= blocks)
+    while (limit < 2.25 * share && teams_for(limit) > blocks) limit *= 1.1;
+  if (teams_for(limit) > blocks) teams_for(share);
+  // teams by the classes' shares of the work (at most one per job), then what is
+  // left over from the smallest jobs' class up
+  int left = blocks, teams[kBatchClasses];
+  double work_left = total;
+  for (int c = 0; c < p.n; ++c) {
+    const int most = std::min(p.job0[c + 1] - p.job0[c], left / p.team[c]);
+    teams[c] = std::min(most, std::max(c == 0 ? 1 : 0, (int)(1.3 * work[(size_t)c] / work_left * left / p.team[c] + 0.5)));
+    left -= teams[c] * p.team[c];
+    work_left -= work[(size_t)c];
+  }
+  for (int c = p.n - 1; c >= 0; --c) {
+    const int more = std::min(p.job0[c + 1] - p.job0[c] - teams[c], left / p.team[c]);
+    teams[c] += more;
+    left -= more * p.team[c];
+  }
+  slot_n->assign((size_t)p.n, 0);
+  for (int c = 0; c < p.n; ++c) {
+    p.block0[c + 1] = p.block0[c] + teams[c] * p.team[c];
+    p.slot0[c + 1] = p.slot0[c] + teams[c];
+    for (int q = p.job0[c]; q < nj; ++q) (*slot_n)[(size_t)c] = std::max((*slot_n)[(size_t)c], jobs[(size_t)q].n);
+  }
+  *plan = p;
+}
+
 // Runs every (graph, permutation) job; jobs[i * k_perms + j] gets its rounds
 // and disagreements.
 int run_batch_jobs(cc_graph* const* gs, int32_t count, int algo, double eps, const uint64_t* seeds, int32_t k_perms,
@@ -695,41 +770,52 @@ int run_batch_jobs(cc_graph* const* gs, int32_t count, int algo, double eps, con
       jb.rounds = 0;
       jb.D = 0;
     }
-  // size classes: one block per job, eight-block teams, or the whole grid
+  // jobs of graphs that a team can take, largest work first, and those that
+  // get the whole grid
   const cc_tuning tune = batch_tuning();
-  std::vector<int64_t> cls[3];
-  for (int64_t q = 0; q < njobs; ++q) {
-    const int64_t n = jobs[(size_t)q].n;
-    cls[n <= tune.batch_small_n ? 0 : (n <= tune.batch_team_n ? 1 : 2)].push_back(q);
-  }
-  const int grid0 = batch_grid_size(gs[0]->device);
-  for (int c = 0; c < 2; ++c) {
-    std::vector<int64_t>& ids = cls[c];
-    if (ids.empty()) continue;
-    std::sort(ids.begin(), ids.end(), [&](int64_t a, int64_t b2) { return jobs[(size_t)a].n > jobs[(size_t)b2].n; });
-    const int team = c == 0 ? 1 : tune.batch_team_blocks;
-    const int teams = grid0 / team;
-    if (teams < 1) return CC_ERR_INTERNAL;
-    const int grid = teams * team;
-    const int64_t n_max = jobs[(size_t)ids[0]].n;
-    const size_t slot = align_up(batch_slot_bytes(n_max, team));
-    void* ws = nullptr;
-    CC_TRY(dalloc(&ws, slot * (size_t)teams, s));
-    std::vector<RoundBuffers> slots((size_t)teams);
-    for (int t = 0; t < teams; ++t) {
-      batch_slot_carve(static_cast<char*>(ws) + slot * (size_t)t, n_max, team, &slots[(size_t)t]);
-      slots[(size_t)t].tune = device_tuning(tune);
-      CC_TRY(cudaMemsetAsync(slots[(size_t)t].ctl, 0, sizeof(Ctl), s));
-    }
+  std::vector<int64_t> ids, whole;
+  for (int64_t q = 0; q < njobs; ++q) (jobs[(size_t)q].n <= tune.batch_team_n ? ids : whole).push_back(q);
+  if (!ids.empty()) {
+    std::sort(ids.begin(), ids.end(), [&](int64_t a, int64_t b2) {
+      return job_work(jobs[(size_t)a]) > job_work(jobs[(size_t)b2]);
+    });
     std::vector<BatchJob> sub(ids.size());
     for (size_t q = 0; q < ids.size(); ++q) sub[q] = jobs[(size_t)ids[q]];
+    int blocks = batch_grid_size(gs[0]->device);
+    BatchPlan plan;
+    std::vector<int64_t> slot_n;
+    std::vector<size_t> at;              // scratch slots: offsets, then the total
+    void* ws = nullptr;
+    for (;; blocks /= 2) {               // fewer teams when their scratch does not fit
+      plan_batch(sub, blocks, tune.batch_team_blocks, &plan, &slot_n);
+      at.assign(1, 0);
+      for (int c = 0; c < plan.n; ++c)
+        for (int t = plan.slot0[c]; t < plan.slot0[c + 1]; ++t)
+          at.push_back(at.back() + align_up(batch_slot_bytes(slot_n[(size_t)c], plan.team[c])));
+      const cudaError_t e = dalloc(&ws, at.back(), s);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorMemoryAllocation || blocks < 2) return from_cuda(e);
+      cudaGetLastError();
+    }
+    std::vector<RoundBuffers> slots((size_t)plan.slot0[plan.n]);
+    for (int c = 0; c < plan.n; ++c)
+      for (int t = plan.slot0[c]; t < plan.slot0[c + 1]; ++t) {
+        RoundBuffers& rb = slots[(size_t)t];
+        batch_slot_carve(static_cast<char*>(ws) + at[(size_t)t], slot_n[(size_t)c], plan.team[c], &rb);
+        rb.tune = device_tuning(tune);
+      }
+    // a class's control blocks in one call (they lie a slot apart)
+    for (int c = 0; c < plan.n; ++c) {
+      const size_t t = (size_t)plan.slot0[c], teams = (size_t)plan.slot0[c + 1] - t;
+      if (teams > 0) CC_TRY(cudaMemset2DAsync(slots[t].ctl, at[t + 1] - at[t], 0, sizeof(Ctl), teams, s));
+    }
     BatchJob* jobs_dev = nullptr;
     RoundBuffers* slots_dev = nullptr;
     CC_TRY(dalloc(&jobs_dev, sizeof(BatchJob) * sub.size(), s));
     CC_TRY(dalloc(&slots_dev, sizeof(RoundBuffers) * slots.size(), s));
     CC_TRY(cudaMemcpyAsync(jobs_dev, sub.data(), sizeof(BatchJob) * sub.size(), cudaMemcpyHostToDevice, s));
     CC_TRY(cudaMemcpyAsync(slots_dev, slots.data(), sizeof(RoundBuffers) * slots.size(), cudaMemcpyHostToDevice, s));
-    CC_TRY(launch_batch(jobs_dev, (int)sub.size(), slots_dev, team, grid, algo, ppm, s));
+    CC_TRY(launch_batch(jobs_dev, slots_dev, plan, algo, ppm, s));
     CC_TRY(cudaMemcpyAsync(sub.data(), jobs_dev, sizeof(BatchJob) * sub.size(), cudaMemcpyDeviceToHost, s));
     dfree(jobs_dev, s);
     dfree(slots_dev, s);
@@ -742,7 +828,7 @@ int run_batch_jobs(cc_graph* const* gs, int32_t count, int algo, double eps, con
       jobs[(size_t)ids[q]].err = 0;
     }
   }
-  for (int64_t q : cls[2]) {   // graphs too large for a team: the whole grid per job
+  for (int64_t q : whole) {   // graphs too large for a team: the whole grid per job
     BatchJob& jb = jobs[(size_t)q];
     int32_t r = 0;
     int64_t d = 0;

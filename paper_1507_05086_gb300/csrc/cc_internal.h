@@ -45,6 +45,8 @@ struct Plan {
 static_assert(sizeof(Plan) == 128, "plan layout");
 constexpr int kPlanCopies = 8;
 
+constexpr int kBatchClasses = 12;      // job classes of a batched launch (BatchPlan)
+
 // Device control block of one clustering job.  Zeroed by the host before
 // each launch; written by the kernels only.
 struct Ctl {
@@ -72,6 +74,7 @@ struct Ctl {
   int32_t best, listed_max, other_max;
   // objective tallies: edges inside clusters, sum over clusters of C(size, 2)
   unsigned long long intra, pairs;
+  int queue[kBatchClasses];       // batched launch, slot 0 only: jobs taken per class
   // results, written by the coordinator at the end
   int64_t round, n_alive;
   int done;
@@ -182,16 +185,36 @@ struct BatchJob {
   int64_t t0, t1;       // result: device clock (%globaltimer, ns) at the job's start and end
 };
 
+// How a batched launch shares its blocks out.  Jobs are sorted by work, largest
+// first, and cut into classes; class c has its own teams (of team[c] blocks, on
+// scratch slots that hold its largest graph) and its own queue.  A team whose
+// queue has run dry takes jobs of the later classes.
+struct BatchPlan {
+  int n;
+  int team[kBatchClasses];
+  int block0[kBatchClasses + 1];   // first block of the class; the grid's size
+  int slot0[kBatchClasses + 1];    // first scratch slot; their number
+  int job0[kBatchClasses + 1];     // first job; their number
+};
+// The plan for a single class of equal teams.
+inline BatchPlan one_class(int jobs, int teams, int team) {
+  BatchPlan p{};
+  p.n = 1;
+  p.team[0] = team;
+  p.block0[1] = teams * team;
+  p.slot0[1] = teams;
+  p.job0[1] = jobs;
+  return p;
+}
+
 // Largest co-resident grid of the batched kernel on this device.
 int batch_grid_size(int device);
 // Per-team scratch of a batched launch, sized for the largest job of the launch.
 size_t batch_slot_bytes(int64_t n_max, int team_size);
 void batch_slot_carve(void* ws, int64_t n_max, int team_size, RoundBuffers* B);
-cudaError_t launch_batch(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int team_size,
-                         int grid, int algo, int64_t eps_ppm, cudaStream_t stream);
-// Team size 1 with an ordinary (not cooperative) launch of `blocks` blocks.
-cudaError_t launch_batch_blocks(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int blocks,
-                                int algo, int64_t eps_ppm, cudaStream_t stream);
+// The slots' control blocks are zero.
+cudaError_t launch_batch(const BatchJob* jobs_dev, const RoundBuffers* slots_dev, const BatchPlan& plan, int algo,
+                         int64_t eps_ppm, cudaStream_t stream);
 
 size_t rounds_workspace_bytes(int64_t n, int32_t max_deg, int grid);
 // Carve a workspace of rounds_workspace_bytes() into RoundBuffers (pointers only).

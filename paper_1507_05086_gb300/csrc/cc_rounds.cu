@@ -2087,10 +2087,10 @@ __device__ __forceinline__ int64_t finish_vertices(const RoundBuffers& B, int32_
 
 // ---------------------------------------------------------------------------
 // Batched engine: many (graph, permutation) jobs in one persistent launch.
-// The grid is cut into teams of G blocks; team t runs jobs t, t + T, ...
-// (jobs arrive sorted by size, largest first).  A job is the whole pipeline:
-// permutation, state set-up, all rounds, objective.  Each team owns one
-// scratch slot, reused job after job.
+// The grid is cut into teams (BatchPlan), and a team takes its next job from
+// its class's queue, then from those of smaller jobs.  A job is the whole
+// pipeline: permutation, state set-up, all rounds, objective.  Each team owns
+// one scratch slot, reused job after job.
 // ---------------------------------------------------------------------------
 
 // pi for the job in k.B, computed by the team: bucket by the top key bits
@@ -2219,29 +2219,39 @@ __device__ bool team_permutation(K<kPerSM>& k, uint64_t seed) {
 
 template <int kPerSM>
 __global__ void __launch_bounds__(kThreads, kPerSM)
-k_batch(BatchJob* __restrict__ jobs, int njobs, const RoundBuffers* __restrict__ slots, int team_size, int algo,
-        int64_t eps_ppm) {
+k_batch(BatchJob* __restrict__ jobs, const RoundBuffers* __restrict__ slots, const __grid_constant__ BatchPlan plan,
+        int algo, int64_t eps_ppm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Shared& S = *reinterpret_cast<Shared*>(smem_raw);
   __shared__ K<kPerSM> k;
   RoundBuffers& rb = k.B;
-  const unsigned G = (unsigned)team_size;
-  const unsigned team = blockIdx.x / G, nteams = gridDim.x / G;
-  if (team >= nteams) return;
-  Ctl* C = slots[team].ctl;
+  int cls = 0;
+  while (cls + 1 < plan.n && (int)blockIdx.x >= plan.block0[cls + 1]) ++cls;
+  const unsigned G = (unsigned)plan.team[cls], rel = blockIdx.x - (unsigned)plan.block0[cls];
+  const RoundBuffers& slot = slots[plan.slot0[cls] + (int)(rel / G)];
+  Ctl* const C = slot.ctl;
   if (threadIdx.x == 0) {
     k.C = C;
     k.S = &S;
     k.G = G;
-    k.bid = blockIdx.x % G;
+    k.bid = rel % G;
     k.epoch = 0;
     S.failed = 0;
     S.plan.state = kDone;
   }
+  // the team's next job (-1: none left), published with the plan
+  auto take_job = [&] {
+    S.plan.k = -1;
+    for (int q = cls; q < plan.n && S.plan.k < 0; ++q) {
+      const int j = plan.job0[q] + atomicAdd(&slots[0].ctl->queue[q], 1);
+      if (j < plan.job0[q + 1]) S.plan.k = j;
+    }
+  };
   __syncthreads();
-  for (int j = (int)team; j < njobs; j += (int)nteams) {
+  if (!k.sync(7, [&] { if (threadIdx.x == 0) take_job(); })) return;
+  for (int j; (j = (int)S.plan.k) >= 0;) {
     if (threadIdx.x == 0) {
-      rb = slots[team];
+      rb = slot;
       const BatchJob& jb = jobs[j];
       rb.n = jb.n;
       rb.nnz = jb.nnz;
@@ -2303,6 +2313,7 @@ k_batch(BatchJob* __restrict__ jobs, int njobs, const RoundBuffers* __restrict__
             jb.err = done && vload(&C->err) == kOk ? 0 : kErrInternal;
             jb.t1 = (int64_t)globaltimer_ns();
             S.plan.state = kDone;
+            take_job();
           }
         }))
       break;
@@ -2481,24 +2492,21 @@ void batch_slot_carve(void* ws, int64_t n_max, int team_size, RoundBuffers* B) {
   B->order = B->order_w;
 }
 
-// One block per job (team size 1): no block waits on another, so an
-// ordinary launch suffices and several batches can share the GPU.
-cudaError_t launch_batch_blocks(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int blocks,
-                                int algo, int64_t eps_ppm, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(k_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
-  if (e != cudaSuccess) return e;
-  k_batch<2><<<blocks, kThreads, sizeof(Shared), stream>>>(const_cast<BatchJob*>(jobs_dev), njobs, slots_dev, 1, algo,
-                                                       eps_ppm);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_batch(const BatchJob* jobs_dev, int njobs, const RoundBuffers* slots_dev, int team_size,
-                         int grid, int algo, int64_t eps_ppm, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(k_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+cudaError_t launch_batch(const BatchJob* jobs_dev, const RoundBuffers* slots_dev, const BatchPlan& plan, int algo,
+                         int64_t eps_ppm, cudaStream_t stream) {
+  const void* const f = (const void*)k_batch<2>;
+  const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   if (e != cudaSuccess) return e;
   BatchJob* jobs = const_cast<BatchJob*>(jobs_dev);
-  void* args[] = {&jobs, &njobs, &slots_dev, &team_size, &algo, &eps_ppm};
-  return cudaLaunchCooperativeKernel((const void*)k_batch<2>, dim3(grid), dim3(kThreads), args, sizeof(Shared), stream);
+  BatchPlan p = plan;
+  void* args[] = {&jobs, &slots_dev, &p, &algo, &eps_ppm};
+  const dim3 grid((unsigned)p.block0[p.n]);
+  // teams of one block wait for no other block: an ordinary launch suffices,
+  // and several batches can share the GPU
+  bool alone = true;
+  for (int c = 0; c < p.n; ++c) alone = alone && p.team[c] == 1;
+  return alone ? cudaLaunchKernel(f, grid, dim3(kThreads), args, sizeof(Shared), stream)
+               : cudaLaunchCooperativeKernel(f, grid, dim3(kThreads), args, sizeof(Shared), stream);
 }
 
 }  // namespace ccg

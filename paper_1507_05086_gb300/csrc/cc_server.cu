@@ -201,8 +201,9 @@ int start_batch(cc_server* sv, Flight& f, int cls, std::vector<Request>& reqs) {
   for (int t = 0; t < teams && e == cudaSuccess; ++t) {
     batch_slot_carve(static_cast<char*>(f.ws) + slot * (size_t)t, n_max, team, &f.slots_host[t]);
     f.slots_host[t].tune = sv->tune;
-    e = cudaMemsetAsync(f.slots_host[t].ctl, 0, sizeof(Ctl), f.stream);
   }
+  // all control blocks in one call (they lie a slot apart)
+  if (e == cudaSuccess) e = cudaMemset2DAsync(f.slots_host[0].ctl, slot, 0, sizeof(Ctl), (size_t)teams, f.stream);
   if (e != cudaSuccess) {
     release_device(f);
     return cuda_status(e);
@@ -231,8 +232,7 @@ int start_batch(cc_server* sv, Flight& f, int cls, std::vector<Request>& reqs) {
     e = cudaMemcpyAsync(f.slots_dev, f.slots_host, sizeof(RoundBuffers) * (size_t)teams, cudaMemcpyHostToDevice,
                         f.stream);
   if (e == cudaSuccess) {
-    e = cls == kSmall ? launch_batch_blocks(f.jobs_dev, (int)f.njobs, f.slots_dev, teams, algo, ppm, f.stream)
-                      : launch_batch(f.jobs_dev, (int)f.njobs, f.slots_dev, team, teams * team, algo, ppm, f.stream);
+    e = launch_batch(f.jobs_dev, f.slots_dev, one_class((int)f.njobs, teams, team), algo, ppm, f.stream);
   }
   // the results land in the pinned copy of the jobs: the copy is asynchronous
   if (e == cudaSuccess)
