@@ -56,6 +56,13 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kRowB = 4;                     // entries in flight per lane (8 spill at 64 registers)
 constexpr int kScanU = 4;                    // list entries per thread per scan step
+// ClusterWild! windows of up to this many tiles per block are selected and
+// attached in one pass (select_attach): planted 10^6 at eps 0.1 6.69 -> 5.70 ms
+// for 211 rounds, R-MAT 20 3.67 -> 3.32 for 102.  Longer windows take as long
+// either way (R-MAT 26: 17.7 / 17.6 / 17.7 / 17.6 ms for 0 / 1 / 2 / 4 tiles),
+// and their rows are better shared out by the list of all actives.
+constexpr int64_t kFuseTiles = 2;
+constexpr int32_t kLongAttach = 8192;        // rows longer than this are walked by the whole grid
 constexpr int kSelU = 2;                     // window entries per thread per selection step
 // Up to this many vertices (64 MB of state words, which L2 holds) selection
 // also reads the bounds and spares the rows of vertices known to have no alive
@@ -224,6 +231,12 @@ struct HeavyList {
   int32_t pick[kHPick];          // vertices whose rows are recounted next
 };
 
+// The rows of a tile's centers (select_attach).
+struct TileRows {
+  int64_t row[kThreads * kSelU];
+  int32_t pos[kThreads * kSelU], len[kThreads * kSelU], rank[kThreads * kSelU];
+};
+
 struct Shared {
   Plan plan;
   Coord co;
@@ -245,6 +258,7 @@ struct Shared {
   union {
     HeavyList hl;
     PermSmem perm;
+    TileRows rows;
   } u;
 };
 
@@ -524,7 +538,7 @@ struct K {
       p.need = c.need;
       p.win_lo = c.win_lo;
       p.win_len = c.win_len;
-      p.th = 0;
+      p.th = (int32_t)c.cursor;         // labels from this rank on are this round's
       p.r0 = -1;
       p.tag = (int32_t)(c.round % kTagCycle) + 1;
     }
@@ -1324,13 +1338,21 @@ struct K {
     int32_t len[kSelU];
     int64_t row[kSelU];
   };
+  // Alive when the round began: not removed, or attached in this round, which
+  // select_attach of other blocks may be doing (cw: ClusterWild!; the tag may
+  // also be that of 15k rounds ago, the rank of the label tells).
+  __device__ __forceinline__ bool was_alive(int32_t v, bool cw) const {
+    const uint32_t t = rtag_of(B.rtag, v);
+    if (t == 0) return true;
+    return cw && t == (uint32_t)P().tag && ldcg(B.st + v) >= kLab + (uint32_t)P().th;
+  }
   __device__ __forceinline__ void sel_vertices(SelTile& T, int64_t base, int64_t e) const {
     T.first = base + (int64_t)threadIdx.x * kSelU;
 #pragma unroll
     for (int q = 0; q < kSelU; ++q) T.v[q] = T.first + q < e ? __ldg(B.order + T.first + q) : -1;
 #pragma unroll
     for (int q = 0; q < kSelU; ++q)
-      if (T.v[q] >= 0 && rtag_of(B.rtag, T.v[q]) != 0) T.v[q] = -1;
+      if (T.v[q] >= 0 && !was_alive(T.v[q], algo == kAlgoCW)) T.v[q] = -1;
   }
   __device__ __forceinline__ void sel_rows(SelTile& T) const {
 #pragma unroll
@@ -1341,7 +1363,7 @@ struct K {
     if (B.n > kStateInL2) return;
 #pragma unroll
     for (int q = 0; q < kSelU; ++q)
-      if (T.v[q] >= 0 && deg_of(ldcg(B.st + T.v[q])) == 0) T.len[q] = 0;
+      if (T.v[q] >= 0 && ldcg(B.st + T.v[q]) == kAlive) T.len[q] = 0;      // (a label is no bound)
   }
 
   // Emits the entries of a tile that are numbered below `need`, the tile's first
@@ -1352,15 +1374,22 @@ struct K {
   // degree 0 as its own cluster.  One scan and one
   // atomic on the packed list counter per tile (solo: none); the tile that
   // reaches need is scanned again without its rest.
-  __device__ __forceinline__ int64_t sel_emit(const SelTile& T, int64_t run, int64_t need, bool solo) {
+  // kFused (select_attach): the rows of up to kLongAttach entries go to the
+  // block's tile list, *cnt rows of *entries together, only longer ones to the
+  // round's; *lost counts the new centers that another block had attached.
+  template <bool kFused>
+  __device__ __forceinline__ int64_t sel_emit(const SelTile& T, int64_t run, int64_t need, bool solo,
+                                              int32_t* cnt = nullptr, int32_t* entries = nullptr,
+                                              int32_t* lost = nullptr) {
     const uint32_t tag = (uint32_t)P().tag;
     // alive << 48 | listed << 36 | entries of the listed rows
     constexpr int kA = 48, kL = 36;
     constexpr int64_t kEM = (int64_t(1) << kL) - 1;
+    auto listed = [](int32_t len) { return len > 0 && (!kFused || len <= kLongAttach); };
     int64_t pk = 0;
 #pragma unroll
     for (int q = 0; q < kSelU; ++q)
-      if (T.v[q] >= 0) pk += (int64_t(1) << kA) + (T.len[q] > 0 ? (int64_t(1) << kL) + T.len[q] : 0);
+      if (T.v[q] >= 0) pk += (int64_t(1) << kA) + (listed(T.len[q]) ? (int64_t(1) << kL) + T.len[q] : 0);
     Scan sc = scan(pk);
     const int64_t alive = sc.tot >> kA;
     int64_t g = run + (sc.ex >> kA);
@@ -1372,7 +1401,7 @@ struct K {
       if (want[q]) {
         if (g == 0) *(solo ? &S->sel_r0 : &C->r0) = (int32_t)(T.first + q);
         if (g == need - 1) *(solo ? &S->sel_cursor : &C->cursor_next) = T.first + q + 1;
-        pk += T.len[q] > 0 ? (int64_t(1) << kL) + T.len[q] : 0;
+        pk += listed(T.len[q]) ? (int64_t(1) << kL) + T.len[q] : 0;
       }
       g += T.v[q] >= 0 ? 1 : 0;
     }
@@ -1383,6 +1412,36 @@ struct K {
       const int64_t wanted = run + alive < need ? alive : need - run;
       S->tal[kTCenters] += (unsigned long long)(algo == kAlgoCW ? wanted : wanted - cnt_tot);
       S->tal[kTEdges] += (unsigned long long)(algo == kAlgoCW ? e_tot : 2 * e_tot);      // C4 reads them twice
+    }
+    if (kFused) {
+      TileRows& R = S->u.rows;
+      int32_t j = (int32_t)(sc.ex >> kL) & 0xFFF, ep = (int32_t)(sc.ex & kEM);
+#pragma unroll
+      for (int q = 0; q < kSelU; ++q) {
+        if (!want[q] || T.len[q] == 0) continue;
+        if (!is_alive(atomicExch(B.st + T.v[q], kActive))) *lost += 1;
+        set_rtag(B.rtag, T.v[q], tag);
+        if (listed(T.len[q])) {
+          R.rank[j] = (int32_t)(T.first + q);
+          R.pos[j] = ep;
+          R.row[j] = T.row[q];
+          R.len[j] = T.len[q];
+          ++j;
+          ep += T.len[q];
+          continue;
+        }
+        const unsigned long long at = atomicAdd(&C->act_pack, (1ull << kPackShift) | (unsigned long long)T.len[q]);
+        const int64_t i = (int64_t)(at >> kPackShift);
+        atomicAdd(&S->tal[kTEdges], (unsigned long long)T.len[q]);
+        if (!CC_IN_BOUNDS(i, B.n, &C->err)) continue;
+        B.act_r[i] = (int32_t)(T.first + q);
+        B.act_e[i] = (int64_t)(at & kPackEdgeMask);
+        B.act_d[i] = T.row[q];
+        B.act_n[i] = T.len[q];
+      }
+      *cnt = (int32_t)cnt_tot;
+      *entries = (int32_t)e_tot;
+      return alive;
     }
     if (cnt_tot == 0) return alive;
     if (threadIdx.x == 0) {
@@ -1463,6 +1522,23 @@ struct K {
     return excl;
   }
 
+  // This thread's share of the window's alive entries in [s, e).
+  __device__ __forceinline__ int32_t count_window(int64_t s, int64_t e) const {
+    const int64_t step = 2 * (int64_t)blockDim.x * kSelU;
+    int32_t cnt = 0;
+    for (int64_t b = s; b < e; b += step) {
+      int32_t v[2 * kSelU];
+#pragma unroll
+      for (int q = 0; q < 2 * kSelU; ++q) {
+        const int64_t i = b + (int64_t)q * blockDim.x + threadIdx.x;
+        v[q] = i < e ? __ldg(B.order + i) : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < 2 * kSelU; ++q) cnt += v[q] >= 0 && was_alive(v[q], algo == kAlgoCW) ? 1 : 0;
+    }
+    return cnt;
+  }
+
   // This block's share of the window; solo: the coordinator block takes all of
   // it, inside a barrier.
   __device__ __noinline__ void select_window(bool solo) {
@@ -1488,20 +1564,10 @@ struct K {
         int32_t cnt = 0;
 #pragma unroll
         for (int q = 0; q < kSelU; ++q) cnt += T.v[q] >= 0 ? 1 : 0;
-        for (int64_t b = s + tile; b < e; b += 2 * tile) {
-          int32_t v[2 * kSelU];
-#pragma unroll
-          for (int q = 0; q < 2 * kSelU; ++q) {
-            const int64_t i = b + (int64_t)q * blockDim.x + threadIdx.x;
-            v[q] = i < e ? __ldg(B.order + i) : -1;
-          }
-#pragma unroll
-          for (int q = 0; q < 2 * kSelU; ++q) cnt += (v[q] >= 0 && rtag_of(B.rtag, v[q]) == 0) ? 1 : 0;
-        }
-        run = lookback(sum_i32(cnt));       // this block's first alive entry is number `run` of the window
+        run = lookback(sum_i32(cnt + count_window(s + tile, e)));       // this block's first alive entry is number `run` of the window
       }
       // emit the alive entries of the window numbered below `need`
-      if (run < need) run += sel_emit(T, run, need, solo);
+      if (run < need) run += sel_emit<false>(T, run, need, solo);
       base += tile;
     } while (base < e && run < need);       // uniform across the block
     if (solo && threadIdx.x == 0) S->sel_total = run;
@@ -1588,6 +1654,27 @@ struct K {
     return false;
   }
 
+  // One batch of a walk over centers' rows (payload: the center's rank, -1: not
+  // a center); returns the vertices attached.
+  template <class Batch>
+  __device__ __forceinline__ int32_t attach_batch(const Words& W, const Batch& X) const {
+    int32_t n = 0;
+    constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+    uint32_t x[kB];
+    // alive (tag 0): try the atomicMin directly; tagged this round (or 15k
+    // rounds ago): the state word decides; removed earlier: nothing to do
+#pragma unroll
+    for (int q = 0; q < kB; ++q) {
+      const bool push = X.w[q] >= 0 && X.aux[q] >= 0 && CC_IN_BOUNDS(X.w[q], B.n, &C->err);
+      x[q] = push ? rtag_of(W.rtag, X.w[q]) : 16u;
+    }
+#pragma unroll
+    for (int q = 0; q < kB; ++q) x[q] = x[q] == 0 ? 0xFFFFFFFFu : (x[q] == W.tag ? ldcg(W.st + X.w[q]) : 0u);
+#pragma unroll
+    for (int q = 0; q < kB; ++q) n += attach_one(W, X.w[q], X.aux[q], x[q]) ? 1 : 0;
+    return n;
+  }
+
   // The entries of the active rows; aux(j) = payload of active j.
   template <class Aux, class F>
   __device__ __forceinline__ void walk_actives(const Aux& aux, F&& f) {
@@ -1606,20 +1693,55 @@ struct K {
     // payload: the center's rank, -1 for a blocked active
     walk_actives([&](int32_t j) { return skip_blocked && ldcg(blocked + j) ? -1 : ldcg(rank + j); },
                  [&](const auto& X) {
-      constexpr int kB = sizeof(X.w) / sizeof(int32_t);
-      uint32_t x[kB];
-      // alive (tag 0): try the atomicMin directly; tagged this round (or 15k
-      // rounds ago): the state word decides; removed earlier: nothing to do
-#pragma unroll
-      for (int q = 0; q < kB; ++q) {
-        const bool push = X.w[q] >= 0 && X.aux[q] >= 0 && CC_IN_BOUNDS(X.w[q], B.n, &C->err);
-        x[q] = push ? rtag_of(W.rtag, X.w[q]) : 16u;
-      }
-#pragma unroll
-      for (int q = 0; q < kB; ++q) x[q] = x[q] == 0 ? 0xFFFFFFFFu : (x[q] == W.tag ? ldcg(W.st + X.w[q]) : 0u);
-#pragma unroll
-      for (int q = 0; q < kB; ++q) attached += attach_one(W, X.w[q], X.aux[q], x[q]) ? 1 : 0;
+      attached += attach_batch(W, X);
     });
+    tally(kTAttached, attached);
+  }
+
+  // ClusterWild!: selection and attachment of a window in one pass.  Every alive
+  // vertex of the window below the k-th is a center whatever the others do, so a
+  // block attaches its own ones' neighbours as soon as it knows their numbers,
+  // without a barrier and without the list of actives in between.  A vertex that
+  // another block's center reaches before its own block makes it a center is
+  // taken back (sel_emit); one that is a center already has the smaller word.
+  // Rows of more than kLongAttach entries, which one block would walk alone, are
+  // left to attach_from_actives.
+  __device__ __noinline__ void select_attach() {
+    int64_t s, e;
+    slice(P().win_lo, P().win_len, &s, &e);
+    const Words W = words();
+    const TileRows& R = S->u.rows;
+    const int64_t tile = (int64_t)blockDim.x * kSelU, need = P().need;
+    const WalkShape shape{B.tune.walk_batches, B.tune.prefetch_ahead};
+    const int warp = (int)(threadIdx.x >> 5), nwarps = kThreads / 32;
+    int64_t base = s, run = 0;
+    int32_t attached = 0;
+    do {
+      SelTile T;
+      sel_vertices(T, base, e);
+      sel_rows(T);
+#pragma unroll
+      for (int q = 0; q < kSelU; ++q)
+        if (T.len[q] > 0) prefetch_l2(B.col + T.row[q]);
+      if (base == s) {
+        int32_t cnt = 0;
+#pragma unroll
+        for (int q = 0; q < kSelU; ++q) cnt += T.v[q] >= 0 ? 1 : 0;
+        run = lookback(sum_i32(cnt + count_window(s + tile, e)));
+      }
+      if (run < need) {
+        int32_t cnt, E, lost = 0;
+        run += sel_emit<true>(T, run, need, false, &cnt, &E, &lost);
+        attached -= lost;
+        __syncthreads();
+        auto at = [&](int32_t j) { return (int64_t)R.pos[j]; };
+        auto load = [&](int32_t j) { return RowItem{(int64_t)R.pos[j], R.row[j], R.len[j], R.rank[j]}; };
+        auto f = [&](const auto& X) { attached += attach_batch(W, X); };
+        if (E <= 64 * nwarps) row_walk<1>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
+        else row_walk<kRowB>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
+      }
+      base += tile;
+    } while (base < e && run < need);       // uniform across the block
     tally(kTAttached, attached);
   }
 
@@ -1924,6 +2046,16 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
       continue;
     }
     if (S.plan.state == kSelect) {
+      if (algo == kAlgoCW && k.G > 1 && S.plan.win_len <= kFuseTiles * (int64_t)k.G * kThreads * kSelU) {
+        k.select_attach();
+        k.flush_round_tallies();
+        if (!k.sync(4, [&] {
+              k.select_decide(false);
+              if (S.plan.state == kRun && S.plan.act_n == 0) k.co_end_round();      // no longer rows left
+            }))
+          goto out;
+        continue;
+      }
       k.select_window(false);
       if (!k.sync(3, [&] {
             k.select_decide(false);
