@@ -14,7 +14,7 @@
 //   clustered ........ kLab + center rank
 //   active ............ kActive / kActCenter / kActNon (undecided or
 //                       ClusterWild! center / C4 center / C4 non-center)
-// An active's rank is kept in arank[v].  A center keeps its active marker for
+// C4 keeps every vertex's rank in arank[v].  A center keeps its active marker for
 // good (its label is its own rank, arank); the actives of the current round
 // are the ones whose rank is >= r0, the round's first active rank.
 //
@@ -56,12 +56,14 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kRowB = 4;                     // entries in flight per lane (8 spill at 64 registers)
 constexpr int kScanU = 4;                    // list entries per thread per scan step
-// ClusterWild! windows of up to this many tiles per block are selected and
-// attached in one pass (select_attach): planted 10^6 at eps 0.1 6.69 -> 5.70 ms
-// for 211 rounds, R-MAT 20 3.67 -> 3.32 for 102.  Longer windows take as long
-// either way (R-MAT 26: 17.7 / 17.6 / 17.7 / 17.6 ms for 0 / 1 / 2 / 4 tiles),
-// and their rows are better shared out by the list of all actives.
-constexpr int64_t kFuseTiles = 2;
+// Windows of up to this many entries per block are selected and attached in one
+// pass (select_attach).  ClusterWild!: planted 10^6 at eps 0.1 6.69 -> 5.47 ms
+// for 211 rounds, R-MAT 20 3.67 -> 3.19 for 102.  C4: planted 0.7M at eps 0.9
+// 1.44 -> 1.23 ms for 22 rounds, R-MAT 24 12.2 -> 11.4 for 145.  Longer windows
+// take as long either way (ClusterWild! on R-MAT 26: 17.7 / 17.6 / 17.7 / 17.6
+// ms for 0 / 1024 / 2048 / 4096; C4 on R-MAT 24: 11.6 / 11.4 / 11.4 for 1024 /
+// 2048 / 8192), and their rows are better shared out by the list of all actives.
+constexpr int64_t kFuseWindow = 2048;
 constexpr int32_t kLongAttach = 8192;        // rows longer than this are walked by the whole grid
 constexpr int kSelU = 2;                     // window entries per thread per selection step
 // Up to this many vertices (64 MB of state words, which L2 holds) selection
@@ -73,6 +75,7 @@ constexpr int kAlgoC4 = 1, kAlgoCW = 2;
 constexpr int kRun = 0, kDone = 1, kSelect = 2, kAbort = 3, kDrawBatch = 6;   // kRun: the active set is there
 constexpr int kRebuildOrder = 7, kRebuildAlive = 8; // heavy list from the degree order, from the alive vertices
 constexpr int kRecount = 9, kRecountLong = 10;      // degree recounts
+constexpr int kResolve = 11;                 // C4: the round's blocked actives are listed
 // where co_delta takes up again, or what it does next
 constexpr int kDScan = 0, kDCounted = 1, kDRebuild = 2, kDPlanned = 3, kDDone = 4;
 constexpr int kHList = kThreads;             // heavy lists up to this long: every block lists all of them
@@ -231,10 +234,11 @@ struct HeavyList {
   int32_t pick[kHPick];          // vertices whose rows are recounted next
 };
 
-// The rows of a tile's centers (select_attach).
+// The rows of a tile's actives (select_attach).
 struct TileRows {
   int64_t row[kThreads * kSelU];
-  int32_t pos[kThreads * kSelU], len[kThreads * kSelU], rank[kThreads * kSelU];
+  int32_t pos[kThreads * kSelU], len[kThreads * kSelU], rank[kThreads * kSelU], v[kThreads * kSelU];
+  uint8_t blocked[kThreads * kSelU];
 };
 
 struct Shared {
@@ -1197,6 +1201,27 @@ struct K {
     co_go_on();
   }
 
+  // Coordinator: the centers that nothing blocked have attached their
+  // neighbours; the round ends, or the blocked actives are next.
+  __device__ __noinline__ void co_blocked() {
+    if (threadIdx.x < 2) S->bcast[threadIdx.x] = (int64_t)vload(threadIdx.x == 0 ? &C->blk_pack : &C->blk_maxlen);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      Plan& p = S->plan;
+      const unsigned long long pk = (unsigned long long)S->bcast[0];
+      p.b_n = (int64_t)(pk >> kPackShift);
+      p.b_E = (int64_t)(pk & kPackEdgeMask);
+      p.undecided = p.b_n;
+      p.state = kResolve;
+      co().fix_iter = 0;
+      co().r_edges += 2 * p.b_E;            // first fixpoint scan, blocked attach / pull
+      const int64_t warps = (int64_t)G * (blockDim.x >> 5);
+      p.by_warp = p.b_n <= warps && S->bcast[1] <= (int64_t)B.tune.warp_resolve_row ? 1 : 0;
+    }
+    __syncthreads();
+    if (P().b_n == 0) co_end_round();
+  }
+
   // ---------------- Sec. 5: the round's binomial batch ------------------------
   // Every block counts its share of the round's draws below the threshold
   // (plan: win_len trials, need = threshold bits, take = every trial
@@ -1330,40 +1355,56 @@ struct K {
   }
 
   // ---------------- active-set selection (Alg. 2: A = next k alive of pi) ----
-  // One tile of the window as one thread sees it: kSelU consecutive entries of
+  // One tile of the window as one thread sees it: kU consecutive entries of
   // pi from rank `first`, their vertices (-1: none or removed) and rows.
+  template <int kU>
   struct SelTile {
     int64_t first;
-    int32_t v[kSelU];
-    int32_t len[kSelU];
-    int64_t row[kSelU];
+    int32_t v[kU];
+    int32_t len[kU];
+    int64_t row[kU];
   };
   // Alive when the round began: not removed, or attached in this round, which
-  // select_attach of other blocks may be doing (cw: ClusterWild!; the tag may
-  // also be that of 15k rounds ago, the rank of the label tells).
-  __device__ __forceinline__ bool was_alive(int32_t v, bool cw) const {
+  // select_attach of other blocks may be doing (the tag may also be that of 15k
+  // rounds ago, the rank of the label tells).
+  __device__ __forceinline__ bool was_alive(int32_t v) const {
     const uint32_t t = rtag_of(B.rtag, v);
     if (t == 0) return true;
-    return cw && t == (uint32_t)P().tag && ldcg(B.st + v) >= kLab + (uint32_t)P().th;
+    return t == (uint32_t)P().tag && ldcg(B.st + v) >= kLab + (uint32_t)P().th;
   }
-  __device__ __forceinline__ void sel_vertices(SelTile& T, int64_t base, int64_t e) const {
-    T.first = base + (int64_t)threadIdx.x * kSelU;
+  template <int kU>
+  __device__ __forceinline__ void sel_vertices(SelTile<kU>& T, int64_t base, int64_t e) const {
+    T.first = base + (int64_t)threadIdx.x * kU;
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q) T.v[q] = T.first + q < e ? __ldg(B.order + T.first + q) : -1;
+    for (int q = 0; q < kU; ++q) T.v[q] = T.first + q < e ? __ldg(B.order + T.first + q) : -1;
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q)
-      if (T.v[q] >= 0 && !was_alive(T.v[q], algo == kAlgoCW)) T.v[q] = -1;
+    for (int q = 0; q < kU; ++q)
+      if (T.v[q] >= 0 && !was_alive(T.v[q])) T.v[q] = -1;
   }
-  __device__ __forceinline__ void sel_rows(SelTile& T) const {
+  template <int kU>
+  __device__ __forceinline__ void sel_rows(SelTile<kU>& T) const {
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q) {
+    for (int q = 0; q < kU; ++q) {
       T.row[q] = T.v[q] >= 0 ? __ldg(B.off + T.v[q]) : 0;
       T.len[q] = T.v[q] >= 0 ? (int32_t)(__ldg(B.off + T.v[q] + 1) - T.row[q]) : 0;
     }
     if (B.n > kStateInL2) return;
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q)
+    for (int q = 0; q < kU; ++q)
       if (T.v[q] >= 0 && ldcg(B.st + T.v[q]) == kAlive) T.len[q] = 0;      // (a label is no bound)
+  }
+
+  // Entry j of the round's list of actives (flag: see blk_flag).
+  __device__ __forceinline__ void put_active(int64_t j, int64_t before, int32_t v, int32_t rank, int64_t row, int32_t len,
+                                             uint8_t flag) {
+    if (!CC_IN_BOUNDS(j, B.n, &C->err)) return;
+    B.act_r[j] = rank;
+    B.act_e[j] = before;
+    B.act_d[j] = row;
+    B.act_n[j] = len;
+    if (algo != kAlgoC4) return;
+    B.act_v[j] = v;
+    B.blk_flag[j] = flag;
   }
 
   // Emits the entries of a tile that are numbered below `need`, the tile's first
@@ -1377,8 +1418,8 @@ struct K {
   // kFused (select_attach): the rows of up to kLongAttach entries go to the
   // block's tile list, *cnt rows of *entries together, only longer ones to the
   // round's; *lost counts the new centers that another block had attached.
-  template <bool kFused>
-  __device__ __forceinline__ int64_t sel_emit(const SelTile& T, int64_t run, int64_t need, bool solo,
+  template <bool kFused, bool kC4 = false, int kU>
+  __device__ __forceinline__ int64_t sel_emit(const SelTile<kU>& T, int64_t run, int64_t need, bool solo,
                                               int32_t* cnt = nullptr, int32_t* entries = nullptr,
                                               int32_t* lost = nullptr) {
     const uint32_t tag = (uint32_t)P().tag;
@@ -1388,15 +1429,15 @@ struct K {
     auto listed = [](int32_t len) { return len > 0 && (!kFused || len <= kLongAttach); };
     int64_t pk = 0;
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q)
+    for (int q = 0; q < kU; ++q)
       if (T.v[q] >= 0) pk += (int64_t(1) << kA) + (listed(T.len[q]) ? (int64_t(1) << kL) + T.len[q] : 0);
     Scan sc = scan(pk);
     const int64_t alive = sc.tot >> kA;
     int64_t g = run + (sc.ex >> kA);
-    bool want[kSelU];
+    bool want[kU];
     pk = 0;
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q) {
+    for (int q = 0; q < kU; ++q) {
       want[q] = T.v[q] >= 0 && g < need;
       if (want[q]) {
         if (g == 0) *(solo ? &S->sel_r0 : &C->r0) = (int32_t)(T.first + q);
@@ -1417,7 +1458,7 @@ struct K {
       TileRows& R = S->u.rows;
       int32_t j = (int32_t)(sc.ex >> kL) & 0xFFF, ep = (int32_t)(sc.ex & kEM);
 #pragma unroll
-      for (int q = 0; q < kSelU; ++q) {
+      for (int q = 0; q < kU; ++q) {
         if (!want[q] || T.len[q] == 0) continue;
         if (!is_alive(atomicExch(B.st + T.v[q], kActive))) *lost += 1;
         set_rtag(B.rtag, T.v[q], tag);
@@ -1426,18 +1467,19 @@ struct K {
           R.pos[j] = ep;
           R.row[j] = T.row[q];
           R.len[j] = T.len[q];
+          if (kC4) {
+            R.v[j] = T.v[q];
+            R.blocked[j] = 0;
+          }
           ++j;
           ep += T.len[q];
           continue;
         }
         const unsigned long long at = atomicAdd(&C->act_pack, (1ull << kPackShift) | (unsigned long long)T.len[q]);
-        const int64_t i = (int64_t)(at >> kPackShift);
-        atomicAdd(&S->tal[kTEdges], (unsigned long long)T.len[q]);
-        if (!CC_IN_BOUNDS(i, B.n, &C->err)) continue;
-        B.act_r[i] = (int32_t)(T.first + q);
-        B.act_e[i] = (int64_t)(at & kPackEdgeMask);
-        B.act_d[i] = T.row[q];
-        B.act_n[i] = T.len[q];
+        put_active((int64_t)(at >> kPackShift), (int64_t)(at & kPackEdgeMask), T.v[q], (int32_t)(T.first + q),
+                   T.row[q], T.len[q], 0);
+        atomicAdd(&S->tal[kTEdges], (unsigned long long)T.len[q] * (kC4 ? 2 : 1));
+        if (kC4) atomicAdd(&S->tal[kTCenters], ~0ull);      // not one yet
       }
       *cnt = (int32_t)cnt_tot;
       *entries = (int32_t)e_tot;
@@ -1457,25 +1499,17 @@ struct K {
       S->bcast[1] = (int64_t)(old & kPackEdgeMask);
     }
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q) {
+    for (int q = 0; q < kU; ++q) {
       if (!want[q] || T.len[q] == 0) continue;
       set_rtag(B.rtag, T.v[q], tag);
       B.st[T.v[q]] = kActive;
-      if (algo == kAlgoC4) B.arank[T.v[q]] = (int32_t)(T.first + q);
     }
     __syncthreads();
     int64_t j = S->bcast[0] + ((sc.ex >> kL) & 0xFFF), ep = S->bcast[1] + (sc.ex & kEM);
 #pragma unroll
-    for (int q = 0; q < kSelU; ++q) {
-      if (!want[q] || T.len[q] == 0 || !CC_IN_BOUNDS(j, B.n, &C->err)) continue;
-      B.act_r[j] = (int32_t)(T.first + q);
-      B.act_e[j] = ep;
-      B.act_d[j] = T.row[q];
-      B.act_n[j] = T.len[q];
-      if (algo == kAlgoC4) {
-        B.act_v[j] = T.v[q];
-        B.blk_flag[j] = 0;
-      }
+    for (int q = 0; q < kU; ++q) {
+      if (!want[q] || T.len[q] == 0) continue;
+      put_active(j, ep, T.v[q], (int32_t)(T.first + q), T.row[q], T.len[q], 0);
       ++j;
       ep += T.len[q];
     }
@@ -1534,7 +1568,7 @@ struct K {
         v[q] = i < e ? __ldg(B.order + i) : -1;
       }
 #pragma unroll
-      for (int q = 0; q < 2 * kSelU; ++q) cnt += v[q] >= 0 && was_alive(v[q], algo == kAlgoCW) ? 1 : 0;
+      for (int q = 0; q < 2 * kSelU; ++q) cnt += v[q] >= 0 && was_alive(v[q]) ? 1 : 0;
     }
     return cnt;
   }
@@ -1557,7 +1591,7 @@ struct K {
     const int64_t tile = (int64_t)blockDim.x * kSelU, need = P().need;
     int64_t base = s, run = 0;
     do {
-      SelTile T;
+      SelTile<kSelU> T;
       sel_vertices(T, base, e);
       sel_rows(T);
       if (base == s && !solo) {
@@ -1624,8 +1658,10 @@ struct K {
 
   // Coordinator: short windows at once (a grid phase would cost a barrier and
   // the same dependent loads); a team of one block has nobody to share with.
+  // Not C4's, whose blocked actives the grid finds in the same phase
+  // (select_attach): R-MAT 18 by the Sec. 5 schedule 13.9 -> 12.8 ms.
   __device__ __noinline__ void select_here() {
-    while (S->plan.state == kSelect && (G == 1 || P().win_len <= kInlineWindow)) {
+    while (S->plan.state == kSelect && (G == 1 || (algo == kAlgoCW && P().win_len <= kInlineWindow))) {
       select_window(true);
       __syncthreads();
       select_decide(true);
@@ -1698,51 +1734,118 @@ struct K {
     tally(kTAttached, attached);
   }
 
-  // ClusterWild!: selection and attachment of a window in one pass.  Every alive
-  // vertex of the window below the k-th is a center whatever the others do, so a
-  // block attaches its own ones' neighbours as soon as it knows their numbers,
-  // without a barrier and without the list of actives in between.  A vertex that
-  // another block's center reaches before its own block makes it a center is
-  // taken back (sel_emit); one that is a center already has the smaller word.
-  // Rows of more than kLongAttach entries, which one block would walk alone, are
-  // left to attach_from_actives.
+  // Selection and attachment of a window in one pass.  ClusterWild!: every alive
+  // vertex of the window below the k-th is a center whatever the others do.  C4:
+  // it is one unless a neighbour of lower rank was alive when the round began
+  // (all of those are active too), which the ranks of pi tell without waiting
+  // for the other blocks' actives; the others are blocked and listed for the
+  // next phase.  So a block attaches its own centers' neighbours as soon as the
+  // look-back tells it their numbers, without barriers and without the list of
+  // actives in between.  A vertex that another block's center reaches before its
+  // own block makes it active is taken back (sel_emit); one that is active
+  // already has the smaller word.  Rows of more than kLongAttach entries, which
+  // one block would walk alone, are left to the passes over that list.
+  // kU entries per thread and tile: one for small graphs, whose windows are short
+  // (planted 10^6 5.71 -> 5.47 ms, R-MAT 20 3.31 -> 3.19), two for large ones (R-MAT
+  // 26: 17.6 ms against 17.9).
+  template <bool kC4, int kU>
   __device__ __noinline__ void select_attach() {
     int64_t s, e;
     slice(P().win_lo, P().win_len, &s, &e);
     const Words W = words();
-    const TileRows& R = S->u.rows;
-    const int64_t tile = (int64_t)blockDim.x * kSelU, need = P().need;
+    TileRows& R = S->u.rows;
+    const int32_t* const arank = B.arank;
+    const int32_t r_lo = P().th;
+    const int64_t tile = (int64_t)blockDim.x * kU, need = P().need;
     const WalkShape shape{B.tune.walk_batches, B.tune.prefetch_ahead};
     const int warp = (int)(threadIdx.x >> 5), nwarps = kThreads / 32;
     int64_t base = s, run = 0;
     int32_t attached = 0;
     do {
-      SelTile T;
+      SelTile<kU> T;
       sel_vertices(T, base, e);
       sel_rows(T);
 #pragma unroll
-      for (int q = 0; q < kSelU; ++q)
+      for (int q = 0; q < kU; ++q)
         if (T.len[q] > 0) prefetch_l2(B.col + T.row[q]);
       if (base == s) {
         int32_t cnt = 0;
 #pragma unroll
-        for (int q = 0; q < kSelU; ++q) cnt += T.v[q] >= 0 ? 1 : 0;
+        for (int q = 0; q < kU; ++q) cnt += T.v[q] >= 0 ? 1 : 0;
         run = lookback(sum_i32(cnt + count_window(s + tile, e)));
       }
       if (run < need) {
         int32_t cnt, E, lost = 0;
-        run += sel_emit<true>(T, run, need, false, &cnt, &E, &lost);
+        run += sel_emit<true, kC4>(T, run, need, false, &cnt, &E, &lost);
         attached -= lost;
         __syncthreads();
-        auto at = [&](int32_t j) { return (int64_t)R.pos[j]; };
-        auto load = [&](int32_t j) { return RowItem{(int64_t)R.pos[j], R.row[j], R.len[j], R.rank[j]}; };
-        auto f = [&](const auto& X) { attached += attach_batch(W, X); };
-        if (E <= 64 * nwarps) row_walk<1>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
-        else row_walk<kRowB>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
+        for (int pass = kC4 ? 0 : 1; pass < 2; ++pass) {
+          auto at = [&](int32_t j) { return (int64_t)R.pos[j]; };
+          auto load = [&](int32_t j) {
+            return RowItem{(int64_t)R.pos[j], R.row[j], R.len[j], kC4 && pass == 1 && R.blocked[j] ? -1 : R.rank[j]};
+          };
+          auto f = [&](const auto& X) {
+            if (!kC4 || pass == 1) {
+              attached += attach_batch(W, X);
+              return;
+            }
+            constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+            uint32_t tg[kB];
+            int32_t ru[kB];
+#pragma unroll
+            for (int q = 0; q < kB; ++q) tg[q] = X.w[q] >= 0 ? rtag_of(W.rtag, X.w[q]) : 16u;
+#pragma unroll
+            for (int q = 0; q < kB; ++q) ru[q] = tg[q] == 0 || tg[q] == W.tag ? ldcg(arank + X.w[q]) : -1;
+#pragma unroll
+            for (int q = 0; q < kB; ++q) {
+              if (ru[q] < r_lo || ru[q] >= X.aux[q]) continue;
+              const uint32_t x = tg[q] == 0 ? 0u : ldcg(W.st + X.w[q]);
+              // active in this round, or attached in it
+              if (is_active(x) || x >= kLab + (uint32_t)r_lo) R.blocked[X.item[q]] = 1;
+            }
+          };
+          if (E <= 64 * nwarps) row_walk<1>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
+          else row_walk<kRowB>(warp, nwarps, cnt, E, B.col, shape, at, load, f);
+          if (kC4 && pass == 0) {
+            __syncthreads();
+            tile_classify(cnt);
+          }
+        }
       }
       base += tile;
     } while (base < e && run < need);       // uniform across the block
     tally(kTAttached, attached);
+  }
+
+  // C4: the actives of the block's tile are centers or go to the blocked list
+  // (and, for the passes that read it, to the list of actives with flag 2).
+  __device__ __forceinline__ void tile_classify(int32_t cnt) {
+    const TileRows& R = S->u.rows;
+    const int lane = threadIdx.x & 31;
+    int32_t centers = 0, nblocked = 0;
+    for (int32_t base = (int32_t)threadIdx.x - lane; base < cnt; base += kThreads) {
+      const int32_t j = base + lane;
+      const bool blocked = j < cnt && R.blocked[j];
+      const int32_t len = blocked ? R.len[j] : 0;
+      if (j < cnt && !blocked) {
+        B.st[R.v[j]] = kActCenter;
+        centers += 1;
+      }
+      if (!__any_sync(FULL, blocked)) continue;
+      const int64_t pk = blocked ? (int64_t(1) << kPackShift) | len : 0, inc = warp_inclusive_sum<int64_t>(pk);
+      unsigned long long old = 0;
+      if (lane == 31) old = atomicAdd(&C->act_pack, (unsigned long long)inc);
+      const int64_t at = (int64_t)__shfl_sync(FULL, old, 31) + inc - pk, i = at >> kPackShift;
+      if (blocked) {
+        put_active(i, at & (int64_t)kPackEdgeMask, R.v[j], R.rank[j], R.row[j], len, 2);
+        nblocked += 1;
+      }
+      warp_append_rows(blocked, (int32_t)i, blocked ? R.row[j] : 0, len, 0x7FFFFFFF, blk_list());
+      const int32_t ml = __reduce_max_sync(FULL, len);
+      if (lane == 0) atomicMax(&C->blk_maxlen, (unsigned long long)ml);
+    }
+    tally(kTCenters, centers);
+    tally(kTBlocked, nblocked);
   }
 
   // ---------------- C4: blocked detection ------------------------------------
@@ -1752,7 +1855,8 @@ struct K {
     const int32_t* const arank = B.arank;
     uint8_t* const blocked = B.blk_flag;
     const int32_t r0 = P().r0;
-    walk_actives([&](int32_t j) { return ldcg(rank + j); }, [&](const auto& X) {
+    // payload: the active's rank, -1 when it is known to be blocked
+    walk_actives([&](int32_t j) { return ldcg(blocked + j) ? -1 : ldcg(rank + j); }, [&](const auto& X) {
       constexpr int kB = sizeof(X.w) / sizeof(int32_t);
       uint32_t tg[kB];
 #pragma unroll
@@ -1783,7 +1887,9 @@ struct K {
       int64_t len = 0, row = 0;
       if (j < an) {
         const int32_t v = ldcg(B.act_v + j);
-        if (ldcg(B.blk_flag + j)) {
+        const uint8_t flag = ldcg(B.blk_flag + j);      // 1: blocked; 2: the same, and listed already
+        if (flag == 2) {
+        } else if (flag) {
           blocked = true;
           row = ldcg(B.act_d + j);
           len = ldcg(B.act_n + j);
@@ -2046,12 +2152,19 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
       continue;
     }
     if (S.plan.state == kSelect) {
-      if (algo == kAlgoCW && k.G > 1 && S.plan.win_len <= kFuseTiles * (int64_t)k.G * kThreads * kSelU) {
-        k.select_attach();
+      if (k.G > 1 && S.plan.win_len <= kFuseWindow * (int64_t)k.G) {
+        if (algo == kAlgoC4) k.template select_attach<true, kPerSM>();
+        else k.template select_attach<false, kPerSM>();
         k.flush_round_tallies();
         if (!k.sync(4, [&] {
               k.select_decide(false);
-              if (S.plan.state == kRun && S.plan.act_n == 0) k.co_end_round();      // no longer rows left
+              // the round goes on with what was left out
+              if (S.plan.state != kRun) return;
+              if (algo == kAlgoCW) {
+                if (S.plan.act_n == 0) k.co_end_round();
+              } else if (S.plan.act_n == (int64_t)(vload(&C->blk_pack) >> kPackShift)) {
+                k.co_blocked();
+              }
             }))
           goto out;
         continue;
@@ -2064,7 +2177,7 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
         goto out;
       continue;
     }
-    {
+    if (S.plan.state == kRun) {
       if (algo == kAlgoCW) {
         k.attach_from_actives(false);
         k.flush_round_tallies();
@@ -2075,29 +2188,17 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
         k.c4_classify();
         k.attach_from_actives(true);
         k.flush_round_tallies();
-        if (!k.sync(4, [&] {
-              if (threadIdx.x < 2) S.bcast[threadIdx.x] = (int64_t)vload(threadIdx.x == 0 ? &C->blk_pack : &C->blk_maxlen);
-              __syncthreads();
-              if (threadIdx.x == 0) {
-                const unsigned long long pk = (unsigned long long)S.bcast[0];
-                S.plan.b_n = (int64_t)(pk >> kPackShift);
-                S.plan.b_E = (int64_t)(pk & kPackEdgeMask);
-                S.plan.undecided = S.plan.b_n;
-                S.co.fix_iter = 0;
-                S.co.r_edges += 2 * S.plan.b_E;       // first fixpoint scan, blocked attach / pull
-                const int64_t warps = (int64_t)k.G * (blockDim.x >> 5);
-                S.plan.by_warp = (S.plan.b_n > 0 && S.plan.b_n <= warps &&
-                               S.bcast[1] <= (int64_t)k.B.tune.warp_resolve_row) ? 1 : 0;
-              }
-              __syncthreads();
-              if (S.plan.b_n == 0) k.co_end_round();       // nothing blocked: the round is over
-            }))
-          goto out;
-        if (S.plan.b_n > 0 && S.plan.by_warp == 1) {
+        if (!k.sync(4, [&] { k.co_blocked(); })) goto out;
+      }
+      continue;
+    }
+    {
+      {
+        if (S.plan.by_warp == 1) {
           k.c4_resolve_by_warp();
           k.flush_round_tallies();
           if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
-        } else if (S.plan.b_n > 0) {
+        } else {
           // the pull slots were set when the list was built; the hit flags are zero
           auto after_decide = [&](long long left) {
             if (threadIdx.x == 0) {
@@ -2230,7 +2331,7 @@ __device__ __forceinline__ int64_t finish_vertices(const RoundBuffers& B, int32_
 // kPermSubBits bits plus an insertion sort inside each bucket.  Also writes
 // the initial state words.
 template <int kPerSM>
-__device__ bool team_permutation(K<kPerSM>& k, uint64_t seed) {
+__device__ bool team_permutation(K<kPerSM>& k, uint64_t seed, bool ranks) {
   const RoundBuffers& B = k.B;
   Shared& S = *k.S;
   const int64_t n = B.n;
@@ -2297,6 +2398,7 @@ __device__ bool team_permutation(K<kPerSM>& k, uint64_t seed) {
           r += (kj < ki || (kj == ki && vj < vi)) ? 1 : 0;
         }
         B.order_w[s0 + r] = vi;
+        if (ranks) B.arank[vi] = (int32_t)(s0 + r);
       }
       __syncthreads();
       continue;
@@ -2343,7 +2445,10 @@ __device__ bool team_permutation(K<kPerSM>& k, uint64_t seed) {
       }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < len; i += blockDim.x) B.order_w[s0 + i] = P.ov[i];
+    for (int i = threadIdx.x; i < len; i += blockDim.x) {
+      B.order_w[s0 + i] = P.ov[i];
+      if (ranks) B.arank[P.ov[i]] = (int32_t)(s0 + i);
+    }
     __syncthreads();
   }
   return k.sync(7);
@@ -2418,7 +2523,7 @@ k_batch(BatchJob* __restrict__ jobs, const RoundBuffers* __restrict__ slots, con
           }
         }))
       break;
-    if (!team_permutation(k, jobs[j].seed)) break;
+    if (!team_permutation(k, jobs[j].seed, algo == kAlgoC4 || algo == kAlgoC4 + 2)) break;
       if (threadIdx.x < kTallies) S.tal[threadIdx.x] = 0;
     __syncthreads();
     run_job(k, algo);
@@ -2460,6 +2565,7 @@ __global__ void k_init_state(RoundBuffers B, int algo, int64_t eps_ppm, uint64_t
     B.size[v] = 0;                     // members per center rank
     B.hit_c[v] = 0;                    // C4 fixpoint flags start (and stay) zero
     B.hit_p[v] = 0;
+    if (algo == kAlgoC4 || algo == kAlgoC4 + 2) B.arank[__ldg(B.order + v)] = (int32_t)v;
   }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rtag_words(n); i += (int64_t)gridDim.x * blockDim.x)
     B.rtag[i] = 0;

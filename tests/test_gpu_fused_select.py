@@ -1,9 +1,10 @@
-"""ClusterWild! selects and attaches a window in one pass: blocks attach while
-others still count, so a vertex may be reached before its own block makes it a
-center, and rows of more than 8192 entries are left to a second pass.  Windows
-around the inline limit and of several tiles per block, rows around 8192 that
-are still alive when windows are long, removal tags that come round again (more
-than 15 rounds).  Labels, rounds and statistics equal the oracle's; exact."""
+"""Selection and attachment of a window run in one pass: blocks attach while
+others still count, so a vertex may be reached before its own block makes it
+active, C4 tells blocked actives by the ranks of pi, and rows of more than 8192
+entries are left to a second pass.  Windows around the inline limit and of
+several tiles per block, rows around 8192 that are still alive when windows are
+long, removal tags that come round again (more than 15 rounds).  Labels, rounds
+and statistics equal the oracle's; exact."""
 import numpy as np
 import pytest
 
@@ -44,9 +45,10 @@ def _ring_and_hubs(gg, n, half, hubs, leaves, seed):
 def test_fused_selection_equals_oracle(cc, gg, ora, n, half, hubs, leaves):
     g = _ring_and_hubs(gg, n, half, hubs, leaves, n)
     with cc.Graph(g.off, g.col) as graph:
-        for algo, a, eps in (("cw", 2, 0.1), ("cw", 2, 0.9), ("cw-est", 4, 0.9)):
+        for algo, a, eps in (("cw", 2, 0.1), ("cw", 2, 0.9), ("cw-est", 4, 0.9), ("c4", 1, 0.1), ("c4", 1, 0.9),
+                             ("c4-est", 3, 0.9)):
             order = ora.permutation(g.n, 11)
-            olab, orr, _, ost = (ora.rounds_bsp(g.off, g.col, order, 2, eps, 11, stats_cap=1_000_000) if a == 4 else
+            olab, orr, _, ost = (ora.rounds_bsp(g.off, g.col, order, a - 2, eps, 11, stats_cap=1_000_000) if a > 2 else
                                  ora.rounds(g.off, g.col, order, a, eps, 1, stats_cap=1_000_000))
             lab, r, d, st = graph.cluster(algo, eps, 11, stats_cap=1_000_000)
             assert np.array_equal(lab, olab) and r == orr and d == ora.disagreements(g.off, g.col, olab), (algo, eps)
