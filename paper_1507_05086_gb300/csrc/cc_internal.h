@@ -66,6 +66,7 @@ struct Ctl {
   long long undecided;
   unsigned long long h_pack;      // heavy-list appends
   unsigned long long nz_pack;     // alive non-isolated vertices counted
+  unsigned long long drawn;       // Sec. 5: successes among the batch's draws
   unsigned long long blk_maxlen;  // C4: longest row of a blocked active this round
   int32_t r0;
   int64_t cursor_next;
@@ -153,8 +154,6 @@ struct RoundBuffers {
   int32_t* b_j;
   int64_t* b_e;
   int64_t* b_d;
-  int64_t* blk_a;              // per-block scratch
-  int64_t* blk_b;
   unsigned long long* desc;    // per-block scan descriptors of the selection (decoupled look-back)
   RoundStat* stats;
   int64_t stats_cap;

@@ -197,6 +197,7 @@ struct Coord {
   int delta_zero;                // a rebuild found no alive vertex with an alive neighbour
   int est;                       // the Sec. 5 schedule: Delta-hat and binomial batches
   int64_t period, rank_cursor;   // rounds per halving of Delta-hat; ranks of pi passed
+  int ahead;                     // the next batch has been drawn
   int32_t withhold;              // test hook (Ctl::withhold)
   int32_t round_ended;           // this barrier ended a round
   int64_t batch_end;             // rank (index in pi) that ends the round's batch
@@ -258,6 +259,7 @@ struct Shared {
   unsigned long long sel_pack;
   int32_t h_picked, h_kept;      // vertices picked for the recount; entries of a compacted list
   int32_t h_best;                // largest exact degree that this block knows of
+  int32_t drawn;                 // Sec. 5: the last batch (Plan::drop) that this block drew its share of
   int64_t nz_cnt;                // alive non-isolated vertices of this block's segment (-1: not looked at yet)
   union {
     HeavyList hl;
@@ -279,6 +281,7 @@ struct K {
   unsigned bid;
   unsigned epoch;
   int algo;                      // C4 or ClusterWild!
+  bool est;                      // by the Sec. 5 schedule
 
   // One round tally of this block; all lanes of the warp call it.
   __device__ __forceinline__ void tally(int which, int32_t x) {
@@ -450,21 +453,6 @@ struct K {
     if (*s > *e) *s = *e;
   }
 
-  // Coordinator: exclusive prefix of blk_a[0..G) in place; returns the total.
-  __device__ int64_t prefix_blocks() {
-    int64_t run = 0;
-    for (unsigned base = 0; base < G; base += blockDim.x) {
-      const unsigned b = base + threadIdx.x;
-      const int64_t x = b < G ? ldcg(B.blk_a + b) : 0;
-      int64_t tot;
-      const int64_t ex = block_exclusive_sum<int64_t>(x, S->scr, &tot);
-      if (b < G) B.blk_a[b] = run + ex;
-      run += tot;
-    }
-    __syncthreads();
-    return run;
-  }
-
   // ---------------- coordinator actions ----------------------------------------
   __device__ void co_init() {
     if (threadIdx.x == 0) {
@@ -492,6 +480,7 @@ struct K {
       if (c.est) c.algo -= 2;
       c.period = c.est ? sec5_period(c.n, c.max_deg, c.eps_ppm) : 0;
       c.rank_cursor = 0;
+      c.ahead = 0;
       c.stats_cap = B.stats_cap;
       Plan& p = S->plan;
       p = Plan{};
@@ -530,6 +519,9 @@ struct K {
         c.k = 0;                          // set from the window's alive count
         c.need = INT64_MAX / 4;
         c.win_len = c.batch_end - c.cursor;
+        // The next batch depends on the cursor alone, not on what this round
+        // removes: it is drawn in this round's first phase.
+        if (c.rank_cursor < c.n) plan_draw(c.round + 1);
       }
       C->act_pack = 0; C->blk_pack = 0; C->blk_maxlen = 0;
       C->r_centers = 0; C->r_attached = 0; C->r_noncenter = 0; C->r_blocked = 0; C->r_edges = 0;
@@ -556,7 +548,17 @@ struct K {
     Coord& c = co();
     Plan& p = S->plan;
     if (c.n_alive <= 0) { p.state = kDone; return 1; }
-    if (c.est) { plan_draw(); return 1; }
+    if (c.est) {
+      c.delta = (int32_t)sec5_delta_hat(c.max_deg, c.period, c.round);
+      if (c.ahead) {                      // drawn during this round's first phase
+        c.ahead = 0;
+        batch_drawn((int64_t)vload(&C->drawn));
+        return 2;
+      }
+      plan_draw(c.round);                 // the first batch: a phase of its own
+      p.state = kDrawBatch;
+      return 1;
+    }
     if (c.round == 0) {                   // every degree is still the full one
       c.delta = c.max_deg;
       if (c.max_deg <= 0) c.delta_zero = 1;
@@ -572,19 +574,26 @@ struct K {
     c.d_th = below(c.delta, c.d_drop);
     return 0;
   }
-  // Sec. 5: the batch is drawn by the grid; no Delta.
-  __device__ __noinline__ void plan_draw() {
-    Coord& c = co();
+  // Sec. 5: plans the draws of round `round` (no Delta): trials, threshold bits,
+  // stream seed; d_lb = 2: every trial succeeds, else 1.
+  __device__ __noinline__ void plan_draw(int64_t round) {
+    const Coord& c = co();
     Plan& p = S->plan;
-    p.state = kDrawBatch;
-    const int64_t dh = sec5_delta_hat(c.max_deg, c.period, c.round);
     bool all;
-    const uint64_t thr = sec5_threshold(c.eps_ppm, dh, &all);
-    c.delta = (int32_t)dh;
-    p.win_len = c.n - c.rank_cursor;                            // trials
-    p.need = (int64_t)thr;                                      // threshold bits
-    p.take = all ? 1 : 0;
-    p.k = (int64_t)perm_key(vload(&C->seed) ^ 0x5851F42D4C957F2Dull, (uint64_t)c.round);   // stream seed
+    p.long_E = (int64_t)sec5_threshold(c.eps_ppm, sec5_delta_hat(c.max_deg, c.period, round), &all);
+    p.long_n = c.n - c.rank_cursor;
+    p.undecided = (int64_t)perm_key(vload(&C->seed) ^ 0x5851F42D4C957F2Dull, (uint64_t)round);
+    p.d_lb = all ? 2 : 1;
+    p.drop = (int32_t)(round & 0x3FFFFFFF);      // tells the blocks that this batch is a new one
+    C->drawn = 0;
+  }
+  // The batch of b ranks of pi from the cursor on.
+  __device__ void batch_drawn(int64_t b) {
+    Coord& c = co();
+    const int64_t end_rank = c.rank_cursor + b;
+    c.batch_end = end_rank < c.al_len ? end_rank : c.al_len;      // entry i of the list has rank i
+    c.rank_cursor = end_rank;
+    if (end_rank > c.n) fail(kErrInternal);
   }
   __device__ __forceinline__ void co_go_on() {
     const int dec = S->dec;
@@ -1223,37 +1232,28 @@ struct K {
   }
 
   // ---------------- Sec. 5: the round's binomial batch ------------------------
-  // Every block counts its share of the round's draws below the threshold
-  // (plan: win_len trials, need = threshold bits, take = every trial
-  // succeeds, k = stream seed); the coordinator adds them up, moves the rank
-  // cursor past the batch and plans the round's single selection window, the
-  // batch's ranks of pi.
-  __device__ __noinline__ bool draw_batch() {
-    const int64_t trials = P().win_len;
-    const uint64_t thr = (uint64_t)P().need, s = (uint64_t)P().k;
+  // The next batch is drawn in the first phase of the round before, which spares
+  // a phase per round (R-MAT 18, 547 rounds: 12.4 -> 10.6 ms).
+  // Every block counts its share of the draws below the threshold (plan: long_n
+  // trials, long_E = threshold bits, undecided = stream seed, d_lb = 2: every
+  // trial succeeds).  The count moves the rank cursor past the batch, whose
+  // ranks of pi are the round's single selection window.
+  __device__ __noinline__ void draw_batch() {
+    const int64_t trials = P().long_n;
+    const uint64_t thr = (uint64_t)P().long_E, s = (uint64_t)P().undecided;
     int64_t cnt = 0;
-    if (P().take) {
+    if (P().d_lb == 2) {
       cnt = bid == 0 && threadIdx.x == 0 ? trials : 0;
     } else {
       for (int64_t j = (int64_t)bid * blockDim.x + threadIdx.x; j < trials; j += (int64_t)G * blockDim.x)
         cnt += sec5_draw(s, (uint64_t)j) < thr ? 1 : 0;
     }
     cnt = block_sum<int64_t>(cnt, S->scr);
-    if (threadIdx.x == 0) B.blk_a[bid] = cnt;
-    return sync(2, [&] {
-      const int64_t b = prefix_blocks();
-      Coord& c = co();
-      const int64_t end_rank = c.rank_cursor + b;
-      // the list entry of rank end_rank ends the batch (entry i has rank i)
-      const int64_t end = end_rank < c.al_len ? end_rank : c.al_len;
-      if (threadIdx.x == 0) {
-        c.batch_end = end;
-        c.rank_cursor = end_rank;
-        if (end_rank > c.n) fail(kErrInternal);
-      }
-      __syncthreads();
-      plan_selection(c.delta);
-    });
+    if (threadIdx.x == 0) {
+      if (cnt) atomicAdd(&C->drawn, (unsigned long long)cnt);
+      S->drawn = P().drop;
+      co().ahead = 1;                     // (the coordinator's)
+    }
   }
 
   // ---------------- rebuild of the heavy list: grid passes ---------------------
@@ -2116,7 +2116,8 @@ template <int kPerSM>
 __device__ void run_job(K<kPerSM>& k, int algo) {
   Shared& S = *k.S;
   Ctl* C = k.C;
-  if (algo >= 3) algo -= 2;             // the Sec. 5 schedule: same rounds, C4 or ClusterWild!
+  const bool est = algo >= 3;           // the Sec. 5 schedule: same rounds, C4 or ClusterWild!
+  if (est) algo -= 2;
   if (k.bid == 0 && threadIdx.x == 0) {
     for (int i = 0; i < 8; ++i) S.co.ph_ns[i] = 0;
     S.co.t0 = globaltimer_ns();
@@ -2124,7 +2125,9 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
   }
   if (threadIdx.x == 0) {
     S.nz_cnt = -1;
+    S.drawn = -1;
     k.algo = algo;
+    k.est = est;
   }
   __syncthreads();
   if (!k.sync(7, [&] { k.co_init(); })) goto out;
@@ -2147,9 +2150,20 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
       if (!k.recount_long()) goto out;
       continue;
     }
-    if (S.plan.state == kDrawBatch) {
-      if (!k.draw_batch()) goto out;
-      continue;
+    if (k.est && S.plan.drop != S.drawn) {
+      k.draw_batch();
+      if (S.plan.state == kDrawBatch) {
+        if (!k.sync(2, [&] {
+              if (threadIdx.x == 0) {
+                S.co.ahead = 0;
+                k.batch_drawn((int64_t)vload(&C->drawn));
+              }
+              __syncthreads();
+              k.plan_selection(S.co.delta);
+            }))
+          goto out;
+        continue;
+      }
     }
     if (S.plan.state == kSelect) {
       if (k.G > 1 && S.plan.win_len <= kFuseWindow * (int64_t)k.G) {
@@ -2618,7 +2632,6 @@ size_t rounds_workspace_bytes(int64_t n, int32_t max_deg, int grid) {
   b += 3 * align_up(nn);                 // blk_flag, hit_c, hit_p
   b += align_up(4 * nn);                 // pull
   b += align_up(4 * nn) + 2 * align_up(8 * nn);       // b_j, b_e, b_d
-  b += 2 * align_up(8 * ((size_t)grid + 1));          // blk_a, blk_b
   b += align_up(8 * kDescStride * ((size_t)grid + 1)); // desc
   return b;
 }
@@ -2649,8 +2662,6 @@ void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* 
   B->b_j = reinterpret_cast<int32_t*>(take(4 * nn));
   B->b_e = reinterpret_cast<int64_t*>(take(8 * nn));
   B->b_d = reinterpret_cast<int64_t*>(take(8 * nn));
-  B->blk_a = reinterpret_cast<int64_t*>(take(8 * ((size_t)grid + 1)));
-  B->blk_b = reinterpret_cast<int64_t*>(take(8 * ((size_t)grid + 1)));
   B->desc = reinterpret_cast<unsigned long long*>(take(8 * kDescStride * ((size_t)grid + 1)));
 }
 
