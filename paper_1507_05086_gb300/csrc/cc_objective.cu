@@ -226,7 +226,10 @@ __global__ void k_nz_count(int64_t n, const int64_t* __restrict__ off, int64_t* 
   }
 }
 
-__global__ void k_nz_scan(int64_t ntiles, int64_t* __restrict__ tile_cnt, int64_t* __restrict__ total) {
+// Block b scans the counts at tile_cnt + b * stride, its sum goes to total[b].
+__global__ void k_nz_scan(int64_t ntiles, int64_t* __restrict__ tile_cnt, int64_t stride,
+                          int64_t* __restrict__ total) {
+  tile_cnt += blockIdx.x * stride;
   __shared__ int64_t scr[33];
   int64_t run = 0;
   for (int64_t base = 0; base < ntiles; base += blockDim.x) {
@@ -237,7 +240,7 @@ __global__ void k_nz_scan(int64_t ntiles, int64_t* __restrict__ tile_cnt, int64_
     if (t < ntiles) tile_cnt[t] = run + ex;
     run += tot;
   }
-  if (threadIdx.x == 0) *total = run;
+  if (threadIdx.x == 0) total[blockIdx.x] = run;
 }
 
 __global__ void k_nz_write(int64_t n, const int64_t* __restrict__ off, const int64_t* __restrict__ tile_off,
@@ -518,7 +521,7 @@ cudaError_t launch_nonempty_rows(int64_t n, const int64_t* off, int32_t* nz_row,
   int64_t* tile = static_cast<int64_t*>(ws);
   const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
   k_nz_count<<<g, kNzTile, 0, stream>>>(n, off, tile);
-  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, count_dev);
+  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, 0, count_dev);
   k_nz_write<<<g, kNzTile, 0, stream>>>(n, off, tile, nz_row, nz_pos, up_at);
   return cudaGetLastError();
 }
@@ -530,11 +533,11 @@ cudaError_t launch_upper_rows(int64_t nz_n, int64_t nnz, const int32_t* nz_row, 
   if (nz_n <= 0) return cudaMemsetAsync(count_dev, 0, 2 * sizeof(unsigned long long), stream);
   const int64_t ntiles = (nz_n + kNzTile - 1) / kNzTile;
   int64_t* tile = static_cast<int64_t*>(ws);
-  int64_t* tile_len = tile + align_up(8 * (size_t)(ntiles + 1)) / 8;
+  const int64_t stride = (int64_t)(align_up(8 * (size_t)(ntiles + 1)) / 8);
+  int64_t* tile_len = tile + stride;
   const int g = (int)(ntiles < (int64_t)num_sms * 4 ? ntiles : (int64_t)num_sms * 4);
   k_up_count<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_pos, up_at, tile, tile_len);
-  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile, reinterpret_cast<int64_t*>(count_dev));
-  k_nz_scan<<<1, 1024, 0, stream>>>(ntiles, tile_len, reinterpret_cast<int64_t*>(count_dev + 1));
+  k_nz_scan<<<2, 1024, 0, stream>>>(ntiles, tile, stride, reinterpret_cast<int64_t*>(count_dev));
   k_up_write<<<g, kNzTile, 0, stream>>>(nz_n, nnz, nz_row, nz_pos, up_at, tile, tile_len, v, row, len, pos, epos);
   return cudaGetLastError();
 }
