@@ -21,7 +21,6 @@ constexpr int kColChunks = 8;
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t stream);
 
 // ---- permutation (cc_perm.cu) ----------------------------------------------
-int perm_bucket_bits(int64_t n);
 size_t perm_workspace_bytes(int64_t n);
 cudaError_t launch_permutation(int64_t n, uint64_t seed, int32_t* order, void* ws, int num_sms,
                                int* err, cudaStream_t stream);

@@ -2,16 +2,21 @@
 //
 // pi lists the vertices by ascending (splitmix64(seed ^ v), v).  The keys are
 // uniform 64-bit values, so a two-level sort suffices:
-//   1. bucket vertices by the top b key bits (b chosen so a bucket holds about
-//      384-768 vertices): a histogram, an exclusive scan and a scatter;
-//   2. sort each bucket in shared memory by the full (key, v): a counting sort
-//      on the next 10 key bits, then an insertion sort per sub-bucket of
-//      about one element, and write its slice of order[].
+//   1. k_bucket_scatter puts the vertices into buckets by the top b key bits (b
+//      chosen so that a bucket holds 2048-4096 vertices).  A bucket has a fixed
+//      place for its expected number and twelve standard deviations more, so
+//      nothing is counted beforehand; what does not fit goes to a spill list.
+//      Above kOneLevelBits bits it runs twice, by the top kCoarseBits bits first.
+//   2. k_bucket_starts: exclusive scan of the buckets' sizes.
+//   3. k_bucket_sort sorts each bucket in shared memory by the full (key, v): a
+//      counting sort on the next 12 key bits, then an insertion sort per
+//      sub-bucket of about one element, and writes its slice of order[].
 // Keys are recomputed from v wherever needed instead of being stored, so the
-// only global traffic is 4 bytes per vertex scattered and 4+4 bytes per vertex
-// read and written by the bucket sort.  A bucket larger than the shared-memory
-// capacity (vanishingly unlikely for a hash) falls back to a rank-by-counting
-// pass that is slow but exact.
+// only global traffic is 4 bytes per vertex scattered (twice, and read once, in
+// two levels) and 4+4+4 bytes per vertex read and written by the bucket sort.
+// Bound by the shared-memory atomics of the two sorts; 10K / 1M / 4.2M / 16.8M /
+// 67M vertices take 20 / 35 / 87 / 290 / 1255 us (36 / 130 / 280 / 730 / 2430 when
+// buckets of 512 were counted and filled by one global atomic per vertex each).
 #include <cstdint>
 
 #include "cc_device.cuh"
@@ -20,67 +25,143 @@
 namespace ccg {
 namespace {
 
-constexpr int kBucketCap = 1536;      // vertices per bucket sorted in shared memory
+constexpr int kMeanMax = 4096;         // expected vertices per bucket, at most
+constexpr int kBucketCap = 4928;       // at least bucket_cap(4096)
+constexpr int kScatterThreads = 512;
 constexpr int kSortThreads = 512;
-constexpr int kMaxOverflow = 1023;    // buckets above capacity handled by the fallback
+constexpr int kSpillCap = 1 << 16;     // vertices that found their bucket full
+// Up to 2^12 buckets (16M vertices) one scatter; above, a chunk holds too few
+// vertices per bucket for neighbouring writes (16M vertices in one level 0.29 ms,
+// in two 0.34; 67M into 2^14 buckets at once 2.4, in two levels 1.26).
+constexpr int kOneLevelBits = 12;
+constexpr int kCoarseBits = 9;
+constexpr int kChunk = 16384;          // vertices per block and scatter, at most
 
 __device__ __forceinline__ uint32_t bucket_of(uint64_t key, int bits) {
   return bits == 0 ? 0u : (uint32_t)(key >> (64 - bits));
 }
 
-__global__ void k_bucket_hist(int64_t n, uint64_t seed, int bits, uint32_t* __restrict__ count) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&count[bucket_of(perm_key(seed, (uint64_t)v), bits)], 1u);
+// Places of a bucket of `mean` expected vertices.
+int64_t bucket_cap(int64_t mean) {
+  int64_t root = 0;
+  while (root * root < mean) ++root;
+  return (mean + 12 * root + 63) & ~int64_t(31);
 }
 
-// Exclusive scan of the nb counts into start[0..nb] (start[nb] = n) and
-// cursor = start, in three steps: every block of kScanTile threads scans its
-// tile of counts (tile totals to tot[]), one block scans the totals, every
-// block adds its tile's offset.
-constexpr int kScanTile = 1024;
-
-__global__ void __launch_bounds__(kScanTile) k_scan_tiles(const uint32_t* __restrict__ count, int64_t nb,
-                                                        int64_t* __restrict__ start, int64_t* __restrict__ tot) {
-  __shared__ int64_t scratch[33];
-  const int64_t i = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
-  int64_t t;
-  const int64_t ex = block_exclusive_sum<int64_t>(i < nb ? (int64_t)count[i] : 0, scratch, &t);
-  if (i < nb) start[i] = ex;
-  if (threadIdx.x == 0) tot[blockIdx.x] = t;
+__device__ __forceinline__ void spill_one(int32_t v, uint32_t* spill) {
+  const uint32_t q = atomicAdd(spill, 1u);
+  if (q < (uint32_t)kSpillCap) spill[1 + q] = (uint32_t)v;
 }
 
-__global__ void k_scan_totals(int64_t ntiles, int64_t nb, int64_t* __restrict__ tot, int64_t* __restrict__ start) {
-  __shared__ int64_t scratch[33];
-  int64_t run = 0;
-  for (int64_t base = 0; base < ntiles; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    int64_t t;
-    const int64_t ex = block_exclusive_sum<int64_t>(i < ntiles ? tot[i] : 0, scratch, &t);
-    if (i < ntiles) tot[i] = run + ex;
-    run += t;
+// A block's share of a scatter: the vertices source(0 .. len) go to the `nb`
+// buckets from `first` on.  They are counted by bucket in shared memory and
+// brought into bucket order there; one atomic takes the places of all of a
+// bucket's vertices, and neighbouring threads write neighbouring places.  (One
+// atomic per vertex, after as many to count the buckets, took 187 of the 280 us
+// of 4.2M vertices: the counters of 8192 buckets lie in 256 lines.  Written
+// straight to their places the vertices of a warp go to 32 pages of memory: 67M
+// into 512 buckets 0.58 ms.)  spilled(v) gets the vertices that found no place.
+struct ScatterSmem {
+  uint32_t* next;                        // [nb] count, then next place in buf
+  uint32_t* delta;                       // [nb] place in the bucket, less the one in buf
+  int32_t* buf;                          // [chunk]
+  __device__ ScatterSmem(uint32_t* raw, int nb)
+      : next(raw), delta(raw + nb), buf(reinterpret_cast<int32_t*>(raw + 2 * nb)) {}
+};
+size_t scatter_smem(int nb, int64_t chunk) { return sizeof(uint32_t) * (2 * (size_t)nb + (size_t)chunk); }
+
+template <class Source, class Spilled>
+__device__ __forceinline__ void scatter_chunk(int len, uint64_t seed, int bits, uint32_t first, int nb, int64_t cap,
+                                              const ScatterSmem& M, uint32_t* __restrict__ count,
+                                              int32_t* __restrict__ tmp, const Source& source,
+                                              const Spilled& spilled) {
+  __shared__ int32_t scr[33];
+  auto bucket = [&](int32_t v) { return bucket_of(perm_key(seed, (uint64_t)v), bits) - first; };
+  for (int b = threadIdx.x; b < nb; b += kScatterThreads) M.next[b] = 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < len; i += kScatterThreads) atomicAdd(&M.next[bucket(source(i))], 1u);
+  __syncthreads();
+  int32_t run = 0;
+  for (int b0 = 0; b0 < nb; b0 += kScatterThreads) {
+    const int b = b0 + threadIdx.x;
+    const int32_t k = b < nb ? (int32_t)M.next[b] : 0;
+    int32_t tot;
+    const int32_t at = run + block_exclusive_sum<int32_t>(k, scr, &tot);
+    run += tot;
+    if (b >= nb) continue;
+    M.next[b] = (uint32_t)at;
+    if (k) M.delta[b] = atomicAdd(count + first + b, (uint32_t)k) - (uint32_t)at;
   }
-  if (threadIdx.x == 0) start[nb] = run;
-}
-
-__global__ void __launch_bounds__(kScanTile) k_scan_add(int64_t nb, const int64_t* __restrict__ tot,
-                                                      int64_t* __restrict__ start, uint32_t* __restrict__ cursor) {
-  const int64_t i = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
-  if (i < nb) {
-    const int64_t s = start[i] + tot[blockIdx.x];
-    start[i] = s;
-    cursor[i] = (uint32_t)s;              // positions are below n < 2^31
+  __syncthreads();
+  for (int i = threadIdx.x; i < len; i += kScatterThreads) {
+    const int32_t v = source(i);
+    M.buf[atomicAdd(&M.next[bucket(v)], 1u)] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < len; i += kScatterThreads) {
+    const int32_t v = M.buf[i];
+    const uint32_t b = bucket(v), at = M.delta[b] + (uint32_t)i;
+    if (at < (uint32_t)cap) tmp[(int64_t)(first + b) * cap + at] = v;
+    else spilled(v);
   }
 }
 
-__global__ void k_bucket_scatter(int64_t n, uint64_t seed, int bits, uint32_t* __restrict__ cursor,
-                                 int32_t* __restrict__ tmp) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t b = bucket_of(perm_key(seed, (uint64_t)v), bits);
-    const int64_t pos = (int64_t)atomicAdd(&cursor[b], 1u);
-    tmp[pos] = (int32_t)v;
+// All vertices, a chunk per block, into the 2^bits buckets of cap places.
+__global__ void __launch_bounds__(kScatterThreads)
+k_bucket_scatter(int64_t n, uint64_t seed, int bits, int cap, int64_t chunk, uint32_t* __restrict__ count,
+                 int32_t* __restrict__ tmp, uint32_t* __restrict__ spill) {
+  extern __shared__ uint32_t sm[];
+  const int64_t c0 = (int64_t)blockIdx.x * chunk;
+  scatter_chunk((int)(n - c0 < chunk ? n - c0 : chunk), seed, bits, 0u, 1 << bits, cap, ScatterSmem(sm, 1 << bits), count,
+                tmp,
+                [&](int i) { return (int32_t)(c0 + i); }, [&](int32_t v) { spill_one(v, spill); });
+}
+
+// The same into the coarse buckets; what finds no place there goes to its
+// bucket of 2^bits directly.
+__global__ void __launch_bounds__(kScatterThreads)
+k_bucket_coarse(int64_t n, uint64_t seed, int64_t coarse_cap, int64_t chunk, uint32_t* __restrict__ coarse_count,
+                int32_t* __restrict__ coarse, int bits, int cap, uint32_t* __restrict__ count,
+                int32_t* __restrict__ tmp, uint32_t* __restrict__ spill) {
+  extern __shared__ uint32_t sm[];
+  const int64_t c0 = (int64_t)blockIdx.x * chunk;
+  scatter_chunk((int)(n - c0 < chunk ? n - c0 : chunk), seed, kCoarseBits, 0u, 1 << kCoarseBits, coarse_cap,
+                ScatterSmem(sm, 1 << kCoarseBits), coarse_count, coarse, [&](int i) { return (int32_t)(c0 + i); }, [&](int32_t v) {
+                  const uint32_t b = bucket_of(perm_key(seed, (uint64_t)v), bits), at = atomicAdd(count + b, 1u);
+                  if (at < (uint32_t)cap) tmp[(int64_t)b * cap + at] = v;
+                  else spill_one(v, spill);
+                });
+}
+
+// Chunk blockIdx.x of coarse bucket blockIdx.y into its part of the 2^bits buckets.
+__global__ void __launch_bounds__(kScatterThreads)
+k_bucket_fine(uint64_t seed, int64_t coarse_cap, const uint32_t* __restrict__ coarse_count,
+              const int32_t* __restrict__ coarse, int bits, int cap, uint32_t* __restrict__ count,
+              int32_t* __restrict__ tmp, uint32_t* __restrict__ spill) {
+  extern __shared__ uint32_t sm[];
+  const int64_t have = coarse_count[blockIdx.y], size = have < coarse_cap ? have : coarse_cap;
+  const int64_t c0 = (int64_t)blockIdx.x * kChunk;
+  if (c0 >= size) return;
+  const int32_t* const from = coarse + (int64_t)blockIdx.y * coarse_cap + c0;
+  const int nb = 1 << (bits - kCoarseBits);
+  scatter_chunk((int)(size - c0 < kChunk ? size - c0 : kChunk), seed, bits, blockIdx.y * (uint32_t)nb, nb, cap,
+                ScatterSmem(sm, nb), count, tmp, [&](int i) { return __ldg(from + i); }, [&](int32_t v) { spill_one(v, spill); });
+}
+
+// start[0..nb] = exclusive scan of the buckets' sizes.
+__global__ void __launch_bounds__(1024) k_bucket_starts(int nb, const uint32_t* __restrict__ count,
+                                                        int64_t* __restrict__ start) {
+  __shared__ int64_t scr[33];
+  const int per = (nb + 1023) / 1024, b0 = (int)threadIdx.x * per;
+  int64_t sum = 0;
+  for (int q = 0; q < per; ++q) sum += b0 + q < nb ? (int64_t)count[b0 + q] : 0;
+  int64_t tot;
+  int64_t run = block_exclusive_sum<int64_t>(sum, scr, &tot);
+  for (int q = 0; q < per && b0 + q < nb; ++q) {
+    start[b0 + q] = run;
+    run += (int64_t)count[b0 + q];
   }
+  if (threadIdx.x == 0) start[nb] = tot;
 }
 
 __device__ __forceinline__ bool kv_less(uint64_t ka, int32_t va, uint64_t kb, int32_t vb) {
@@ -91,124 +172,132 @@ __device__ __forceinline__ bool kv_less(uint64_t ka, int32_t va, uint64_t kb, in
 // top `bits` bits and the next kSubBits bits are still uniform, so a counting
 // sort on those bits spreads the bucket over kSub sub-buckets of about one
 // element each; one thread then finishes each sub-bucket with an insertion
-// sort on the full (key, v).
-constexpr int kSubBits = 10;
+// sort on the 32 key bits below, which stand beside the vertex in shared memory
+// (equal ones: on the full key and the vertex).  The bucket is read twice, for
+// the counts and for the places: a copy of it in shared memory would halve the
+// blocks per SM.
+constexpr int kSubBits = 12;
 constexpr int kSub = 1 << kSubBits;
-// the sub-bucket counts are scanned two per thread
-static_assert(2 * kSortThreads >= kSub, "k_bucket_sort needs 2 * kSortThreads >= kSub");
+static_assert(kSub % kSortThreads == 0, "every thread scans the same number of sub-buckets");
+
+struct SortSmem {
+  uint32_t k[kBucketCap];
+  int32_t v[kBucketCap];
+  int32_t cnt[kSub];
+  int32_t scr[33];
+};
+
+__device__ __forceinline__ bool sub_less(uint64_t seed, uint32_t ka, int32_t va, uint32_t kb, int32_t vb) {
+  return ka != kb ? ka < kb : kv_less(perm_key(seed, (uint64_t)va), va, perm_key(seed, (uint64_t)vb), vb);
+}
 
 __global__ void __launch_bounds__(kSortThreads)
-k_bucket_sort(uint64_t seed, int bits, int64_t nb, const int64_t* __restrict__ start,
-              const int32_t* __restrict__ tmp, int32_t* __restrict__ order, int* __restrict__ overflow) {
-  __shared__ uint64_t sk[kBucketCap];
-  __shared__ int32_t sv[kBucketCap];
-  __shared__ uint64_t ok_[kBucketCap];
-  __shared__ int32_t ov[kBucketCap];
-  __shared__ int32_t cnt[kSub + 1];
-  __shared__ int64_t scr[33];
-  const int shift = 64 - bits - kSubBits;
-  for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
-    const int64_t s0 = start[b], len = start[b + 1] - s0;
-    if (len <= 0) continue;
-    if (len > kBucketCap) {   // handled by k_bucket_sort_large
-      if (threadIdx.x == 0) {
-        int slot = atomicAdd(overflow, 1);
-        if (slot < kMaxOverflow) overflow[1 + slot] = (int)b;
+k_bucket_sort(uint64_t seed, int bits, int nb, int cap, const int64_t* __restrict__ start,
+              const int32_t* __restrict__ tmp, int32_t* __restrict__ order, const uint32_t* __restrict__ spill,
+              int* __restrict__ err) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  SortSmem& S = *reinterpret_cast<SortSmem*>(raw);
+  constexpr int kPer = kSub / kSortThreads;
+  const uint32_t spilled = *spill;
+  if (spilled > (uint32_t)kSpillCap) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(err, kOk, kErrInternal);
+    return;
+  }
+  for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+    const int64_t s0 = start[b];
+    const int len = (int)(start[b + 1] - s0);
+    const int32_t* const in = tmp + (int64_t)b * cap;
+    if (len > cap) {
+      // a bucket with spilled vertices (next to impossible for a hash): each
+      // one's position is the number of smaller ones, by counting
+      auto member = [&](int i) -> int32_t { return i < cap ? in[i] : (int32_t)spill[1 + i - cap]; };
+      const int all = cap + (int)spilled;
+      for (int i = threadIdx.x; i < all; i += kSortThreads) {
+        const int32_t vi = member(i);
+        const uint64_t ki = perm_key(seed, (uint64_t)vi);
+        if ((int)bucket_of(ki, bits) != b) continue;
+        int64_t r = 0;
+        for (int j = 0; j < all; ++j) {
+          const int32_t vj = member(j);
+          const uint64_t kj = perm_key(seed, (uint64_t)vj);
+          r += (int)bucket_of(kj, bits) == b && kv_less(kj, vj, ki, vi) ? 1 : 0;
+        }
+        order[s0 + r] = vi;
       }
       continue;
     }
-    for (int i = threadIdx.x; i < kSub; i += blockDim.x) cnt[i] = 0;
+    auto sub_of = [&](uint64_t key) { return (int)((key << bits) >> (64 - kSubBits)); };
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) S.cnt[threadIdx.x + q * kSortThreads] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-      const int32_t v = tmp[s0 + i];
-      const uint64_t k = perm_key(seed, (uint64_t)v);
-      sv[i] = v;
-      sk[i] = k;
-      atomicAdd(&cnt[(int)((k >> shift) & (kSub - 1))], 1);
-    }
+    for (int i = threadIdx.x; i < len; i += kSortThreads) atomicAdd(&S.cnt[sub_of(perm_key(seed, (uint64_t)in[i]))], 1);
     __syncthreads();
-    // exclusive scan of the sub-bucket counts (two per thread)
+    // exclusive scan of the sub-bucket counts
     {
-      const int i0 = threadIdx.x * 2;
-      const int c0 = i0 < kSub ? cnt[i0] : 0, c1 = i0 + 1 < kSub ? cnt[i0 + 1] : 0;
-      int64_t tot;
-      const int64_t ex = block_exclusive_sum<int64_t>(c0 + c1, scr, &tot);
-      if (i0 < kSub) cnt[i0] = (int)ex;
-      if (i0 + 1 < kSub) cnt[i0 + 1] = (int)ex + c0;
-      if (threadIdx.x == 0) cnt[kSub] = (int)tot;
+      int32_t c[kPer], sum = 0, tot;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        c[q] = S.cnt[threadIdx.x * kPer + q];
+        sum += c[q];
+      }
+      int32_t run = block_exclusive_sum<int32_t>(sum, S.scr, &tot);
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        S.cnt[threadIdx.x * kPer + q] = run;
+        run += c[q];
+      }
     }
     __syncthreads();
     // scatter into sub-buckets (arbitrary order inside a sub-bucket); the
     // counters end at the next sub-bucket's start
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-      const uint64_t k = sk[i];
-      const int pos = atomicAdd(&cnt[(int)((k >> shift) & (kSub - 1))], 1);
-      ok_[pos] = k;
-      ov[pos] = sv[i];
+    for (int i = threadIdx.x; i < len; i += kSortThreads) {
+      const int32_t v = in[i];
+      const uint64_t key = perm_key(seed, (uint64_t)v);
+      const int pos = atomicAdd(&S.cnt[sub_of(key)], 1);
+      S.k[pos] = (uint32_t)((key << (bits + kSubBits)) >> 32);
+      S.v[pos] = v;
     }
     __syncthreads();
     // sub-bucket q now spans [q == 0 ? 0 : cnt[q-1], cnt[q]): insertion sort
-    for (int q = threadIdx.x; q < kSub; q += blockDim.x) {
-      const int lo = q == 0 ? 0 : cnt[q - 1], hi = cnt[q];
+    for (int q = threadIdx.x; q < kSub; q += kSortThreads) {
+      const int lo = q == 0 ? 0 : S.cnt[q - 1], hi = S.cnt[q];
       for (int i = lo + 1; i < hi; ++i) {
-        const uint64_t k = ok_[i];
-        const int32_t v = ov[i];
+        const uint32_t k = S.k[i];
+        const int32_t v = S.v[i];
         int j = i - 1;
-        while (j >= lo && kv_less(k, v, ok_[j], ov[j])) {
-          ok_[j + 1] = ok_[j];
-          ov[j + 1] = ov[j];
+        while (j >= lo && sub_less(seed, k, v, S.k[j], S.v[j])) {
+          S.k[j + 1] = S.k[j];
+          S.v[j + 1] = S.v[j];
           --j;
         }
-        ok_[j + 1] = k;
-        ov[j + 1] = v;
+        S.k[j + 1] = k;
+        S.v[j + 1] = v;
       }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < len; i += blockDim.x) order[s0 + i] = ov[i];
+    for (int i = threadIdx.x; i < len; i += kSortThreads) order[s0 + i] = S.v[i];
     __syncthreads();
   }
 }
 
-// Exact fallback for buckets above kBucketCap: each element's position is the
-// number of bucket elements smaller than it.
-__global__ void k_bucket_sort_large(uint64_t seed, const int* __restrict__ overflow,
-                                    const int64_t* __restrict__ start, const int32_t* __restrict__ tmp,
-                                    int32_t* __restrict__ order, int* __restrict__ err) {
-  const int cnt = overflow[0];
-  if (cnt > kMaxOverflow) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(err, kOk, kErrInternal);
-    return;
-  }
-  for (int q = 0; q < cnt; ++q) {
-    const int64_t b = overflow[1 + q];
-    const int64_t s0 = start[b], len = start[b + 1] - s0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t vi = tmp[s0 + i];
-      const uint64_t ki = perm_key(seed, (uint64_t)vi);
-      int64_t r = 0;
-      for (int64_t j = 0; j < len; ++j) {
-        const int32_t vj = tmp[s0 + j];
-        r += kv_less(perm_key(seed, (uint64_t)vj), vj, ki, vi) ? 1 : 0;
-      }
-      order[s0 + r] = vi;
-    }
-  }
+// Bucket sizes: 2048 to 4096 expected vertices, fewer (512 at least) while there
+// are not two buckets per SM.
+int bucket_bits(int64_t n) {
+  int bits = 0;
+  while ((n >> bits) > kMeanMax) ++bits;
+  while ((1 << bits) < 304 && (n >> (bits + 1)) >= 512) ++bits;
+  return bits;
 }
 
 }  // namespace
 
-int perm_bucket_bits(int64_t n) {
-  int bits = 0;
-  while (bits < 40 && (n >> bits) > 768) ++bits;
-  return bits;
-}
-
 size_t perm_workspace_bytes(int64_t n) {
-  const int64_t nb = int64_t(1) << perm_bucket_bits(n);
-  return align_up(sizeof(uint32_t) * nb) + align_up(sizeof(int64_t) * (nb + 1)) +
-         align_up(sizeof(int64_t) * nb) + align_up(sizeof(int32_t) * (n > 0 ? n : 1)) +
-         align_up(sizeof(int) * (kMaxOverflow + 1)) + align_up(sizeof(int64_t) * ((nb + kScanTile - 1) / kScanTile));
+  const int bits = bucket_bits(n);
+  const int64_t nb = int64_t(1) << bits;
+  const int64_t nc = bits > kOneLevelBits ? int64_t(1) << kCoarseBits : 0;
+  return align_up(sizeof(uint32_t) * (nc + nb + 1 + kSpillCap)) + align_up(sizeof(int64_t) * (nb + 1)) +
+         align_up(sizeof(int32_t) * nb * bucket_cap((n >> bits) + 1)) +
+         align_up(sizeof(int32_t) * nc * bucket_cap((n >> kCoarseBits) + 1));
 }
 
 // order[0..n) = pi for `seed`.  ws must hold perm_workspace_bytes(n).  A
@@ -216,32 +305,48 @@ size_t perm_workspace_bytes(int64_t n) {
 cudaError_t launch_permutation(int64_t n, uint64_t seed, int32_t* order, void* ws, int num_sms,
                                int* err, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
-  const int bits = perm_bucket_bits(n);
-  const int64_t nb = int64_t(1) << bits;
+  const int bits = bucket_bits(n), nb = 1 << bits, cap = (int)bucket_cap((n >> bits) + 1);
+  const int nc = bits > kOneLevelBits ? 1 << kCoarseBits : 0;
   char* p = static_cast<char*>(ws);
-  uint32_t* count = reinterpret_cast<uint32_t*>(p); p += align_up(sizeof(uint32_t) * nb);
-  int64_t* start = reinterpret_cast<int64_t*>(p);   p += align_up(sizeof(int64_t) * (nb + 1));
-  uint32_t* cursor = reinterpret_cast<uint32_t*>(p); p += align_up(sizeof(int64_t) * nb);
-  int32_t* tmp = reinterpret_cast<int32_t*>(p);     p += align_up(sizeof(int32_t) * n);
-  int* overflow = reinterpret_cast<int*>(p);         p += align_up(sizeof(int) * (kMaxOverflow + 1));
-  int64_t* tot = reinterpret_cast<int64_t*>(p);
-  const int64_t stiles = (nb + kScanTile - 1) / kScanTile;
-  cudaError_t e = cudaMemsetAsync(count, 0, sizeof(uint32_t) * nb, stream);
+  uint32_t* coarse_count = reinterpret_cast<uint32_t*>(p);
+  uint32_t* count = coarse_count + nc;
+  uint32_t* spill = count + nb;                              // their number, then the vertices
+  p += align_up(sizeof(uint32_t) * ((size_t)nc + nb + 1 + kSpillCap));
+  int64_t* start = reinterpret_cast<int64_t*>(p);
+  p += align_up(sizeof(int64_t) * ((size_t)nb + 1));
+  int32_t* tmp = reinterpret_cast<int32_t*>(p);
+  p += align_up(sizeof(int32_t) * (size_t)nb * cap);
+  int32_t* coarse = reinterpret_cast<int32_t*>(p);
+  cudaError_t e = cudaMemsetAsync(coarse_count, 0, sizeof(uint32_t) * ((size_t)nc + nb + 1), stream);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(overflow, 0, sizeof(int), stream);
+  // chunks: two per SM at least
+  const int64_t share = (n + (int64_t)num_sms * 2 - 1) / ((int64_t)num_sms * 2);
+  const int64_t chunk = share < 2048 ? 2048 : (share < kChunk ? share : kChunk);
+  const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
+  if (nc == 0) {
+    const size_t smem = scatter_smem(nb, chunk);
+    e = cudaFuncSetAttribute(k_bucket_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_bucket_scatter<<<grid, kScatterThreads, smem, stream>>>(n, seed, bits, cap, chunk, count, tmp, spill);
+  } else {
+    const int64_t coarse_cap = bucket_cap((n >> kCoarseBits) + 1);
+    size_t smem = scatter_smem(nc, chunk);
+    e = cudaFuncSetAttribute(k_bucket_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_bucket_coarse<<<grid, kScatterThreads, smem, stream>>>(n, seed, coarse_cap, chunk, coarse_count, coarse, bits, cap,
+                                                          count, tmp, spill);
+    const dim3 fine((unsigned)((coarse_cap + kChunk - 1) / kChunk), (unsigned)nc);
+    smem = scatter_smem(nb / nc, kChunk);
+    e = cudaFuncSetAttribute(k_bucket_fine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_bucket_fine<<<fine, kScatterThreads, smem, stream>>>(
+        seed, coarse_cap, coarse_count, coarse, bits, cap, count, tmp, spill);
+  }
+  k_bucket_starts<<<1, 1024, 0, stream>>>(nb, count, start);
+  e = cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
   if (e != cudaSuccess) return e;
-  const int64_t want = (n + 255) / 256;
-  const int grid = (int)(want < (int64_t)num_sms * 8 ? want : (int64_t)num_sms * 8);
-  k_bucket_hist<<<grid, 256, 0, stream>>>(n, seed, bits, count);
-  k_scan_tiles<<<(unsigned)stiles, kScanTile, 0, stream>>>(count, nb, start, tot);
-  k_scan_totals<<<1, 1024, 0, stream>>>(stiles, nb, tot, start);
-  k_scan_add<<<(unsigned)stiles, kScanTile, 0, stream>>>(nb, tot, start, cursor);
-  k_bucket_scatter<<<grid, 256, 0, stream>>>(n, seed, bits, cursor, tmp);
-  const int sgrid = (int)(nb < (int64_t)num_sms * 4 ? nb : (int64_t)num_sms * 4);
-  k_bucket_sort<<<sgrid, kSortThreads, 0, stream>>>(seed, bits, nb, start, tmp, order, overflow);
-  // The fallback kernel returns at once when no bucket overflowed, so it
-  // always runs; this keeps the host free of a sync.
-  k_bucket_sort_large<<<num_sms, 256, 0, stream>>>(seed, overflow, start, tmp, order, err);
+  k_bucket_sort<<<nb < num_sms * 4 ? nb : num_sms * 4, kSortThreads, sizeof(SortSmem), stream>>>(
+      seed, bits, nb, cap, start, tmp, order, spill, err);
   return cudaGetLastError();
 }
 
