@@ -227,11 +227,7 @@ int cc_graph_destroy(cc_graph* g) {
   dfree(g->nz_pos, s);
   dfree(g->dsort, s);
   dfree(g->dge, s);
-  dfree(g->up_v, s);
   dfree(g->up_row, s);
-  dfree(g->up_len, s);
-  dfree(g->up_pos, s);
-  dfree(g->up_epos, s);
   dfree(g->perm_ws, s);
   dfree(g->order, s);
   dfree(g->round_ws, s);
@@ -357,15 +353,15 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
       void* dws = nullptr;
       if ((rc = from_cuda(dalloc(&g->dsort, 4 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&g->dge, 8 * ((size_t)g->max_deg + 2), s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_v, 4 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_row, 8 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_len, 4 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_pos, 4 * nz, s))) != CC_OK ||
-          (rc = from_cuda(dalloc(&g->up_epos, 4 * nz, s))) != CC_OK ||
+          (rc = from_cuda(dalloc(&g->up_row, 24 * nz, s))) != CC_OK ||
           (rc = from_cuda(dalloc(&dws, degree_order_workspace_bytes(g->max_deg), s))) != CC_OK) {
         dfree(dws, s); dfree(vws, s); dfree(nws, s); dfree(up_at, s);
         break;
       }
+      g->up_v = reinterpret_cast<int32_t*>(g->up_row + nz);
+      g->up_len = g->up_v + nz;
+      g->up_pos = reinterpret_cast<uint32_t*>(g->up_len + nz);
+      g->up_epos = g->up_pos + nz;
       rc = from_cuda(launch_degree_order(g->nz_n, g->nz_row, g->off, g->max_deg, g->dsort, g->dge, dws, g->num_sms, s));
       dfree(dws, s);
       if (rc != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }

@@ -25,8 +25,8 @@ struct cc_graph {
   int32_t* dsort = nullptr;
   int64_t* dge = nullptr;
   // the upper part of every row, each edge once (arrays of nz_n entries)
+  int64_t* up_row = nullptr;       // the allocation; the others lie behind
   int32_t* up_v = nullptr;
-  int64_t* up_row = nullptr;
   int32_t* up_len = nullptr;
   uint32_t* up_pos = nullptr;
   uint32_t* up_epos = nullptr;
