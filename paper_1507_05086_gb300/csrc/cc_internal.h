@@ -103,8 +103,8 @@ Tuning batch_settings(int64_t* small_n, int64_t* team_n, int* team_blocks);
 // The upper part of every row (columns above the row's vertex), which holds
 // each edge once: per row with a non-empty upper part its vertex, the CSR
 // position and length of the part, its first unit (unit_walk in
-// cc_device.cuh) and the entries before it (row_walk; batched jobs, whose rows
-// are short).  The objective walks it.
+// cc_device.cuh) and the entries before it (row_walk: batched jobs, whose rows
+// are short, and the largest graphs).  The objective walks it.
 struct UpperRows {
   const int32_t* v;
   const int64_t* row;

@@ -48,16 +48,18 @@ __global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int
   if (threadIdx.x == 0 && pairs) atomicAdd(out + 1, (unsigned long long)pairs);
 }
 
-// Edges (u, w) with id[u] == id[w] in [lo, hi), every edge read from its lower end only
-// (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 23
+// Edges (u, w) with id[u] == id[w] in [lo, hi), every edge read from its lower
+// end only (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 23
 // (130M edges, 0.49 ms, 265e9 edges/s) L2 runs at 65 % and L1 at 70 % of their
 // throughput, above the 236e9 reads/s of a library gather from a 32 MiB table.
 // With sig, a 4-bit signature per vertex decides first, so that ids are read
 // only where the signatures agree.  Whole objective of a ClusterWild! labelling
 // of R-MAT 22 / 24 / 26: both ends of every edge 0.59 / 2.43 / 12.5 ms, upper
-// ends over 128-edge batches (lbs_for_each) 0.40 / 1.52 / 7.6 ms, this 0.32 /
-// 1.22 / 5.8 ms.  Three blocks per SM at 40 registers spill: 0.49 / 1.90 / 7.4;
-// four units per batch at three blocks: 0.37 / 1.41 / 5.7.
+// ends over 128-edge batches (lbs_for_each) 0.40 / 1.52 / 7.6 ms, by units of 32
+// entries 0.32 / 1.22 / 5.8 ms.  Three blocks per SM at 40 registers spill: 0.49 /
+// 1.90 / 7.4; four units per batch at three blocks: 0.37 / 1.41 / 5.7.  By rows
+// (row_walk) 0.37 ms at R-MAT 22 but 5.3 at R-MAT 26, where the ids come from
+// DRAM: with sig the walk is by rows, else by units.
 template <bool kSig>
 __global__ void __launch_bounds__(kObjThreads, kObjBlocks) k_intra(UpperRows up, const int32_t* __restrict__ col,
                                                       uint32_t lo, uint32_t hi,
@@ -65,29 +67,41 @@ __global__ void __launch_bounds__(kObjThreads, kObjBlocks) k_intra(UpperRows up,
                                                       const uint32_t* __restrict__ sig, unsigned long long* out) {
   __shared__ int64_t scr[33];
   int64_t cnt = 0;
-  unit_walk((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, ((int64_t)gridDim.x * blockDim.x) >> 5, up.n,
-            up.units, col, WalkShape{}, [&](int64_t j) { return __ldg(up.pos + j); },
-            [&](int64_t j) {
-              const uint32_t x = __ldg(id + __ldg(up.v + j));
-              return UnitItem{__ldg(up.pos + j), __ldg(up.len + j), __ldg(up.row + j),
-                              (int32_t)(x >= lo && x < hi ? x : 0xFFFFFFFFu)};
-            },
-            [&](const UnitBatch& X) {
-    uint32_t x[kUnitB];
+  auto center = [&](int64_t j) {
+    const uint32_t x = __ldg(id + __ldg(up.v + j));
+    return (int32_t)(x >= lo && x < hi ? x : 0xFFFFFFFFu);
+  };
+  auto count = [&](const auto& X) {
+    constexpr int kB = sizeof(X.w) / sizeof(int32_t);
+    uint32_t x[kB];
     if (kSig) {
 #pragma unroll
-      for (int q = 0; q < kUnitB; ++q) x[q] = X.w[q] >= 0 ? __ldg(sig + (X.w[q] >> 3)) >> ((X.w[q] & 7) * 4) : 0;
+      for (int q = 0; q < kB; ++q) x[q] = X.w[q] >= 0 ? __ldg(sig + (X.w[q] >> 3)) >> ((X.w[q] & 7) * 4) : 0;
 #pragma unroll
-      for (int q = 0; q < kUnitB; ++q)
+      for (int q = 0; q < kB; ++q)
         if (X.w[q] >= 0 && ((x[q] ^ cluster_sig((uint32_t)X.aux[q])) & 15u) == 0)
           cnt += __ldg(id + X.w[q]) == (uint32_t)X.aux[q] ? 1 : 0;
     } else {
 #pragma unroll
-      for (int q = 0; q < kUnitB; ++q) x[q] = X.w[q] >= 0 ? __ldg(id + X.w[q]) : 0;
+      for (int q = 0; q < kB; ++q) x[q] = X.w[q] >= 0 ? __ldg(id + X.w[q]) : 0;
 #pragma unroll
-      for (int q = 0; q < kUnitB; ++q) cnt += X.w[q] >= 0 && x[q] == (uint32_t)X.aux[q] ? 1 : 0;
+      for (int q = 0; q < kB; ++q) cnt += X.w[q] >= 0 && x[q] == (uint32_t)X.aux[q] ? 1 : 0;
     }
-  });
+  };
+  const int gwarp = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
+  const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+  if (kSig) {
+    row_walk<kUnitB>(gwarp, nwarps, (int32_t)up.n, up.edges, col, WalkShape{},
+                     [&](int32_t j) { return (int64_t)__ldg(up.epos + j); },
+                     [&](int32_t j) {
+                       return RowItem{(int64_t)__ldg(up.epos + j), __ldg(up.row + j), __ldg(up.len + j), center(j)};
+                     },
+                     count);
+  } else {
+    unit_walk(gwarp, nwarps, up.n, up.units, col, WalkShape{}, [&](int64_t j) { return __ldg(up.pos + j); },
+              [&](int64_t j) { return UnitItem{__ldg(up.pos + j), __ldg(up.len + j), __ldg(up.row + j), center(j)}; },
+              count);
+  }
   cnt = block_sum<int64_t>(cnt, scr);
   if (threadIdx.x == 0 && cnt) atomicAdd(out, (unsigned long long)cnt);
 }

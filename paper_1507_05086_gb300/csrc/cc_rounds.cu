@@ -79,10 +79,12 @@ constexpr int kResolve = 11;                 // C4: the round's blocked actives 
 // where co_delta takes up again, or what it does next
 constexpr int kDScan = 0, kDCounted = 1, kDRebuild = 2, kDPlanned = 3, kDDone = 4;
 constexpr int kHList = kThreads;             // heavy lists up to this long: every block lists all of them
-constexpr int kHere = 16 * kThreads;         // heavy lists up to this long are looked at inside the barrier
+// Heavy lists up to this long, one read of the block, are looked at inside the
+// barrier (10K Erdos-Renyi 583 us of rounds, R-MAT 24 11.2 ms; 8192: 647, 11.5;
+// 1024: 589, 11.2, and planted 10^6 5.7 ms against 5.6).
+constexpr int kHere = kScanU * kThreads;
 constexpr int kHRows = 1024;                 // rows that one block recounts at once
 constexpr int kHPick = 4096;                 // vertices that one block picks at once
-constexpr int kInlineWindow = 1024;          // selection windows up to this long are scanned inside the barrier
 constexpr int kInlineEdges = 8192;           // recounts up to this many entries run inside the barrier
 constexpr int32_t kLongRow = 1024;           // rows above this are not recounted by one block alone
 constexpr int32_t kTightest = 8;             // heavy lists reach down to 1 - 2^-8 of the largest bound at most
@@ -723,57 +725,36 @@ struct K {
   __device__ __noinline__ void look_here() {
     Coord& c = co();
     const int len = (int)c.h_len;
-    constexpr int step = kScanU * kThreads;
     int32_t v[kScanU], ub[kScanU], top = 0, alive = 0;
-    const auto read = [&](int base) {
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const int i = base + q * kThreads + (int)threadIdx.x;
-        v[q] = i < len ? ldcg(hv() + i) : -1;
-      }
+    for (int q = 0; q < kScanU; ++q) {
+      const int i = q * kThreads + (int)threadIdx.x;
+      v[q] = i < len ? ldcg(hv() + i) : -1;
+    }
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const uint32_t x = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
-        ub[q] = is_alive(x) ? (int32_t)deg_of(x) : 0;
-      }
-    };
-#pragma unroll 1
-    for (int base = 0; base < len; base += step) {
-      read(base);
-#pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        top = ub[q] > top ? ub[q] : top;
-        alive += ub[q] > 0 ? 1 : 0;
-      }
+    for (int q = 0; q < kScanU; ++q) {
+      const uint32_t x = v[q] >= 0 ? ldcg(B.st + v[q]) : 0u;
+      ub[q] = is_alive(x) ? (int32_t)deg_of(x) : 0;
+      top = ub[q] > top ? ub[q] : top;
+      alive += ub[q] > 0 ? 1 : 0;
     }
     if (threadIdx.x == 0) S->h_picked = S->h_kept = 0;
     top = max_i32(top);
     // a second look costs no barrier here: a fraction of the recent fall
     const int32_t th = c.d_lb < 0 ? below(top, c.d_drop >> 2) : c.d_lb + 1;
-    const bool pack = sum_i32(alive) < len - (len >> 2);    // a quarter has left
+    const bool pack = sum_i32(alive) < len - (len >> 2);    // a quarter has left (every entry is read by now)
     int32_t other = 0;
-#pragma unroll 1
-    for (int base = 0; base < len; base += step) {
-      if (len > step) read(base);                        // a longer list is read again (L2)
-      if (pack) __syncthreads();                         // the step is read before it is written over
 #pragma unroll
-      for (int q = 0; q < kScanU; ++q) {
-        const bool take = v[q] >= 0 && ub[q] >= th;      // th >= 1
-        other = !take && ub[q] > other ? ub[q] : other;
-        const unsigned m = __ballot_sync(FULL, take);
-        if (m) {
-          int at = 0;
-          if ((threadIdx.x & 31) == 0) at = atomicAdd(&S->h_picked, __popc(m));
-          at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
-          if (take && at < kHPick) S->u.hl.pick[at] = v[q];
-        }
-        if (!pack) continue;
-        const unsigned k = __ballot_sync(FULL, ub[q] > 0);
-        int at = 0;
-        if (k && (threadIdx.x & 31) == 0) at = atomicAdd(&S->h_kept, __popc(k));
-        at = __shfl_sync(FULL, at, 0) + __popc(k & ((1u << (threadIdx.x & 31)) - 1u));
-        if (ub[q] > 0) hv()[at] = v[q];
-      }
+    for (int q = 0; q < kScanU; ++q) {
+      const bool take = v[q] >= 0 && ub[q] >= th;        // th >= 1
+      other = !take && ub[q] > other ? ub[q] : other;
+      pick(take, v[q]);
+      if (!pack) continue;
+      const unsigned k = __ballot_sync(FULL, ub[q] > 0);
+      int at = 0;
+      if (k && (threadIdx.x & 31) == 0) at = atomicAdd(&S->h_kept, __popc(k));
+      at = __shfl_sync(FULL, at, 0) + __popc(k & ((1u << (threadIdx.x & 31)) - 1u));
+      if (ub[q] > 0) hv()[at] = v[q];
     }
     other = max_i32(other);
     if (threadIdx.x == 0) {
@@ -1656,12 +1637,10 @@ struct K {
     __syncthreads();
   }
 
-  // Coordinator: short windows at once (a grid phase would cost a barrier and
-  // the same dependent loads); a team of one block has nobody to share with.
-  // Not C4's, whose blocked actives the grid finds in the same phase
-  // (select_attach): R-MAT 18 by the Sec. 5 schedule 13.9 -> 12.8 ms.
+  // A team of one block has nobody to share a window with: it selects inside the
+  // barrier.
   __device__ __noinline__ void select_here() {
-    while (S->plan.state == kSelect && (G == 1 || (algo == kAlgoCW && P().win_len <= kInlineWindow))) {
+    while (S->plan.state == kSelect && G == 1) {
       select_window(true);
       __syncthreads();
       select_decide(true);
