@@ -161,7 +161,7 @@ int ensure_cluster_ws(cc_graph* g) {
     CC_TRY(dalloc(&g->perm_ws, pb, g->stream));
     g->perm_ws_bytes = pb;
   }
-  if (!g->grid) g->grid = rounds_grid_size(g->device, g->nnz);
+  if (!g->grid) g->grid = rounds_grid_size(g->device, g->nnz, g->max_deg);
   const size_t rb = rounds_workspace_bytes(g->n, g->max_deg, g->grid);
   if (g->round_ws_bytes < rb) {
     dfree(g->round_ws, g->stream);

@@ -218,7 +218,7 @@ size_t rounds_workspace_bytes(int64_t n, int32_t max_deg, int grid);
 // Carve a workspace of rounds_workspace_bytes() into RoundBuffers (pointers only).
 void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* b);
 // Largest co-resident grid for the persistent round kernel on this device.
-int rounds_grid_size(int device, int64_t nnz);
+int rounds_grid_size(int device, int64_t nnz, int32_t max_deg);
 cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint64_t seed, int grid,
                           cudaStream_t stream, int32_t withhold = 0);
 // labels_out[v] = center vertex id (order[center rank]) when labels_out is

@@ -2644,20 +2644,26 @@ void rounds_carve(void* ws, int64_t n, int32_t max_deg, int grid, RoundBuffers* 
   B->desc = reinterpret_cast<unsigned long long*>(take(8 * kDescStride * ((size_t)grid + 1)));
 }
 
-// Blocks of k_rounds per SM.  Rounds of small graphs are a chain of barriers and
+// Blocks of k_rounds per SM.  Rounds of few entries are a chain of barriers and
 // dependent reads: one block per SM, whose barrier has half the arrivals and
-// whose 128 registers spill nothing, is faster (R-MAT 20, 31M entries: 3.39 ms
-// against 3.98; R-MAT 22, 128M: 5.04 / 5.82; planted 0.7M, 24M: 2.20 / 2.48).
-// From here on the walks of a round are long enough for the entries in flight of
-// twice as many warps to count (planted 4M, 137M entries: 4.02 / 3.86 ms; R-MAT
-// 26, 2.1G: 20.1 / 17.8).
-constexpr int64_t kTwoPerSM = int64_t(1) << 27;
-inline int blocks_per_sm(int64_t nnz) { return nnz < kTwoPerSM ? 1 : 2; }
+// whose 128 registers spill nothing, is faster; longer walks want the entries in
+// flight of twice as many warps.  The rounds of a run grow with log Delta, so the
+// measure is entries / log2 of the largest degree (one / two blocks per SM, ms):
+//   planted 2M  68M / 6    C4  2.50 / 2.57        R-MAT 21   64M / 16  C4  4.78 / 5.44
+//   planted 3M 103M / 6    CW  2.22 / 2.14        R-MAT 23  260M / 17  CW  5.88 / 6.15
+//   planted 4M 137M / 6    C4  3.77 / 3.43        R-MAT 24  520M / 18  C4 11.83 / 11.65
+//   planted 8M 275M / 6    CW  4.48 / 3.56        R-MAT 24             CW  8.61 / 8.63
+constexpr int64_t kTwoPerSM = int64_t(1) << 24;
+inline int blocks_per_sm(int64_t nnz, int32_t max_deg) {
+  int log = 1;
+  while (log < 31 && (max_deg >> (log + 1)) != 0) ++log;
+  return nnz / log < kTwoPerSM ? 1 : 2;
+}
 
-int rounds_grid_size(int device, int64_t nnz) {
+int rounds_grid_size(int device, int64_t nnz, int32_t max_deg) {
   int sms = 0, per = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  if (blocks_per_sm(nnz) == 1) return sms;
+  if (blocks_per_sm(nnz, max_deg) == 1) return sms;
   cudaFuncSetAttribute(k_rounds<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rounds<2>, kThreads, sizeof(Shared));
   if (per < 1) per = 1;
@@ -2675,7 +2681,7 @@ cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint
   if (b.n <= 0) return cudaSuccess;
   RoundBuffers arg = b;
   void* args[] = {&arg};
-  const void* const f = blocks_per_sm(b.nnz) == 1 ? (const void*)k_rounds<1> : (const void*)k_rounds<2>;
+  const void* const f = blocks_per_sm(b.nnz, b.max_deg) == 1 ? (const void*)k_rounds<1> : (const void*)k_rounds<2>;
   e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(kThreads), args, sizeof(Shared),
