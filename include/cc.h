@@ -223,11 +223,11 @@ int cc_last_timings(const cc_graph* g, float* ms_out);
 /*
  * Device-side breakdown of the last clustering's round kernel (always
  * recorded; globaltimer at every grid barrier).  ms_out[0..min(cap,7)) =
- * milliseconds spent in: Delta from the heavy list (grid scans) and the
- * count pass of its rebuild, the rebuild's compaction and refill, the Sec. 5
- * batch draws, active-set selection, centers + attachment (C4: detection
- * and classification too), C4 fixpoint and blocked actives, removal and
- * degree updates.  (Zeros for CC_ALGO_C4_ASYNC.)
+ * milliseconds spent in: rebuilds of the heavy list from the alive vertices,
+ * from the degree order, the first Sec. 5 batch draw, the selection of long
+ * windows, selection + attachment and attachment (C4: detection and
+ * classification too), C4 blocked actives, recounts of degrees.  (Zeros for
+ * CC_ALGO_C4_ASYNC.)
  */
 int cc_last_phase_times(const cc_graph* g, double* ms_out, int32_t cap);
 
@@ -322,8 +322,9 @@ int cc_server_destroy(cc_server* s);
  *   walk_batches     edge walker: 128-entry batches per warp chunk, 1..8 (4)
  *   prefetch_ahead   edge walker: batches of a long row prefetched into L2,
  *                    0..8 (2)
- *   inline_heavy     exact Delta: heavy lists up to this long are scanned
- *                    inside the grid barrier by one block, 0..65536 (8192)
+ *   inline_heavy     exact Delta: heavy lists up to this long (and 2048) are
+ *                    looked at inside the grid barrier by one block, 0..65536
+ *                    (8192)
  *   inline_decide    C4: blocked lists up to this long are decided inside the
  *                    barrier, 0..65536 (4096)
  *   inline_rebuild   Delta rebuild: degree-order segments up to this long are

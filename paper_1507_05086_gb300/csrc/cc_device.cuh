@@ -33,11 +33,6 @@ __host__ __device__ __forceinline__ uint64_t perm_key(uint64_t seed, uint64_t v)
 template <class T>
 __device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -47,9 +42,6 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -187,25 +179,6 @@ __device__ __forceinline__ int32_t block_sum_i32(int32_t x, int32_t* scratch) {
   if (lane == 0) scratch[warp] = x;
   __syncthreads();
   return __reduce_add_sync(FULL, lane < (int)((blockDim.x + 31) >> 5) ? scratch[lane] : 0);
-}
-
-template <class T>
-__device__ __forceinline__ T block_max(T x, T* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = (blockDim.x + 31) >> 5;
-  x = warp_max(x);
-  __syncthreads();
-  if (lane == 0) scratch[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    T w = lane < nwarps ? scratch[lane] : scratch[0];
-    w = warp_max(w);
-    if (lane == 0) scratch[0] = w;
-  }
-  __syncthreads();
-  T r = scratch[0];
-  __syncthreads();
-  return r;
 }
 
 // ---------------------------------------------------------------------------

@@ -122,7 +122,7 @@ struct RoundBuffers {
   const int32_t* order;
   uint32_t* st;                // per-vertex state word
   uint32_t* rtag;              // per-vertex removal tag, 4 bits (8 vertices per word)
-  int32_t* arank;              // C4: rank of every vertex (the inverse of order)
+  int32_t* arank;              // C4: rank of every vertex (above 2^24 vertices: of the actives)
   // the actives: vertex, rank, entries before the row (row_walk in
   // cc_device.cuh), CSR row start, row length.  (C4 without rounds: act_e / act_d as in RowList.)
   // The blocked list holds active-list indices, entries before the row and

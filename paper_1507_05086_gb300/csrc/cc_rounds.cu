@@ -14,7 +14,7 @@
 //   clustered ........ kLab + center rank
 //   active ............ kActive / kActCenter / kActNon (undecided or
 //                       ClusterWild! center / C4 center / C4 non-center)
-// C4 keeps every vertex's rank in arank[v].  A center keeps its active marker for
+// C4 keeps every vertex's rank in arank[v] (above kStateInL2 vertices: an active's).  A center keeps its active marker for
 // good (its label is its own rank, arank); the actives of the current round
 // are the ones whose rank is >= r0, the round's first active rank.
 //
@@ -69,7 +69,11 @@ constexpr int kSelU = 2;                     // window entries per thread per se
 // Up to this many vertices (64 MB of state words, which L2 holds) selection
 // also reads the bounds and spares the rows of vertices known to have no alive
 // neighbour; above, those rows cost less than a random DRAM read per active.
+// C4 holds the inverse of pi up to here: beyond, its random writes (2.4 ms at 2^26)
+// and reads cost as much as the phases that it spares (set-up and rounds of C4 on
+// R-MAT 25 / 26 16.8 / 25.3 ms, with it 16.7 / 26.2).
 constexpr int64_t kStateInL2 = int64_t(1) << 24;
+constexpr int kInlineWindow = 1024;          // without it, windows up to this long are selected inside the barrier
 constexpr int64_t kDescStride = 16;          // look-back descriptors: one per 128-byte line
 constexpr int kAlgoC4 = 1, kAlgoCW = 2;
 constexpr int kRun = 0, kDone = 1, kSelect = 2, kAbort = 3, kDrawBatch = 6;   // kRun: the active set is there
@@ -324,6 +328,8 @@ struct K {
   }
 
   __device__ __forceinline__ const Plan& P() const { return S->plan; }
+  // Whether windows can be selected and attached in one pass (C4: by the inverse of pi).
+  __device__ __forceinline__ bool fused() const { return algo == kAlgoCW || B.n <= kStateInL2; }
   // The current heavy list (its buffer changes when the grid cuts it down).
   __device__ __forceinline__ int32_t* hv() const { return S->plan.hv_sel ? B.hv2 : B.hv; }
   __device__ __forceinline__ Coord& co() const { return S->co; }
@@ -1484,6 +1490,7 @@ struct K {
       if (!want[q] || T.len[q] == 0) continue;
       set_rtag(B.rtag, T.v[q], tag);
       B.st[T.v[q]] = kActive;
+      if (algo == kAlgoC4 && !fused()) B.arank[T.v[q]] = (int32_t)(T.first + q);
     }
     __syncthreads();
     int64_t j = S->bcast[0] + ((sc.ex >> kL) & 0xFFF), ep = S->bcast[1] + (sc.ex & kEM);
@@ -1637,10 +1644,10 @@ struct K {
     __syncthreads();
   }
 
-  // A team of one block has nobody to share a window with: it selects inside the
-  // barrier.
+  // Inside the barrier select a team of one block, which has nobody to share a
+  // window with, and short windows that cannot be attached in the same pass.
   __device__ __noinline__ void select_here() {
-    while (S->plan.state == kSelect && G == 1) {
+    while (S->plan.state == kSelect && (G == 1 || (!fused() && P().win_len <= kInlineWindow))) {
       select_window(true);
       __syncthreads();
       select_decide(true);
@@ -2145,7 +2152,9 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
       }
     }
     if (S.plan.state == kSelect) {
-      if (k.G > 1 && S.plan.win_len <= kFuseWindow * (int64_t)k.G) {
+      // (a round that has begun to attach goes on that way: only select_attach
+      // takes back what its centers have reached)
+      if (k.G > 1 && k.fused() && (S.plan.win_len <= kFuseWindow * (int64_t)k.G || S.plan.win_lo != (int64_t)S.plan.th)) {
         if (algo == kAlgoC4) k.template select_attach<true, kPerSM>();
         else k.template select_attach<false, kPerSM>();
         k.flush_round_tallies();
@@ -2558,7 +2567,7 @@ __global__ void k_init_state(RoundBuffers B, int algo, int64_t eps_ppm, uint64_t
     B.size[v] = 0;                     // members per center rank
     B.hit_c[v] = 0;                    // C4 fixpoint flags start (and stay) zero
     B.hit_p[v] = 0;
-    if (algo == kAlgoC4 || algo == kAlgoC4 + 2) B.arank[__ldg(B.order + v)] = (int32_t)v;
+    if ((algo == kAlgoC4 || algo == kAlgoC4 + 2) && n <= kStateInL2) B.arank[__ldg(B.order + v)] = (int32_t)v;
   }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rtag_words(n); i += (int64_t)gridDim.x * blockDim.x)
     B.rtag[i] = 0;

@@ -54,3 +54,24 @@ def test_fused_selection_equals_oracle(cc, gg, ora, n, half, hubs, leaves):
             assert np.array_equal(lab, olab) and r == orr and d == ora.disagreements(g.off, g.col, olab), (algo, eps)
             for f in STAT_FIELDS:
                 assert np.array_equal(st[f], ost[f]), (algo, eps, f)
+
+
+def test_second_window_of_a_round_in_small_teams(cc, gg, ora):
+    """Teams of two blocks fuse windows of up to 4096 entries.  In the last rounds
+    of 7000 cliques a window of that length holds a handful of alive vertices;
+    when it holds too few, the round goes on with a longer one whose vertices the
+    first window's centers may have reached."""
+    i, j = np.triu_indices(10, 1)
+    base = (np.arange(7000) * 10)[:, None]
+    g = gg.from_edges(70_000, (base + i).ravel(), (base + j).ravel())
+    default = cc.get_batch_tuning()
+    with cc.Graph(g.off, g.col) as graph:
+        try:
+            cc.set_batch_tuning(dict(default, batch_team_blocks=2))
+            for first in range(0, 600, 150):
+                D, R = cc.batch_jobs([graph], "cw", 0.5, np.array([first], np.uint64), 150)
+                for q in range(150):
+                    lab, r, _, _ = ora.rounds(g.off, g.col, ora.permutation(g.n, first + q), 2, 0.5, 1)
+                    assert R[0, q] == r and D[0, q] == ora.disagreements(g.off, g.col, lab), first + q
+        finally:
+            cc.set_batch_tuning(default)
