@@ -200,7 +200,11 @@ k_bucket_sort(uint64_t seed, int bits, int nb, int cap, const int64_t* __restric
   constexpr int kPer = kSub / kSortThreads;
   const uint32_t spilled = *spill;
   if (spilled > (uint32_t)kSpillCap) {
+    // reported; the kernels that follow find vertices in order all the same
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(err, kOk, kErrInternal);
+    const int64_t n = start[nb];
+    for (int64_t i = blockIdx.x * (int64_t)kSortThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSortThreads)
+      order[i] = (int32_t)i;
     return;
   }
   for (int b = blockIdx.x; b < nb; b += gridDim.x) {

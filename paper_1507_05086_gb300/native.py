@@ -279,6 +279,7 @@ class Graph:
         _check("cc_last_timings", self._lib.cc_last_timings(self._h, ctypes.cast(ms, ctypes.c_void_p)))
         return tuple(float(x) for x in ms)
 
+    # delta_scan / delta_rebuild: heavy-list rebuilds; removal_decrement: recounts of degrees
     PHASES = ("delta_scan", "delta_rebuild", "sec5_draws", "select", "centers_attach",
               "c4_fixpoint", "removal_decrement")
 
