@@ -1015,7 +1015,9 @@ struct K {
       pick(take, v[q]);                     // room for a whole step is left (below)
     }
     __syncthreads();
-    if (S->h_picked > k.limit || (last && S->h_picked > 0)) {    // uniform
+    const int picked = S->h_picked;
+    __syncthreads();                        // all have read it: the next step's picks may add to it
+    if (picked > k.limit || (last && picked > 0)) {      // the same in every thread: recount_picked has barriers
       recount_picked();
       if (S->h_best >= k.th) k.th = S->h_best + 1;
       k.limit = k.limit * 4 < kHPick / 2 ? k.limit * 4 : kHPick / 2;
