@@ -1440,8 +1440,9 @@ struct K {
     if (threadIdx.x == 0) {
       // ClusterWild!: every one is a center; C4: so far those without neighbours
       const int64_t wanted = run + alive < need ? alive : need - run;
-      S->tal[kTCenters] += (unsigned long long)(algo == kAlgoCW ? wanted : wanted - cnt_tot);
-      S->tal[kTEdges] += (unsigned long long)(algo == kAlgoCW ? e_tot : 2 * e_tot);      // C4 reads them twice
+      // (other threads add to both below, for their long rows)
+      atomicAdd(&S->tal[kTCenters], (unsigned long long)(algo == kAlgoCW ? wanted : wanted - cnt_tot));
+      atomicAdd(&S->tal[kTEdges], (unsigned long long)(algo == kAlgoCW ? e_tot : 2 * e_tot));      // C4 reads them twice
     }
     if (kFused) {
       TileRows& R = S->u.rows;
