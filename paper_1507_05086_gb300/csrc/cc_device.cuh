@@ -618,6 +618,7 @@ __device__ __forceinline__ void row_walk(int gwarp, int nwarps, int32_t nitems, 
                                          const int32_t* __restrict__ col, WalkShape shape, const At& at,
                                          const Load& load, F&& f, G&& g) {
   constexpr int32_t kFar = 1 << 30;     // relative positions from here on lie behind the chunk
+  const auto near = [](int64_t x) { return (int32_t)(x < -kFar ? -kFar : x < kFar ? x : kFar); };
   constexpr int kW = 32 * kB;
   const int lane = threadIdx.x & 31;
   // up to 2 * shape.batches batches per chunk, fewer when the list is short
@@ -629,7 +630,8 @@ __device__ __forceinline__ void row_walk(int gwarp, int nwarps, int32_t nitems, 
     const int32_t cend = E - cs < chunk ? (int32_t)(E - cs) : chunk;
     int32_t j0 = nitems > 32 ? warp_item_at(at, nitems, cs) : 0;       // a short list is one window
     for (int32_t e = 0; e < cend; j0 += 32) {
-      // the window: starts and ends relative to the chunk
+      // the window: starts and ends relative to the chunk, from kFar before it to
+      // kFar behind it (a short list's first rows may end 2^31 entries before it)
       int32_t p = kFar, end = kFar, aux = 0;
       int64_t rel = 0;                  // CSR position of the chunk's first entry, were it in this row
       if (j0 + lane < nitems) {
@@ -637,8 +639,8 @@ __device__ __forceinline__ void row_walk(int gwarp, int nwarps, int32_t nitems, 
         const int64_t d = it.pos - cs;
         rel = it.row - d;
         aux = it.aux;
-        p = d < kFar ? (int32_t)d : kFar;
-        end = d + it.len < kFar ? (int32_t)(d + it.len) : kFar;
+        p = near(d);
+        end = near(d + it.len);
       }
       int32_t wend = __shfl_sync(FULL, end, 31);
       wend = wend < cend ? wend : cend;
