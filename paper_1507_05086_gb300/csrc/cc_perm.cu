@@ -36,6 +36,7 @@ constexpr int kSpillCap = 1 << 16;     // vertices that found their bucket full
 constexpr int kOneLevelBits = 12;
 constexpr int kCoarseBits = 9;
 constexpr int kChunk = 16384;          // vertices per block and scatter, at most
+constexpr int kBitsMax = 19;           // buckets of 2^31 - 1 vertices (bucket_bits)
 
 __device__ __forceinline__ uint32_t bucket_of(uint64_t key, int bits) {
   return bits == 0 ? 0u : (uint32_t)(key >> (64 - bits));
@@ -68,7 +69,7 @@ struct ScatterSmem {
   __device__ ScatterSmem(uint32_t* raw, int nb)
       : next(raw), delta(raw + nb), buf(reinterpret_cast<int32_t*>(raw + 2 * nb)) {}
 };
-size_t scatter_smem(int nb, int64_t chunk) { return sizeof(uint32_t) * (2 * (size_t)nb + (size_t)chunk); }
+constexpr size_t scatter_smem(int nb, int64_t chunk) { return sizeof(uint32_t) * (2 * (size_t)nb + (size_t)chunk); }
 
 template <class Source, class Spilled>
 __device__ __forceinline__ void scatter_chunk(int len, uint64_t seed, int bits, uint32_t first, int nb, int64_t cap,
@@ -293,6 +294,21 @@ int bucket_bits(int64_t n) {
   return bits;
 }
 
+// One launch, checked at once: a later success of cudaFuncSetAttribute clears
+// the error of a refused launch.  The limit of a kernel's dynamic shared memory
+// belongs to the kernel, not to the call, and other threads launch it for graphs
+// of other sizes: every call sets the kernel's own largest need, `most`.
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, size_t most, cudaStream_t stream,
+                   A... args) {
+  if (most > 0) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) return e;
+  }
+  kernel<<<grid, threads, smem, stream>>>(args...);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 size_t perm_workspace_bytes(int64_t n) {
@@ -328,30 +344,24 @@ cudaError_t launch_permutation(int64_t n, uint64_t seed, int32_t* order, void* w
   const int64_t chunk = share < 2048 ? 2048 : (share < kChunk ? share : kChunk);
   const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
   if (nc == 0) {
-    const size_t smem = scatter_smem(nb, chunk);
-    e = cudaFuncSetAttribute(k_bucket_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = launch(k_bucket_scatter, grid, kScatterThreads, scatter_smem(nb, chunk),
+               scatter_smem(1 << kOneLevelBits, kChunk), stream, n, seed, bits, cap, chunk, count, tmp, spill);
     if (e != cudaSuccess) return e;
-    k_bucket_scatter<<<grid, kScatterThreads, smem, stream>>>(n, seed, bits, cap, chunk, count, tmp, spill);
   } else {
     const int64_t coarse_cap = bucket_cap((n >> kCoarseBits) + 1);
-    size_t smem = scatter_smem(nc, chunk);
-    e = cudaFuncSetAttribute(k_bucket_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = launch(k_bucket_coarse, grid, kScatterThreads, scatter_smem(nc, chunk), scatter_smem(1 << kCoarseBits, kChunk),
+               stream, n, seed, coarse_cap, chunk, coarse_count, coarse, bits, cap, count, tmp, spill);
     if (e != cudaSuccess) return e;
-    k_bucket_coarse<<<grid, kScatterThreads, smem, stream>>>(n, seed, coarse_cap, chunk, coarse_count, coarse, bits, cap,
-                                                          count, tmp, spill);
     const dim3 fine((unsigned)((coarse_cap + kChunk - 1) / kChunk), (unsigned)nc);
-    smem = scatter_smem(nb / nc, kChunk);
-    e = cudaFuncSetAttribute(k_bucket_fine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = launch(k_bucket_fine, fine, kScatterThreads, scatter_smem(nb / nc, kChunk),
+               scatter_smem(1 << (kBitsMax - kCoarseBits), kChunk), stream, seed, coarse_cap, coarse_count, coarse,
+               bits, cap, count, tmp, spill);
     if (e != cudaSuccess) return e;
-    k_bucket_fine<<<fine, kScatterThreads, smem, stream>>>(
-        seed, coarse_cap, coarse_count, coarse, bits, cap, count, tmp, spill);
   }
-  k_bucket_starts<<<1, 1024, 0, stream>>>(nb, count, start);
-  e = cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+  e = launch(k_bucket_starts, 1, 1024, 0, 0, stream, nb, count, start);
   if (e != cudaSuccess) return e;
-  k_bucket_sort<<<nb < num_sms * 4 ? nb : num_sms * 4, kSortThreads, sizeof(SortSmem), stream>>>(
-      seed, bits, nb, cap, start, tmp, order, spill, err);
-  return cudaGetLastError();
+  return launch(k_bucket_sort, nb < num_sms * 4 ? nb : num_sms * 4, kSortThreads, sizeof(SortSmem), sizeof(SortSmem),
+                stream, seed, bits, nb, cap, start, tmp, order, spill, err);
 }
 
 }  // namespace ccg
