@@ -262,6 +262,12 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     if (cudaGetDevice(&g->device) != cudaSuccess) { rc = CC_ERR_CUDA; break; }
     cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->device);
     cudaStream_t s = g->stream;
+    // first error of the launches and copies below that nothing else reports
+    // (their calls return, and so clear, the error of a refused launch); what the
+    // caller's own calls left behind is not this graph's
+    cudaGetLastError();
+    cudaError_t queued = cudaSuccess;
+    auto queue = [&](cudaError_t e) { if (queued == cudaSuccess) queued = e; };
     // nnz = off[n]
     int64_t nnz = 0;
     if (dev) {
@@ -287,8 +293,8 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
       if (i32) {
         int32_t* tmp = nullptr;
         if ((rc = from_cuda(dalloc(&tmp, 4 * (size_t)(n + 1), s))) != CC_OK) break;
-        cudaMemcpyAsync(tmp, row_offsets, 4 * (size_t)(n + 1), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
-        launch_offsets_i32_to_i64(n, tmp, g->off, s);
+        queue(cudaMemcpyAsync(tmp, row_offsets, 4 * (size_t)(n + 1), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        queue(launch_offsets_i32_to_i64(n, tmp, g->off, s));
         dfree(tmp, s);
       } else if ((rc = from_cuda(cudaMemcpyAsync(g->off, row_offsets, 8 * (size_t)(n + 1), cudaMemcpyHostToDevice, s))) != CC_OK) {
         break;
@@ -327,9 +333,10 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
     if ((rc = from_cuda(dalloc(&vws, validate_workspace_bytes(), s))) != CC_OK) break;
     int* vflags_dev = reinterpret_cast<int*>(static_cast<char*>(vws) + align_up(8 * sizeof(unsigned long long)));
     int vflags[2] = {0, 0};
-    launch_validate_offsets(n, nnz, g->off, vws, g->num_sms, s);
-    cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s);
-    if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) { dfree(vws, s); break; }
+    queue(launch_validate_offsets(n, nnz, g->off, vws, g->num_sms, s));
+    queue(cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s));
+    queue(cudaStreamSynchronize(s));
+    if ((rc = from_cuda(queued)) != CC_OK) { dfree(vws, s); break; }
     if (vflags[0] != 0) { dfree(vws, s); rc = CC_ERR_INVALID_GRAPH; break; }
     g->max_deg = vflags[1];
     // non-empty rows (for the edge-balanced passes over the whole CSR)
@@ -343,9 +350,10 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
       break;
     }
     int64_t* nz_dev = reinterpret_cast<int64_t*>(static_cast<char*>(nws) + nonempty_workspace_bytes(n) - 256);
-    launch_nonempty_rows(n, g->off, g->nz_row, g->nz_pos, up_at, nws, nz_dev, g->num_sms, s);
-    cudaMemcpyAsync(&g->nz_n, nz_dev, 8, cudaMemcpyDeviceToHost, s);
-    if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }
+    queue(launch_nonempty_rows(n, g->off, g->nz_row, g->nz_pos, up_at, nws, nz_dev, g->num_sms, s));
+    queue(cudaMemcpyAsync(&g->nz_n, nz_dev, 8, cudaMemcpyDeviceToHost, s));
+    queue(cudaStreamSynchronize(s));
+    if ((rc = from_cuda(queued)) != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }
     // the non-isolated vertices by degree (for the round kernel's Delta) and
     // the memory of the rows' upper parts (for the objective)
     {
@@ -367,23 +375,24 @@ int cc_graph_create(int64_t n, const void* row_offsets, const int32_t* col_idx, 
       if (rc != CC_OK) { dfree(vws, s); dfree(nws, s); dfree(up_at, s); break; }
     }
     for (int c = 0; c < chunks; ++c) {
-      if (g->col_ready[c]) cudaStreamWaitEvent(s, g->col_ready[c], 0);
-      launch_validate_edges(n, cut[c], cut[c + 1], c == chunks - 1, g->nz_row, g->nz_pos, g->nz_n, g->col, up_at, vws,
-                            g->num_sms, s);
+      if (g->col_ready[c]) queue(cudaStreamWaitEvent(s, g->col_ready[c], 0));
+      queue(launch_validate_edges(n, cut[c], cut[c + 1], c == chunks - 1, g->nz_row, g->nz_pos, g->nz_n, g->col, up_at,
+                                  vws, g->num_sms, s));
     }
     unsigned long long* up_dev = reinterpret_cast<unsigned long long*>(nz_dev);
     unsigned long long up_pack[2] = {0, 0};
-    launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_v, g->up_row, g->up_len, g->up_pos,
-                      g->up_epos, nws, up_dev, g->num_sms, s);
-    cudaMemcpyAsync(up_pack, up_dev, sizeof(up_pack), cudaMemcpyDeviceToHost, s);
+    queue(launch_upper_rows(g->nz_n, nnz, g->nz_row, g->nz_pos, up_at, g->up_v, g->up_row, g->up_len, g->up_pos,
+                            g->up_epos, nws, up_dev, g->num_sms, s));
+    queue(cudaMemcpyAsync(up_pack, up_dev, sizeof(up_pack), cudaMemcpyDeviceToHost, s));
     if (flags & CC_VALIDATE_EXACT)
-      launch_validate_reverse(nnz, g->off, g->nz_row, g->nz_pos, g->nz_n, g->col, vws, g->num_sms, s);
-    cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s);
+      queue(launch_validate_reverse(nnz, g->off, g->nz_row, g->nz_pos, g->nz_n, g->col, vws, g->num_sms, s));
+    queue(cudaMemcpyAsync(vflags, vflags_dev, sizeof(vflags), cudaMemcpyDeviceToHost, s));
     dfree(vws, s);
     dfree(nws, s);
     dfree(up_at, s);
-    if ((rc = from_cuda(cudaStreamSynchronize(s))) != CC_OK) break;
-    if ((rc = from_cuda(cudaGetLastError())) != CC_OK) break;
+    queue(cudaStreamSynchronize(s));
+    queue(cudaGetLastError());
+    if ((rc = from_cuda(queued)) != CC_OK) break;
     if (vflags[0] != 0) { rc = CC_ERR_INVALID_GRAPH; break; }
     g->up_n = (int64_t)(up_pack[0] >> 33);
     g->up_units = (int64_t)(up_pack[0] & ((1ull << 33) - 1));
