@@ -475,7 +475,7 @@ static int cluster_async(cc_graph* g, uint64_t seed, int32_t* labels_out, int32_
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[1], s));
   CC_TRY(launch_async_c4(b, g->async_grid, lab, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[2], s));
-  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), g->rows(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   if (labels_out && !dev) CC_TRY(cudaMemcpyAsync(labels_out, lab, 4 * (size_t)g->n, cudaMemcpyDeviceToHost, s));
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[3], s));
   CC_TRY(cudaMemcpyAsync(g->ctl_host, b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -571,10 +571,10 @@ int cc_cluster_ex(cc_graph* g, int algo, double eps, uint64_t seed, int32_t* lab
   const bool dev = is_device_ptr(labels_out);
   if (labels_out && !dev) {
     if ((rc = ensure_labels_tmp(g)) != CC_OK) return rc;
-    CC_TRY(launch_finalize_labels(b, g->labels_tmp, disagreements_out != nullptr, g->num_sms, s));
+    CC_TRY(launch_finalize_labels(b, g->rows(), g->labels_tmp, disagreements_out != nullptr, g->num_sms, s));
     CC_TRY(cudaMemcpyAsync(labels_out, g->labels_tmp, 4 * (size_t)g->n, cudaMemcpyDeviceToHost, s));
   } else {
-    CC_TRY(launch_finalize_labels(b, labels_out, disagreements_out != nullptr, g->num_sms, s));
+    CC_TRY(launch_finalize_labels(b, g->rows(), labels_out, disagreements_out != nullptr, g->num_sms, s));
   }
   if (g->timing) CC_TRY(cudaEventRecord(g->ev[3], s));
   CC_TRY(cudaMemcpyAsync(g->ctl_host, b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -655,7 +655,7 @@ int cc_disagreements(cc_graph* g, const int32_t* labels, int64_t* out) {
     CC_TRY(cudaMemcpyAsync(g->labels_tmp, labels, 4 * (size_t)g->n, cudaMemcpyHostToDevice, s));
     lab = g->labels_tmp;
   }
-  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
+  CC_TRY(launch_disagreements(g->n, g->col, g->upper(), g->rows(), lab, g->obj_ws, g->obj_out, g->num_sms, s));
   CC_TRY(cudaMemcpyAsync(g->obj_host, g->obj_out, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   CC_TRY(cudaStreamSynchronize(s));
   if (g->obj_host[2]) return CC_ERR_INVALID_ARG;

@@ -32,6 +32,7 @@ struct cc_graph {
   uint32_t* up_epos = nullptr;
   int64_t up_n = 0, up_units = 0, up_edges = 0;
   ccg::UpperRows upper() const { return ccg::UpperRows{up_v, up_row, up_len, up_pos, up_epos, up_n, up_units, up_edges}; }
+  ccg::FullRows rows() const { return ccg::FullRows{nz_row, nz_pos, nz_n, nnz}; }
   // cached workspaces (grown on demand)
   void* perm_ws = nullptr;
   size_t perm_ws_bytes = 0;

@@ -114,6 +114,14 @@ struct UpperRows {
   int64_t n, units, edges;
 };
 
+// The non-empty rows: vertex and first CSR entry of each (they lie one behind the
+// other).  The objective of graphs with short rows walks them.
+struct FullRows {
+  const int32_t* v;
+  const int64_t* pos;
+  int64_t n, nnz;
+};
+
 struct RoundBuffers {
   int64_t n, nnz;
   int32_t max_deg;
@@ -224,23 +232,24 @@ cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint
 // labels_out[v] = center vertex id (order[center rank]) when labels_out is
 // not null; with `objective` also the two terms of D: ctl->pairs = sum_c
 // C(s_c, 2) and ctl->intra = the number of edges inside clusters.
-cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, bool objective, int num_sms,
-                                   cudaStream_t stream);
+cudaError_t launch_finalize_labels(const RoundBuffers& b, const FullRows& all, int32_t* labels_out, bool objective,
+                                   int num_sms, cudaStream_t stream);
 
 // ---- objective and validation (cc_objective.cu) ------------------------------
 size_t objective_workspace_bytes(int64_t n);
 // out[0] = edges inside clusters, out[1] = sum_c C(s_c, 2), out[2] = 1 if a
 // label was outside [0, n).  out: 3 device words.
-cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows& up,
+cudaError_t launch_disagreements(int64_t n, const int32_t* col, const UpperRows& up, const FullRows& all,
                                  const int32_t* labels, void* ws, unsigned long long* out, int num_sms,
                                  cudaStream_t stream);
 // *out += the number of edges (u, w) with id[u] == id[w] in [lo, hi); `sig` (or null): a
 // 4-bit signature of id per vertex, eight to a word, that is equal when the
 // ids are.
-cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const uint32_t* id, const uint32_t* sig, uint32_t lo,
-                         uint32_t hi, unsigned long long* out, int num_sms, cudaStream_t stream);
-// Vertices above which the objective reads signatures before ids.
-bool intra_wants_signatures(int64_t n);
+cudaError_t launch_intra(const int32_t* col, const UpperRows& up, const FullRows& all, const uint32_t* id,
+                         const uint32_t* sig, uint32_t lo, uint32_t hi, unsigned long long* out, int num_sms,
+                         cudaStream_t stream);
+// Whether the objective of a graph of n vertices reads signatures before ids.
+bool intra_wants_signatures(int64_t n, const UpperRows& up);
 size_t validate_workspace_bytes();
 // Validation in two steps sharing ws (validate_workspace_bytes()): offsets
 // first (zeroes ws), then the entries over the non-empty rows.  The int pair

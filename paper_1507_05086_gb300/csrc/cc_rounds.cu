@@ -2700,16 +2700,16 @@ cudaError_t launch_rounds(const RoundBuffers& b, int algo, int64_t eps_ppm, uint
                                      stream);
 }
 
-cudaError_t launch_finalize_labels(const RoundBuffers& b, int32_t* labels_out, bool objective, int num_sms,
-                                   cudaStream_t stream) {
+cudaError_t launch_finalize_labels(const RoundBuffers& b, const FullRows& all, int32_t* labels_out, bool objective,
+                                   int num_sms, cudaStream_t stream) {
   if (b.n <= 0) return cudaSuccess;
   const int64_t want = (b.n + 255) / 256;
   const int grid = (int)(want < 2048 ? want : 2048);
-  const bool sig = intra_wants_signatures(b.n);
+  const bool sig = intra_wants_signatures(b.n, b.up);
   k_finalize_labels<<<grid, 256, 0, stream>>>(b, labels_out, objective, sig);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !objective) return e;
-  return launch_intra(b.col, b.up, b.st, sig ? b.rtag : nullptr, kLab, kAlive, &b.ctl->intra, num_sms, stream);
+  return launch_intra(b.col, b.up, all, b.st, sig ? b.rtag : nullptr, kLab, kAlive, &b.ctl->intra, num_sms, stream);
 }
 
 int batch_grid_size(int device) {
