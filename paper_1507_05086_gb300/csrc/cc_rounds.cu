@@ -89,6 +89,11 @@ constexpr int kHList = kThreads;             // heavy lists up to this long: eve
 constexpr int kHere = kScanU * kThreads;
 constexpr int kHRows = 1024;                 // rows that one block recounts at once
 constexpr int kHPick = 4096;                 // vertices that one block picks at once
+// Picked rows of more than kManyEdges entries together: about kFewEdges of them are
+// recounted first (300 cliques of 300, ClusterWild! at eps 0.05 / 0.01: 5.5 / 18.8 ms
+// without, 2.4 / 6.1 with; 16384: 2.3 / 5.8, 49152: 2.9 / 7.8.  Where no row can be
+// left out it costs: R-MAT 24 and 26 and batches of Chung-Lu graphs 0.5 %).
+constexpr int kManyEdges = 24576, kFewEdges = 2048;
 constexpr int kInlineEdges = 8192;           // recounts up to this many entries run inside the barrier
 constexpr int32_t kLongRow = 1024;           // rows above this are not recounted by one block alone
 constexpr int32_t kTightest = 8;             // heavy lists reach down to 1 - 2^-8 of the largest bound at most
@@ -855,15 +860,61 @@ struct K {
     return sc.tot;
   }
 
-  // Block-wide: recount of every picked vertex; the largest degree known to the
-  // block, and to the team so far, goes to S->h_best.
+  // Block-wide: the rows from `first` on of S->u.hl whose vertex has a bound above
+  // `known`, moved to the list's front; returns their entries, *items their number.
+  __device__ __noinline__ int64_t drop_known(int first, int items, int32_t known, int* kept) {
+    constexpr int kPer = kHRows / kThreads;
+    HeavyList& hl = S->u.hl;
+    int32_t v[kPer], len[kPer];
+    int64_t row[kPer], mine = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = first + threadIdx.x * kPer + q;
+      v[q] = i < items ? hl.v[i] : -1;
+      len[q] = v[q] >= 0 ? hl.len[i] : 0;
+      row[q] = v[q] >= 0 ? hl.row[i] : 0;
+      if (v[q] >= 0 && (int32_t)deg_of(ldcg(B.st + v[q])) <= known) v[q] = -1;
+      mine += v[q] >= 0 ? (int64_t(1) << kPackShift) | len[q] : 0;
+    }
+    const Scan sc = scan(mine);             // every row has been read by now
+    int64_t ex = sc.ex;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      if (v[q] < 0) continue;
+      const int j = (int)(ex >> kPackShift);
+      hl.pos[j] = ex & (int64_t)kPackEdgeMask;
+      hl.row[j] = row[q];
+      hl.len[j] = len[q];
+      hl.v[j] = v[q];
+      hl.cnt[j] = 0;
+      ex += (int64_t(1) << kPackShift) | len[q];
+    }
+    *kept = (int)(sc.tot >> kPackShift);
+    __syncthreads();
+    return sc.tot & (int64_t)kPackEdgeMask;
+  }
+
+  // Block-wide: recount of the picked vertices; the largest degree known to the
+  // block, and to the team so far, goes to S->h_best.  Of long lists of entries a few
+  // rows are recounted first: where degrees are equal and few of them fall in a round
+  // (cliques at small eps), no other vertex's bound is above what these have.
   __device__ __noinline__ void recount_picked() {
     const int n = S->h_picked;
     int32_t best = -1;
     int64_t edges = 0;
     for (int base = 0; base < n; base += kHRows) {
-      const int items = n - base < kHRows ? n - base : kHRows;
-      const int64_t E = prepare_rows(base, items, G > 1);
+      int items = n - base < kHRows ? n - base : kHRows;
+      int64_t E = prepare_rows(base, items, G > 1);
+      if (E > kManyEdges) {
+        const int few = (int)(items * (int64_t)kFewEdges / E) + 1;
+        if (few < items) {
+          const int64_t first = S->u.hl.pos[few];
+          const int32_t b = block_recount(few, first);
+          best = b > best ? b : best;
+          edges += first;
+          E = drop_known(few, items, best, &items);
+        }
+      }
       const int32_t b = block_recount(items, E);
       best = b > best ? b : best;
       edges += E;
