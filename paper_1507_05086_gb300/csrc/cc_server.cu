@@ -346,13 +346,18 @@ void dispatcher(cc_server* sv) {
   std::unique_lock<std::mutex> lk(sv->mu);
   std::vector<Request> batch;
   for (;;) {
-    // reap finished batches
-    for (auto& f : sv->fl) {
-      if (!f.busy) continue;
-      const cudaError_t q = cudaEventQuery(f.done);
-      if (q == cudaErrorNotReady) continue;
-      if (q != cudaSuccess) cudaGetLastError();
-      finish_batch(sv, f, q);
+    // reap finished batches (the flights are this thread's alone: the events are
+    // asked without the lock, which submit waits for)
+    lk.unlock();
+    cudaError_t ev[kStreams];
+    for (int i = 0; i < kStreams; ++i) {
+      ev[i] = sv->fl[i].busy ? cudaEventQuery(sv->fl[i].done) : cudaErrorNotReady;
+      if (ev[i] != cudaSuccess && ev[i] != cudaErrorNotReady) cudaGetLastError();
+    }
+    lk.lock();
+    for (int i = 0; i < kStreams; ++i) {
+      if (ev[i] == cudaErrorNotReady) continue;
+      finish_batch(sv, sv->fl[i], ev[i]);
       sv->cv_done.notify_all();
     }
     bool any_busy = false;
