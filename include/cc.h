@@ -324,7 +324,7 @@ int cc_server_destroy(cc_server* s);
  *                    0..8 (2)
  *   inline_heavy     exact Delta: heavy lists up to this long (and 2048) are
  *                    looked at inside the grid barrier by one block, 0..65536
- *                    (8192)
+ *                    (2048; more is the same)
  *   inline_decide    C4: blocked lists up to this long are decided inside the
  *                    barrier, 0..65536 (4096)
  *   inline_rebuild   Delta rebuild: degree-order segments up to this long are

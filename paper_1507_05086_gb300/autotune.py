@@ -2,8 +2,8 @@
 
 The settings cut the work differently (edge-walker chunks and prefetch
 depth, which heavy-list scans, Delta rebuild segments and C4 blocked sets
-run inside a grid barrier, the heavy-list threshold, and the size classes
-and team size of batched jobs); none changes a result.  This module picks
+run inside a grid barrier, the heavy-list threshold, and the largest team
+of batched jobs); none changes a result.  This module picks
 them by measurement, per device and per class of graph, and keeps the
 choices in a JSON cache so that a later process reuses them:
 
@@ -32,14 +32,13 @@ ROUND_KNOBS = {
     "walk_batches": (1, 2, 4, 8),
     "prefetch_ahead": (0, 1, 2, 4),
     "heavy_shift": (1, 2),
-    "inline_heavy": (2048, 8192, 32768),
+    "inline_heavy": (0, 512, 2048),
     "inline_rebuild": (2048, 8192, 32768),
     "inline_decide": (1024, 4096, 16384),
     "warp_resolve_row": (256, 1024, 4096),
 }
 BATCH_KNOBS = {
     "batch_team_blocks": (4, 8, 16),
-    "batch_small_n": (1 << 14, 1 << 15, 1 << 16, 1 << 17),
 }
 
 
@@ -165,10 +164,10 @@ def batch_class(graphs) -> str:
 
 def tune_batch(graphs, algo: str = "cw", eps: float = 0.5, k_perms: int = 2, cache: str | None = None,
                budget_s: float = 60.0, force: bool = False, knobs=None):
-    """Size classes and team size of batched jobs for a batch like `graphs`
-    (timed on those graphs, k_perms permutations each): from the cache, else
-    by coordinate descent.  Applies the choice process-wide
-    (cc_set_batch_tuning) and returns the cache entry."""
+    """Largest team of batched jobs for a batch like `graphs` (timed on those
+    graphs, k_perms permutations each): from the cache, else by coordinate
+    descent.  Applies the choice process-wide (cc_set_batch_tuning) and returns
+    the cache entry, of which only the knobs tuned here are taken."""
     import numpy as np
     import torch
     dev = device_key()
@@ -176,8 +175,9 @@ def tune_batch(graphs, algo: str = "cw", eps: float = 0.5, k_perms: int = 2, cac
     hit = None if force else lookup(cache, dev, "batch", cls)
     base = native.default_tuning().to_dict()
     if hit is not None:
-        native.set_batch_tuning(dict(base, **hit["tuning"]))
-        return dict(hit, source="cache", batch_class=cls, device=dev)
+        chosen = {k: v for k, v in hit["tuning"].items() if k in (knobs or BATCH_KNOBS)}
+        native.set_batch_tuning(dict(base, **chosen))
+        return dict(hit, tuning=chosen, source="cache", batch_class=cls, device=dev)
     seeds = np.arange(len(graphs), dtype=np.uint64) * 7 + 1
     ref = {}
 

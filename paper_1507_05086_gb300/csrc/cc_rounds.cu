@@ -98,7 +98,7 @@ constexpr int kInlineEdges = 8192;           // recounts up to this many entries
 constexpr int32_t kLongRow = 1024;           // rows above this are not recounted by one block alone
 constexpr int32_t kTightest = 8;             // heavy lists reach down to 1 - 2^-8 of the largest bound at most
 // Defaults of the run-time schedule settings (Tuning; cc_tuning in the C ABI)
-constexpr int32_t kInlineH = 8192;           // heavy lists up to this size are scanned by the coordinator
+constexpr int32_t kInlineH = kHere;          // heavy lists up to this size (and kHere) are looked at by the coordinator
 constexpr int32_t kInlineDecide = 4096;      // C4 blocked lists up to this size are decided by the coordinator
 constexpr int32_t kInlineRebuild = 8192;     // heavy-list rebuilds over prefixes up to this size run in the coordinator
 constexpr int32_t kHeavyShift = 1;           // heavy-list threshold tau = max(1, D >> kHeavyShift)
