@@ -1,6 +1,8 @@
 // cc_device.cuh -- device-side building blocks shared by the library's kernels:
-// the permutation hash, a grid barrier with a bounded wait, warp/block scans
-// and the edge-balanced list walker used by every adjacency pass.
+// the permutation hash, bounded waits, warp/block scans and the edge-balanced
+// walks over adjacency rows: row_walk (the round kernel, the objective above 2^24
+// vertices), unit_walk (the objective below) and lbs_for_each (validation, graphs
+// with short rows, C4 without rounds).
 #pragma once
 
 #include <cstdint>
@@ -287,8 +289,6 @@ __device__ __forceinline__ int64_t warp_upper_bound(const int64_t* a, int64_t n,
 // inside the batch, so a batch spanning a few rows costs one group, not
 // kLbsK (every item owns at least one edge, so kLbsK groups always suffice,
 // and the item after the batch's last one is always among those loaded).
-// With vmap, the per-item payload is vmap[vtx[j]] - vsub instead of vtx[j]
-// (one load per item, not per edge).
 //
 // With colp (the CSR column array; the walk's CSR position of virtual edge e
 // of item j is e + delta[j], or e without delta), the column ids of the
@@ -297,8 +297,7 @@ __device__ __forceinline__ int64_t warp_upper_bound(const int64_t* a, int64_t n,
 template <class F>
 __device__ __forceinline__ void lbs_chunk(const int64_t* epos, int64_t nitems, int64_t c0, int64_t cend, LbsWarp* ws,
                                           F& f, const int64_t* delta, const int32_t* vtx,
-                                          const uint32_t* vmap = nullptr, uint32_t vsub = 0,
-                                          const int32_t* colp = nullptr, int64_t E = 0, int pf_ahead = kLbsPfAhead) {
+                                          const int32_t* colp, int64_t E) {
   const int lane = threadIdx.x & 31;
   int64_t j0 = warp_upper_bound(epos, nitems, c0) - 1;
   // cached item (warp-uniform): valid when cur_j == j0
@@ -323,8 +322,8 @@ __device__ __forceinline__ void lbs_chunk(const int64_t* epos, int64_t nitems, i
         L.ri[t] = 0;
         if (base + lane + 32 * t < cend) L.valid |= 1u << t;
       }
-      if (colp && pf_ahead > 0 && lane < kLbsW / 32) {
-        const int64_t pe = base + (int64_t)pf_ahead * kLbsW + 32 * lane;
+      if (colp && kLbsPfAhead > 0 && lane < kLbsW / 32) {
+        const int64_t pe = base + (int64_t)kLbsPfAhead * kLbsW + 32 * lane;
         if (pe < cur_end && pe < E) prefetch_l2(colp + pe + cur_dlt);
       }
       f(L);
@@ -352,15 +351,6 @@ __device__ __forceinline__ void lbs_chunk(const int64_t* epos, int64_t nitems, i
     }
     if (lane == 0) ws->next = -1;
     __syncwarp();
-    if (vmap) {
-      // payload of the items that own edges of this batch, and of the one
-      // that starts the next batch (it may be kept for that batch)
-#pragma unroll
-      for (int t = 0; t < kLbsK; ++t) {
-        const int i = lane + 32 * t;
-        if (s[t] <= base + kLbsW) ws->vtx[i] = (int32_t)(ldcg(vmap + ws->vtx[i]) - vsub);
-      }
-    }
 #pragma unroll
     for (int t = 0; t < kLbsK; ++t) {
       const int i = lane + 32 * t;
@@ -423,7 +413,7 @@ __device__ __forceinline__ void lbs_chunk(const int64_t* epos, int64_t nitems, i
       cur_vtx = vtx ? ws->vtx[m] : 0;
       // the next batches of that item: start streaming them
       if (colp) {
-        for (int a = 1; a <= pf_ahead; ++a) {
+        for (int a = 1; a <= kLbsPfAhead; ++a) {
           const int64_t pe = base + (int64_t)a * kLbsW + 32 * lane;
           if (lane < kLbsW / 32 && pe >= cur_start && pe < cur_end && pe < E) prefetch_l2(colp + pe + cur_dlt);
         }
@@ -435,32 +425,21 @@ __device__ __forceinline__ void lbs_chunk(const int64_t* epos, int64_t nitems, i
   }
 }
 
-// gwarp / nwarps: this warp's index among, and the number of, the warps that
-// share the walk (the whole grid, or one team of blocks).  The walk covers
-// the virtual edges [E0, E); warp w takes chunks w, w + nwarps, ...
-template <class F>
-__device__ __forceinline__ void lbs_for_each_in(int64_t gwarp, int64_t nwarps, const int64_t* epos, int64_t nitems,
-                                                int64_t E, LbsWarp* ws, F&& f, const int64_t* delta = nullptr,
-                                                const int32_t* vtx = nullptr, int64_t E0 = 0,
-                                                const uint32_t* vmap = nullptr, uint32_t vsub = 0,
-                                                const int32_t* colp = nullptr, WalkShape shape = WalkShape{}) {
-  if (E <= E0) return;
-  // up to shape.batches batches per chunk, fewer when the list is short, so
-  // that short lists still spread over many warps
-  int64_t nb = (E - E0) / (nwarps * (int64_t)kLbsW * 2);
-  nb = nb < 1 ? 1 : (nb > shape.batches ? shape.batches : nb);
-  const int64_t kChunk = (int64_t)kLbsW * nb;
-  for (int64_t c0 = E0 + gwarp * kChunk; c0 < E; c0 += nwarps * kChunk)
-    lbs_chunk(epos, nitems, c0, c0 + kChunk < E ? c0 + kChunk : E, ws, f, delta, vtx, vmap, vsub, colp, E,
-              shape.pf_ahead);
-}
-
+// The walk covers the virtual edges [E0, E); warp w of the grid takes chunks w,
+// w + nwarps, ... of up to kLbsBatches batches, fewer when the list is short, so
+// that short lists still spread over many warps.
 template <class F>
 __device__ __forceinline__ void lbs_for_each(const int64_t* epos, int64_t nitems, int64_t E, LbsWarp* ws, F&& f,
                                              const int64_t* delta = nullptr, const int32_t* vtx = nullptr,
                                              int64_t E0 = 0, const int32_t* colp = nullptr) {
-  lbs_for_each_in(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((int64_t)gridDim.x * blockDim.x) >> 5,
-                  epos, nitems, E, ws, f, delta, vtx, E0, nullptr, 0, colp);
+  if (E <= E0) return;
+  const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int64_t nb = (E - E0) / (nwarps * (int64_t)kLbsW * 2);
+  nb = nb < 1 ? 1 : (nb > kLbsBatches ? kLbsBatches : nb);
+  const int64_t kChunk = (int64_t)kLbsW * nb;
+  for (int64_t c0 = E0 + gwarp * kChunk; c0 < E; c0 += nwarps * kChunk)
+    lbs_chunk(epos, nitems, c0, c0 + kChunk < E ? c0 + kChunk : E, ws, f, delta, vtx, colp, E);
 }
 
 // ---------------------------------------------------------------------------
@@ -480,7 +459,7 @@ __device__ __forceinline__ void lbs_for_each(const int64_t* epos, int64_t nitems
 //
 // at(j) = pos of item j; load(j) = the item's data, read once per window of
 // items; f(X) gets the batch: the column of this lane's entry of each unit
-// (-1: none) and, the same in all lanes, the unit's item and payload.  All 32
+// (-1: none) and, the same in all lanes, the unit's payload.  All 32
 // lanes call f together.
 // ---------------------------------------------------------------------------
 constexpr int kUnitB = 8;
@@ -496,8 +475,6 @@ struct UnitItem {
 struct UnitBatch {
   int32_t w[kUnitB];     // column of this lane's entry, -1 when there is none
   int32_t aux[kUnitB];   // payload of the unit's item
-  int32_t item[kUnitB];  // the unit's item relative to j0
-  int64_t j0;
 };
 
 // Number of items whose pos is <= x (pos ascending), by a 33-ary search of the warp.
@@ -530,14 +507,14 @@ __device__ __forceinline__ void unit_walk(int64_t gwarp, int64_t nwarps, int64_t
   for (int64_t c0 = gwarp * chunk; c0 < U; c0 += nwarps * chunk) {
     const int64_t cend = c0 + chunk < U ? c0 + chunk : U;
     UnitBatch X;
-    X.j0 = warp_count_upto(at, nitems, (uint32_t)c0) - 1;
+    int64_t j0 = warp_count_upto(at, nitems, (uint32_t)c0) - 1;
     UnitItem it;
     uint32_t wend = 0;                  // first unit after the window's items
     for (int64_t t = c0; t < cend; t += kUnitB) {
       const int64_t tend = t + kUnitB < cend ? t + kUnitB : cend;
       if (t == c0 || tend > (int64_t)wend) {
-        if (t != c0) X.j0 += __popc(__ballot_sync(FULL, it.pos <= (uint32_t)t)) - 1;
-        const int64_t j = X.j0 + lane;
+        if (t != c0) j0 += __popc(__ballot_sync(FULL, it.pos <= (uint32_t)t)) - 1;
+        const int64_t j = j0 + lane;
         it = UnitItem{0xFFFFFFFFu, 0, 0, 0};
         if (j < nitems) it = load(j);
         const uint32_t e = it.pos + (uint32_t)units_of(it.len);
@@ -552,7 +529,6 @@ __device__ __forceinline__ void unit_walk(int64_t gwarp, int64_t nwarps, int64_t
         const int32_t len = __shfl_sync(FULL, it.len, i);
         const int64_t row = __shfl_sync(FULL, it.row, i);
         X.aux[q] = __shfl_sync(FULL, it.aux, i);
-        X.item[q] = i;
         const int32_t k = (int32_t)((uint32_t)x - p) * 32 + lane;
         X.w[q] = x < cend && k < len ? __ldg(col + row + k) : -1;
         // lane q looks shape.pf_ahead batches ahead in the same row

@@ -193,7 +193,6 @@ static_assert(kPlanWords == 32, "one warp reads the plan");
 struct Coord {
   int64_t n, n_alive, cursor, al_len, k, round, stats_cap, eps_ppm;
   int64_t need, win_lo, win_len, r_edges, fix_iter;
-  int64_t clusters;              // centers opened so far
   int64_t h_len;                 // heavy list length
   int64_t nz_len;                // alive non-isolated vertices, as of the last look at all of them
   int32_t tau, delta, max_deg;
@@ -202,7 +201,6 @@ struct Coord {
   int32_t d_other;               // largest bound among the others
   int32_t tight;                 // the heavy list reaches down to ub - (ub >> tight)
   int32_t tau_next;              // the raised tau of a planned look
-  int32_t hv_sel;                // which of the two heavy-list buffers is current
   int32_t d_top, d_drop;         // largest bound at the first look; how far Delta fell below it lately
   int algo, rebuilds_in_row;
   int delta_zero;                // a rebuild found no alive vertex with an alive neighbour
@@ -481,10 +479,8 @@ struct K {
       c.delta_zero = 0;
       c.d_drop = 0;
       c.tight = 1;
-      c.hv_sel = 0;
       c.r_edges = 0;
       c.round = 0;
-      c.clusters = 0;
       c.rebuilds_in_row = 0;
       c.algo = vload(&C->algo);
       c.eps_ppm = vload(&C->eps_ppm);
@@ -1240,7 +1236,6 @@ struct K {
       c.r_edges = 0;
       if (centers_seen != centers) fail(kErrInternal);
       c.n_alive -= removed;
-      c.clusters += centers;
       if (c.n_alive < 0) fail(kErrInternal);
       c.round = r + 1;
       c.rebuilds_in_row = 0;
@@ -2249,47 +2244,44 @@ __device__ void run_job(K<kPerSM>& k, int algo) {
       }
       continue;
     }
-    {
-      {
-        if (S.plan.by_warp == 1) {
-          k.c4_resolve_by_warp();
-          k.flush_round_tallies();
-          if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
+    // kResolve: C4's blocked actives
+    if (S.plan.by_warp == 1) {
+      k.c4_resolve_by_warp();
+      k.flush_round_tallies();
+      if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
+    } else {
+      // the pull slots were set when the list was built; the hit flags are zero
+      auto after_decide = [&](long long left) {
+        if (threadIdx.x == 0) {
+          S.plan.undecided = left;
+          S.co.fix_iter += 1;
+          if (S.co.fix_iter > 1) S.co.r_edges += S.plan.b_E;
+          if (S.co.fix_iter > S.plan.b_n + 1) { k.fail(kErrInternal); S.plan.undecided = 0; }
+        }
+      };
+      while (S.plan.undecided > 0) {
+        k.c4_fix_scan();
+        if (S.plan.b_n <= k.B.tune.inline_decide) {
+          // a short blocked list: the coordinator decides inside the barrier
+          if (!k.sync(5, [&] {
+                const long long left = block_sum<int64_t>(k.c4_fix_decide(threadIdx.x, blockDim.x), S.scr);
+                after_decide(left);
+              }))
+            goto out;
         } else {
-          // the pull slots were set when the list was built; the hit flags are zero
-          auto after_decide = [&](long long left) {
-            if (threadIdx.x == 0) {
-              S.plan.undecided = left;
-              S.co.fix_iter += 1;
-              if (S.co.fix_iter > 1) S.co.r_edges += S.plan.b_E;
-              if (S.co.fix_iter > S.plan.b_n + 1) { k.fail(kErrInternal); S.plan.undecided = 0; }
-            }
-          };
-          while (S.plan.undecided > 0) {
-            k.c4_fix_scan();
-            if (S.plan.b_n <= k.B.tune.inline_decide) {
-              // a short blocked list: the coordinator decides inside the barrier
-              if (!k.sync(5, [&] {
-                    const long long left = block_sum<int64_t>(k.c4_fix_decide(threadIdx.x, blockDim.x), S.scr);
-                    after_decide(left);
-                  }))
-                goto out;
-            } else {
-              if (!k.sync(5, [&] { if (threadIdx.x == 0) C->undecided = 0; })) goto out;
-              const long long left = block_sum<int64_t>(
-                  k.c4_fix_decide((int64_t)k.bid * blockDim.x + threadIdx.x, (int64_t)k.G * blockDim.x), S.scr);
-              if (threadIdx.x == 0 && left)
-                atomicAdd(reinterpret_cast<unsigned long long*>(&C->undecided), (unsigned long long)left);
-              if (!k.sync(5, [&] { after_decide((long long)vload(&C->undecided)); })) goto out;
-            }
-          }
-          k.c4_blocked_attach();
-          if (!k.sync(5)) goto out;
-          k.c4_pull_finalize();
-          k.flush_round_tallies();
-          if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
+          if (!k.sync(5, [&] { if (threadIdx.x == 0) C->undecided = 0; })) goto out;
+          const long long left = block_sum<int64_t>(
+              k.c4_fix_decide((int64_t)k.bid * blockDim.x + threadIdx.x, (int64_t)k.G * blockDim.x), S.scr);
+          if (threadIdx.x == 0 && left)
+            atomicAdd(reinterpret_cast<unsigned long long*>(&C->undecided), (unsigned long long)left);
+          if (!k.sync(5, [&] { after_decide((long long)vload(&C->undecided)); })) goto out;
         }
       }
+      k.c4_blocked_attach();
+      if (!k.sync(5)) goto out;
+      k.c4_pull_finalize();
+      k.flush_round_tallies();
+      if (!k.sync(5, [&] { k.co_end_round(); })) goto out;
     }
   }
 out:
@@ -2581,7 +2573,7 @@ k_batch(BatchJob* __restrict__ jobs, const RoundBuffers* __restrict__ slots, con
         }))
       break;
     if (!team_permutation(k, jobs[j].seed, algo == kAlgoC4 || algo == kAlgoC4 + 2)) break;
-      if (threadIdx.x < kTallies) S.tal[threadIdx.x] = 0;
+    if (threadIdx.x < kTallies) S.tal[threadIdx.x] = 0;
     __syncthreads();
     run_job(k, algo);
     if (S.plan.state == kAbort) {
