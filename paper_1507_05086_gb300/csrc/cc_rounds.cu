@@ -1408,11 +1408,13 @@ struct K {
     if (t == 0) return true;
     return t == (uint32_t)P().tag && ldcg(B.st + v) >= kLab + (uint32_t)P().th;
   }
+  // (pi is read at L2: a batched job writes it in the same kernel, over the order of
+  // the job before it)
   template <int kU>
   __device__ __forceinline__ void sel_vertices(SelTile<kU>& T, int64_t base, int64_t e) const {
     T.first = base + (int64_t)threadIdx.x * kU;
 #pragma unroll
-    for (int q = 0; q < kU; ++q) T.v[q] = T.first + q < e ? __ldg(B.order + T.first + q) : -1;
+    for (int q = 0; q < kU; ++q) T.v[q] = T.first + q < e ? ldcg(B.order + T.first + q) : -1;
 #pragma unroll
     for (int q = 0; q < kU; ++q)
       if (T.v[q] >= 0 && !was_alive(T.v[q])) T.v[q] = -1;
@@ -1603,7 +1605,7 @@ struct K {
 #pragma unroll
       for (int q = 0; q < 2 * kSelU; ++q) {
         const int64_t i = b + (int64_t)q * blockDim.x + threadIdx.x;
-        v[q] = i < e ? __ldg(B.order + i) : -1;
+        v[q] = i < e ? ldcg(B.order + i) : -1;
       }
 #pragma unroll
       for (int q = 0; q < 2 * kSelU; ++q) cnt += v[q] >= 0 && was_alive(v[q]) ? 1 : 0;
