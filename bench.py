@@ -157,13 +157,13 @@ def measured_hbm_peak():
 # DRAM traffic of the round kernel per algorithmic byte, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum, a one-pass metric set, of the
 # four k_rounds launches of `bench.py --steps 1 --warmup 1` on the
-# default workload, R-MAT scale 26, eps 0.5: ClusterWild! 30.40 and 30.35 GB against
-# 7.17 GB algorithmic, C4 35.95 and 37.01 GB against 8.91 GB), keyed by a digest of the
+# default workload, R-MAT scale 26, eps 0.5: ClusterWild! 31.23 and 30.85 GB against
+# 7.17 GB algorithmic, C4 36.63 and 38.29 GB against 8.91 GB), keyed by a digest of the
 # kernel's code (comments and blank lines left out): a changed kernel reports
 # traffic null until it is captured again.
 ROUNDS_SOURCES = ("paper_1507_05086_gb300/csrc/cc_rounds.cu", "paper_1507_05086_gb300/csrc/cc_device.cuh",
                   "paper_1507_05086_gb300/csrc/cc_internal.h")
-ROUNDS_TRAFFIC_PER_BYTE = {"8fe2bf2f2fe41bd9": (30.40e9 + 35.95e9 + 30.35e9 + 37.01e9) / (2 * (7.17e9 + 8.91e9))}
+ROUNDS_TRAFFIC_PER_BYTE = {"ff3d783a48521c86": (31.23e9 + 36.63e9 + 30.85e9 + 38.29e9) / (2 * (7.17e9 + 8.91e9))}
 
 
 def rounds_sources_digest() -> str:

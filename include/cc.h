@@ -200,9 +200,9 @@ int cc_batch_run(cc_graph* const* gs, int32_t count, int algo, double eps,
 /*
  * cc_batch_jobs -- the jobs of cc_batch_run without the best-of-k reduction:
  * D_out[i * k_perms + j] and rounds_out[i * k_perms + j] (host arrays, either
- * may be NULL) for graph i under seed seeds[i] + j.  Small graphs run one per
- * thread block, medium graphs one per team of blocks, all in one launch per
- * size class; graphs above 2^21 vertices run on the whole GPU one at a time.
+ * may be NULL) for graph i under seed seeds[i] + j.  Jobs run on teams of one to
+ * batch_team_blocks thread blocks, by their sizes and their number, all in one
+ * launch; graphs above 2^21 vertices run on the whole GPU one at a time.
  * All graphs must live on the same device.
  */
 int cc_batch_jobs(cc_graph* const* gs, int32_t count, int algo, double eps,

@@ -49,8 +49,8 @@ __global__ void k_sizes_pairs(int64_t n, const int32_t* __restrict__ labels, int
 }
 
 // Edges (u, w) with id[u] == id[w] in [lo, hi), every edge read from its lower
-// end only (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 23
-// (130M edges, 0.49 ms, 265e9 edges/s) L2 runs at 65 % and L1 at 70 % of their
+// end only (half of the CSR's entries).  Bound by the random id reads in L2: at R-MAT 24
+// (260M edges, 1.04 ms, 250e9 edges/s) L2 runs at 66 % and L1 at 69 % of their
 // throughput, above the 236e9 reads/s of a library gather from a 32 MiB table.
 // With sig, a 4-bit signature per vertex decides first, so that ids are read
 // only where the signatures agree.  Whole objective of a ClusterWild! labelling
